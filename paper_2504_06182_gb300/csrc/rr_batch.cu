@@ -76,31 +76,35 @@ __global__ void k_classify(rr_instance *inst, int count, int nclass, int max_sid
     s_classify(hw_blk(), inst, count, nclass, max_side, classCount, classList);
 }
 
-// 16-bit slot links (sides up to 256) and 32-bit ones; narrow (shared-memory
-// slots only) and wide (overflow slots in global memory, for the instances
-// the narrow pass handed over).
-__global__ void k_sim16(rr_instance *inst, JobWS *wsv, int count, const int *classList, const int *classCount,
-                        int slotCap, int lineCap)
+// The simulation: one block per instance (of a size class's list, or of the
+// whole call).
+template <int MODE>
+__device__ __forceinline__ void sim_of_block(rr_instance *inst, JobWS *wsv, int count, const int *classList,
+                                             const int *classCount, int side, int counters)
 {
-    sim_body<int16_t, false>(hw_blk(), inst, wsv, count, classList, classCount, slotCap, lineCap);
+    extern __shared__ int4 sim_smem[];
+    int q = blockIdx.x;
+    if (classList) {
+        if (q >= *classCount) return;
+        q = classList[q];
+    }
+    if (q >= count) return;
+    sim_block<MODE>(&inst[q], wsv[q], (char *)sim_smem, side, counters);
 }
 
-__global__ void k_sim32(rr_instance *inst, JobWS *wsv, int count, const int *classList, const int *classCount,
-                        int slotCap, int lineCap)
+// sides up to 256
+__global__ void __launch_bounds__(SIM_MAX_THREADS, 6) k_sim(rr_instance *inst, JobWS *wsv, int count,
+                                                            const int *classList, const int *classCount, int side,
+                                                            int counters)
 {
-    sim_body<int32_t, false>(hw_blk(), inst, wsv, count, classList, classCount, slotCap, lineCap);
+    sim_of_block<SIM_SMALL>(inst, wsv, count, classList, classCount, side, counters);
 }
 
-__global__ void k_sim16w(rr_instance *inst, JobWS *wsv, int count, const int *classList, const int *classCount,
-                         int slotCap, int lineCap)
+__global__ void __launch_bounds__(SIM_MAX_THREADS, 4) k_sim_big(rr_instance *inst, JobWS *wsv, int count,
+                                                                const int *classList, const int *classCount, int side,
+                                                                int counters)
 {
-    sim_body<int16_t, true>(hw_blk(), inst, wsv, count, classList, classCount, slotCap, lineCap);
-}
-
-__global__ void k_sim32w(rr_instance *inst, JobWS *wsv, int count, const int *classList, const int *classCount,
-                         int slotCap, int lineCap)
-{
-    sim_body<int32_t, true>(hw_blk(), inst, wsv, count, classList, classCount, slotCap, lineCap);
+    sim_of_block<SIM_BIG>(inst, wsv, count, classList, classCount, side, counters);
 }
 
 int guard_cap_batch(long long cap)

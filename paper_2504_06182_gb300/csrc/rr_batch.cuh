@@ -8,20 +8,9 @@
 // list of paths through it in id order, and from it the de-duplicated
 // successor lists and in-degrees.
 //
-// Alg. 4 itself runs as an event-driven simulation, one warp per instance.
-// The lowest-id unfinished move is always ready (nothing earlier is
-// unfinished), so it is always the first member ("leader") of the batch. With
-// the leader's token at (r, c) moving in direction d, the other members are
-// the ready moves stepping in direction d whose tokens lie on row r (set A)
-// or on column c (set B): the one of A and B holding the smaller id wins,
-// because pairwise row-or-column sharing with three or more tokens forces
-// them onto one line. While the members advance together the batch can only
-// change when a member turns or finishes, or when the leader's row (vertical
-// d) or column (horizontal d) reaches a waiting ready move of direction d.
-// Between such events every batch is the same, so runs of identical batches
-// are written in one go.
-#include <type_traits>
+// Alg. 4 itself runs as an event-driven simulation (below).
 #pragma once
+#include <type_traits>
 #include "rr_internal.cuh"
 
 namespace rrk {
@@ -94,13 +83,16 @@ __device__ inline void s_bsetup(const Blk B, rr_instance *inst, JobWS *wsv, int 
             ws.rowCur = (int32_t *)arena_alloc(A, 4ull * (m + 1), &ok);
             ws.rowList = (int32_t *)arena_alloc(A, 4ull * (k + 1), &ok);
             ws.firstH = (int32_t *)arena_alloc(A, 4ull * cells, &ok);
-            ws.succCnt = (int32_t *)arena_alloc(A, 4ull * (k + 1), &ok);
+            ws.multiPos = (uint32_t *)arena_alloc(A, 4ull * (k + 1), &ok);
             ws.indeg = (int32_t *)arena_alloc(A, 4ull * (k + 1), &ok);
             ws.rec = (int4 *)arena_alloc(A, 32ull * (k + 1), &ok);
             ws.succ4 = ws.rec + 1;
             ws.ready0 = (int32_t *)arena_alloc(A, 4ull * (k + 1) + 16, &ok);
-            ws.slotOvf = arena_alloc(A, 40ull * (k + 1), &ok);
-            ws.ovfFree = (int32_t *)arena_alloc(A, 4ull * (k + 1), &ok);
+            ws.slotOvf = arena_alloc(A, sim_wide_bytes(k), &ok);
+            ws.multiNo = (int32_t *)arena_alloc(A, 4ull * (k + 1), &ok);
+            ws.multi = ws.colList;               // both lists are free again once they have been swept
+            ws.multiId = ws.rowList;
+            ws.nmulti = 0;
             ws.nextAt = nullptr;
             ws.succ = nullptr;
             ws.lbStatus = (unsigned long long *)arena_alloc(A, 8ull * ((k + LB_TILE - 1) / LB_TILE), &ok);
@@ -156,13 +148,16 @@ __device__ inline void s_bsetup(const Blk B, rr_instance *inst, JobWS *wsv, int 
             ws.rowCur = (int32_t *)arena_alloc(A, 4ull * (m + 1), &ok);
             ws.rowList = (int32_t *)arena_alloc(A, 4ull * (k + 1), &ok);
             ws.firstH = (int32_t *)arena_alloc(A, 4ull * cells, &ok);
-            ws.succCnt = (int32_t *)arena_alloc(A, 4ull * (k + 1), &ok);
+            ws.multiPos = (uint32_t *)arena_alloc(A, 4ull * (k + 1), &ok);
             ws.indeg = (int32_t *)arena_alloc(A, 4ull * (k + 1), &ok);
             ws.rec = (int4 *)arena_alloc(A, 32ull * (k + 1), &ok);   // record, successors: one 32 B sector
             ws.succ4 = ws.rec + 1;
             ws.ready0 = (int32_t *)arena_alloc(A, 4ull * (k + 1) + 16, &ok);
-            ws.slotOvf = arena_alloc(A, 40ull * (k + 1), &ok);
-            ws.ovfFree = (int32_t *)arena_alloc(A, 4ull * (k + 1), &ok);
+            ws.slotOvf = arena_alloc(A, sim_wide_bytes(k), &ok);
+            ws.multiNo = (int32_t *)arena_alloc(A, 4ull * (k + 1), &ok);
+            ws.multi = ws.colList;               // both lists are free again once they have been swept
+            ws.multiId = ws.rowList;
+            ws.nmulti = 0;
             // a path has at most as many distinct successors as vertices: they
             // are stored at the path's vertex offset, so no count pass or scan
             ws.succ = (int32_t *)arena_alloc(A, 4ull * (tp + 1), &ok);
@@ -334,6 +329,64 @@ __device__ inline void s_pairoff_lookback(const Blk B, rr_instance *inst, JobWS 
     }
 }
 
+constexpr int INTMAX = 0x7fffffff;
+
+// Sort a[0..n) of int32 ascending with one warp: in registers up to 32, else
+// by a bitonic network whose comparators all point up (each merge begins with
+// a mirrored step), so that no padding is needed: in buf (cap words) when the
+// list fits there, else in place.
+__device__ inline void warp_sort32(int32_t *a, int n, int32_t *buf, int cap)
+{
+    const int lane = threadIdx.x & 31;
+    if (n <= 1) return;
+    if (n <= 32) {
+        int v = lane < n ? a[lane] : 0x7fffffff;
+#pragma unroll
+        for (int kk = 2; kk <= 32; kk <<= 1) {
+#pragma unroll
+            for (int jj = kk >> 1; jj > 0; jj >>= 1) {
+                const int o = __shfl_xor_sync(FULL, v, jj);
+                const bool up = (lane & kk) == 0, low = (lane & jj) == 0;
+                v = (low == up) ? min(v, o) : max(v, o);
+            }
+        }
+        if (lane < n) a[lane] = v;
+        __syncwarp();
+        return;
+    }
+    int32_t *t = n <= cap ? buf : a;
+    if (t != a)
+        for (int i = lane; i < n; i += 32) t[i] = a[i];
+    __syncwarp();
+    auto order = [&](int i, int j) {
+        if (j > i && j < n) {
+            const int x = t[i], y = t[j];
+            if (x > y) { t[i] = y; t[j] = x; }
+        }
+    };
+    for (int k = 2; (k >> 1) < n; k <<= 1) {
+        for (int i = lane; i < n; i += 32) order(i, i ^ (k - 1));
+        __syncwarp();
+        for (int j = k >> 2; j > 0; j >>= 1) {
+            for (int i = lane; i < n; i += 32) order(i, i ^ j);
+            __syncwarp();
+        }
+    }
+    if (t != a)
+        for (int i = lane; i < n; i += 32) a[i] = t[i];
+    __syncwarp();
+}
+
+// A pointer loaded from memory, known to be global: loads and stores through
+// it need not tell shared memory apart.
+template <class T> __device__ __forceinline__ T *as_global(T *p)
+{
+#ifdef __CUDA_ARCH__
+    __builtin_assume(__isGlobal(p));
+#endif
+    return p;
+}
+
 // ---------------------------------------------------------------- Gamma
 // Vertex (r, c) is covered by the vertical parts of the moves ending in
 // column c (the corner of an L-move included) and by the horizontal parts of
@@ -400,48 +453,10 @@ __device__ inline void s_gfill(const Blk B, rr_instance *inst, JobWS *wsv, int c
     }
 }
 
-// Sort a[0..n) of int32 ascending with one warp (registers up to 32, else a
-// shared-memory bitonic network over buf, sized for the next power of two).
-__device__ inline void warp_sort32(int32_t *a, int n, int32_t *buf)
-{
-    const int lane = threadIdx.x & 31;
-    if (n <= 1) return;
-    if (n <= 32) {
-        int v = lane < n ? a[lane] : 0x7fffffff;
-#pragma unroll
-        for (int kk = 2; kk <= 32; kk <<= 1) {
-#pragma unroll
-            for (int jj = kk >> 1; jj > 0; jj >>= 1) {
-                const int o = __shfl_xor_sync(FULL, v, jj);
-                const bool up = (lane & kk) == 0, low = (lane & jj) == 0;
-                v = (low == up) ? min(v, o) : max(v, o);
-            }
-        }
-        if (lane < n) a[lane] = v;
-        __syncwarp();
-        return;
-    }
-    int P = 1;
-    while (P < n) P <<= 1;
-    for (int i = lane; i < P; i += 32) buf[i] = i < n ? a[i] : 0x7fffffff;
-    __syncwarp();
-    for (int k = 2; k <= P; k <<= 1)
-        for (int j = k >> 1; j > 0; j >>= 1) {
-            for (int i = lane; i < P; i += 32) {
-                const int ij = i ^ j;
-                if (ij > i) {
-                    const int x = buf[i], y = buf[ij];
-                    if ((x > y) == ((i & k) == 0)) { buf[i] = y; buf[ij] = x; }
-                }
-            }
-            __syncwarp();
-        }
-    for (int i = lane; i < n; i += 32) a[i] = buf[i];
-    __syncwarp();
-}
-
 // Order every column list and row list by id (one warp per list). Lists of
-// red-rec plans are mostly ascending already.
+// red-rec plans are mostly ascending already, and hold no more moves than
+// the line has traps; a longer list (any move list may be batched) does not
+// fit the buffer and is sorted in place.
 __device__ inline void s_gsort(const Blk B, rr_instance *inst, JobWS *wsv, int count, int bufLen)
 {
     extern __shared__ int32_t sortbuf[];
@@ -461,7 +476,7 @@ __device__ inline void s_gsort(const Blk B, rr_instance *inst, JobWS *wsv, int c
         bool sorted = true;
         for (int i = lane; i + 1 < len; i += 32) sorted &= a[i] < a[i + 1];
         if (__all_sync(FULL, sorted)) continue;
-        warp_sort32(a, len, buf);
+        warp_sort32(a, len, buf, bufLen);
     }
 }
 
@@ -579,7 +594,7 @@ __device__ inline void s_gsweep_v(const Blk B, rr_instance *inst, JobWS *wsv, in
 // four successors (registers) and then against the rest already written
 // (read back from out, which only this thread writes). The path's entries
 // are read 16 bytes at a time once aligned.
-__device__ inline int distinct_succ(const int32_t *seq, int len, int32_t *out, int32_t *indeg)
+__device__ inline int distinct_succ(const int32_t *seq, int len, int32_t *out, JobWS &ws)
 {
     int cnt = 0;
     int32_t last = -1, b0 = -1, b1 = -1, b2 = -1, b3 = -1;
@@ -591,7 +606,11 @@ __device__ inline int distinct_succ(const int32_t *seq, int len, int32_t *out, i
             if (out[u] == v) return;
         if (cnt == 0) b0 = v; else if (cnt == 1) b1 = v; else if (cnt == 2) b2 = v; else if (cnt == 3) b3 = v;
         out[cnt++] = v;
-        atomicAdd(&indeg[v], 1);
+        if (atomicAdd(&ws.indeg[v], 1) == 1) {    // a second predecessor: it needs a counter
+            const int x = atomicAdd(&ws.nmulti, 1);
+            ws.multiId[x] = v;
+            ws.multiNo[v] = x;
+        }
     };
     int t = 0;
     const int head = min(len, (int)((4u - (unsigned)(((uintptr_t)seq >> 2) & 3u)) & 3u));
@@ -605,7 +624,8 @@ __device__ inline int distinct_succ(const int32_t *seq, int len, int32_t *out, i
 }
 
 // Distinct successors of every path, written at the path's vertex offset,
-// their count, and the in-degree of every successor.
+// their count, the in-degree of every successor, and a number for every move
+// with several predecessors.
 __device__ inline void s_bsucc(const Blk B, rr_instance *inst, JobWS *wsv, int count)
 {
     const int q = B.y;
@@ -616,14 +636,15 @@ __device__ inline void s_bsucc(const Blk B, rr_instance *inst, JobWS *wsv, int c
     const int64_t k = I->n_moves;
     for (int64_t b = B.x * blockDim.x + threadIdx.x; b < k; b += (int64_t)B.gx * blockDim.x) {
         const int lo = ws.pairOff[b], hi = ws.pairOff[b + 1];
-        ws.succCnt[b] = distinct_succ(ws.nextAt + lo, hi - lo, ws.succ + lo, ws.indeg);
+        ws.rec[2 * b].z = distinct_succ(ws.nextAt + lo, hi - lo, ws.succ + lo, ws);   // until the records are made
     }
 }
 
-// Per-move records for the simulation: packed geometry, successor count and
-// the first four successors (flagged when the successor has no other
-// predecessor); later successors are flagged in place. Moves without
-// predecessors are listed as initially ready.
+// Per-move records for the simulation: geometry, successor count and the
+// first four successors (the flagged id of a successor without other
+// predecessors, else the number of its counter); later successors are
+// replaced in place. The in-degrees of the numbered moves start the
+// simulation's counters; moves without predecessors are listed as ready.
 __device__ inline void s_brec(const Blk B, rr_instance *inst, JobWS *wsv, int count)
 {
     const int q = B.y;
@@ -634,496 +655,24 @@ __device__ inline void s_brec(const Blk B, rr_instance *inst, JobWS *wsv, int co
     const int64_t k = I->n_moves;
     for (int64_t b = B.x * blockDim.x + threadIdx.x; b < k; b += (int64_t)B.gx * blockDim.x) {
         const rr_move p = I->moves[b];
-        const int lo = ws.pairOff[b], hi = lo + ws.succCnt[b];
-        int4 r;
-        r.x = (p.src_row & 0xffff) | (p.src_col << 16);
-        r.y = (p.dst_row & 0xffff) | (p.dst_col << 16);
-        r.z = hi - lo;
-        r.w = lo + 4;
+        const int lo = ws.pairOff[b], hi = lo + ws.rec[2 * b].z;
         int v[4] = {-1, -1, -1, -1};
         for (int e = lo; e < hi; ++e) {
             const int32_t sId = ws.succ[e];
-            const int32_t f = sId | (ws.indeg[sId] == 1 ? SUCC_SINGLE : 0);
+            const int32_t f = ws.indeg[sId] == 1 ? sId | SUCC_SINGLE : ws.multiNo[sId];
             if (e - lo < 4) v[e - lo] = f; else ws.succ[e] = f;
         }
+        const int4 r = move_rec(p, hi - lo, lo + 4, hi - lo == 1 && v[0] == (int)(SUCC_SINGLE | (b + 1)));
         ws.rec[2 * b] = r;
         ws.rec[2 * b + 1] = make_int4(v[0], v[1], v[2], v[3]);
-        if (ws.indeg[b] == 0) ws.ready0[atomicAdd(&ws.ready0[k], 1)] = (int32_t)b;
-    }
-}
-
-// ---------------------------------------------------------- simulation
-//
-// The ready moves other than the leader live in a slot table (structure of
-// arrays; shared memory up to its capacity, then a global overflow area with
-// the same layout); the leader is held in registers (LeaderState).
-// The moves of the current batch other than the leader ("members") are kept
-// in a persistent array sorted by id; every other ready move ("static") is
-// linked into two lists, one per (direction, row) and one per (direction,
-// column), and flagged in per-direction bitmaps of non-empty rows (vertical
-// directions) or columns (horizontal ones) for pickup detection.
-//
-// Members always share one line (a row or a column) and one direction. At a
-// segment boundary the candidates of the leader's row are the statics of that
-// row list plus the members if they form that row (likewise for its column);
-// so a segment walks two lists, usually short, and merges the newcomers. The
-// batch is dissolved back into the lists only when the leader's line or
-// direction no longer matches the members'.
-
-constexpr int KEY_LIVE = 1 << 22;
-constexpr int KEY_MEM = 1 << 23;
-constexpr int INTMAX = 0x7fffffff;
-
-template <typename IX> struct SlotSoA {
-    int32_t *key;     // row | col << 10 | dir << 20 | KEY_LIVE [| KEY_MEM]; 0 when free
-    int32_t *id;      // move id, INT_MAX when free
-    int16_t *t;       // elementary steps done (paths are shorter than 2 048 steps)
-    int16_t *legEnd;  // t at the end of the current straight leg
-    int16_t *dstRow;  // destination row: where the last (vertical) leg ends
-    IX *rp, *rn, *cp, *cn;        // static-list links (slot indices, -1)
-    // a move's successors are read from its record when it finishes: only
-    // the leader and the members ever finish
-};
-
-// The narrow simulation (WIDE false) keeps every slot in shared memory and
-// gives up on an instance that needs more (it is retried by the wide one);
-// the wide simulation spills slots beyond the shared capacity C to a global
-// overflow area. Peak demand on red-rec plans is two ready moves per column
-// (one chain head per vertical direction), within the shared capacity.
-template <typename IX, bool WIDE> struct Sim {
-    using ix = IX;
-    static constexpr bool wide = WIDE;
-    SlotSoA<IX> sm, gm;
-    int C, m, n, Wm, Wn;
-    int16_t *freeStk;
-    int32_t *map;
-    IX *rowHead, *colHead;          // [4][m], [4][n] static lists
-    int32_t *ovfFree;               // recycled overflow slots (global)
-    uint32_t *rowBits, *colBits;    // [2][Wm] (dirs 0, 1), [2][Wn] (dirs 2, 3)
-    int32_t *Mid, *Msl;             // members sorted by id
-    long long *Kb;                  // sort / merge buffer
-    int32_t *sbuf;
-};
-
-// A slot field: shared memory below the capacity C, the global overflow area
-// above it. Loads and stores branch on the index (rather than selecting a
-// pointer) so that the common shared-memory case stays a shared access.
-template <typename T> struct SlotRef {
-    T *s, *g;
-    int i, C;
-    __device__ __forceinline__ operator T() const { return i < C ? s[i] : g[i - C]; }
-    __device__ __forceinline__ SlotRef &operator=(T v)
-    {
-        if (i < C) s[i] = v; else g[i - C] = v;
-        return *this;
-    }
-};
-template <bool WIDE, typename T> struct SlotAt {
-    static __device__ __forceinline__ T &at(T *s, T *, int i, int) { return s[i]; }
-};
-template <typename T> struct SlotAt<true, T> {
-    static __device__ __forceinline__ SlotRef<T> at(T *s, T *g, int i, int C) { return SlotRef<T>{s, g, i, C}; }
-};
-#define SLOTF(X, f, i)                                                                         \
-    (SlotAt<std::decay_t<decltype(X)>::wide, std::remove_reference_t<decltype(*(X).sm.f)>>::at( \
-        (X).sm.f, (X).gm.f, (int)(i), (X).C))
-
-__device__ __forceinline__ int key_of(int r, int c, int d) { return r | (c << 10) | (d << 20) | KEY_LIVE; }
-__device__ __forceinline__ int key_r(int k) { return k & 1023; }
-__device__ __forceinline__ int key_c(int k) { return (k >> 10) & 1023; }
-__device__ __forceinline__ int key_d(int k) { return (k >> 20) & 3; }
-
-// a % b for 0 <= a <= 32 < 2^24 and b >= 1: a float quotient, corrected
-// by one either way (exact: the error of the product is far below 1)
-__device__ __forceinline__ int small_mod(int a, int b)
-{
-    const int q = __float2int_rz((float)a * __frcp_rn((float)b));
-    int r = a - q * b;
-    if (r < 0) r += b;
-    if (r >= b) r -= b;
-    return r;
-}
-
-template <class S>
-__device__ __forceinline__ void bits_set(const S &X, int d, int r, int c)
-{
-    using IX = typename S::ix;
-    if (d < 2) atomicOr(&X.rowBits[d * X.Wm + (r >> 5)], 1u << (r & 31));
-    else atomicOr(&X.colBits[(d - 2) * X.Wn + (c >> 5)], 1u << (c & 31));
-}
-
-// Static-list maintenance. push/remove touch the row list and the column
-// list of the slot's current key; callers that run them on several lanes at
-// once must guarantee distinct lists (see dissolve()).
-template <class S>
-__device__ void push_row(const S &X, int si, int key)
-{
-    using IX = typename S::ix;
-    IX *h = &X.rowHead[key_d(key) * X.m + key_r(key)];
-    SLOTF(X, rp, si) = (IX)-1; SLOTF(X, rn, si) = *h;
-    if (*h >= 0) SLOTF(X, rp, *h) = (IX)si;
-    *h = (IX)si;
-    if (key_d(key) < 2) atomicOr(&X.rowBits[key_d(key) * X.Wm + (key_r(key) >> 5)], 1u << (key_r(key) & 31));
-}
-template <class S>
-__device__ void push_col(const S &X, int si, int key)
-{
-    using IX = typename S::ix;
-    IX *h = &X.colHead[key_d(key) * X.n + key_c(key)];
-    SLOTF(X, cp, si) = (IX)-1; SLOTF(X, cn, si) = *h;
-    if (*h >= 0) SLOTF(X, cp, *h) = (IX)si;
-    *h = (IX)si;
-    if (key_d(key) >= 2) atomicOr(&X.colBits[(key_d(key) - 2) * X.Wn + (key_c(key) >> 5)], 1u << (key_c(key) & 31));
-}
-template <class S>
-__device__ void unlink_row(const S &X, int si, int key)
-{
-    using IX = typename S::ix;
-    const int p = SLOTF(X, rp, si), q = SLOTF(X, rn, si);
-    IX *h = &X.rowHead[key_d(key) * X.m + key_r(key)];
-    if (p >= 0) SLOTF(X, rn, p) = (IX)q; else *h = (IX)q;
-    if (q >= 0) SLOTF(X, rp, q) = (IX)p;
-    if (*h < 0 && key_d(key) < 2) atomicAnd(&X.rowBits[key_d(key) * X.Wm + (key_r(key) >> 5)], ~(1u << (key_r(key) & 31)));
-}
-template <class S>
-__device__ void unlink_col(const S &X, int si, int key)
-{
-    using IX = typename S::ix;
-    const int p = SLOTF(X, cp, si), q = SLOTF(X, cn, si);
-    IX *h = &X.colHead[key_d(key) * X.n + key_c(key)];
-    if (p >= 0) SLOTF(X, cn, p) = (IX)q; else *h = (IX)q;
-    if (q >= 0) SLOTF(X, cp, q) = (IX)p;
-    if (*h < 0 && key_d(key) >= 2) atomicAnd(&X.colBits[(key_d(key) - 2) * X.Wn + (key_c(key) >> 5)], ~(1u << (key_c(key) & 31)));
-}
-
-// Link a slot into its row list and its column list (both head loads first:
-// the two lists are independent).
-template <class S>
-__device__ __forceinline__ void push_both(const S &X, int si, int key)
-{
-    using IX = typename S::ix;
-    IX *hr = &X.rowHead[key_d(key) * X.m + key_r(key)];
-    IX *hc = &X.colHead[key_d(key) * X.n + key_c(key)];
-    const int oldR = *hr, oldC = *hc;
-    SLOTF(X, rp, si) = (IX)-1; SLOTF(X, rn, si) = (IX)oldR;
-    SLOTF(X, cp, si) = (IX)-1; SLOTF(X, cn, si) = (IX)oldC;
-    if (oldR >= 0) SLOTF(X, rp, oldR) = (IX)si;
-    if (oldC >= 0) SLOTF(X, cp, oldC) = (IX)si;
-    *hr = (IX)si;
-    *hc = (IX)si;
-    if (key_d(key) < 2) atomicOr(&X.rowBits[key_d(key) * X.Wm + (key_r(key) >> 5)], 1u << (key_r(key) & 31));
-    else atomicOr(&X.colBits[(key_d(key) - 2) * X.Wn + (key_c(key) >> 5)], 1u << (key_c(key) & 31));
-}
-// Lanes in `pend` link their slots, one lane at a time (two of them may
-// share a list).
-template <class S>
-__device__ __forceinline__ void push_lanes(const S &X, unsigned pend, int si, int key)
-{
-    using IX = typename S::ix;
-    const int lane = threadIdx.x & 31;
-    for (; pend; pend &= pend - 1) {
-        if (lane == __ffs(pend) - 1) push_both(X, si, key);
-        __syncwarp();
-    }
-}
-
-// First i in 1..maxq with bit (pos + i*delta) set, or 0 (delta = +-1)
-// (warp-uniform arguments; every lane calls it). The bits of the range
-// [lo, hi] are read a word per lane, 32 words (1 024 bits) per round, and
-// the nearest set bit is found with a ballot and ffs / clz; a range within
-// one word needs no vote.
-__device__ inline int bit_scan(const uint32_t *b, int limit, int pos, int delta, int maxq)
-{
-    const int lane = threadIdx.x & 31;
-    const int lo = delta > 0 ? pos + 1 : max(0, pos - maxq);
-    const int hi = delta > 0 ? min(limit - 1, pos + maxq) : pos - 1;
-    if (lo > hi) return 0;
-    const int w0 = lo >> 5, w1 = hi >> 5;
-    auto masked = [&](int w) {
-        uint32_t v = b[w];
-        if (w == w0) v &= ~0u << (lo & 31);
-        if (w == w1) v &= 0xffffffffu >> (31 - (hi & 31));
-        return v;
-    };
-    if (w0 == w1) {
-        const uint32_t v = masked(w0);
-        if (!v) return 0;
-        const int y = delta > 0 ? (w0 << 5) + __ffs(v) - 1 : (w0 << 5) + 31 - __clz(v);
-        return delta > 0 ? y - pos : pos - y;
-    }
-    const int nw = w1 - w0 + 1;
-    for (int r = 0; r < nw; r += 32) {
-        // rounds run outward from pos: ascending words when delta > 0
-        const int idx = r + lane;
-        const int w = delta > 0 ? w0 + idx : w1 - idx;
-        const uint32_t v = idx < nw ? masked(w) : 0u;
-        const unsigned bal = __ballot_sync(FULL, v != 0u);
-        if (bal) {
-            const int src = __ffs(bal) - 1;   // the word nearest pos
-            const uint32_t vv = __shfl_sync(FULL, v, src);
-            const int ws = delta > 0 ? w0 + r + src : w1 - r - src;
-            const int y = delta > 0 ? (ws << 5) + __ffs(vv) - 1 : (ws << 5) + 31 - __clz(vv);
-            return delta > 0 ? y - pos : pos - y;
+        const int in = ws.indeg[b];
+        if (in > 1) {
+            const int x = ws.multiNo[b];
+            ws.multi[x] = in | (r.y & 8191) << MULTI_BITS;
+            ws.multiPos[x] = (uint32_t)r.x;
         }
+        if (in == 0) ws.ready0[atomicAdd(&ws.ready0[k], 1)] = (int32_t)b;
     }
-    return 0;
-}
-
-// Lowest move id held in slots [0, hi) and its slot (warp-cooperative).
-template <class S>
-__device__ int lowest_slot(const S &X, int hi)
-{
-    using IX = typename S::ix;
-    const int lane = threadIdx.x & 31;
-    int best = INTMAX, bs = -1;
-    for (int i = lane; i < hi; i += 32) {
-        const int id = SLOTF(X, id, i);
-        if (id < best) { best = id; bs = i; }
-    }
-#pragma unroll
-    for (int o = 16; o; o >>= 1) {
-        const int ob = __shfl_xor_sync(FULL, best, o), os = __shfl_xor_sync(FULL, bs, o);
-        if (ob < best || (ob == best && os < bs)) { best = ob; bs = os; }
-    }
-    return best == INTMAX ? -1 : bs;
-}
-
-// Sort a[0..n) ascending: registers for n <= 32, else a shared-memory
-// bitonic network (a must have room for the next power of two).
-__device__ inline void warp_sort64(long long *a, int n)
-{
-    const int lane = threadIdx.x & 31;
-    if (n <= 1) return;
-    if (n <= 32) {
-        long long v = lane < n ? a[lane] : 0x7fffffffffffffffll;
-#pragma unroll
-        for (int kk = 2; kk <= 32; kk <<= 1) {
-#pragma unroll
-            for (int jj = kk >> 1; jj > 0; jj >>= 1) {
-                const long long o = __shfl_xor_sync(FULL, v, jj);
-                const bool up = (lane & kk) == 0, low = (lane & jj) == 0;
-                v = (low == up) ? (v < o ? v : o) : (v > o ? v : o);
-            }
-        }
-        if (lane < n) a[lane] = v;
-        __syncwarp();
-        return;
-    }
-    int P = 1;
-    while (P < n) P <<= 1;
-    for (int i = n + lane; i < P; i += 32) a[i] = 0x7fffffffffffffffll;
-    __syncwarp();
-    for (int k = 2; k <= P; k <<= 1) {
-        for (int j = k >> 1; j > 0; j >>= 1) {
-            for (int i = lane; i < P; i += 32) {
-                const int ij = i ^ j;
-                if (ij > i) {
-                    const long long x = a[i], y = a[ij];
-                    const bool up = (i & k) == 0;
-                    if ((x > y) == up) { a[i] = y; a[ij] = x; }
-                }
-            }
-            __syncwarp();
-        }
-    }
-}
-
-// Allocate `cnt` slots (warp-cooperative); lane `rank` < cnt gets a slot.
-// freeTop / ovfUsed / hi are warp-uniform.
-template <class S>
-__device__ __forceinline__ int alloc_slot(const S &X, int rank, int cnt, int &freeTop, int &ovfFreeTop,
-                                          int &ovfUsed, int &hi, int kmax, int *err)
-{
-    using IX = typename S::ix;
-    int si = -1;
-    const int fromStack = min(cnt, freeTop);
-    const int fromOvf = min(cnt - fromStack, ovfFreeTop);
-    if (rank < fromStack) si = X.freeStk[freeTop - 1 - rank];
-    else if (rank < fromStack + fromOvf) si = X.ovfFree[ovfFreeTop - 1 - (rank - fromStack)];
-    else if (rank < cnt) si = X.C + ovfUsed + (rank - fromStack - fromOvf);
-    freeTop -= fromStack;
-    ovfFreeTop -= fromOvf;
-    ovfUsed += cnt - fromStack - fromOvf;
-    // the overflow area holds kmax + 1 slots, and slot indices must stay
-    // representable in the link type: beyond either, no slot (nothing is
-    // written) and the run ends with an error
-    // (narrow: the shared capacity; beyond it the instance is handed to the
-    // wide simulation)
-    const int lastOk = S::wide ? min(X.C + kmax, sizeof(IX) == 2 ? 32767 : 0x7fffffff) : X.C - 1;
-    if (si > lastOk) si = -1;
-    if (ovfUsed > kmax || X.C + ovfUsed > lastOk + 1) *err = S::wide ? RR_ERR_INTERNAL : RR_SIM_RETRY;
-    hi = S::wide ? X.C + ovfUsed : X.C;   // every slot ever used lies below
-    return si;
-}
-
-// A newly ready move: fill its slot (the caller links it into the lists).
-template <class S>
-__device__ __forceinline__ int fill_slot(const S &X, int si, int id, int4 r)
-{
-    using IX = typename S::ix;
-    // the first leg: along the source row if the move changes column, else
-    // along the column (an L-path runs row first, then column)
-    const int sr = r.x & 0xffff, sc = r.x >> 16, dr = r.y & 0xffff, dc = r.y >> 16;
-    const int d = dc != sc ? (dc > sc ? 3 : 2) : (dr > sr ? 1 : 0);
-    const int key = key_of(sr, sc, d);
-    SLOTF(X, key, si) = key;
-    SLOTF(X, id, si) = id;
-    SLOTF(X, t, si) = 0;
-    SLOTF(X, legEnd, si) = (int16_t)(dc != sc ? iabs(dc - sc) : iabs(dr - sr));
-    SLOTF(X, dstRow, si) = (int16_t)dr;
-    X.map[id & (MAPN - 1)] = si;
-    return key;
-}
-
-// Pull a move's own record toward L1: it is read when the move finishes.
-__device__ __forceinline__ void prefetch_rec(const JobWS &ws, int id)
-{
-    asm volatile("prefetch.global.L1 [%0];" ::"l"(ws.rec + 2 * id));
-}
-
-// Pull the records of a move's first successors toward L1: they are read when
-// the move finishes, a few batches later.
-__device__ __forceinline__ void prefetch_succ(const JobWS &ws, int4 s4, int nsucc)
-{
-    const int v[4] = {s4.x, s4.y, s4.z, s4.w};
-#pragma unroll
-    for (int e = 0; e < 4; ++e)
-        if (e < nsucc) {
-            const int4 *a = ws.rec + 2 * (v[e] & SUCC_ID);
-            asm volatile("prefetch.global.L1 [%0];" ::"l"(a));
-        }
-}
-
-// Turn the members back into statics (warp-cooperative). Members share one
-// line, so their perpendicular lists are distinct and are pushed in
-// parallel; the shared line list gets the members as one spliced chain.
-template <class S>
-__device__ void dissolve(const S &X, int nm, bool rowLine)
-{
-    using IX = typename S::ix;
-    const int lane = threadIdx.x & 31;
-    if (nm <= 0) return;
-    const int k0 = SLOTF(X, key, X.Msl[0]) & ~KEY_MEM;
-    IX *lineHead = rowLine ? &X.rowHead[key_d(k0) * X.m + key_r(k0)] : &X.colHead[key_d(k0) * X.n + key_c(k0)];
-    const int oldHead = *lineHead;
-    __syncwarp();
-    for (int u = lane; u < nm; u += 32) {
-        const int si = X.Msl[u];
-        const int key = SLOTF(X, key, si) & ~KEY_MEM;
-        SLOTF(X, key, si) = key;
-        const int prv = u == 0 ? -1 : X.Msl[u - 1], nxt = u == nm - 1 ? oldHead : X.Msl[u + 1];
-        if (rowLine) { SLOTF(X, rp, si) = (IX)prv; SLOTF(X, rn, si) = (IX)nxt; push_col(X, si, key); }
-        else { SLOTF(X, cp, si) = (IX)prv; SLOTF(X, cn, si) = (IX)nxt; push_row(X, si, key); }
-    }
-    __syncwarp();
-    if (lane == 0) {
-        if (oldHead >= 0) { if (rowLine) SLOTF(X, rp, oldHead) = (IX)X.Msl[nm - 1]; else SLOTF(X, cp, oldHead) = (IX)X.Msl[nm - 1]; }
-        *lineHead = (IX)X.Msl[0];
-        bits_set(X, key_d(k0), key_r(k0), key_c(k0));
-    }
-    __syncwarp();
-}
-
-// The leader (the lowest unfinished move, which is always ready) lives in
-// warp-uniform registers and holds no slot: its key (position, direction),
-// steps done, the end of its current leg, its destination row, and the
-// successor part of its record (count, overflow offset, first four), loaded
-// when it becomes the leader so that the load has long completed when it
-// finishes.
-struct LeaderState {
-    int key = 0, t = 0, legEnd = 0, dstRow = 0, nsu = 0, ov = 0;
-    int4 s4 = {-1, -1, -1, -1};
-    bool pref = false;   // its successors' records still to be prefetched
-};
-
-// A ready move becomes the leader: its state moves from its slot (already
-// out of the lists and the members) into the registers and the slot is freed.
-template <class S>
-__device__ __forceinline__ void leader_from_slot(const S &X, const JobWS &ws, int si, int &L, LeaderState &Ld,
-                                                 int &freeTop, int &ovfFreeTop)
-{
-    using IX = typename S::ix;
-    const int lane = threadIdx.x & 31;
-    L = SLOTF(X, id, si);
-    Ld.key = SLOTF(X, key, si) & ~KEY_MEM;
-    Ld.t = SLOTF(X, t, si);
-    Ld.legEnd = SLOTF(X, legEnd, si);
-    Ld.dstRow = SLOTF(X, dstRow, si);
-    const int4 own = ws.rec[2 * L];
-    Ld.s4 = ws.rec[2 * L + 1];
-    Ld.nsu = own.z;
-    Ld.ov = own.w;
-    Ld.pref = true;
-    __syncwarp();
-    if (lane == 0) {
-        if (X.map[L & (MAPN - 1)] == si) X.map[L & (MAPN - 1)] = -1;
-        SLOTF(X, key, si) = 0;
-        SLOTF(X, id, si) = INTMAX;
-        if (si < X.C) X.freeStk[freeTop] = (int16_t)si; else X.ovfFree[ovfFreeTop] = si;
-    }
-    if (si < X.C) ++freeTop; else ++ovfFreeTop;
-    __syncwarp();
-}
-
-// A move that became ready just now becomes the leader straight from its
-// record (the first leg as fill_slot sets it).
-__device__ __forceinline__ void leader_from_rec(const JobWS &ws, int id, int4 r, int &L, LeaderState &Ld)
-{
-    const int sr = r.x & 0xffff, sc = r.x >> 16, dr = r.y & 0xffff, dc = r.y >> 16;
-    const int d = dc != sc ? (dc > sc ? 3 : 2) : (dr > sr ? 1 : 0);
-    L = id;
-    Ld.key = key_of(sr, sc, d);
-    Ld.t = 0;
-    Ld.legEnd = dc != sc ? iabs(dc - sc) : iabs(dr - sr);
-    Ld.dstRow = dr;
-    Ld.nsu = r.z;
-    Ld.ov = r.w;
-    Ld.s4 = ws.rec[2 * id + 1];
-    Ld.pref = true;
-}
-
-// One round of successor entries, at most one per lane (warp-cooperative):
-// e is a flagged successor id, or ~index into the successor array. Each
-// entry decrements its move's in-degree (unless the move has no other
-// predecessor); moves that become ready take a slot and join the static
-// lists, except the move handId (the next leader once the leader has
-// finished), whose record is handed back in handRec with hand set.
-template <class S>
-__device__ __forceinline__ void release_round(const S &X, const JobWS &ws, bool has, int32_t e, int handId,
-                                              int &hand, int4 &handRec, int &freeTop, int &ovfFreeTop,
-                                              int &ovfUsed, int &hi, int kmax, int *err)
-{
-    using IX = typename S::ix;
-    const int lane = threadIdx.x & 31;
-    const unsigned lt = (1u << lane) - 1u;
-    int ready = -1;
-    int4 r = make_int4(0, 0, 0, 0);
-    if (has) {
-        if (e < 0) e = ws.succ[~e];
-        const int id = e & SUCC_ID;
-        r = ws.rec[2 * id];   // fetched with the counter update
-        if ((e & SUCC_SINGLE) || atomicSub(&ws.indeg[id], 1) == 1) ready = id;
-    }
-    const unsigned hb = __ballot_sync(FULL, ready >= 0 && ready == handId);
-    if (hb) {
-        const int src = __ffs(hb) - 1;
-        handRec.x = __shfl_sync(FULL, r.x, src);
-        handRec.y = __shfl_sync(FULL, r.y, src);
-        handRec.z = __shfl_sync(FULL, r.z, src);
-        handRec.w = __shfl_sync(FULL, r.w, src);
-        hand = 1;
-        if (lane == src) ready = -1;
-    }
-    const unsigned bal = __ballot_sync(FULL, ready >= 0);
-    const int cnt = __popc(bal);
-    if (cnt) {
-        const int si = alloc_slot(X, __popc(bal & lt), cnt, freeTop, ovfFreeTop, ovfUsed, hi, kmax, err);
-        int key = 0;
-        if (ready >= 0 && si >= 0) key = fill_slot(X, si, ready, r);
-        __syncwarp();
-        push_lanes(X, __ballot_sync(FULL, ready >= 0 && si >= 0), si, key);
-    }
-    __syncwarp();
 }
 
 // Instance order by side, largest first: a counting sort on max(m, n)
@@ -1188,730 +737,899 @@ __device__ inline void s_classify(const Blk B, rr_instance *inst, int count, int
     }
 }
 
-template <typename IX, bool WIDE>
-__device__ __forceinline__ void sim_body(const Blk B, rr_instance *inst, JobWS *wsv, int count, const int *classList,
-                                         const int *classCount, int slotCap, int lineCap)
+// ---------------------------------------------------------- simulation
+//
+// Alg. 4 with the local constraint set of Sec. IV, as an event-driven
+// simulation: one block per instance, its first warp simulates and logs, its
+// other warps write the batches.
+//
+// The lowest-id unfinished move is always ready (nothing earlier is
+// unfinished), so it is always the first member ("leader") of the batch. With
+// the leader's token at (r, c) moving in direction d, the other members are
+// the ready moves stepping in direction d whose tokens lie on row r (set A)
+// or on column c (set B): the one of A and B holding the smaller id wins,
+// because pairwise row-or-column sharing with three or more tokens forces
+// them onto one line. While the members advance together the batch can only
+// change when the leg of one of them ends, or when the leader reaches a line
+// across its way that holds a waiting ready move of direction d. Between such
+// events every batch is the same: a segment.
+//
+// What bounds it: one warp's chain of dependent instructions (segments follow
+// one another strictly; a 256 x 256 grid has about 29 000, its batches 724
+// 000). So the state is laid out to keep that chain short:
+//  - Coordinates are directed: a move of direction d has a position `along`
+//    its way, mirrored for the two negative directions so that it always
+//    grows, and `across` it. The leader's line across the way (its row, for a
+//    vertical direction) is the set of equal `along`, its line of motion the
+//    set of equal `across`.
+//  - Ready moves outside the batch ("statics") stand in one table per
+//    direction, `along` and `across` in the halves of a word, holes marked.
+//    Two 16-byte loads per lane cover 256 statics; one fused add-and-minimum
+//    on 16-bit halves per static tells whether any stands on one of the
+//    leader's two lines and how far the next line ahead is. There are no
+//    lists to walk or to maintain: a move enters by two stores, its entry
+//    taken from a stack by one atomic, so that lanes need no vote among them.
+//  - The batch's other members advance by a common clock: a member keeps its
+//    `along` minus the clock and the clock at which its leg ends, so a segment
+//    that none of them ends does not touch them. They are kept in no order
+//    (the writers sort), with the smallest id and the first end in registers.
+//  - The leader lives in warp-uniform registers. When it finishes, the next
+//    leader is nearly always the next id, released at that moment: its record
+//    is loaded while its predecessor still runs.
+//  - In-degrees of the moves with several predecessors are counted in shared
+//    memory as far as they fit (a global atomic's answer takes about 700
+//    cycles); their predecessors name the counter, not the move, so that a
+//    count that does not reach zero touches nothing else. Moves with one
+//    predecessor need no count.
+//  - A segment is logged in 16 bytes plus its members' ids where these
+//    changed, into memory that the conflict graph no longer needs. The other
+//    warps of the block turn the log into batches and members while the
+//    simulation runs on, each warp 32 segments at a time, with stores of
+//    consecutive words.
+
+// ------------------------------------------------------------- the writers
+
+// A segment's kseg batches of ns moves at batch op0 and member mem0: the
+// leader L (the smallest id) and the ns - 1 moves of list[], in no order.
+// One warp; buf holds the next power of two of ns words. Batches are written
+// as consecutive words (three per batch), members likewise.
+__device__ inline void write_segment(rr_op *ops, int32_t *mem, unsigned op0, unsigned mem0, int kseg, int ns, int d,
+                                     int L, const int32_t *list, int32_t *buf)
 {
-    extern __shared__ int4 smem_i4[];
-    int q = B.x;                  // without a class list: every instance
-    if (classList) {
-        if ((int)B.x >= *classCount) return;
-        q = classList[B.x];
-    }
-    if (q >= count) return;
-    rr_instance *I = &inst[q];
-    if (WIDE ? I->status != RR_SIM_RETRY : !live(I)) return;
-    JobWS &ws = wsv[q];
-    const int k = (int)I->n_moves;
-    const int m = I->m, n = I->n;
     const int lane = threadIdx.x & 31;
-    const unsigned lt = (1u << lane) - 1u;
-    if (k == 0) { if (lane == 0) { I->n_ops = 0; I->n_members = 0; } return; }
-    if (WIDE) {
-        // the narrow pass consumed in-degrees before giving up: recount them
-        // from the successor lists, then start over
-        for (int b = lane; b < k; b += 32) ws.indeg[b] = 0;
+    int32_t *o = (int32_t *)(ops + op0);
+    for (int w = lane; w < 3 * kseg; w += 32) {
+        const int q = (int)(((unsigned)w * 43691u) >> 17), f = w - 3 * q;      // w / 3 for w < 2^16
+        o[w] = f == 0 ? d : f == 1 ? (int32_t)(mem0 + (unsigned)(q * ns)) : ns;
+    }
+    int32_t *mp = mem + mem0;
+    const int total = kseg * ns;
+    if (ns == 1) {
+        for (int i = lane; i < total; i += 32) mp[i] = L;
+        return;
+    }
+    // lane's place in the cycle of ns members, and what 32 places on means
+    const float inv = __frcp_rn((float)ns);
+    auto mod = [&](int a) {
+        int r = a - __float2int_rz((float)a * inv) * ns;
+        if (r < 0) r += ns;
+        if (r >= ns) r -= ns;
+        return r;
+    };
+    int u = mod(lane);
+    const int step = mod(32);
+    if (ns <= 32) {
+        int v = lane == 0 ? L : lane < ns ? list[lane - 1] : INTMAX;
+        int r = 0;
+        for (int j = 0; j < ns; ++j) r += __shfl_sync(FULL, v, j) < v;
+        if (lane < ns) buf[r] = v;
         __syncwarp();
-        for (int b = lane; b < k; b += 32) {
-            const int lo = ws.pairOff[b], cnt = ws.succCnt[b];
-            for (int e = 0; e < cnt; ++e) atomicAdd(&ws.indeg[ws.succ[lo + e] & SUCC_ID], 1);
+        v = lane < ns ? buf[lane] : 0;
+        for (int i0 = 0; i0 < total; i0 += 32) {
+            const int x = __shfl_sync(FULL, v, u);
+            if (i0 + lane < total) mp[i0 + lane] = x;
+            u += step;
+            if (u >= ns) u -= ns;
         }
+    } else {
+        for (int i = lane; i < ns; i += 32) buf[i] = i == 0 ? L : list[i - 1];
         __syncwarp();
+        warp_sort32(buf, ns, buf, ns);
+        for (int i = lane; i < total; i += 32) {
+            mp[i] = buf[u];
+            u += step;
+            if (u >= ns) u -= ns;
+        }
+    }
+    __syncwarp();
+}
+
+constexpr int SIM_POLLS = 1 << 22;      // a writer's polls without progress before it gives up
+
+// Header of a logged segment: its first batch and first member, where its
+// members' ids lie, and the leader (30 bits) with the direction. Lengths
+// follow from the next header.
+__device__ inline void run_writers(SimCtl *C, rr_instance *I, const int32_t *log, int32_t *buf)
+{
+    const int lane = threadIdx.x & 31;
+    const uint4 *hdr = (const uint4 *)log;
+    const unsigned long long cap_ops = (unsigned long long)I->cap_ops, cap_mem = (unsigned long long)I->cap_members;
+    rr_op *ops = as_global(I->ops);
+    int32_t *mem = as_global(I->members);
+    volatile int *pub = &C->pub, *fin = &C->fin;
+    for (;;) {
+        int s0 = 0;
+        if (lane == 0) s0 = atomicAdd(&C->next, 32);
+        s0 = __shfl_sync(FULL, s0, 0);
+        int have = 0;
+        for (int polls = 0;; ++polls) {
+            const int f = *fin;
+            __threadfence_block();
+            have = *pub;
+            if (__all_sync(FULL, have >= s0 + 32 || f)) break;
+            if (polls > SIM_POLLS) { if (lane == 0) set_status(I, RR_ERR_TIMEOUT); return; }
+            __nanosleep(2000);
+        }
+        have = __shfl_sync(FULL, have, 0);
         __threadfence_block();
-        if (lane == 0) I->status = RR_OK;
+        const int cnt = min(32, have - s0);
+        if (cnt <= 0) return;
+        uint4 h = make_uint4(0u, 0u, 0u, 0u);
+        int kseg = 0, ns = 0;
+        if (lane < cnt) {
+            h = hdr[s0 + lane];
+            const uint2 nx = *(const uint2 *)&hdr[s0 + lane + 1];
+            kseg = (int)(nx.x - h.x);
+            ns = (int)((nx.y - h.y) / (unsigned)max(kseg, 1));
+            // a batch list that does not fit ends as RR_ERR_CAPACITY: nothing of it is written
+            if (nx.x > cap_ops || nx.y > cap_mem) kseg = 0;
+        }
+        for (int j = 0; j < cnt; ++j) {
+            const int kj = __shfl_sync(FULL, kseg, j), nj = __shfl_sync(FULL, ns, j);
+            const unsigned op0 = __shfl_sync(FULL, h.x, j), mem0 = __shfl_sync(FULL, h.y, j);
+            const unsigned lo = __shfl_sync(FULL, h.z, j), l = __shfl_sync(FULL, h.w, j);
+            if (kj > 0)
+                write_segment(ops, mem, op0, mem0, kj, nj, (int)(l >> 30), (int)(l & 0x3fffffffu), log + lo, buf);
+        }
+    }
+}
+
+// ---------------------------------------------------------- the simulation
+
+// Position words: `along` in the low half, `across` in the high one, both
+// plus one, so that neither is zero; a hole of the table is all ones.
+constexpr uint32_t HOLE = 0xffffffffu;
+
+// The vertical leg after a horizontal one (direction d) that ended at p.
+struct Leg { int d; uint32_t pos; int rem; };
+__device__ __forceinline__ Leg second_leg(int d, uint32_t p, int dstRow)
+{
+    const int row = (int)(p >> 16) - 1, al = (int)(p & 0xffffu);
+    Leg g;
+    g.d = dstRow > row ? 1 : 0;
+    g.pos = dir_pos(g.d, row, d == 2 ? MIRROR - 1 - al : al - 1);
+    g.rem = iabs(dstRow - row);
+    return g;
+}
+
+// Which of eight position words match w in the halves of `half`.
+__device__ __forceinline__ unsigned match8(uint4 a, uint4 b, uint32_t w, uint32_t half)
+{
+    const uint32_t x[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+    unsigned m = 0;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) m |= ((x[i] ^ w) & half) == 0u ? 1u << i : 0u;
+    return m;
+}
+// Minimum, half by half, of v and the eight words plus w.
+__device__ __forceinline__ uint32_t min8(uint4 a, uint4 b, uint32_t w, uint32_t v)
+{
+    v = __viaddmin_u16x2(a.x, w, v);
+    v = __viaddmin_u16x2(a.y, w, v);
+    v = __viaddmin_u16x2(a.z, w, v);
+    v = __viaddmin_u16x2(a.w, w, v);
+    v = __viaddmin_u16x2(b.x, w, v);
+    v = __viaddmin_u16x2(b.y, w, v);
+    v = __viaddmin_u16x2(b.z, w, v);
+    v = __viaddmin_u16x2(b.w, w, v);
+    return v;
+}
+
+// Memory operations of the lanes that `c` holds for, predicated rather than
+// branched around: in one warp's serial code a branch and the point where its
+// lanes meet again cost 15 to 20 cycles each, and the code below has little
+// else between them.
+#ifdef __CUDA_ARCH__
+__device__ __forceinline__ uint32_t sh_addr(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
+#define RR_IF(instr) "{ .reg .pred q; setp.ne.u32 q, %0, 0; @q " instr " }"
+__device__ __forceinline__ int sh_add_if(bool c, void *p, int v)
+{
+    int r = 0;
+    asm volatile("{ .reg .pred q; setp.ne.u32 q, %1, 0; @q atom.shared.add.u32 %0, [%2], %3; }"
+                 : "+r"(r) : "r"((unsigned)c), "r"(sh_addr(p)), "r"(v) : "memory");
+    return r;
+}
+__device__ __forceinline__ int ld_u16_if(bool c, const uint16_t *p)
+{
+    unsigned short r = 0;
+    asm volatile("{ .reg .pred q; setp.ne.u32 q, %1, 0; @q ld.shared.u16 %0, [%2]; }"
+                 : "+h"(r) : "r"((unsigned)c), "r"(sh_addr(p)) : "memory");
+    return r;
+}
+__device__ __forceinline__ void st_if(bool c, uint16_t *p, int v)
+{
+    asm volatile(RR_IF("st.shared.u16 [%1], %2;") ::"r"((unsigned)c), "r"(sh_addr(p)), "h"((unsigned short)v) : "memory");
+}
+__device__ __forceinline__ void st_if(bool c, void *p, uint32_t v)
+{
+    asm volatile(RR_IF("st.shared.u32 [%1], %2;") ::"r"((unsigned)c), "r"(sh_addr(p)), "r"(v) : "memory");
+}
+__device__ __forceinline__ void st_if(bool c, int2 *p, int x, int y)
+{
+    asm volatile(RR_IF("st.shared.v2.u32 [%1], {%2, %3};") ::"r"((unsigned)c), "r"(sh_addr(p)), "r"(x), "r"(y) : "memory");
+}
+__device__ __forceinline__ int4 ldg_if(bool c, const int4 *p)
+{
+    int4 v = make_int4(0, 0, 0, 0);
+    asm volatile("{ .reg .pred q; setp.ne.u32 q, %4, 0; @q ld.global.v4.u32 {%0, %1, %2, %3}, [%5]; }"
+                 : "+r"(v.x), "+r"(v.y), "+r"(v.z), "+r"(v.w) : "r"((unsigned)c), "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ int2 ldg_if(bool c, const int2 *p)
+{
+    int2 v = make_int2(0, 0);
+    asm volatile("{ .reg .pred q; setp.ne.u32 q, %2, 0; @q ld.global.v2.u32 {%0, %1}, [%3]; }"
+                 : "+r"(v.x), "+r"(v.y) : "r"((unsigned)c), "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ int ldg_if(bool c, const void *p)
+{
+    int v = 0;
+    asm volatile("{ .reg .pred q; setp.ne.u32 q, %1, 0; @q ld.global.u32 %0, [%2]; }"
+                 : "+r"(v) : "r"((unsigned)c), "l"(p) : "memory");
+    return v;
+}
+// Bring a record's first half, or a word, into L1 without a register waiting
+// for it: an asynchronous copy to a place in shared memory that nothing
+// reads. (prefetch.global.L1 stops at L2 here: a load after it takes 300 to
+// 500 cycles, after this copy 40.)
+__device__ __forceinline__ void touch_rec_if(bool c, const int4 *rec, int id, uint32_t dump)
+{
+    asm volatile(RR_IF("cp.async.ca.shared.global [%1], [%2], 16;") ::"r"((unsigned)c), "r"(dump),
+                 "l"(rec + 2 * (size_t)id) : "memory");
+}
+__device__ __forceinline__ void touch_word_if(bool c, const void *p, uint32_t dump)
+{
+    asm volatile(RR_IF("cp.async.ca.shared.global [%1], [%2], 4;") ::"r"((unsigned)c), "r"(dump), "l"(p) : "memory");
+}
+__device__ __forceinline__ void touch_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+#undef RR_IF
+#else   // host-side stand-ins
+static inline uint32_t sh_addr(const void *) { return 0; }
+static inline int sh_add_if(bool c, void *p, int v) { int r = 0; if (c) { r = *(int *)p; *(int *)p = (int)((unsigned)r + (unsigned)v); } return r; }
+static inline int ld_u16_if(bool c, const uint16_t *p) { return c ? *p : 0; }
+static inline void st_if(bool c, uint16_t *p, int v) { if (c) *p = (uint16_t)v; }
+static inline void st_if(bool c, void *p, uint32_t v) { if (c) *(uint32_t *)p = v; }
+static inline void st_if(bool c, int2 *p, int x, int y) { if (c) *p = make_int2(x, y); }
+static inline int4 ldg_if(bool c, const int4 *p) { return c ? *p : make_int4(0, 0, 0, 0); }
+static inline int2 ldg_if(bool c, const int2 *p) { return c ? *p : make_int2(0, 0); }
+static inline int ldg_if(bool c, const void *p) { return c ? *(const int *)p : 0; }
+static inline void touch_rec_if(bool, const int4 *, int, uint32_t) {}
+static inline void touch_word_if(bool, const void *, uint32_t) {}
+static inline void touch_wait() {}
+#endif
+
+// The largest of the lanes' values (usually all the same): a value that the
+// compiler knows to be uniform, so that branches on it, and on what is
+// computed from it, need no bookkeeping for lanes that might diverge.
+__device__ __forceinline__ uint32_t uni(uint32_t v) { return __reduce_max_sync(FULL, v); }
+
+// Words the log must have left at the start of 32 segments: their headers and
+// the one after them, a list of ids for each.
+#define LOG_SLACK(lineCap) (4u * 34u + 32u * (unsigned)(lineCap))
+
+// One simulation by one warp. SIM_SMALL: tables in shared memory, at most 256
+// entries per direction (one load of every lane covers them); SIM_BIG: the
+// same with more entries; both end with RR_SIM_RETRY when an instance has
+// more ready moves of a direction than entries. SIM_WIDE: tables in global
+// memory, room for every move.
+enum { SIM_SMALL, SIM_BIG, SIM_WIDE };
+
+template <int MODE>
+struct Sim {
+    using ST = typename std::conditional<MODE == SIM_WIDE, int32_t, uint16_t>::type;
+    uint32_t *pos;            // position words, a table of cap entries per direction
+    int2 *ir;                 // id, steps left in the leg
+    ST *stk;                  // free entries (numbers within the table)
+    int cap;                  // (the wide tables have sizes of their own, C->wcap from C->wbase on)
+    int2 *mie;                // members: id, clock at the end of the leg
+    uint32_t *mpos;           // members: position word, `along` minus the clock
+    SimCtl *C;
+    const int4 *rec;
+    const int32_t *succ, *multiId;
+    const uint32_t *multiPos;
+    int32_t *multi;           // in-degree counters in global memory (with their moves' first legs)
+    unsigned *cnt;            // the first ncnt of them in shared memory, two per word
+    int ncnt;
+    bool allShared;           // all of them
+    uint32_t dump;            // shared address for the touches
+
+    __device__ __forceinline__ int base(int d) const { return MODE == SIM_WIDE ? C->wbase[d] : d * cap; }
+    __device__ __forceinline__ int size(int d) const { return MODE == SIM_WIDE ? C->wcap[d] : cap; }
+
+    // The moves of the lanes with c become statics.
+    __device__ __forceinline__ void enter(bool c, int d, uint32_t p, int id, int rem)
+    {
+        if constexpr (MODE == SIM_WIDE) {
+            if (c) {
+                const int b = base(d), e = b + stk[b + atomicSub(&C->nfree[d], 1) - 1];
+                pos[e] = p;
+                ir[e] = make_int2(id, rem);
+            }
+        } else {
+            const int o = sh_add_if(c, &C->nfree[d], -1) - 1;
+            const bool none = c && o < 0, ok = c && o >= 0;
+            st_if(none, &C->full, 1u);             // no room: the run will end with RR_SIM_RETRY
+            sh_add_if(none, &C->nfree[d], 1);
+            const int e = d * cap + ld_u16_if(ok, stk + d * cap + o);
+            st_if(ok, pos + e, p);
+            st_if(ok, ir + e, id, rem);
+        }
     }
 
-    // shared-memory layout (mirrored by the launcher's size computation)
-    Sim<IX, WIDE> X;
-    X.C = slotCap; X.m = m; X.n = n; X.Wm = (m + 31) >> 5; X.Wn = (n + 31) >> 5;
-    const int lbuf = 2 * (lineCap + 2);
-    X.Kb = (long long *)smem_i4;
-    int32_t *p32 = (int32_t *)(X.Kb + lbuf);
-    X.sm.key = p32; p32 += slotCap;
-    X.sm.id = p32; p32 += slotCap;
-    X.map = p32; p32 += MAPN;
-    X.Mid = p32; p32 += lineCap + 2;
-    X.Msl = p32; p32 += lineCap + 2;
-    X.sbuf = p32; p32 += SBUF;
-    X.rowBits = (uint32_t *)p32; p32 += 2 * ((lineCap + 31) >> 5);
-    X.colBits = (uint32_t *)p32; p32 += 2 * ((lineCap + 31) >> 5);
-    IX *pix = (IX *)p32;
-    X.sm.rp = pix; pix += slotCap;
-    X.sm.rn = pix; pix += slotCap;
-    X.sm.cp = pix; pix += slotCap;
-    X.sm.cn = pix; pix += slotCap;
-    X.rowHead = pix; pix += 4 * lineCap;
-    X.colHead = pix; pix += 4 * lineCap;
-    int16_t *p16 = (int16_t *)pix;
-    X.sm.t = p16; p16 += slotCap;
-    X.sm.legEnd = p16; p16 += slotCap;
-    X.sm.dstRow = p16; p16 += slotCap;
-    X.freeStk = p16;
-    X.ovfFree = ws.ovfFree;
-    {   // overflow slots (global), same structure
-        char *g = (char *)ws.slotOvf;
-        const size_t K1 = (size_t)k + 1;
-        X.gm.key = (int32_t *)g;           g += 4 * K1;
-        X.gm.id = (int32_t *)g;            g += 4 * K1;
-        IX **fl[4] = {&X.gm.rp, &X.gm.rn, &X.gm.cp, &X.gm.cn};
-        for (int u = 0; u < 4; ++u) { *fl[u] = (IX *)g; g += sizeof(IX) * K1; }
-        X.gm.t = (int16_t *)g;             g += 2 * K1;
-        X.gm.legEnd = (int16_t *)g;        g += 2 * K1;
-        X.gm.dstRow = (int16_t *)g;
+    // A finished move of each lane with c hands one predecessor fewer to the
+    // successor entry v: a move without other predecessors (flagged id) is
+    // ready now, another counts down. The moves that become ready enter their
+    // tables, except the next leader: true in its lane. (Every lane calls.)
+    __device__ __forceinline__ bool release(bool c, int32_t v, int handId)
+    {
+        const bool single = c && (v & SUCC_SINGLE), multi_ = c && !(v & SUCC_SINGLE);
+        const int x = v & SUCC_ID;
+        const int sh = (x & 1) * 16;
+        int old = (sh_add_if(multi_ && x < ncnt, cnt + (x >> 1), -(1 << sh)) >> sh) & 0xffff;
+        if (!allShared) {
+            if (multi_ && x >= ncnt) old = atomicSub(&multi[x], 1) & MULTI_COUNT;
+            __syncwarp();
+        }
+        const bool soon = multi_ && old == 2, last = multi_ && old == 1;
+        touch_word_if(soon, multiId + x, dump);           // next time it is ready
+        touch_word_if(soon, multiPos + x, dump);
+        touch_word_if(soon, multi + x, dump);
+        bool h = single && x == handId;
+        const bool fresh = single && !h;
+        if (__any_sync(FULL, fresh || last)) {
+            const int2 r = ldg_if(fresh, (const int2 *)(rec + 2 * (size_t)x));
+            int id = ldg_if(last, (const void *)(multiId + x)), p = ldg_if(last, (const void *)(multiPos + x));
+            int y = ldg_if(last, (const void *)(multi + x)) >> MULTI_BITS;
+            if (fresh) { id = x; p = r.x; y = r.y; }
+            h |= last && id == handId;
+            enter((fresh || last) && !h, y & 3, (uint32_t)p, id, y >> 2 & 2047);
+        }
+        return h;
     }
-    for (int i = lane; i < slotCap; i += 32) { X.sm.key[i] = 0; X.sm.id[i] = INTMAX; X.freeStk[i] = (int16_t)(slotCap - 1 - i); }
-    for (int i = lane; i < MAPN; i += 32) X.map[i] = -1;
-    for (int i = lane; i < 4 * m; i += 32) X.rowHead[i] = (IX)-1;
-    for (int i = lane; i < 4 * n; i += 32) X.colHead[i] = (IX)-1;
-    for (int i = lane; i < 2 * X.Wm; i += 32) X.rowBits[i] = 0u;
-    for (int i = lane; i < 2 * X.Wn; i += 32) X.colBits[i] = 0u;
-    int freeTop = slotCap, ovfFreeTop = 0, ovfUsed = 0, hi = slotCap, err = 0;
-    __syncwarp();
+
+    __device__ __forceinline__ int run(rr_instance *I, JobWS &ws, int32_t *log, unsigned logWords, int lineCap,
+                                       int32_t *buf, int32_t *ids);
+};
+
+template <int MODE>
+__device__ __forceinline__ int Sim<MODE>::run(rr_instance *I, JobWS &ws, int32_t *log, unsigned logWords, int lineCap,
+                                              int32_t *buf, int32_t *ids)
+{
+    const int lane = threadIdx.x & 31;
+    const unsigned lt = (1u << lane) - 1u;
+    const int k = (int)I->n_moves;
+    int err = RR_OK;
 
     // moves without predecessors become statics
-    const int32_t *ready0 = ws.ready0;
-    const int nready0 = ready0[k];
-    for (int base = 0; base < nready0; base += 32) {
-        const int cnt = min(32, nready0 - base);
-        int id = -1;
-        int4 r = make_int4(0, 0, 0, 0);
-        if (lane < cnt) { id = ready0[base + lane]; r = ws.rec[2 * id]; }
-        const int si = alloc_slot(X, lane, cnt, freeTop, ovfFreeTop, ovfUsed, hi, k, &err);
-        int key = 0;
-        if (lane < cnt && si >= 0) key = fill_slot(X, si, id, r);
+    {
+        const int n0 = ws.ready0[k];
+        for (int b = 0; b < n0; b += 32) {
+            const bool c = b + lane < n0;
+            const int id = c ? ws.ready0[b + lane] : 0;
+            const int4 r = ldg_if(c, rec + 2 * (size_t)id);
+            enter(c, r.y & 3, (uint32_t)r.x, id, r.y >> 2 & 2047);
+        }
         __syncwarp();
-        push_lanes(X, __ballot_sync(FULL, lane < cnt && si >= 0), si, key);
     }
+    // the leader: id, direction, position word, clock at the end of its leg,
+    // destination row, successors
+    int L = -1, d = 0, lend = 0, ldst = 0, nsu = 0, ov = 0;
+    uint32_t lpos = 0;
+    bool chain = false;       // its only successor is the next id, which waits for nothing else
+    int4 s4 = make_int4(0, 0, 0, 0);
+    // members: nm of them, of direction dm, on the line `along - clock ==
+    // line` (prim) or `across == line`; the clock at their first leg end
+    int nm = 0, dm = -1, line = 0, minEnd = INTMAX;
+    bool prim = true, changed = false;
+    int clk = 0;              // elementary steps so far: also the number of batches
+    unsigned nmem = 0;
+    // the log: headers from its start, ids from its end
+    uint4 *hdr = (uint4 *)log;
+    unsigned nseg = 0, idTop = logWords, list = 0;
+    bool logging = idTop >= LOG_SLACK(lineCap);
+    // housekeeping every 32 segments: publish, check the bounds
+    int left = 32;
+    long long guard = (g_guard_cap > 0 ? g_guard_cap : I->n_steps + 2ll * k + 16) + 1;
+    if (guard < 32) left = (int)guard;
+    guard -= left;
+    // this lane's eight entries of a table's first 256 (a lane beyond the
+    // table reads the last eight too: that changes no minimum)
+    int groups = size(0) >> 3, off = 8 * min(lane, groups - 1);
 
-    const int64_t cap_ops = I->cap_ops, cap_mem = I->cap_members;
-    rr_op *ops = I->ops;
-    int32_t *mem = I->members;
-    int64_t nop = 0, nmem = 0;
-    int overflow = 0;
-    int Ls = lowest_slot(X, hi);
-    int L = Ls >= 0 ? SLOTF(X, id, Ls) : -1;
-    // the leader: warp-uniform registers, no slot (see LeaderState)
-    LeaderState Ld;
-    if (err) {
-        // out of slots already (narrow pass): handed to the wide pass
-    } else if (L != 0) err = RR_ERR_INTERNAL;
-    else {
-        if (lane == 0) { const int kk = SLOTF(X, key, Ls); unlink_row(X, Ls, kk); unlink_col(X, Ls, kk); }
+    auto set_leg = [&](uint32_t y) {
+        d = (int)(y & 3u);
+        lend = clk + (int)(y >> 2 & 2047u);
+        ldst = (int)(y >> 13 & 1023u);
+        chain = (y >> 23) != 0u;
+    };
+    auto on_clock = [&](uint32_t p) { return (p & 0xffff0000u) | ((p + (uint32_t)clk) & 0xffffu); };
+    auto dissolve = [&]() {
+        for (int u0 = 0; u0 < nm; u0 += 32) {
+            const int u = min(u0 + lane, nm - 1);
+            const int2 ie = mie[u];
+            enter(u0 + lane < nm, dm, on_clock(mpos[u]), ie.x, ie.y - clk);
+        }
+        nm = 0;
+        minEnd = INTMAX;
+        changed = true;
         __syncwarp();
-        leader_from_slot(X, ws, Ls, L, Ld, freeTop, ovfFreeTop);
-    }
-    // members: nm of them (leader excluded), on one line of type rowLine at
-    // index lineIdx, direction dm
-    int nm = 0, dm = -1, lineIdx = -1;
-    bool rowLine = true;
-    const int64_t guard_max = g_guard_cap > 0 ? g_guard_cap : I->n_steps + 2ll * k + 16;
-    int64_t guard = 0;
-    // records of up to 32 newcomers: fetched when they join, their
-    // successors' records prefetched in the next segment
-    int4 nrec = make_int4(0, 0, 0, 0), ns4 = nrec;
-    int npref = 0;
-
-    while (!err && L < k) {
-        if (++guard > guard_max) { err = RR_ERR_TIMEOUT; break; }
-        const int lr = key_r(Ld.key), lc = key_c(Ld.key), d = key_d(Ld.key);
-        const int remL = Ld.legEnd - Ld.t;
-        const int sgn = (d == 1 || d == 3) ? 1 : -1;
-        // members still on the leader's line in the leader's direction?
-        if (nm > 0 && !(dm == d && (rowLine ? lineIdx == lr : lineIdx == lc))) { dissolve(X, nm, rowLine); nm = 0; }
-        // smallest static id on the leader's row and column (lane 0 walks;
-        // nothing to walk when both lists are empty)
-        int minA = INTMAX, minB = INTMAX;
-        const int hA = X.rowHead[d * m + lr], hB = X.colHead[d * n + lc];
-        if (hA >= 0 || hB >= 0) {
+    };
+    // a record a little later into L1
+    auto look_ahead = [&]() {
+        touch_rec_if(lane == 0, rec, min(L + 4, k), dump);
+    };
+    // the lowest unfinished move, wherever it waits, becomes the leader (rare:
+    // nearly always it is released when its predecessor finishes); false when
+    // there is none
+    auto find_leader = [&]() {
+        int best = INTMAX, where = -1, place = 0;
+        for (int u = lane; u < nm; u += 32) {
+            const int id = mie[u].x;
+            if (id < best) { best = id; where = 4; place = u; }
+        }
+        for (int q = 0; q < 4; ++q)
+            for (int e0 = base(q) + 4 * lane; e0 < base(q) + size(q); e0 += 128) {
+                const uint4 a = *(const uint4 *)(pos + e0);
+                const uint32_t x[4] = {a.x, a.y, a.z, a.w};
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+                    if (x[i] != HOLE && ir[e0 + i].x < best) { best = ir[e0 + i].x; where = q; place = e0 + i; }
+            }
+        const int least = __reduce_min_sync(FULL, best);
+        if (least == INTMAX) return false;
+        // (ids are distinct: one lane has it)
+        where = (int)uni(best == least ? (uint32_t)where : 0u);
+        place = (int)uni(best == least ? (uint32_t)place : 0u);
+        L = least;
+        const int4 r = rec[2 * (size_t)L];
+        s4 = rec[2 * (size_t)L + 1];
+        nsu = r.z;
+        ov = r.w;
+        set_leg(uni((uint32_t)r.y));
+        if (where < 4) {
+            d = where;
+            lpos = uni(pos[place]);
+            lend = clk + (int)uni((uint32_t)ir[place].y);
+            const int fr = C->nfree[d], tb = base(d);
+            __syncwarp();
             if (lane == 0) {
-                int walk = 0;
-                for (int p = hA; p >= 0 && walk <= lineCap; p = SLOTF(X, rn, p), ++walk) minA = min(minA, SLOTF(X, id, p));
-                for (int p = hB; p >= 0 && walk <= 2 * lineCap; p = SLOTF(X, cn, p), ++walk) minB = min(minB, SLOTF(X, id, p));
-                if (walk > 2 * lineCap) err = RR_ERR_INTERNAL;
-            }
-            minA = __shfl_sync(FULL, minA, 0);
-            minB = __shfl_sync(FULL, minB, 0);
-            err = __shfl_sync(FULL, err, 0);
-            if (err) break;
-        }
-        if (nm > 0) { if (rowLine) minA = min(minA, X.Mid[0]); else minB = min(minB, X.Mid[0]); }
-        // the previous segment's newcomers: their records have arrived,
-        // their successors' records are prefetched now
-        if (lane < npref) prefetch_succ(ws, ns4, nrec.z);
-        npref = 0;
-        if (minA != INTMAX || minB != INTMAX) {
-            const bool chooseRow = minA < minB;
-            if (nm > 0 && chooseRow != rowLine) { dissolve(X, nm, rowLine); nm = 0; }
-            // newcomers: every static of the chosen line (the list empties)
-            const int h = chooseRow ? X.rowHead[d * m + lr] : X.colHead[d * n + lc];
-            int nc = 0;
-            if (lane == 0) {
-                for (int p = h; p >= 0 && nc <= lineCap; p = chooseRow ? SLOTF(X, rn, p) : SLOTF(X, cn, p))
-                    X.Kb[nc++] = ((long long)SLOTF(X, id, p) << 32) | (unsigned)p;
-                if (chooseRow) {
-                    X.rowHead[d * m + lr] = (IX)-1;
-                    if (d < 2) atomicAnd(&X.rowBits[d * X.Wm + (lr >> 5)], ~(1u << (lr & 31)));
-                } else {
-                    X.colHead[d * n + lc] = (IX)-1;
-                    if (d >= 2) atomicAnd(&X.colBits[(d - 2) * X.Wn + (lc >> 5)], ~(1u << (lc & 31)));
-                }
-            }
-            nc = __shfl_sync(FULL, nc, 0);
-            if (nm + nc > lineCap) { err = RR_ERR_INTERNAL; break; }
-            __syncwarp();
-            // unlink each newcomer from its perpendicular list (distinct lists)
-            for (int u = lane; u < nc; u += 32) {
-                const int si = (int)(X.Kb[u] & 0xffffffff);
-                const int key = SLOTF(X, key, si);
-                if (chooseRow) unlink_col(X, si, key); else unlink_row(X, si, key);
-                SLOTF(X, key, si) = key | KEY_MEM;
-                const int id = (int)(X.Kb[u] >> 32);
-                if (u < 32) { nrec = ws.rec[2 * id]; ns4 = ws.rec[2 * id + 1]; }
-                else prefetch_rec(ws, id);
-            }
-            __syncwarp();
-            // merge the newcomers into the sorted members (keys id << 32 | slot)
-            if (nc > 0 && nm <= 32 && nc <= 32) {
-                // the usual case, one member and one newcomer per lane: each
-                // newcomer's id is broadcast in turn; a member's rank grows by
-                // the newcomers below it, a newcomer's rank is the members
-                // below it (one vote) plus the newcomers below it (ids are
-                // distinct)
-                const int mId = lane < nm ? X.Mid[lane] : INTMAX;
-                const int mSl = lane < nm ? X.Msl[lane] : 0;
-                const long long kn = lane < nc ? X.Kb[lane] : 0ll;
-                const int nId = lane < nc ? (int)(kn >> 32) : INTMAX;
-                int rM = lane, rN = 0;
-                for (int j = 0; j < nc; ++j) {
-                    const int o = __shfl_sync(FULL, nId, j);
-                    rM += o < mId;
-                    rN += o < nId;
-                    const int below = __popc(__ballot_sync(FULL, mId < o));
-                    if (lane == j) rN += below;
-                }
-                __syncwarp();
-                if (lane < nm) { X.Mid[rM] = mId; X.Msl[rM] = mSl; }
-                if (lane < nc) { X.Mid[rN] = nId; X.Msl[rN] = (int)(kn & 0xffffffff); }
-                nm += nc;
-            } else if (nc > 0) {
-                const int tot = nm + nc;
-                long long *out = X.Kb + (lineCap + 2);
-                if (nc <= 32) {
-                    // few newcomers (the usual case): ranks by counting
-                    for (int u = lane; u < nm; u += 32) {
-                        const long long key = ((long long)X.Mid[u] << 32) | (unsigned)X.Msl[u];
-                        int r = 0;
-                        for (int j = 0; j < nc; ++j) r += X.Kb[j] < key;
-                        out[u + r] = key;
-                    }
-                    if (lane < nc) {
-                        const long long key = X.Kb[lane];
-                        int r = 0;
-                        for (int j = 0; j < nc; ++j) r += X.Kb[j] < key;
-                        int lo = 0, hi2 = nm;
-                        while (lo < hi2) {
-                            const int md = (lo + hi2) >> 1;
-                            if ((((long long)X.Mid[md] << 32) | (unsigned)X.Msl[md]) < key) lo = md + 1; else hi2 = md;
-                        }
-                        out[r + lo] = key;
-                    }
-                } else {
-                    warp_sort64(X.Kb, nc);
-                    for (int u = lane; u < nm; u += 32) {      // member u: rank among newcomers
-                        const long long key = ((long long)X.Mid[u] << 32) | (unsigned)X.Msl[u];
-                        int lo = 0, hi2 = nc;
-                        while (lo < hi2) { const int md = (lo + hi2) >> 1; if (X.Kb[md] < key) lo = md + 1; else hi2 = md; }
-                        out[u + lo] = key;
-                    }
-                    for (int u = lane; u < nc; u += 32) {      // newcomer u: rank among members
-                        const long long key = X.Kb[u];
-                        int lo = 0, hi2 = nm;
-                        while (lo < hi2) {
-                            const int md = (lo + hi2) >> 1;
-                            if ((((long long)X.Mid[md] << 32) | (unsigned)X.Msl[md]) < key) lo = md + 1; else hi2 = md;
-                        }
-                        out[u + lo] = key;
-                    }
-                }
-                __syncwarp();
-                for (int u = lane; u < tot; u += 32) { X.Mid[u] = (int)(out[u] >> 32); X.Msl[u] = (int)(out[u] & 0xffffffff); }
-                nm = tot;
-            }
-            npref = min(nc, 32);
-            rowLine = chooseRow;
-            lineIdx = chooseRow ? lr : lc;
-            dm = d;
-            __syncwarp();
-        }
-        // segment length: shortest remaining leg, next pickup
-        int kseg = remL;
-        // up to 32 members: lane u keeps member u's slot, id, key, steps and
-        // leg end in registers from here through the advance
-        const bool regM = nm > 0 && nm <= 32;
-        int mSi = -1, mId = 0, mKey = 0, mT = 0, mLe = 0;
-        if (nm > 0) {
-            int remM = INTMAX;
-            if (regM) {
-                if (lane < nm) {
-                    mSi = X.Msl[lane];
-                    mId = X.Mid[lane];
-                    mKey = SLOTF(X, key, mSi);
-                    mT = SLOTF(X, t, mSi);
-                    mLe = SLOTF(X, legEnd, mSi);
-                    remM = mLe - mT;
-                }
-            } else {
-                for (int u = lane; u < nm; u += 32) { const int si = X.Msl[u]; remM = min(remM, SLOTF(X, legEnd, si) - SLOTF(X, t, si)); }
-            }
-            kseg = min(kseg, __reduce_min_sync(FULL, remM));   // one warp reduction
-        }
-        if (kseg > 1) {   // a static move of direction d the leader's line reaches
-            const int hit = d >= 2 ? bit_scan(X.colBits + (d - 2) * X.Wn, n, lc, sgn, kseg - 1)
-                                   : bit_scan(X.rowBits + d * X.Wm, m, lr, sgn, kseg - 1);
-            if (hit > 0) kseg = hit;
-        }
-        if (kseg < 1) { err = RR_ERR_INTERNAL; break; }
-        const int ns = nm + 1;
-
-        // kseg identical batches: the leader, then the members in ascending id
-        // (a segment holds at most 2 048 batches of at most lineCap + 1 moves,
-        // so offsets within it fit 32 bits; the first-member field is the
-        // low 32 bits of the member count, as the ABI's int32 field holds it)
-        const int addm = kseg * ns;
-        if (!overflow && nop + kseg <= cap_ops && nmem + addm <= cap_mem) {
-            rr_op *op = ops + nop;
-            int32_t *mp = mem + nmem;
-            const int32_t f0 = (int32_t)nmem;
-            if (ns == 1) {
-                for (int i = lane; i < kseg; i += 32) { op[i] = rr_op{d, f0 + i, 1}; mp[i] = L; }
-            } else {
-                for (int i = lane; i < kseg; i += 32) op[i] = rr_op{d, f0 + i * ns, ns};
-                int u = small_mod(lane, ns);
-                const int step = small_mod(32, ns);
-                for (int i = lane; i < addm; i += 32) {
-                    mp[i] = u == 0 ? L : X.Mid[u - 1];
-                    u += step;
-                    if (u >= ns) u -= ns;
-                }
+                pos[place] = HOLE;
+                stk[tb + fr] = (ST)(place - tb);
+                C->nfree[d] = fr + 1;
             }
         } else {
-            overflow = 1;
-        }
-        nop += kseg;
-        nmem += addm;
-
-        // advance by kseg steps along the current legs (no batch move's leg
-        // ends before the segment does); at a leg's end a move finishes on
-        // its destination row or turns toward it. The leader first (its
-        // registers), then the members: finished members release their
-        // successors, members whose leg ended leave the batch and become
-        // statics, the others stay members.
-        if (Ld.pref) {   // the leader's record has arrived by now
-            prefetch_succ(ws, Ld.s4, lane == 0 ? Ld.nsu : 0);
-            Ld.pref = false;
-        }
-        bool lfin = false;
-        {
-            const int t = Ld.t + kseg;
-            const int r_ = lr + (d == 1 ? kseg : d == 0 ? -kseg : 0);
-            const int c_ = lc + (d == 3 ? kseg : d == 2 ? -kseg : 0);
-            int d_ = d;
-            Ld.t = t;
-            if (t == Ld.legEnd) {
-                if (r_ == Ld.dstRow) lfin = true;
-                else { d_ = Ld.dstRow > r_ ? 1 : 0; Ld.legEnd = t + iabs(Ld.dstRow - r_); }
-            }
-            Ld.key = key_of(r_, c_, d_);
-        }
-        // once the leader has finished, L + 1 (if it becomes ready now) is the
-        // next leader and takes no slot
-        const int handId = lfin ? L + 1 : -1;
-        int hand = 0;
-        int4 handRec = make_int4(0, 0, 0, 0);
-        int nkeep = 0;
-        for (int u0 = 0; u0 < nm; u0 += 32) {
-            const int u = u0 + lane;
-            bool fin = false, turn = false;
-            const bool act = u < nm;
-            int si = -1, nsu = 0, newKey = 0, ov = 0;
-            int4 fs4 = make_int4(0, 0, 0, 0);
-            if (act) {
-                si = regM ? mSi : X.Msl[u];
-                const int key = regM ? mKey : SLOTF(X, key, si);
-                const int t = (regM ? mT : SLOTF(X, t, si)) + kseg;
-                const int le = regM ? mLe : SLOTF(X, legEnd, si);
-                int d_ = key_d(key);
-                const int r_ = key_r(key) + (d_ == 1 ? kseg : d_ == 0 ? -kseg : 0);
-                const int c_ = key_c(key) + (d_ == 3 ? kseg : d_ == 2 ? -kseg : 0);
-                int rem = le - t;
-                SLOTF(X, t, si) = (int16_t)t;
-                if (rem == 0) {
-                    const int dr = SLOTF(X, dstRow, si);
-                    fin = r_ == dr;
-                    d_ = dr > r_ ? 1 : 0;
-                    rem = iabs(dr - r_);
-                }
-                if (fin) {
-                    const int id = regM ? mId : SLOTF(X, id, si);
-                    const int4 own = ws.rec[2 * id];
-                    fs4 = ws.rec[2 * id + 1];
-                    nsu = own.z;
-                    ov = own.w;
-                } else {
-                    turn = d_ != d;
-                    newKey = key_of(r_, c_, d_) | (turn ? 0 : KEY_MEM);
-                    SLOTF(X, key, si) = newKey;
-                    if (t + rem != le) SLOTF(X, legEnd, si) = (int16_t)(t + rem);
-                }
-            }
-            // survivors keep their order (stable compaction: straight into the
-            // member arrays when they are held in registers, else into Kb)
-            const bool keep = act && !fin && !turn;
-            const unsigned kb = __ballot_sync(FULL, keep);
-            if (regM) {
-                __syncwarp();
-                if (keep) { X.Mid[__popc(kb & lt)] = mId; X.Msl[__popc(kb & lt)] = si; }
-            } else if (keep) {
-                X.Kb[nkeep + __popc(kb & lt)] = ((long long)X.Mid[u] << 32) | (unsigned)si;
-            }
-            nkeep += __popc(kb);
-            // members whose leg ended become statics
-            push_lanes(X, __ballot_sync(FULL, turn), si, newKey);
-            if (!__any_sync(FULL, fin)) continue;     // nothing finished in this chunk
-            const int off = warp_incl_scan(nsu) - nsu;
-            const int total = __shfl_sync(FULL, off + nsu, 31);
-            // free the finished moves' slots first (their successors may take
-            // them; shared-memory slots are recycled)
-            if (fin) {
-                const int id = SLOTF(X, id, si);
-                if (X.map[id & (MAPN - 1)] == si) X.map[id & (MAPN - 1)] = -1;
-                SLOTF(X, key, si) = 0;
-                SLOTF(X, id, si) = INTMAX;
-            }
-            const bool recyc = fin && si < X.C, recycO = fin && si >= X.C;
-            const unsigned fb = __ballot_sync(FULL, recyc), fo = __ballot_sync(FULL, recycO);
-            if (recyc) X.freeStk[freeTop + __popc(fb & lt)] = (int16_t)si;
-            if (recycO) X.ovfFree[ovfFreeTop + __popc(fo & lt)] = si;
-            freeTop += __popc(fb);
-            ovfFreeTop += __popc(fo);
+            d = dm;
+            const int2 ie = mie[place];
+            lpos = uni(on_clock(mpos[place]));
+            lend = (int)uni((uint32_t)ie.y);
+            --nm;
+            const int2 le = mie[nm];
+            const uint32_t lp = mpos[nm];
             __syncwarp();
-            // successor entries of the finished members, in rounds of SBUF
-            for (int base = 0; base < total; base += SBUF) {
-                if (fin) {
-                    for (int e = max(0, base - off); e < nsu && off + e < base + SBUF; ++e)
-                        X.sbuf[off + e - base] = e == 0 ? fs4.x : e == 1 ? fs4.y : e == 2 ? fs4.z : e == 3 ? fs4.w
-                                                                                                : ~(ov + e - 4);
-                }
-                __syncwarp();
-                const int nb = min(SBUF, total - base);
-                for (int b0 = 0; b0 < nb; b0 += 32) {
-                    const bool has = b0 + lane < nb;
-                    release_round(X, ws, has, has ? X.sbuf[b0 + lane] : 0, handId, hand, handRec, freeTop,
-                                  ovfFreeTop, ovfUsed, hi, k, &err);
-                }
-            }
+            if (lane == 0) { mie[place] = le; mpos[place] = lp; }
+            __syncwarp();
+            int me = INTMAX;
+            for (int u = lane; u < nm; u += 32) me = min(me, mie[u].y);
+            minEnd = __reduce_min_sync(FULL, me);
+            changed = true;
         }
-        // the finished leader's successors, straight from its registers
-        if (lfin && Ld.nsu == 1 && (Ld.s4.x & SUCC_SINGLE)) {
-            // one successor, with no other predecessor: ready now (uniform)
-            const int sid = Ld.s4.x & SUCC_ID;
-            const int4 r = ws.rec[2 * sid];
-            if (sid == handId) { hand = 1; handRec = r; }
-            else {
-                const int si = alloc_slot(X, lane, 1, freeTop, ovfFreeTop, ovfUsed, hi, k, &err);
-                if (lane == 0 && si >= 0) push_both(X, si, fill_slot(X, si, sid, r));
-                __syncwarp();
-            }
-        } else if (lfin) {
-            for (int e0 = 0; e0 < Ld.nsu; e0 += 32) {
-                const int e = e0 + lane;
-                const int32_t v = e == 0 ? Ld.s4.x : e == 1 ? Ld.s4.y : e == 2 ? Ld.s4.z : e == 3 ? Ld.s4.w
-                                                                                            : ~(Ld.ov + e - 4);
-                release_round(X, ws, e < Ld.nsu, v, handId, hand, handRec, freeTop, ovfFreeTop, ovfUsed, hi, k,
-                              &err);
-            }
-        }
-        if (!regM)
-            for (int u = lane; u < nkeep; u += 32) { X.Mid[u] = (int)(X.Kb[u] >> 32); X.Msl[u] = (int)(X.Kb[u] & 0xffffffff); }
-        nm = nkeep;
-        // a line moving across itself carries its index along
-        if (rowLine && d < 2) lineIdx += sgn * kseg;
-        if (!rowLine && d >= 2) lineIdx += sgn * kseg;
         __syncwarp();
-        if (lfin && !err) {
-            // next leader: the lowest unfinished id. L + 1, if it became ready
-            // just now, takes over at once; otherwise the lowest id still held
-            // (usually L + 1): a member leaves the front of the members, a
-            // static its lists
-            if (hand) leader_from_rec(ws, L + 1, handRec, L, Ld);
+        look_ahead();
+        return true;
+    };
+
+    if (!find_leader() || L != 0) err = RR_ERR_INTERNAL;
+    int evEnd = lend;         // the first leg end of the batch
+    while (!err) {
+        // the statics of the leader's direction: the distance to the nearest
+        // line ahead that holds one, 0 when one stands on a line of the leader's
+        const int tb = base(d);
+        if (MODE == SIM_WIDE) { groups = size(d) >> 3; off = 8 * min(lane, groups - 1); }
+        const uint32_t nadd = 0x10000u - lpos;
+        uint4 a = *(const uint4 *)(pos + tb + off), b = *(const uint4 *)(pos + tb + off + 4);
+        uint32_t v = min8(a, b, nadd, HOLE);
+        if (MODE != SIM_SMALL)
+            for (int g = lane + 32; g < groups; g += 32) {
+                const uint4 a2 = *(const uint4 *)(pos + tb + 8 * g), b2 = *(const uint4 *)(pos + tb + 8 * g + 4);
+                v = min8(a2, b2, nadd, v);
+            }
+        int pick = (int)__reduce_min_sync(FULL, v < 0x10000u ? 0u : v & 0xffffu);
+        if (pick == 0) {
+            const unsigned ba = __ballot_sync(FULL, (v & 0xffffu) == 0u), bc = __ballot_sync(FULL, v < 0x10000u);
+            bool choose;
+            if (bc == 0u && (nm == 0 || prim)) choose = true;
+            else if (ba == 0u && (nm == 0 || !prim)) choose = false;
             else {
-                int cand = -1;
-                const int nx = L + 1;
-                if (nx < k) {
-                    const int si = X.map[nx & (MAPN - 1)];
-                    if (si >= 0 && SLOTF(X, id, si) == nx) cand = si;
+                // candidates on both lines: the smaller smallest id decides
+                int ma = INTMAX, mc = INTMAX;
+                for (int g = lane; g < groups; g += 32) {
+                    const int e = tb + 8 * g;
+                    if (MODE != SIM_SMALL) { a = *(const uint4 *)(pos + e); b = *(const uint4 *)(pos + e + 4); }
+                    for (unsigned q = match8(a, b, lpos, 0xffffu); q; q &= q - 1) ma = min(ma, ir[e + __ffs(q) - 1].x);
+                    for (unsigned q = match8(a, b, lpos, 0xffff0000u); q; q &= q - 1) mc = min(mc, ir[e + __ffs(q) - 1].x);
                 }
-                if (cand < 0) cand = lowest_slot(X, hi);
-                if (cand < 0) L = k;
-                else {
-                    const int kk = SLOTF(X, key, cand);
-                    if (kk & KEY_MEM) {
-                        if (nm == 0 || X.Msl[0] != cand) { err = RR_ERR_INTERNAL; break; }
-                        __syncwarp();
-                        for (int u = lane; u + 1 < nm; u += 32) X.Kb[u] = ((long long)X.Mid[u + 1] << 32) | (unsigned)X.Msl[u + 1];
-                        __syncwarp();
-                        --nm;
-                        for (int u = lane; u < nm; u += 32) { X.Mid[u] = (int)(X.Kb[u] >> 32); X.Msl[u] = (int)(X.Kb[u] & 0xffffffff); }
-                    } else if (lane == 0) {
-                        unlink_row(X, cand, kk);
-                        unlink_col(X, cand, kk);
+                for (int u = lane; u < nm; u += 32) {
+                    const int id = mie[u].x;
+                    if (prim) ma = min(ma, id); else mc = min(mc, id);
+                }
+                choose = __reduce_min_sync(FULL, ma) < __reduce_min_sync(FULL, mc);
+                if (nm > 0 && choose != prim) dissolve();
+            }
+            if (choose ? ba : bc) {
+                // the chosen line's statics join the members
+                int me = minEnd, fr = C->nfree[d];
+                __syncwarp();
+                const uint32_t half = choose ? 0xffffu : 0xffff0000u;
+                for (int g0 = 0; g0 < groups; g0 += 32) {
+                    const int e0 = tb + 8 * (g0 + lane);
+                    unsigned q = 0;
+                    if (MODE == SIM_SMALL) {
+                        q = lane < groups ? match8(a, b, lpos, half) : 0u;
+                    } else if (g0 + lane < groups) {
+                        q = match8(*(const uint4 *)(pos + e0), *(const uint4 *)(pos + e0 + 4), lpos, half);
+                    }
+                    for (unsigned bal = __ballot_sync(FULL, q != 0u); bal; bal = __ballot_sync(FULL, q != 0u)) {
+                        const int n = __popc(bal);
+                        if (nm + n > lineCap) { err = RR_ERR_INTERNAL; break; }
+                        const bool c = q != 0u;
+                        const int i = c ? 31 - __clz(q) : 0, e = e0 + i, rank = __popc(bal & lt), u = nm + rank;
+                        q &= ~(1u << i);
+                        if constexpr (MODE == SIM_WIDE) {
+                            if (c) {
+                                const int2 x = ir[e];
+                                mie[u] = make_int2(x.x, x.y + clk);
+                                mpos[u] = (pos[e] & 0xffff0000u) | ((pos[e] - (uint32_t)clk) & 0xffffu);
+                                pos[e] = HOLE;
+                                stk[tb + fr + rank] = (ST)(e - tb);
+                                me = min(me, x.y + clk);
+                            }
+                        } else {
+                            const int ec = c ? e : tb;
+                            const int2 x = ir[ec];
+                            const uint32_t p = pos[ec];
+                            const int end = x.y + clk;
+                            st_if(c, mie + u, x.x, end);
+                            st_if(c, mpos + u, (p & 0xffff0000u) | ((p - (uint32_t)clk) & 0xffffu));
+                            st_if(c, pos + e, HOLE);
+                            st_if(c, stk + tb + fr + rank, e - tb);
+                            if (c) me = min(me, end);
+                            // its record and its likeliest successor's: read when it finishes
+                            touch_rec_if(c, rec, x.x, dump);
+                            touch_rec_if(c, rec, x.x + 1, dump);
+                        }
+                        nm += n;
+                        fr += n;
+                    }
+                    if (MODE == SIM_SMALL || err) break;
+                }
+                if (err) break;
+                if (lane == 0) C->nfree[d] = fr;
+                minEnd = __reduce_min_sync(FULL, me);
+                prim = choose;
+                dm = d;
+                line = choose ? (int)(lpos & 0xffffu) - clk : (int)(lpos >> 16);
+                changed = true;
+                __syncwarp();
+            }
+            evEnd = min(lend, minEnd);
+            // the nearest line ahead of the leader's own (those that have just
+            // joined along its line of motion are further than its leg's end)
+            v = min8(a, b, nadd - 1u, HOLE);
+            if (MODE != SIM_SMALL)
+                for (int g = lane; g < groups; g += 32) {
+                    const uint4 a2 = *(const uint4 *)(pos + tb + 8 * g), b2 = *(const uint4 *)(pos + tb + 8 * g + 4);
+                    v = min8(a2, b2, nadd - 1u, v);
+                }
+            pick = (int)__reduce_min_sync(FULL, v & 0xffffu) + 1;
+        }
+        // the segment: up to the first leg end or the nearest line ahead
+        const int kseg = min(pick, evEnd - clk);
+        if (logging) {
+            if (changed) {
+                changed = false;
+                idTop -= (unsigned)nm;
+                list = idTop;
+                for (int u0 = 0; u0 < nm; u0 += 32)
+                    if (u0 + lane < nm) log[list + u0 + lane] = mie[u0 + lane].x;
+            }
+            if (lane == 0) hdr[nseg] = make_uint4((unsigned)clk, nmem, list, (unsigned)L | (unsigned)d << 30);
+            ++nseg;
+        } else {
+            const unsigned long long o1 = (unsigned long long)clk + kseg, m1 = nmem + (unsigned long long)kseg * (nm + 1);
+            if (o1 <= (unsigned long long)I->cap_ops && m1 <= (unsigned long long)I->cap_members) {
+                for (int u = lane; u < nm; u += 32) ids[u] = mie[u].x;
+                __syncwarp();
+                write_segment(as_global(I->ops), as_global(I->members), (unsigned)clk, nmem, kseg, nm + 1, d, L, ids, buf);
+            }
+        }
+        // everything in the batch advances
+        nmem += (unsigned)(kseg * (nm + 1));
+        clk += kseg;
+        lpos += (uint32_t)kseg;
+        if (--left == 0) {
+            if (guard <= 0) { err = RR_ERR_TIMEOUT; break; }
+            if (kseg < 1) { err = RR_ERR_INTERNAL; break; }
+            if (MODE != SIM_WIDE && *(volatile int *)&C->full) break;
+            left = guard < 32 ? (int)guard : 32;
+            guard -= left;
+            if (logging) {
+                // a header follows the published segments (it says where they
+                // end); without room for the next 32 segments the rest is
+                // written here, above
+                if (lane == 0) hdr[nseg] = make_uint4((unsigned)clk, nmem, 0u, 0u);
+                __syncwarp();
+                __threadfence_block();
+                if (lane == 0) *(volatile int *)&C->pub = (int)nseg;
+                logging = 4u * nseg + LOG_SLACK(lineCap) <= idTop;
+            }
+        }
+        if (clk != evEnd) continue;
+        bool fin = false, moved = false;
+        int4 nr = make_int4(0, 0, 0, 0), ns4 = nr;
+        if (clk == lend) {
+            // the next id's record (an entry beyond the last one exists)
+            nr = rec[2 * (size_t)(L + 1)];
+            ns4 = rec[2 * (size_t)(L + 1) + 1];
+            moved = true;
+            if (d < 2 || ldst == (int)(lpos >> 16) - 1) fin = true;
+            else {
+                const Leg g = second_leg(d, lpos, ldst);
+                d = g.d; lpos = g.pos; lend = clk + g.rem;
+            }
+        }
+        // once the leader has finished, the next id (if it becomes ready now)
+        // is the next leader and enters no table
+        const int handId = fin ? L + 1 : -1;
+        bool hand = false;
+        if (clk == minEnd) {
+            // members whose leg ended leave: they turn (into the tables) or
+            // finish (and release their successors)
+            int nk = 0, me = INTMAX;
+            for (int u0 = 0; u0 < nm; u0 += 32) {
+                const int u = u0 + lane;
+                const bool act = u < nm;
+                const int2 ie = mie[act ? u : u0];
+                const uint32_t p = mpos[act ? u : u0];
+                const bool ended = act && ie.y == clk, keep = act && ie.y != clk;
+                const unsigned kb = __ballot_sync(FULL, keep);
+                me = keep ? min(me, ie.y) : me;
+                const int w = nk + __popc(kb & lt);
+                if (nk != u0 || kb != FULL) {                          // some move up
+                    __syncwarp();
+                    st_if(keep, mie + w, ie.x, ie.y);
+                    st_if(keep, mpos + w, p);
+                    if (__any_sync(FULL, ended)) {
+                        int4 r = ldg_if(ended, rec + 2 * (size_t)ie.x), s = ldg_if(ended, rec + 2 * (size_t)ie.x + 1);
+                        if (dm >= 2) {
+                            const int dst = r.y >> 13 & 1023;
+                            const bool turn = ended && dst != (int)(p >> 16) - 1;
+                            const Leg g = second_leg(dm, on_clock(p), dst);
+                            enter(turn, g.d, g.pos, ie.x, g.rem);
+                            if (turn) r.z = 0;
+                        }
+                        const int most = (int)uni((uint32_t)r.z);
+                        for (int e = 0; e < most; ++e) {
+                            int32_t v = e == 0 ? s.x : e == 1 ? s.y : e == 2 ? s.z : s.w;
+                            if (e >= 4) v = ldg_if(e < r.z, (const void *)(succ + r.w + e - 4));
+                            hand |= release(e < r.z, v, handId);
+                        }
                     }
                     __syncwarp();
-                    leader_from_slot(X, ws, cand, L, Ld, freeTop, ovfFreeTop);
                 }
+                nk += __popc(kb);
+            }
+            nm = nk;
+            minEnd = __reduce_min_sync(FULL, me);
+            changed = true;
+        }
+        if (fin) {
+            if (chain) hand = true;
+            else {
+                const int n = (int)uni((uint32_t)nsu);
+                for (int e0 = 0; e0 < n; e0 += 32) {
+                    const int e = e0 + lane;
+                    int32_t v = e == 0 ? s4.x : e == 1 ? s4.y : e == 2 ? s4.z : s4.w;
+                    if (n > 4) {
+                        const int w = ldg_if(e >= 4 && e < n, (const void *)(succ + ov + e - 4));
+                        v = e >= 4 ? w : v;
+                    }
+                    hand |= release(e < n, v, handId);
+                }
+                hand = __any_sync(FULL, hand);
+                __syncwarp();
+            }
+            if (hand) {
+                L = handId;
+                lpos = uni((uint32_t)nr.x);
+                set_leg(uni((uint32_t)nr.y));
+                nsu = nr.z;
+                ov = nr.w;
+                s4 = ns4;
+                look_ahead();
+            } else if (!find_leader()) {
+                break;
             }
         }
-        __syncwarp();
+        // members no longer on the leader's line or in its direction?
+        if (moved && nm > 0 && !(dm == d && line == (prim ? (int)(lpos & 0xffffu) - clk : (int)(lpos >> 16)))) dissolve();
+        evEnd = min(lend, minEnd);
     }
+    // the log's end: a header with the totals, everything published
+    touch_wait();
+    __syncwarp();
+    if (logging && lane == 0) hdr[nseg] = make_uint4((unsigned)clk, nmem, 0u, 0u);
     if (lane == 0) {
-        I->n_ops = nop;
+        I->n_ops = clk;
         I->n_members = nmem;
-        if (err) I->status = err;
-        else if (nmem != I->n_steps) I->status = RR_ERR_INTERNAL;
-        else if (overflow) I->status = RR_ERR_CAPACITY;
     }
+    if (MODE != SIM_WIDE && *(volatile int *)&C->full) err = RR_SIM_RETRY;
+    if (!err && (long long)nmem != I->n_steps) err = RR_ERR_INTERNAL;
+    if (!err && ((int64_t)clk > I->cap_ops || (int64_t)nmem > I->cap_members)) err = RR_ERR_CAPACITY;
+    __syncwarp();
+    __threadfence_block();
+    if (lane == 0) {
+        *(volatile int *)&C->pub = (int)nseg;
+        __threadfence_block();
+        *(volatile int *)&C->fin = 1;
+    }
+    __syncwarp();
+    return err;
 }
 
-// ------------------------------------------------- small-grid simulation
-//
-// Alg. 4 for one small instance with the ready set in warp registers. At most
-// SMALL_CAP moves may be ready at once: two per lane, slot j = 32 p + lane of
-// plane p, kept sorted by move id, so that slot 0 holds the leader (the
-// lowest unfinished id) and a ballot in slot order lists candidates in id
-// order. Every segment is recomputed from the registers: the batch is the
-// leader plus every ready move of its direction on its row (set A) or on its
-// column (set B), whichever holds the lower id (the same rule as sim_body);
-// the segment ends at the first leg end of a batch move or where the leader
-// reaches a row (vertical moves) or column (horizontal ones) holding a ready
-// move of its direction. Finishing moves release their successors (in-degrees
-// in shared memory) and the ready set is re-sorted through shared memory.
-// The move records are staged in shared memory first. An instance with more
-// than SMALL_MAX_MOVES moves, or more than SMALL_CAP ready at once, is left to
-// sim_body (status RR_SIM_RETRY: its wide pass redoes it from the start).
-constexpr int SMALL_CAP = 64;
-constexpr int SMALL_MAX_MOVES = 2048;
-constexpr int SMALL_SBUF = 128;   // successor entries released per round
+// A block's shared memory (sim_smem_bytes), the tables apart.
+struct SimLayout {
+    int MC;                   // room of the members
+    int2 *mie;
+    uint32_t *mpos;
+    SimCtl *C;
+    int32_t *bufs, *ids;      // a sort buffer per warp, a list of ids
+    int32_t *dump;            // 16 bytes that nothing reads
+    unsigned *cnt;
+    __device__ __forceinline__ SimLayout(char *smem, int side)
+    {
+        MC = (side + 7) & ~7;
+        mie = (int2 *)(smem + 14 * 4 * sim_cap(side));
+        mpos = (uint32_t *)(mie + MC);
+        C = (SimCtl *)(mpos + MC);
+        bufs = (int32_t *)(C + 1);
+        ids = bufs + sim_pow2(side) * (int)(blockDim.x >> 5);
+        dump = ids + MC;
+        cnt = (unsigned *)(dump + 4);
+    }
+};
 
-__host__ __device__ inline size_t small_smem_bytes()
+template <int MODE>
+__device__ __forceinline__ int sim_run(Sim<MODE> &S, rr_instance *I, JobWS &ws, const SimLayout &Y, int counters)
 {
-    return 32ull * SMALL_MAX_MOVES + 4ull * SMALL_MAX_MOVES +      // records, in-degrees
-           16ull * SMALL_CAP + 4ull * SMALL_CAP +                  // re-sort staging, sorted survivor ids
-           4ull * (SMALL_CAP + 32) + 4ull * SMALL_SBUF + 4ull * (SMALL_CAP + 2);   // new ids, successors, batch
+    S.mie = Y.mie; S.mpos = Y.mpos; S.C = Y.C;
+    S.rec = as_global(ws.rec); S.succ = as_global(ws.succ); S.multi = as_global(ws.multi);
+    S.multiId = as_global(ws.multiId); S.multiPos = as_global(ws.multiPos);
+    S.cnt = Y.cnt;
+    S.dump = sh_addr(Y.dump);
+    S.ncnt = min(counters, ws.nmulti);
+    S.allShared = counters >= ws.nmulti;
+    // the log: the chains of the conflict graph are no longer needed
+    return S.run(I, ws, as_global(ws.nextAt), (unsigned)((4 * (ws.P + 1) + 255) / 256 * 64), Y.MC, Y.bufs, Y.ids);
 }
 
-struct SmallSlot { int32_t id, key, rem, dst; };
-
-__device__ __forceinline__ SmallSlot small_from_rec(int id, int4 r)
+// The tables in global memory, for an instance that outgrew shared memory.
+static __device__ __noinline__ int sim_wide(rr_instance *I, JobWS *ws, char *smem, int side, int counters)
 {
-    const int sr = r.x & 0xffff, sc = r.x >> 16, dr = r.y & 0xffff, dc = r.y >> 16;
-    const int d = dc != sc ? (dc > sc ? 3 : 2) : (dr > sr ? 1 : 0);
-    return SmallSlot{id, key_of(sr, sc, d), dc != sc ? iabs(dc - sc) : iabs(dr - sr), dr};
+    const size_t n = sim_wide_entries(I->n_moves);
+    Sim<SIM_WIDE> S;
+    S.pos = (uint32_t *)ws->slotOvf;
+    S.ir = (int2 *)(S.pos + n);
+    S.stk = (int32_t *)(S.ir + n);
+    S.cap = 0;
+    return sim_run(S, I, *ws, SimLayout(smem, side), counters);
 }
 
-// Returns with I->status unchanged (done), RR_SIM_RETRY (left to sim_body) or
-// an error status. One warp; `sm` is this warp's shared memory.
-__device__ inline void sim_small(rr_instance *I, JobWS &ws, char *sm)
+// The whole simulation of one instance by one block (every thread calls it):
+// warp 0 simulates, the others write, warp 0 writes too once it is done.
+// An instance that outgrows the shared-memory tables starts over with its
+// tables in global memory (the batches written so far are the same ones).
+template <int MODE>
+__device__ __forceinline__ void sim_block(rr_instance *I, JobWS &ws, char *smem, int side, int counters)
 {
-    const int lane = threadIdx.x & 31;
-    const unsigned lt = (1u << lane) - 1u;
-    if (!live(I)) return;
+    const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int k = (int)I->n_moves;
-    if (k == 0) { if (lane == 0) { I->n_ops = 0; I->n_members = 0; } return; }
-    if (k > SMALL_MAX_MOVES) { if (lane == 0) I->status = RR_SIM_RETRY; return; }
-    int4 *recs = (int4 *)sm;                                   // 2 per move: geometry, first successors
-    int32_t *indeg = (int32_t *)(recs + 2 * SMALL_MAX_MOVES);
-    SmallSlot *stage = (SmallSlot *)(indeg + SMALL_MAX_MOVES);
-    int32_t *survIds = (int32_t *)(stage + SMALL_CAP);
-    int32_t *newIds = survIds + SMALL_CAP;
-    int32_t *sbuf = newIds + SMALL_CAP + 32;
-    int32_t *bat = sbuf + SMALL_SBUF;
-    for (int i = lane; i < 2 * k; i += 32) recs[i] = ws.rec[i];
-    for (int i = lane; i < k; i += 32) indeg[i] = ws.indeg[i];
-    __syncwarp();
-
-    // the initially ready moves, sorted by id
-    const int n0 = ws.ready0[k];
-    if (n0 > SMALL_CAP) { if (lane == 0) I->status = RR_SIM_RETRY; return; }
-    for (int i = lane; i < n0; i += 32) newIds[i] = ws.ready0[i];
-    __syncwarp();
-    SmallSlot S0{INTMAX, 0, 0, 0}, S1{INTMAX, 0, 0, 0};
-    for (int i = lane; i < n0; i += 32) {
-        const int id = newIds[i];
-        int r = 0;
-        for (int j = 0; j < n0; ++j) r += newIds[j] < id;
-        stage[r] = small_from_rec(id, recs[2 * id]);
+    if (!live(I)) return;                       // the same in every thread: set before this kernel or a barrier
+    if (k == 0) {
+        if (threadIdx.x == 0) { I->n_ops = 0; I->n_members = 0; }
+        return;
     }
-    __syncwarp();
-    if (lane < n0) S0 = stage[lane];
-    if (32 + lane < n0) S1 = stage[32 + lane];
-    __syncwarp();
+    const int cap = sim_cap(side);
+    const SimLayout Y(smem, side);
+    Sim<MODE> S;
+    S.pos = (uint32_t *)smem;
+    S.ir = (int2 *)(S.pos + 4 * cap);
+    S.stk = (uint16_t *)(S.ir + 4 * cap);
+    S.cap = cap;
+    SimCtl *C = Y.C;
 
-    const int64_t cap_ops = I->cap_ops, cap_mem = I->cap_members;
-    rr_op *ops = I->ops;
-    int32_t *mem = I->members;
-    int64_t nop = 0, nmem = 0;
-    int overflow = 0, err = 0, done = 0;
-    const int64_t guard_max = g_guard_cap > 0 ? g_guard_cap : I->n_steps + 2ll * k + 16;
-    for (int64_t guard = 0;; ++guard) {
-        if (guard >= guard_max) { err = RR_ERR_TIMEOUT; break; }
-        const int Lid = __shfl_sync(FULL, S0.id, 0);
-        if (Lid == INTMAX) break;
-        const int Lkey = __shfl_sync(FULL, S0.key, 0);
-        const int d = key_d(Lkey), lr = key_r(Lkey), lc = key_c(Lkey);
-        const bool vert = d < 2;
-        const int sgn = (d == 1 || d == 3) ? 1 : -1;
-        // candidates: ready moves of direction d, the leader excluded
-        const bool same0 = S0.id != INTMAX && key_d(S0.key) == d && lane != 0;
-        const bool same1 = S1.id != INTMAX && key_d(S1.key) == d;
-        const unsigned bR0 = __ballot_sync(FULL, same0 && key_r(S0.key) == lr);
-        const unsigned bC0 = __ballot_sync(FULL, same0 && key_c(S0.key) == lc);
-        const unsigned bR1 = __ballot_sync(FULL, same1 && key_r(S1.key) == lr);
-        const unsigned bC1 = __ballot_sync(FULL, same1 && key_c(S1.key) == lc);
-        unsigned m0 = 0u, m1 = 0u;
-        if (bR0 | bC0) {
-            const int f = __ffs(bR0 | bC0) - 1;
-            const bool row = (bR0 >> f) & 1u;
-            m0 = row ? bR0 : bC0;
-            m1 = row ? bR1 : bC1;
-        } else if (bR1 | bC1) {
-            const int f = __ffs(bR1 | bC1) - 1;
-            const bool row = (bR1 >> f) & 1u;
-            m1 = row ? bR1 : bC1;
+    for (int pass = 0;; ++pass) {
+        if (threadIdx.x < 4) C->nfree[threadIdx.x] = pass == 0 ? cap : 0;
+        if (threadIdx.x == 0) {
+            C->full = C->pub = C->next = C->fin = 0;
+            C->status = RR_OK;
         }
-        const bool in0 = lane == 0 || ((m0 >> lane) & 1u), in1 = (m1 >> lane) & 1u;
-        const int ns = 1 + __popc(m0) + __popc(m1);
-        // segment length: the first leg end in the batch, the nearest ready
-        // move of direction d on a line ahead of the leader
-        auto limit = [&](const SmallSlot &S, bool inB, bool same) {
-            if (inB) return S.rem;
-            if (same) {
-                const int dist = (vert ? key_r(S.key) - lr : key_c(S.key) - lc) * sgn;
-                if (dist > 0) return dist;
-            }
-            return INTMAX;
-        };
-        const int kseg = __reduce_min_sync(FULL, min(limit(S0, in0, same0), limit(S1, in1, same1)));
-        if (kseg < 1 || kseg == INTMAX) { err = RR_ERR_INTERNAL; break; }
-        // kseg identical batches: ids in rank order (leader first, then slot order)
-        const int64_t addm = (int64_t)kseg * ns;
-        if (!overflow && nop + kseg <= cap_ops && nmem + addm <= cap_mem) {
-            for (int i = lane; i < kseg; i += 32) ops[nop + i] = rr_op{d, (int32_t)(nmem + (int64_t)i * ns), ns};
-            // the batch's ids in rank order: the leader, then the members in
-            // slot (id) order
-            if (in0) bat[lane == 0 ? 0 : 1 + __popc(m0 & lt)] = S0.id;
-            if (in1) bat[1 + __popc(m0) + __popc(m1 & lt)] = S1.id;
-            __syncwarp();
-            if (ns <= 32) {
-                // lane r writes the r-th member of every batch of the segment
-                const int v = lane < ns ? bat[lane] : 0;
-                if (lane < ns)
-                    for (int i = 0; i < kseg; ++i) mem[nmem + (int64_t)i * ns + lane] = v;
-                __syncwarp();
-            } else {
-                int u = small_mod(lane, ns);
-                const int step = small_mod(32, ns);
-                for (int64_t i = lane; i < addm; i += 32) {
-                    mem[nmem + i] = bat[u];
-                    u += step;
-                    if (u >= ns) u -= ns;
-                }
-                __syncwarp();
+        // entries are handed out from a table's start
+        if (pass == 0) {
+            for (int i = threadIdx.x; i < 4 * cap; i += blockDim.x) {
+                S.pos[i] = HOLE;
+                S.stk[i] = (uint16_t)(cap - 1 - i % cap);
             }
         } else {
-            overflow = 1;
-        }
-        nop += kseg;
-        nmem += addm;
-        // advance the batch; at a leg end a move turns toward its
-        // destination row or finishes there
-        bool fin0 = false, fin1 = false;
-        auto advance = [&](SmallSlot &S, bool inB) {
-            if (!inB) return false;
-            int r = key_r(S.key), c = key_c(S.key), dd = key_d(S.key);
-            if (dd == 0) r -= kseg; else if (dd == 1) r += kseg; else if (dd == 2) c -= kseg; else c += kseg;
-            S.rem -= kseg;
-            if (S.rem == 0) {
-                if (r == S.dst) { S.key = key_of(r, c, dd); return true; }
-                dd = S.dst > r ? 1 : 0;
-                S.rem = iabs(S.dst - r);
+            // as many entries per direction as there are legs of it (rounded
+            // up to eight, at least eight)
+            __syncthreads();
+            for (int b = threadIdx.x; b < k; b += blockDim.x) {
+                const int4 r = ws.rec[2 * (size_t)b];
+                const int d = r.y & 3, dst = r.y >> 13 & 1023, row = (int)((uint32_t)r.x >> 16) - 1;
+                atomicAdd(&C->nfree[d], 1);
+                if (d >= 2 && dst != row) atomicAdd(&C->nfree[dst > row ? 1 : 0], 1);
             }
-            S.key = key_of(r, c, dd);
-            return false;
-        };
-        fin0 = advance(S0, in0);
-        fin1 = advance(S1, in1);
-        const unsigned f0 = __ballot_sync(FULL, fin0), f1 = __ballot_sync(FULL, fin1);
-        if (!(f0 | f1)) continue;
-        done += __popc(f0) + __popc(f1);
-        // release the finished moves' successors, one finished move at a time
-        // (lane e takes successor e); newly ready ids go to newIds
-        int nn = 0;
-        for (unsigned fm0 = f0, fm1 = f1; fm0 | fm1;) {
-            int src, pl;
-            if (fm0) { src = __ffs(fm0) - 1; fm0 &= fm0 - 1; pl = 0; }
-            else { src = __ffs(fm1) - 1; fm1 &= fm1 - 1; pl = 1; }
-            const int a0 = __shfl_sync(FULL, S0.id, src), a1 = __shfl_sync(FULL, S1.id, src);
-            const int fid = pl ? a1 : a0;
-            const int4 g = recs[2 * fid];
-            const int32_t *s4 = (const int32_t *)&recs[2 * fid + 1];
-            for (int e0 = 0; e0 < g.z; e0 += 32) {
-                const int e = e0 + lane;
-                int ready = -1;
-                if (e < g.z) {
-                    const int v = e < 4 ? s4[e] : ws.succ[g.w + e - 4];
-                    const int sid = v & SUCC_ID;
-                    if ((v & SUCC_SINGLE) || atomicSub(&indeg[sid], 1) == 1) ready = sid;
+            __syncthreads();
+            if (threadIdx.x == 0) {
+                int at = 0;
+                for (int d = 0; d < 4; ++d) {
+                    C->wbase[d] = at;
+                    C->nfree[d] = C->wcap[d] = max(8, (C->nfree[d] + 7) & ~7);
+                    at += C->wcap[d];
                 }
-                const unsigned bal = __ballot_sync(FULL, ready >= 0);
-                if (ready >= 0 && nn + __popc(bal & lt) < 32) newIds[nn + __popc(bal & lt)] = ready;
-                nn += __popc(bal);
             }
+            __syncthreads();
+            const size_t n = sim_wide_entries(k);
+            uint32_t *p = (uint32_t *)ws.slotOvf;
+            int32_t *st = (int32_t *)(p + 3 * n);
+            for (int d = 0; d < 4; ++d)
+                for (int i = threadIdx.x; i < C->wcap[d]; i += blockDim.x) {
+                    p[C->wbase[d] + i] = HOLE;
+                    st[C->wbase[d] + i] = C->wcap[d] - 1 - i;
+                }
+            // the first pass counted in-degrees down: start over
+            for (int x = threadIdx.x; x < ws.nmulti; x += blockDim.x) ws.multi[x] = (ws.multi[x] & ~MULTI_COUNT) | ws.indeg[ws.multiId[x]];
         }
-        // the ready set again, sorted: survivors keep their order, newly ready
-        // moves go between them by id
-        const bool sv0 = S0.id != INTMAX && !fin0, sv1 = S1.id != INTMAX && !fin1;
-        const unsigned b0v = __ballot_sync(FULL, sv0), b1v = __ballot_sync(FULL, sv1);
-        const int nsv = __popc(b0v) + __popc(b1v);
-        if (nn > 32 || nsv + nn > SMALL_CAP) { if (lane == 0) I->status = RR_SIM_RETRY; return; }
-        __syncwarp();
-        const int myNew = lane < nn ? newIds[lane] : INTMAX;
-        int c0 = 0, c1 = 0, posNew = 0;
-        for (int t = 0; t < nn; ++t) {
-            const int id = __shfl_sync(FULL, myNew, t);
-            const int below = __popc(__ballot_sync(FULL, sv0 && S0.id < id)) +
-                              __popc(__ballot_sync(FULL, sv1 && S1.id < id)) +
-                              __popc(__ballot_sync(FULL, myNew < id));
-            if (lane == t) posNew = below;
-            c0 += sv0 && id < S0.id;
-            c1 += sv1 && id < S1.id;
+        __syncthreads();
+        unsigned short *c16 = (unsigned short *)Y.cnt;
+        const int ncnt = min(counters, ws.nmulti);
+        for (int i = threadIdx.x; i < ncnt; i += blockDim.x) c16[i] = (unsigned short)(ws.multi[i] & MULTI_COUNT);
+        __syncthreads();
+        if (wid == 0) {
+            const int st = pass == 0 ? sim_run(S, I, ws, Y, counters) : sim_wide(I, &ws, smem, side, counters);
+            if (lane == 0) C->status = st;
+            __syncwarp();
         }
-        if (sv0) stage[__popc(b0v & lt) + c0] = S0;
-        if (sv1) stage[__popc(b0v) + __popc(b1v & lt) + c1] = S1;
-        if (lane < nn) stage[posNew] = small_from_rec(myNew, recs[2 * myNew]);
-        __syncwarp();
-        const int T = nsv + nn;
-        S0 = lane < T ? stage[lane] : SmallSlot{INTMAX, 0, 0, 0};
-        S1 = 32 + lane < T ? stage[32 + lane] : SmallSlot{INTMAX, 0, 0, 0};
-        __syncwarp();
-    }
-    if (lane == 0) {
-        I->n_ops = nop;
-        I->n_members = nmem;
-        if (err) I->status = err;
-        else if (done != k || nmem != I->n_steps) I->status = RR_ERR_INTERNAL;
-        else if (overflow) I->status = RR_ERR_CAPACITY;
+        run_writers(C, I, as_global(ws.nextAt), Y.bufs + sim_pow2(side) * wid);
+        __syncthreads();
+        const int st = C->status;
+        if (st != RR_SIM_RETRY || pass == 1 || k < SIM_WIDE_MIN) {
+            if (threadIdx.x == 0 && st != RR_OK) I->status = st == RR_SIM_RETRY ? RR_ERR_INTERNAL : st;
+            break;
+        }
+        __syncthreads();
     }
 }
-
 
 } // namespace rrk

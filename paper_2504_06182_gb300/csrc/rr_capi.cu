@@ -29,10 +29,8 @@ __global__ void k_classify(rr_instance *, int, int, int, int *, int *);
 __global__ void k_order(const rr_instance *, int, int *);
 __global__ void k_gather(const rr_instance *, const int *, rr_instance *);
 __global__ void k_scatter(rr_instance *, const int *, const rr_instance *, int);
-__global__ void k_sim16(rr_instance *, JobWS *, int, const int *, const int *, int, int);
-__global__ void k_sim32(rr_instance *, JobWS *, int, const int *, const int *, int, int);
-__global__ void k_sim16w(rr_instance *, JobWS *, int, const int *, const int *, int, int);
-__global__ void k_sim32w(rr_instance *, JobWS *, int, const int *, const int *, int, int);
+__global__ void k_sim(rr_instance *, JobWS *, int, const int *, const int *, int, int);
+__global__ void k_sim_big(rr_instance *, JobWS *, int, const int *, const int *, int, int);
 }  // namespace rrk
 
 using namespace rrk;
@@ -43,7 +41,7 @@ static_assert(sizeof(rr_instance) == 128, "rr_instance layout is part of the ABI
 static constexpr int SMALL_CALL = 8;
 
 // Kernels launched with more than the default 48 KB of dynamic shared memory.
-enum { SM_GSORT, SM_GSWEEP_H, SM_GSWEEP_V, SM_SIM16, SM_SIM32, SM_SIM16W, SM_SIM32W, SM_BIRD, SM_ONE, SM_NKERNEL };
+enum { SM_GSORT, SM_GSWEEP_H, SM_GSWEEP_V, SM_SIM, SM_SIM_BIG, SM_BIRD, SM_ONE, SM_NKERNEL };
 
 struct rr_ctx {
     int device;
@@ -139,8 +137,7 @@ static int smem_limits(int dev, int *out)
         int optin = 0;
         cudaError_t e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
         const void *fn[SM_NKERNEL] = {(const void *)k_gsort, (const void *)k_gsweep_h, (const void *)k_gsweep_v,
-                                      (const void *)k_sim16, (const void *)k_sim32, (const void *)k_sim16w,
-                                      (const void *)k_sim32w, (const void *)k_bird, one_kernel()};
+                                      (const void *)k_sim, (const void *)k_sim_big, (const void *)k_bird, one_kernel()};
         for (int i = 0; e == cudaSuccess && i < SM_NKERNEL; ++i) {
             cudaFuncAttributes fa;
             e = cudaFuncGetAttributes(&fa, fn[i]);
@@ -356,6 +353,22 @@ static int launch_plan(rr_ctx *ctx, rr_instance *d_inst, JobWS *ws, int count, i
     return RR_OK;
 }
 
+// A simulation block: its warps (one simulates, the others write) and its
+// in-degree counters in shared memory. A call over few grids leaves most of
+// the machine idle: more writers, and counters for every move that needs one.
+struct SimShape { int warps, counters; size_t smem; };
+static SimShape sim_shape(const rr_ctx *ctx, int count, int side)
+{
+    SimShape s;
+    const bool few = count <= ctx->nsm;
+    const int limit = std::min(ctx->smemLimit[SM_SIM], ctx->smemLimit[SM_SIM_BIG]);
+    s.warps = few ? 4 : 2;
+    const int room = (limit - (int)sim_smem_bytes(side, s.warps, 0)) / 2 - 8;
+    s.counters = std::max(0, std::min(side * side / (few ? 4 : 12), room)) & ~7;
+    s.smem = sim_smem_bytes(side, s.warps, s.counters);
+    return s;
+}
+
 // Simulation launch shapes: per size class on forked streams, or one launch
 // over every instance of the call on its stream.
 enum { SIM_CLASSES = 0, SIM_ONE = 1 };
@@ -403,10 +416,8 @@ static int launch_batch(rr_ctx *ctx, rr_instance *d_inst, JobWS *ws, int count, 
     k_bsucc<<<dim3(pathBlocks, count), 256, 0, s>>>(d_inst, ws, count);
     mark(ctx, s, "k_brec");
     k_brec<<<dim3(pathBlocks, count), 256, 0, s>>>(d_inst, ws, count);
-    // simulation: one warp per instance, launched per size class on forked
-    // streams so that each class's shared memory fits its own grids; slot
-    // table, static lists and buffers live in shared memory (layout mirrored
-    // in k_sim)
+    // simulation: one block per instance, launched per size class on forked
+    // streams so that each class's shared memory fits its own grids
     // one launch over all instances (a small call, or the largest grids of a
     // pipelined call), or size classes each on a stream of its own so that
     // each gets shared memory for its own sides
@@ -426,28 +437,13 @@ static int launch_batch(rr_ctx *ctx, rr_instance *d_inst, JobWS *ws, int count, 
         cudaStream_t cs = one ? s : ctx->classStream[c];
         if (!one) CUDA_TRY(cudaStreamWaitEvent(cs, ctx->evFork, 0));
         const int side = class_side(max_side, c, nclass);
-        // ready moves never exceed two per column here (one chain head each
-        // way); beyond the capacity slots spill to the global overflow area
-        const int slotCap = 2 * side + 8, lineCap = side;
-        // links are 16-bit up to side 256: about 2 * side moves are ready at
-        // once, far below 32 768; an instance that would need more slots
-        // ends with an internal error instead of wrapping an index
-        const bool narrow = lineCap <= 256;
-        const size_t simSmem = sim_smem_bytes(slotCap, lineCap, narrow ? 2 : 4);
-        if (simSmem > (size_t)std::min(ctx->smemLimit[narrow ? SM_SIM16 : SM_SIM32],
-                                       ctx->smemLimit[narrow ? SM_SIM16W : SM_SIM32W]))
-            return fail(ctx, RR_ERR_ARG, "simulation shared memory %zu too large", simSmem);
+        const SimShape sh = sim_shape(ctx, count, side);
+        if (sh.smem > (size_t)std::min(ctx->smemLimit[SM_SIM], ctx->smemLimit[SM_SIM_BIG]))
+            return fail(ctx, RR_ERR_ARG, "simulation shared memory %zu too large", sh.smem);
         const int *list = one ? nullptr : ctx->d_classList + (size_t)c * count;
         const int *cnt = one ? nullptr : ctx->d_classCount + c;
-        // the narrow pass, then the wide one for the instances it handed over
-        // (its blocks of other instances return at once)
-        if (narrow) {
-            k_sim16<<<count, 32, simSmem, cs>>>(d_inst, ws, count, list, cnt, slotCap, lineCap);
-            k_sim16w<<<count, 32, simSmem, cs>>>(d_inst, ws, count, list, cnt, slotCap, lineCap);
-        } else {
-            k_sim32<<<count, 32, simSmem, cs>>>(d_inst, ws, count, list, cnt, slotCap, lineCap);
-            k_sim32w<<<count, 32, simSmem, cs>>>(d_inst, ws, count, list, cnt, slotCap, lineCap);
-        }
+        (side <= 256 ? k_sim : k_sim_big)<<<count, 32 * sh.warps, sh.smem, cs>>>(d_inst, ws, count, list, cnt, side,
+                                                                                 sh.counters);
         if (!one) {
             CUDA_TRY(cudaEventRecord(ctx->evJoin[c], cs));
             CUDA_TRY(cudaStreamWaitEvent(s, ctx->evJoin[c], 0));
@@ -455,7 +451,7 @@ static int launch_batch(rr_ctx *ctx, rr_instance *d_inst, JobWS *ws, int count, 
     }
     mark(ctx, s, nullptr);
     CUDA_TRY(cudaGetLastError());
-    ctx->nlaunch += (one ? 9 : 10) + 2 * nclass;
+    ctx->nlaunch += (one ? 9 : 10) + nclass;
     return RR_OK;
 }
 

@@ -77,18 +77,22 @@ struct JobWS {
     int64_t P;             // total path vertices (sum of path length + 1)
     int32_t *pairOff;      // k + 1
     int32_t *nextAt;       // P
-    int32_t *succCnt;      // k: distinct successors of each path
     int32_t *succ;         // P: a path's successors at its vertex offset (pairOff)
     int32_t *indeg;        // k
-    int4 *rec;             // k: packed geometry, successor count, overflow offset
+    int4 *rec;             // k + 1 (the last unused): see move_rec
     int4 *succ4;           // k: first four successors (flagged, -1 padded)
     int32_t *ready0;       // k + 1: moves without predecessors; [k] = their count
     // Gamma by sweeps: moves ending in each column, L-moves starting on each row
     int32_t *colOff, *colCur, *colList;   // n + 1, n, k
     int32_t *rowOff, *rowCur, *rowList;   // m + 1, m, k
     int32_t *firstH;       // m * n: lowest-id L-move crossing each vertex, -1
-    void *slotOvf;         // k simulation slots beyond the shared-memory ones
-    int32_t *ovfFree;      // k: recycled overflow slots
+    void *slotOvf;         // the wide simulation's tables
+    // the moves with several predecessors, by number: in-degree and first leg
+    // (MULTI_BITS), id, position word
+    int32_t *multi, *multiId;
+    uint32_t *multiPos;
+    int32_t *multiNo;      // k: a move's number among them
+    int32_t nmulti;        // how many there are
     // path-vertex offsets by the multi-block scan (large move lists only):
     // one status word per tile, the tile counter
     unsigned long long *lbStatus;
@@ -111,30 +115,80 @@ __host__ __device__ inline int class_side(int max_side, int c, int nclass)
     return s < 32 ? 32 : s;
 }
 
-// Shared memory of one batching-simulation block (one warp, one instance):
-// sort / merge buffer, slot table, id map, members, successor buffer,
-// pickup bitmaps, list links and heads (ix bytes each), step counters and
-// the free-slot stack. The kernel's layout follows this order.
-constexpr int MAPN = 256;       // id -> slot cache for finding the next leader
-constexpr int SBUF = 256;       // successor entries released per round
-__host__ __device__ inline size_t sim_smem_bytes(int slotCap, int lineCap, int ix)
-{
-    const size_t S = (size_t)slotCap, L = (size_t)lineCap;
-    return 8 * 2 * (L + 2) +                                            // Kb
-           4 * (2 * S + MAPN + 2 * (L + 2) + SBUF + 4 * ((L + 31) / 32)) +  // key id, map, Mid Msl, sbuf, bits
-           (size_t)ix * (4 * S + 8 * L) +                                // rp rn cp cn, row and column heads
-           2 * 4 * S +                                                   // t, legEnd, dstRow, free stack
-           64;
-}
+// Block-wide state of a simulation in shared memory.
+struct SimCtl {
+    int nfree[4];             // free entries of each direction's table
+    int wbase[4], wcap[4];    // the wide tables: first entry, entries
+    int full;                 // a table was full
+    int pub;                  // segments of the log that the writers may write
+    int next;                 // first segment not yet taken by a writer (by 32)
+    int fin;                  // the simulation has ended: pub is final
+    int status;               // its end: RR_OK, RR_SIM_RETRY or an error
+    int pad[3];
+};
 
-// Status of an instance between the two simulation passes: the narrow pass
-// (shared-memory slots only) ran out of slots and the wide pass redoes it.
-// The wide pass always follows in the same launch sequence, so callers never
-// see it.
+// Table entries per direction in shared memory. Red-rec and bird plans have
+// at most one ready move per column and vertical direction, nearly all of
+// them at the start; up to side 256 one load of every lane covers a table.
+__host__ __device__ inline int sim_cap(int side)
+{
+    const int c = (side + (side <= 256 ? 63 : 31)) & ~7;
+    return side <= 256 && c > 256 ? 256 : c;
+}
+__host__ __device__ inline int sim_pow2(int side)
+{
+    int p = 32;
+    while (p < side) p <<= 1;
+    return p;
+}
+// Shared memory of a simulation block for grids of at most `side`: the
+// tables, the members, the control words, a sort buffer per warp, a list of
+// ids, 16 bytes nothing reads, the in-degree counters.
+__host__ __device__ inline size_t sim_smem_bytes(int side, int warps, int counters)
+{
+    const size_t M = (size_t)((side + 7) & ~7);
+    return 14 * 4 * (size_t)sim_cap(side) + 12 * M + sizeof(SimCtl) + 4 * ((size_t)sim_pow2(side) * warps + M) + 16 +
+           2 * (size_t)((counters + 7) & ~7);
+}
+constexpr int SIM_MAX_THREADS = 128;
+
+// Workspace of the wide simulation: tables in global memory with room for
+// every move, at most two legs each. Only instances with more ready moves
+// than a shared-memory table holds (at least 64) can need it.
+constexpr int SIM_WIDE_MIN = 65;
+__host__ __device__ inline size_t sim_wide_entries(long long k) { return 2 * (size_t)k + 32; }
+__host__ __device__ inline size_t sim_wide_bytes(long long k) { return k < SIM_WIDE_MIN ? 0 : 16 * sim_wide_entries(k); }
+
+// End of the narrow simulation when an instance needs more table entries
+// than shared memory holds: the wide one starts over in the same block, so
+// callers never see it.
 constexpr int32_t RR_SIM_RETRY = 100;
 
+// A move's record (two int4): the position word of its source; its first
+// leg's direction (2 bits) and length (11 bits), its destination row (10
+// bits) and whether its only successor is the next id, without other
+// predecessors; its number of successors; where those after the fourth lie;
+// then the first four successors. The position of a token that moves in direction d: the
+// coordinate along its way, mirrored for the negative directions so that it
+// grows, and the one across it, both plus one, in the halves of a word.
+constexpr int MIRROR = 1025;
+constexpr int MULTI_BITS = 11, MULTI_COUNT = (1 << MULTI_BITS) - 1;   // a path has at most 2 047 predecessors
+__device__ __forceinline__ uint32_t dir_pos(int d, int row, int col)
+{
+    const int x = d < 2 ? row : col, al = (d & 1) ? x + 1 : MIRROR - 1 - x;
+    return (uint32_t)al | (uint32_t)((d < 2 ? col : row) + 1) << 16;
+}
+__device__ __forceinline__ int4 move_rec(rr_move p, int nsucc, int more, bool chain)
+{
+    const int hl = p.dst_col - p.src_col, vl = p.dst_row - p.src_row;
+    const int d = hl ? (hl > 0 ? 3 : 2) : (vl > 0 ? 1 : 0), len = hl ? (hl > 0 ? hl : -hl) : (vl > 0 ? vl : -vl);
+    return make_int4((int)dir_pos(d, p.src_row, p.src_col), d | len << 2 | p.dst_row << 13 | (chain ? 1 << 23 : 0),
+                     nsucc, more);
+}
+
 // Successor entries carry this flag when the successor has a single
-// predecessor: it becomes ready as soon as that predecessor finishes.
+// predecessor: it becomes ready as soon as that predecessor finishes. Other
+// entries hold the number of the successor's in-degree counter.
 constexpr int32_t SUCC_SINGLE = 1 << 30;
 constexpr int32_t SUCC_ID = SUCC_SINGLE - 1;
 

@@ -9,10 +9,9 @@
 // same functions the separate kernels run (rr_plan.cuh, rr_bird.cuh,
 // rr_batch.cuh), given block coordinates x = 0, gx = 1 so that each
 // grid-stride loop covers all of its work with this block's warps; the
-// single-warp stages (pairing, simulation) run on warp 0 and the two-warp
-// bird stage on warps 0-1 while the other warps wait at the next barrier.
-// The simulation keeps the ready set in registers (sim_small) while it stays
-// within SMALL_CAP moves and falls back to the general one otherwise.
+// pairing runs on warp 0 and the two-warp bird stage on warps 0-1 while the
+// other warps wait at the next barrier. In the simulation warp 0 simulates
+// and the other warps write the batches.
 // The descriptor comes in as a kernel parameter and the final one is written
 // to mapped host memory, so a call is one launch and one synchronisation.
 #include <algorithm>
@@ -23,7 +22,7 @@
 namespace rrk {
 
 __global__ void __launch_bounds__(ONE_THREADS) k_one(rr_instance h, rr_instance *I, JobWS *ws, Arena A, int flags,
-                                                      int side, int P2, rr_instance *hostOut)
+                                                      int side, int P2, int counters, rr_instance *hostOut)
 {
     extern __shared__ int4 one_smem[];
     const Blk B{0, 0, 1};
@@ -71,24 +70,16 @@ __global__ void __launch_bounds__(ONE_THREADS) k_one(rr_instance h, rr_instance 
         __syncthreads();
         s_brec(B, I, ws, 1);
         __syncthreads();
-        // the ready set in registers when it stays small; else the general
-        // simulation (narrow pass, then the wide one if that runs out of slots)
-        if (wid == 0) sim_small(I, ws[0], (char *)one_smem);
+        sim_block<SIM_SMALL>(I, ws[0], (char *)one_smem, side, counters);
         __syncthreads();
-        const bool general = I->status == RR_SIM_RETRY;
-        __syncthreads();
-        if (general) {
-            if (threadIdx.x == 0) I->status = RR_OK;
-            __syncthreads();
-            const int slotCap = 2 * side + 8, lineCap = side;
-            if (wid == 0) sim_body<int16_t, false>(B, I, ws, 1, nullptr, nullptr, slotCap, lineCap);
-            __syncthreads();
-            if (wid == 0) sim_body<int16_t, true>(B, I, ws, 1, nullptr, nullptr, slotCap, lineCap);
-            __syncthreads();
-        }
     }
     if (threadIdx.x < sizeof(rr_instance) / 4) ((volatile int32_t *)hostOut)[threadIdx.x] = ((int32_t *)I)[threadIdx.x];
 }
+
+// In-degree counters of the simulation: enough for every move with several
+// predecessors of a bird plan (about a fifth of the traps), so that none of
+// them is counted in global memory.
+static int one_counters(int side) { return std::min(32768, side * side / 4 + 64); }
 
 // Dynamic shared memory of k_one for grids up to `side`: the largest
 // request of its stages (pairing, bird, the Gamma sorts and sweeps with
@@ -107,8 +98,7 @@ size_t one_smem_bytes(int side, int flags)
     if (flags & RR_WITH_BATCH) {
         b = std::max(b, warps * 4 * (size_t)P2);                              // k_gsort
         b = std::max(b, warps * 12 * (size_t)side);                           // k_gsweep_v (h needs a third)
-        b = std::max(b, sim_smem_bytes(2 * side + 8, side, 2));
-        b = std::max(b, small_smem_bytes());
+        b = std::max(b, sim_smem_bytes(side, (int)warps, one_counters(side)));
     }
     return b;
 }
@@ -120,7 +110,7 @@ int one_launch(rr_instance h, rr_instance *d_inst, JobWS *d_ws, Arena A, int fla
 {
     int P2 = 32;
     while (P2 < side) P2 <<= 1;
-    k_one<<<1, ONE_THREADS, smem, s>>>(h, d_inst, d_ws, A, flags, side, P2, hostOut);
+    k_one<<<1, ONE_THREADS, smem, s>>>(h, d_inst, d_ws, A, flags, side, P2, one_counters(side), hostOut);
     return cudaGetLastError() == cudaSuccess ? RR_OK : RR_ERR_CUDA;
 }
 

@@ -5,6 +5,13 @@
 
 namespace rrk {
 
+// Batching of one move list begins: its descriptor arrives as a kernel
+// parameter and the arena starts afresh.
+__global__ void k_batch_begin(rr_instance h, rr_instance *I, Arena A)
+{
+    if (threadIdx.x == 0) { *I = h; *A.top = 0; }
+}
+
 __global__ void k_bsetup(rr_instance *inst, JobWS *wsv, int count, Arena A, int lookback)
 {
     s_bsetup(hw_blk(), inst, wsv, count, A, lookback);

@@ -112,7 +112,7 @@ __device__ inline void s_bsetup(const Blk B, rr_instance *inst, JobWS *wsv, int 
     __syncthreads();
     long long P = 0, steps = 0;
     for (int64_t b = threadIdx.x; b < k; b += blockDim.x) {
-        const rr_move p = I->moves[b];
+        const rr_move p = load_move(&I->moves[b]);
         if (p.src_row < 0 || p.src_row >= m || p.dst_row < 0 || p.dst_row >= m || p.src_col < 0 ||
             p.src_col >= n || p.dst_col < 0 || p.dst_col >= n || (p.src_row == p.dst_row && p.src_col == p.dst_col))
             s_bad = 1;
@@ -170,7 +170,7 @@ __device__ inline void s_bsetup(const Blk B, rr_instance *inst, JobWS *wsv, int 
     if (!live(I)) return;
     // pairOff = exclusive scan of (len + 1); zero the counters
     for (int64_t b = threadIdx.x; b < k; b += blockDim.x) {
-        const rr_move p = I->moves[b];
+        const rr_move p = load_move(&I->moves[b]);
         ws.pairOff[b] = iabs(p.dst_col - p.src_col) + iabs(p.dst_row - p.src_row) + 1;
         ws.indeg[b] = 0;
     }
@@ -239,7 +239,7 @@ __device__ inline void s_pairoff_lookback(const Blk B, rr_instance *inst, JobWS 
             const int64_t b = b0 + u;
             v[u] = 0;
             if (b < k) {
-                const rr_move p = I->moves[b];
+                const rr_move p = load_move(&I->moves[b]);
                 bad |= p.src_row < 0 || p.src_row >= m || p.dst_row < 0 || p.dst_row >= m || p.src_col < 0 ||
                        p.src_col >= n || p.dst_col < 0 || p.dst_col >= n ||
                        (p.src_row == p.dst_row && p.src_col == p.dst_col);
@@ -409,7 +409,7 @@ __device__ inline void s_gcount(const Blk B, rr_instance *inst, JobWS *wsv, int 
     JobWS &ws = wsv[q];
     const int64_t k = I->n_moves;
     for (int64_t b = B.x * blockDim.x + threadIdx.x; b < k; b += (int64_t)B.gx * blockDim.x) {
-        const rr_move p = I->moves[b];
+        const rr_move p = load_move(&I->moves[b]);
         atomicAdd(&ws.colCur[p.dst_col], 1);
         if (p.src_col != p.dst_col) atomicAdd(&ws.rowCur[p.src_row], 1);
     }
@@ -447,7 +447,7 @@ __device__ inline void s_gfill(const Blk B, rr_instance *inst, JobWS *wsv, int c
     JobWS &ws = wsv[q];
     const int64_t k = I->n_moves;
     for (int64_t b = B.x * blockDim.x + threadIdx.x; b < k; b += (int64_t)B.gx * blockDim.x) {
-        const rr_move p = I->moves[b];
+        const rr_move p = load_move(&I->moves[b]);
         ws.colList[atomicAdd(&ws.colCur[p.dst_col], 1)] = (int32_t)b;
         if (p.src_col != p.dst_col) ws.rowList[atomicAdd(&ws.rowCur[p.src_row], 1)] = (int32_t)b;
     }
@@ -498,7 +498,7 @@ __device__ inline void s_gsweep_h(const Blk B, rr_instance *inst, JobWS *wsv, in
         __syncwarp();
         for (int e = ws.rowOff[r]; e < ws.rowOff[r + 1]; ++e) {
             const int b = ws.rowList[e];
-            const rr_move p = I->moves[b];
+            const rr_move p = load_move(&I->moves[b]);
             const int step = p.dst_col > p.src_col ? 1 : -1;
             const int hl = iabs(p.dst_col - p.src_col);
             const int base = ws.pairOff[b];
@@ -542,7 +542,7 @@ __device__ inline void s_gsweep_v(const Blk B, rr_instance *inst, JobWS *wsv, in
         __syncwarp();
         for (int e = ws.colOff[c]; e < ws.colOff[c + 1]; ++e) {
             const int b = ws.colList[e];
-            const rr_move p = I->moves[b];
+            const rr_move p = load_move(&I->moves[b]);
             const int step = p.dst_row > p.src_row ? 1 : -1;
             const int hl = iabs(p.dst_col - p.src_col), vl = iabs(p.dst_row - p.src_row);
             const int base = ws.pairOff[b] + hl;
@@ -571,7 +571,7 @@ __device__ inline void s_gsweep_v(const Blk B, rr_instance *inst, JobWS *wsv, in
             for (; (v >= 0 || h >= 0) && steps <= k; ++steps) {   // a chain holds each move at most once
                 const bool takeV = h < 0 || (v >= 0 && v < h);
                 const int x = takeV ? v : h;
-                const rr_move p = I->moves[x];
+                const rr_move p = load_move(&I->moves[x]);
                 const int e = ws.pairOff[x] + (takeV ? iabs(p.dst_col - p.src_col) + iabs(r - p.src_row)
                                                      : iabs(c - p.src_col));
                 const int nx = (takeV && e == lastPos[r]) ? -1 : ws.nextAt[e];
@@ -654,7 +654,7 @@ __device__ inline void s_brec(const Blk B, rr_instance *inst, JobWS *wsv, int co
     JobWS &ws = wsv[q];
     const int64_t k = I->n_moves;
     for (int64_t b = B.x * blockDim.x + threadIdx.x; b < k; b += (int64_t)B.gx * blockDim.x) {
-        const rr_move p = I->moves[b];
+        const rr_move p = load_move(&I->moves[b]);
         const int lo = ws.pairOff[b], hi = lo + ws.rec[2 * b].z;
         int v[4] = {-1, -1, -1, -1};
         for (int e = lo; e < hi; ++e) {
@@ -940,7 +940,6 @@ __device__ __forceinline__ uint32_t min8(uint4 a, uint4 b, uint32_t w, uint32_t 
 // lanes meet again cost 15 to 20 cycles each, and the code below has little
 // else between them.
 #ifdef __CUDA_ARCH__
-__device__ __forceinline__ uint32_t sh_addr(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
 #define RR_IF(instr) "{ .reg .pred q; setp.ne.u32 q, %0, 0; @q " instr " }"
 __device__ __forceinline__ int sh_add_if(bool c, void *p, int v)
 {
@@ -989,23 +988,8 @@ __device__ __forceinline__ int ldg_if(bool c, const void *p)
                  : "+r"(v) : "r"((unsigned)c), "l"(p) : "memory");
     return v;
 }
-// Bring a record's first half, or a word, into L1 without a register waiting
-// for it: an asynchronous copy to a place in shared memory that nothing
-// reads. (prefetch.global.L1 stops at L2 here: a load after it takes 300 to
-// 500 cycles, after this copy 40.)
-__device__ __forceinline__ void touch_rec_if(bool c, const int4 *rec, int id, uint32_t dump)
-{
-    asm volatile(RR_IF("cp.async.ca.shared.global [%1], [%2], 16;") ::"r"((unsigned)c), "r"(dump),
-                 "l"(rec + 2 * (size_t)id) : "memory");
-}
-__device__ __forceinline__ void touch_word_if(bool c, const void *p, uint32_t dump)
-{
-    asm volatile(RR_IF("cp.async.ca.shared.global [%1], [%2], 4;") ::"r"((unsigned)c), "r"(dump), "l"(p) : "memory");
-}
-__device__ __forceinline__ void touch_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 #undef RR_IF
 #else   // host-side stand-ins
-static inline uint32_t sh_addr(const void *) { return 0; }
 static inline int sh_add_if(bool c, void *p, int v) { int r = 0; if (c) { r = *(int *)p; *(int *)p = (int)((unsigned)r + (unsigned)v); } return r; }
 static inline int ld_u16_if(bool c, const uint16_t *p) { return c ? *p : 0; }
 static inline void st_if(bool c, uint16_t *p, int v) { if (c) *p = (uint16_t)v; }
@@ -1014,10 +998,12 @@ static inline void st_if(bool c, int2 *p, int x, int y) { if (c) *p = make_int2(
 static inline int4 ldg_if(bool c, const int4 *p) { return c ? *p : make_int4(0, 0, 0, 0); }
 static inline int2 ldg_if(bool c, const int2 *p) { return c ? *p : make_int2(0, 0); }
 static inline int ldg_if(bool c, const void *p) { return c ? *(const int *)p : 0; }
-static inline void touch_rec_if(bool, const int4 *, int, uint32_t) {}
-static inline void touch_word_if(bool, const void *, uint32_t) {}
-static inline void touch_wait() {}
 #endif
+
+__device__ __forceinline__ void touch_rec_if(bool c, const int4 *rec, int id, uint32_t dump)
+{
+    touch_if(c, rec + 2 * (size_t)id, dump);
+}
 
 // The largest of the lanes' values (usually all the same): a value that the
 // compiler knows to be uniform, so that branches on it, and on what is
@@ -1092,9 +1078,9 @@ struct Sim {
             __syncwarp();
         }
         const bool soon = multi_ && old == 2, last = multi_ && old == 1;
-        touch_word_if(soon, multiId + x, dump);           // next time it is ready
-        touch_word_if(soon, multiPos + x, dump);
-        touch_word_if(soon, multi + x, dump);
+        touch_if(soon, multiId + x, dump);           // next time it is ready
+        touch_if(soon, multiPos + x, dump);
+        touch_if(soon, multi + x, dump);
         bool h = single && x == handId;
         const bool fresh = single && !h;
         if (__any_sync(FULL, fresh || last)) {

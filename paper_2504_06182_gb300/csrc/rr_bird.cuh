@@ -371,7 +371,7 @@ __device__ inline void s_bird(const Blk B, rr_instance *inst, JobWS *wsv, int co
             else if (k >= ku_start) pos = kd_end + (k - ku_start);
             else continue;
             const long long o = base + pos;
-            if (o < I->cap_moves) I->moves[o] = rr_move{row, col, r0 + k, j};
+            if (o < I->cap_moves) store_move(&I->moves[o], row, col, r0 + k, j);
             steps += iabs(r0 + k - row) + iabs(j - col);
         }
         // the chosen tokens leave the reservoirs

@@ -9,11 +9,13 @@
 
 namespace rrk {
 __global__ void k_plan_setup(rr_instance *, JobWS *, int, int, Arena);
-__global__ void k_transpose(rr_instance *, JobWS *, int);
-__global__ void k_colstats(rr_instance *, JobWS *, int, int);
-__global__ void k_pair(rr_instance *, JobWS *, int);
-__global__ void k_emit_cols(rr_instance *, JobWS *, int);
-__global__ void k_emit_recv(rr_instance *, JobWS *, int);
+__global__ void k_plan_begin(rr_instance, rr_instance *, JobWS *, int, Arena);
+__global__ void k_batch_begin(rr_instance, rr_instance *, Arena);
+__global__ void k_transpose(rr_instance *, JobWS *, int, int);
+__global__ void k_colstats(rr_instance *, JobWS *, int, int, int);
+__global__ void k_pair(rr_instance *, JobWS *, int, int);
+__global__ void k_emit_cols(rr_instance *, JobWS *, int, int);
+__global__ void k_emit_recv(rr_instance *, JobWS *, int, int);
 __global__ void k_bird(rr_instance *, JobWS *, int, int);
 __global__ void k_bsetup(rr_instance *, JobWS *, int, Arena, int);
 __global__ void k_pairoff_lookback(rr_instance *, JobWS *, int, Arena);
@@ -311,22 +313,28 @@ static size_t bird_smem_bytes(int max_side)
 // red-rec (Alg. 1), or with RR_BIRD the bird algorithm (Alg. 2), which shares
 // red-rec's column phase; RR_STRICT_RESERVOIR selects the strict reading of
 // target sub-rectangles for either.
+// `first`: the descriptor of a call over one grid, not on the device yet.
 static int launch_plan(rr_ctx *ctx, rr_instance *d_inst, JobWS *ws, int count, int max_side, cudaStream_t s,
-                       int flags)
+                       int flags, const rr_instance *first = nullptr)
 {
     const bool bird = (flags & RR_BIRD) != 0;
     const int strict = (flags & RR_STRICT_RESERVOIR) ? 1 : 0;
     const Arena A = arena_of(ctx);
-    const int colBlocks = clampi(std::max(1, budget(ctx, 4096) / count), 1, (max_side + 7) / 8);
+    const int colBlocks = clampi(std::max(1, budget(ctx, 8192) / count), 1, (max_side + 7) / 8);
     const int tiles = ((max_side + 31) / 32) * ((max_side + 31) / 32);
     const int trBlocks = clampi(std::max(1, budget(ctx, 4096) / count), 1, (tiles + 7) / 8);
-    const int recvBlocks = clampi(std::max(1, budget(ctx, 2048) / count), 1, max_side);
+    const int recvBlocks = clampi(std::max(1, budget(ctx, 8192) / count), 1, (max_side * ((max_side + 31) / 32) + 7) / 8);
+    // warps of a block on each instance: all eight, fewer in calls over very
+    // many grids (see hw_blk_shared)
+    const int per = count <= 4096 ? 8 : count <= 8192 ? 4 : count <= 16384 ? 2 : 1;
+    const int rows = (count * per + 7) / 8;
     mark(ctx, s, "k_plan_setup");
-    k_plan_setup<<<(count + 127) / 128, 128, 0, s>>>(d_inst, ws, count, max_side, A);
+    if (first) k_plan_begin<<<1, 32, 0, s>>>(*first, d_inst, ws, max_side, A);
+    else k_plan_setup<<<(count + 127) / 128, 128, 0, s>>>(d_inst, ws, count, max_side, A);
     mark(ctx, s, "k_transpose");
-    k_transpose<<<dim3(trBlocks, count), 256, 0, s>>>(d_inst, ws, count);
+    k_transpose<<<dim3(trBlocks, rows), 256, 0, s>>>(d_inst, ws, count, per);
     mark(ctx, s, "k_colstats");
-    k_colstats<<<dim3(colBlocks, count), 256, 0, s>>>(d_inst, ws, count, strict);
+    k_colstats<<<dim3(colBlocks, rows), 256, 0, s>>>(d_inst, ws, count, strict, per);
     if (bird) {
         const size_t birdSmem = bird_smem_bytes(max_side);
         if (birdSmem > (size_t)ctx->smemLimit[SM_BIRD])
@@ -334,19 +342,19 @@ static int launch_plan(rr_ctx *ctx, rr_instance *d_inst, JobWS *ws, int count, i
         mark(ctx, s, "k_bird");
         k_bird<<<count, 64, birdSmem, s>>>(d_inst, ws, count, max_side);
         mark(ctx, s, "k_emit_cols");
-        k_emit_cols<<<dim3(colBlocks, count), 256, 0, s>>>(d_inst, ws, count);
+        k_emit_cols<<<dim3(colBlocks, rows), 256, 0, s>>>(d_inst, ws, count, per);
         mark(ctx, s, nullptr);
         CUDA_TRY(cudaGetLastError());
         ctx->nlaunch += 5;
         return RR_OK;
     }
-    const size_t pairSmem = (size_t)max_side * 30 + 64;
+    const size_t pairSmem = (size_t)max_side * PAIR_BYTES + 64;
     mark(ctx, s, "k_pair");
-    k_pair<<<count, 32, pairSmem, s>>>(d_inst, ws, count);
+    k_pair<<<count, 32, pairSmem, s>>>(d_inst, ws, count, count <= ctx->nsm ? 1 : 0);
     mark(ctx, s, "k_emit_cols");
-    k_emit_cols<<<dim3(colBlocks, count), 256, 0, s>>>(d_inst, ws, count);
+    k_emit_cols<<<dim3(colBlocks, rows), 256, 0, s>>>(d_inst, ws, count, per);
     mark(ctx, s, "k_emit_recv");
-    k_emit_recv<<<dim3(recvBlocks, count), 256, 0, s>>>(d_inst, ws, count);
+    k_emit_recv<<<dim3(recvBlocks, rows), 256, 0, s>>>(d_inst, ws, count, per);
     mark(ctx, s, nullptr);
     CUDA_TRY(cudaGetLastError());
     ctx->nlaunch += 6;
@@ -461,6 +469,12 @@ static bool rect_ok(int m, int n, rr_rect R)
            R.r1 <= m && R.c0 >= 0 && R.c0 < R.c1 && R.c1 <= n;
 }
 
+// Planning alone runs as one block up to this side: below it the kernels'
+// launches and boundaries cost more than the blocks they would spread over
+// give (whole calls at sides 32 / 64 / 96: 55 / 89 / 132 us in one launch, 71 /
+// 95 / 118 us in six).
+static constexpr int ONE_PLAN_SIDE = 64;
+
 static int plan_one(rr_ctx *ctx, const void *d_grid, int layout, int m, int n, rr_rect rect, rr_move *d_moves,
                     int64_t cap, int64_t *n_moves, cudaStream_t stream, int flags, const char *name)
 {
@@ -473,16 +487,25 @@ static int plan_one(rr_ctx *ctx, const void *d_grid, int layout, int m, int n, r
     h.grid = d_grid; h.layout = layout; h.m = m; h.n = n; h.rect = rect;
     h.moves = d_moves; h.cap_moves = cap;
     ctx->nmarks = 0;
-    CUDA_TRY(cudaMemsetAsync(ctx->d_top, 0, sizeof(unsigned long long), stream));
-    CUDA_TRY(cudaMemcpyAsync(ctx->d_one, &h, sizeof(h), cudaMemcpyHostToDevice, stream));
-    int st = launch_plan(ctx, ctx->d_one, ctx->d_ws, 1, std::max(m, n), stream, flags);
-    if (st != RR_OK) return st;
-    CUDA_TRY(cudaMemcpyAsync(&h, ctx->d_one, sizeof(h), cudaMemcpyDeviceToHost, stream));
+    const int side = std::max(m, n);
+    int st;
+    if (side <= ONE_PLAN_SIDE) {
+        mark(ctx, stream, "k_one");
+        st = one_launch(h, ctx->d_one, ctx->d_ws, arena_of(ctx), flags, side, one_smem_bytes(side, flags), ctx->d_hone, stream);
+        if (st != RR_OK) return fail(ctx, st, "%s: launch: %s", name, cudaGetErrorString(cudaGetLastError()));
+        mark(ctx, stream, nullptr);
+        ctx->nlaunch += 1;
+    } else {
+        st = launch_plan(ctx, ctx->d_one, ctx->d_ws, 1, side, stream, flags, &h);
+        if (st != RR_OK) return st;
+        CUDA_TRY(cudaMemcpyAsync(ctx->h_one, ctx->d_one, sizeof(h), cudaMemcpyDeviceToHost, stream));
+    }
     CUDA_TRY(cudaStreamSynchronize(stream));
-    *n_moves = h.n_moves;
-    if (h.status < 0)
-        return fail(ctx, h.status, "%s: device status %d (n_moves=%lld)", name, h.status, (long long)h.n_moves);
-    return h.status;
+    const volatile rr_instance *r = ctx->h_one;
+    *n_moves = r->n_moves;
+    st = r->status;
+    if (st < 0) return fail(ctx, st, "%s: device status %d (n_moves=%lld)", name, st, (long long)*n_moves);
+    return st;
 }
 
 extern "C" int rr_plan(rr_ctx *ctx, const void *d_grid, int layout, int m, int n, rr_rect rect,
@@ -518,16 +541,18 @@ extern "C" int rr_batch(rr_ctx *ctx, const rr_move *d_moves, int64_t n_moves, in
     h.ops = d_ops; h.cap_ops = cap_ops; h.members = d_members; h.cap_members = cap_members;
     h.status = RR_OK;
     ctx->nmarks = 0;
-    CUDA_TRY(cudaMemsetAsync(ctx->d_top, 0, sizeof(unsigned long long), stream));
-    CUDA_TRY(cudaMemcpyAsync(ctx->d_one, &h, sizeof(h), cudaMemcpyHostToDevice, stream));
+    k_batch_begin<<<1, 32, 0, stream>>>(h, ctx->d_one, arena_of(ctx));
+    ctx->nlaunch += 1;
     int st = launch_batch(ctx, ctx->d_one, ctx->d_ws, 1, std::max(m, n), stream, SIM_ONE, nullptr, nullptr);
     if (st != RR_OK) return st;
-    CUDA_TRY(cudaMemcpyAsync(&h, ctx->d_one, sizeof(h), cudaMemcpyDeviceToHost, stream));
+    CUDA_TRY(cudaMemcpyAsync(ctx->h_one, ctx->d_one, sizeof(h), cudaMemcpyDeviceToHost, stream));
     CUDA_TRY(cudaStreamSynchronize(stream));
-    *n_ops = h.n_ops;
-    *n_members = h.n_members;
-    if (h.status < 0) return fail(ctx, h.status, "rr_batch: device status %d", h.status);
-    return h.status;
+    const volatile rr_instance *r = ctx->h_one;
+    *n_ops = r->n_ops;
+    *n_members = r->n_members;
+    st = r->status;
+    if (st < 0) return fail(ctx, st, "rr_batch: device status %d", st);
+    return st;
 }
 
 extern "C" int rr_plan_one(rr_ctx *ctx, const void *d_grid, int layout, int m, int n, rr_rect rect, int flags,

@@ -13,9 +13,24 @@ constexpr unsigned FULL = 0xffffffffu;
 // rr_bird.cuh and rr_batch.cuh): the hardware's when a stage runs as a
 // kernel of its own; x = 0, gx = 1 when one block runs the whole path of one
 // grid (the single-grid kernel), so that every grid-stride loop covers all
-// of its items.
-struct Blk { int x, y, gx; };
-__device__ __forceinline__ Blk hw_blk() { return Blk{(int)blockIdx.x, (int)blockIdx.y, (int)gridDim.x}; }
+// of its items. Stages that give a warp an item use w and nw: this warp's
+// first item and the number of warps on this instance.
+struct Blk { int x, y, gx, w, nw; };
+__device__ __forceinline__ Blk hw_blk()
+{
+    const int wpb = blockDim.x >> 5;
+    return Blk{(int)blockIdx.x, (int)blockIdx.y, (int)gridDim.x, (int)blockIdx.x * wpb + (int)(threadIdx.x >> 5),
+               (int)gridDim.x * wpb};
+}
+// The same with `per` warps of a block on each instance, hence several
+// instances per block: for calls over very many grids, whose instances would
+// otherwise take a whole block each, most of it idle when they are narrow.
+__device__ __forceinline__ Blk hw_blk_shared(int per)
+{
+    const int wpb = blockDim.x >> 5, wid = threadIdx.x >> 5;
+    return Blk{(int)blockIdx.x, (int)blockIdx.y * (wpb / per) + wid / per, (int)gridDim.x,
+               (int)blockIdx.x * per + wid % per, (int)gridDim.x * per};
+}
 
 // Column classification after the column phase (Alg. 1 first loop, solved for
 // every column of non-negative surplus at once as in Sec. III.D).
@@ -44,18 +59,22 @@ struct Event {
     int32_t i, j;       // donor, receiver
     int32_t x, a;       // tokens exchanged, of which a come from above the band
     int32_t t0, b0;     // donor pool cursors (nearest-first index) before the exchange
-    int32_t next;       // next event with the same receiver, -1
+    int32_t at;         // of the p-th slot: the event there when ordered by receiver (saturation
+                        // order) and, within a receiver, by time
 };
 
 // A receiver unit, in the order receivers become saturated.
 struct RecvInfo {
     int32_t j;
-    int32_t ev_first;   // first event whose receiver is j (linked by Event::next)
-    int32_t ncontrib;   // events in that list
+    int32_t ev_first;   // its events' first slot (Event::at)
+    int32_t ncontrib;   // its events
     int32_t nT;         // sources above the band (mandatory + chosen)
     int32_t kd_end, ku_start, nmoves;
     int32_t pad;
 };
+
+// Shared memory of the pairing stage per column.
+constexpr int PAIR_BYTES = 42;
 
 struct Arena {
     char *base;
@@ -200,6 +219,8 @@ __device__ __forceinline__ void *arena_alloc(const Arena &A, unsigned long long 
     return A.base + off;
 }
 
+__host__ __device__ constexpr unsigned long long arena_pad(unsigned long long bytes) { return (bytes + 255ull) & ~255ull; }
+
 __device__ __forceinline__ int warp_incl_scan(int v)
 {
     const int lane = threadIdx.x & 31;
@@ -211,21 +232,15 @@ __device__ __forceinline__ int warp_incl_scan(int v)
     return v;
 }
 
-__device__ __forceinline__ int warp_sum(int v)
-{
-#pragma unroll
-    for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(FULL, v, o);
-    return v;
-}
+__device__ __forceinline__ int warp_sum(int v) { return __reduce_add_sync(FULL, v); }
 
+// (two 32-bit reductions: the upper halves, then the lower ones of the lanes
+// that hold the largest upper half)
 __device__ __forceinline__ unsigned long long warp_max_u64(unsigned long long v)
 {
-#pragma unroll
-    for (int o = 16; o; o >>= 1) {
-        unsigned long long u = __shfl_xor_sync(FULL, v, o);
-        v = u > v ? u : v;
-    }
-    return v;
+    const unsigned hi = __reduce_max_sync(FULL, (unsigned)(v >> 32));
+    const unsigned lo = __reduce_max_sync(FULL, (unsigned)(v >> 32) == hi ? (unsigned)v : 0u);
+    return (unsigned long long)hi << 32 | lo;
 }
 
 // Bits of rows [lo, hi) that fall in word w (rows 32w .. 32w+31).
@@ -241,6 +256,23 @@ __device__ __forceinline__ uint32_t row_mask(int w, int lo, int hi)
 __device__ __forceinline__ int iabs(int v) { return v < 0 ? -v : v; }
 __device__ __forceinline__ int isgn(int v) { return (v > 0) - (v < 0); }
 
+// A move of a list in one 16-byte access where the list is aligned for it
+// (an array of rr_move need not be): four 4-byte accesses of a warp's moves
+// touch each of their sectors four times.
+__device__ __forceinline__ rr_move load_move(const rr_move *p)
+{
+    if (((uintptr_t)p & 15) == 0) {
+        const int4 v = *reinterpret_cast<const int4 *>(p);
+        return rr_move{v.x, v.y, v.z, v.w};
+    }
+    return *p;
+}
+__device__ __forceinline__ void store_move(rr_move *p, int sr, int sc, int dr, int dc)
+{
+    if (((uintptr_t)p & 15) == 0) *reinterpret_cast<int4 *>(p) = make_int4(sr, sc, dr, dc);
+    else *p = rr_move{sr, sc, dr, dc};
+}
+
 // Direction codes of rr_op.
 __device__ __forceinline__ int step_dir(int sr, int sc, int dr, int dc, int t)
 {
@@ -255,6 +287,24 @@ __device__ __forceinline__ void path_cell(int sr, int sc, int dr, int dc, int t,
     if (t <= hl) { *r = sr; *c = sc + t * isgn(dc - sc); }
     else { *r = sr + (t - hl) * isgn(dr - sr); *c = dc; }
 }
+
+// Bring the 32 bytes around a word into L1 without a register waiting for
+// them (lanes that c holds for): an asynchronous copy of the word to a place
+// in shared memory that nothing reads, `dump`. (prefetch.global.L1 stops at
+// L2 here: a load after it takes 300 to 500 cycles, after this copy 40.)
+#ifdef __CUDA_ARCH__
+__device__ __forceinline__ uint32_t sh_addr(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
+__device__ __forceinline__ void touch_if(bool c, const void *p, uint32_t dump)
+{
+    asm volatile("{ .reg .pred q; setp.ne.u32 q, %0, 0; @q cp.async.ca.shared.global [%1], [%2], 4; }"
+                 ::"r"((unsigned)c), "r"(dump), "l"(p) : "memory");
+}
+__device__ __forceinline__ void touch_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+#else   // host-side stand-ins
+static inline uint32_t sh_addr(const void *) { return 0; }
+static inline void touch_if(bool, const void *, uint32_t) {}
+static inline void touch_wait() {}
+#endif
 
 // Test hook: when positive, the pairing loop and the batching simulation
 // stop after this many iterations with RR_ERR_TIMEOUT, as when their own

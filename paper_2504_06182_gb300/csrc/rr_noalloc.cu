@@ -16,12 +16,13 @@
 #include "rr_internal.cuh"
 
 namespace rrk {
-__global__ void k_plan_setup(rr_instance *, JobWS *, int, int, Arena);
-__global__ void k_transpose(rr_instance *, JobWS *, int);
-__global__ void k_colstats(rr_instance *, JobWS *, int, int);
-__global__ void k_pair(rr_instance *, JobWS *, int);
-__global__ void k_emit_cols(rr_instance *, JobWS *, int);
-__global__ void k_emit_recv(rr_instance *, JobWS *, int);
+__global__ void k_plan_begin(rr_instance, rr_instance *, JobWS *, int, Arena);
+__global__ void k_plan_block(rr_instance, rr_instance *, JobWS *, Arena, int);
+__global__ void k_transpose(rr_instance *, JobWS *, int, int);
+__global__ void k_colstats(rr_instance *, JobWS *, int, int, int);
+__global__ void k_pair(rr_instance *, JobWS *, int, int);
+__global__ void k_emit_cols(rr_instance *, JobWS *, int, int);
+__global__ void k_emit_recv(rr_instance *, JobWS *, int, int);
 }  // namespace rrk
 
 using namespace rrk;
@@ -49,6 +50,10 @@ static constexpr size_t noalloc_worst_case()
 }
 static_assert(noalloc_worst_case() <= RR_NOALLOC_SCRATCH_BYTES - OFF_ARENA,
               "the fixed workspace must hold the largest accepted plan");
+
+// Grids up to this side are planned by one block in one launch (side 32:
+// 62 us against 72 us for six kernels; from side 96 on the kernels are faster).
+static constexpr int ONE_BLOCK_SIDE = 64;
 
 // Device address of the scratch array, looked up once per device (host
 // code must not use the symbol itself: it names a host-side stand-in).
@@ -92,20 +97,23 @@ extern "C" int rr_plan_noalloc(const void *d_grid, int layout, int m, int n, rr_
     memset(&h, 0, sizeof(h));
     h.grid = d_grid; h.layout = layout; h.m = m; h.n = n; h.rect = rect;
     h.moves = d_moves; h.cap_moves = cap;
-    // the previous call's contents remain: reset the bump pointer and the descriptor
-    if (cudaMemsetAsync(A.top, 0, sizeof(unsigned long long), stream) != cudaSuccess) return RR_ERR_CUDA;
-    if (cudaMemcpyAsync(d_inst, &h, sizeof(h), cudaMemcpyHostToDevice, stream) != cudaSuccess) return RR_ERR_CUDA;
-
+    // (the previous call's contents remain: the first kernel resets the bump
+    // pointer and the descriptor)
     const int side = m > n ? m : n;
-    const int colBlocks = (side + 7) / 8;
-    const int tiles = ((side + 31) / 32) * ((side + 31) / 32);
-    const int trBlocks = (tiles + 7) / 8;
-    k_plan_setup<<<1, 128, 0, stream>>>(d_inst, d_ws, 1, side, A);
-    k_transpose<<<dim3(trBlocks, 1), 256, 0, stream>>>(d_inst, d_ws, 1);
-    k_colstats<<<dim3(colBlocks, 1), 256, 0, stream>>>(d_inst, d_ws, 1, 0);
-    k_pair<<<1, 32, (size_t)side * 30 + 64, stream>>>(d_inst, d_ws, 1);
-    k_emit_cols<<<dim3(colBlocks, 1), 256, 0, stream>>>(d_inst, d_ws, 1);
-    k_emit_recv<<<dim3(side, 1), 256, 0, stream>>>(d_inst, d_ws, 1);
+    const size_t pairSmem = (size_t)side * PAIR_BYTES + 64;
+    if (side <= ONE_BLOCK_SIDE) {
+        k_plan_block<<<1, 256, pairSmem, stream>>>(h, d_inst, d_ws, A, side);
+    } else {
+        const int colBlocks = (side + 7) / 8;
+        const int tiles = ((side + 31) / 32) * ((side + 31) / 32);
+        const int trBlocks = (tiles + 7) / 8;
+        k_plan_begin<<<1, 32, 0, stream>>>(h, d_inst, d_ws, side, A);
+        k_transpose<<<dim3(trBlocks, 1), 256, 0, stream>>>(d_inst, d_ws, 1, 8);
+        k_colstats<<<dim3(colBlocks, 1), 256, 0, stream>>>(d_inst, d_ws, 1, 0, 8);
+        k_pair<<<1, 32, pairSmem, stream>>>(d_inst, d_ws, 1, 1);
+        k_emit_cols<<<dim3(colBlocks, 1), 256, 0, stream>>>(d_inst, d_ws, 1, 8);
+        k_emit_recv<<<dim3((side * ((side + 31) / 32) + 7) / 8, 1), 256, 0, stream>>>(d_inst, d_ws, 1, 8);
+    }
     if (cudaGetLastError() != cudaSuccess) return RR_ERR_CUDA;
     if (cudaMemcpyAsync(&h, d_inst, sizeof(h), cudaMemcpyDeviceToHost, stream) != cudaSuccess) return RR_ERR_CUDA;
     if (cudaStreamSynchronize(stream) != cudaSuccess) return RR_ERR_CUDA;

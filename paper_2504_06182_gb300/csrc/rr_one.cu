@@ -25,8 +25,8 @@ __global__ void __launch_bounds__(ONE_THREADS) k_one(rr_instance h, rr_instance 
                                                       int side, int P2, int counters, rr_instance *hostOut)
 {
     extern __shared__ int4 one_smem[];
-    const Blk B{0, 0, 1};
     const int wid = threadIdx.x >> 5;
+    const Blk B{0, 0, 1, wid, ONE_THREADS / 32};
     const bool bird = (flags & RR_BIRD) != 0, batch = (flags & RR_WITH_BATCH) != 0;
     if (threadIdx.x == 0) {
         *I = h;
@@ -44,7 +44,7 @@ __global__ void __launch_bounds__(ONE_THREADS) k_one(rr_instance h, rr_instance 
         __syncthreads();
         s_emit_cols(B, I, ws, 1);
     } else {
-        if (wid == 0) s_pair(B, I, ws, 1);
+        if (wid == 0) s_pair(B, I, ws, 1, 1);
         __syncthreads();
         s_emit_cols(B, I, ws, 1);
         __syncthreads();
@@ -89,7 +89,7 @@ size_t one_smem_bytes(int side, int flags)
     int P2 = 32;
     while (P2 < side) P2 <<= 1;
     const size_t warps = ONE_THREADS / 32;
-    size_t b = (size_t)side * 30 + 64;                                       // pairing
+    size_t b = (size_t)side * PAIR_BYTES + 64;                               // pairing
     if (flags & RR_BIRD) {
         size_t cap = 1;
         while (cap < (size_t)side) cap <<= 1;

@@ -1,6 +1,7 @@
 // rr_plan.cu -- kernels of the red-rec planner (arXiv 2504.06182, Alg. 1):
 // each runs one stage of rr_plan.cuh over the instance array, blockIdx.y
-// selecting the instance (blockIdx.x for the one-block-per-instance stages).
+// selecting the instance (blockIdx.x for the one-block-per-instance stages);
+// `per` warps of a block on each instance where a warp takes an item.
 #include "rr_plan.cuh"
 
 namespace rrk {
@@ -10,29 +11,60 @@ __global__ void k_plan_setup(rr_instance *inst, JobWS *wsv, int count, int max_s
     s_plan_setup(hw_blk(), inst, wsv, count, max_side, A);
 }
 
-__global__ void k_transpose(rr_instance *inst, JobWS *wsv, int count)
+// Planning of one grid begins: its descriptor arrives as a kernel parameter
+// (no copy before it) and the arena starts afresh.
+__global__ void k_plan_begin(rr_instance h, rr_instance *I, JobWS *ws, int max_side, Arena A)
 {
-    s_transpose(hw_blk(), inst, wsv, count);
+    if (threadIdx.x == 0) { *I = h; *A.top = 0; }
+    __syncthreads();
+    s_plan_setup(hw_blk(), I, ws, 1, max_side, A);
 }
 
-__global__ void k_colstats(rr_instance *inst, JobWS *wsv, int count, int strict)
+// Red-rec planning of one small grid by one block, block barriers instead of
+// kernel boundaries (the single-grid kernel without bird and batching).
+__global__ void __launch_bounds__(256) k_plan_block(rr_instance h, rr_instance *I, JobWS *ws, Arena A, int side)
 {
-    s_colstats(hw_blk(), inst, wsv, count, strict);
+    const int wid = threadIdx.x >> 5;
+    const Blk B{0, 0, 1, wid, 8};
+    if (threadIdx.x == 0) { *I = h; *A.top = 0; }
+    __syncthreads();
+    s_plan_setup(B, I, ws, 1, side, A);
+    __syncthreads();
+    s_transpose(B, I, ws, 1);
+    __syncthreads();
+    s_colstats(B, I, ws, 1, 0);
+    __syncthreads();
+    if (wid == 0) s_pair(B, I, ws, 1, 1);
+    __syncthreads();
+    s_emit_cols(B, I, ws, 1);
+    s_emit_recv(B, I, ws, 1);
 }
 
-__global__ void k_pair(rr_instance *inst, JobWS *wsv, int count)
+__global__ void k_transpose(rr_instance *inst, JobWS *wsv, int count, int per)
 {
-    s_pair(hw_blk(), inst, wsv, count);
+    s_transpose(hw_blk_shared(per), inst, wsv, count);
 }
 
-__global__ void k_emit_cols(rr_instance *inst, JobWS *wsv, int count)
+__global__ void k_colstats(rr_instance *inst, JobWS *wsv, int count, int strict, int per)
 {
-    s_emit_cols(hw_blk(), inst, wsv, count);
+    s_colstats(hw_blk_shared(per), inst, wsv, count, strict);
 }
 
-__global__ void k_emit_recv(rr_instance *inst, JobWS *wsv, int count)
+__global__ void k_pair(rr_instance *inst, JobWS *wsv, int count, int warm)
 {
-    s_emit_recv(hw_blk(), inst, wsv, count);
+    s_pair(hw_blk(), inst, wsv, count, warm);
+}
+
+__global__ void k_emit_cols(rr_instance *inst, JobWS *wsv, int count, int per)
+{
+    s_emit_cols(hw_blk_shared(per), inst, wsv, count);
+}
+
+// (more resident warps are worth more here than registers: 95 of them left
+// room for 16 warps per SM)
+__global__ void __launch_bounds__(256, 5) k_emit_recv(rr_instance *inst, JobWS *wsv, int count, int per)
+{
+    s_emit_recv(hw_blk_shared(per), inst, wsv, count);
 }
 
 int guard_cap_plan(long long cap)

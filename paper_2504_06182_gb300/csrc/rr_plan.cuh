@@ -12,47 +12,59 @@
 
 namespace rrk {
 
-// ----------------------------------------------------------------- helpers
-
-// Row of the l-th nearest-to-band pool atom above (top) / below (bottom).
-__device__ __forceinline__ int pool_top_row(const ColInfo &D, const int16_t *rows, int r0, int l)
-{
-    return D.kind == KIND_OUTER_FULL ? r0 - 1 - l : (int)rows[D.tbase - l];
-}
-__device__ __forceinline__ int pool_bot_row(const ColInfo &D, const int16_t *rows, int r1, int l)
-{
-    return D.kind == KIND_OUTER_FULL ? r1 + l : (int)rows[D.bbase + l];
-}
-
 // ------------------------------------------------------------ validation
 
 __device__ inline void s_plan_setup(const Blk B, rr_instance *inst, JobWS *wsv, int count, int max_side, Arena A)
 {
-    const int q = B.x * blockDim.x + threadIdx.x;
-    if (q >= count) return;
+    const int q = B.x * blockDim.x + threadIdx.x, lane = threadIdx.x & 31;
     rr_instance *I = &inst[q];
-    JobWS &ws = wsv[q];
-    I->n_moves = 0; I->n_steps = 0; I->n_ops = 0; I->n_members = 0;
-    I->status = RR_OK;
-    const int m = I->m, n = I->n;
-    const rr_rect R = I->rect;
-    if (m < 1 || n < 1 || m > max_side || n > max_side || m > RR_MAX_SIDE || n > RR_MAX_SIDE || R.r0 < 0 || R.r0 >= R.r1 || R.r1 > m ||
-        R.c0 < 0 || R.c0 >= R.c1 || R.c1 > n || !I->grid || (I->layout != RR_U8 && I->layout != RR_BITS32) ||
-        I->cap_moves < 0 || (I->cap_moves > 0 && !I->moves)) {
-        I->status = RR_ERR_ARG;
-        return;
+    int m = 0, n = 0, h = 0, tw = 0;
+    if (q < count) {
+        I->n_moves = 0; I->n_steps = 0; I->n_ops = 0; I->n_members = 0;
+        m = I->m; n = I->n;
+        const rr_rect R = I->rect;
+        const bool bad = m < 1 || n < 1 || m > max_side || n > max_side || m > RR_MAX_SIDE || n > RR_MAX_SIDE ||
+                         R.r0 < 0 || R.r0 >= R.r1 || R.r1 > m || R.c0 < 0 || R.c0 >= R.c1 || R.c1 > n || !I->grid ||
+                         (I->layout != RR_U8 && I->layout != RR_BITS32) || I->cap_moves < 0 ||
+                         (I->cap_moves > 0 && !I->moves);
+        I->status = bad ? RR_ERR_ARG : RR_OK;
+        h = R.r1 - R.r0;
+        tw = R.c1 - R.c0;
+        if (bad) m = n = h = tw = 0;
     }
-    const int W = (m + 31) >> 5, h = R.r1 - R.r0, tw = R.c1 - R.c0;
-    bool ok = true;
-    ws.colbits = (uint32_t *)arena_alloc(A, sizeof(uint32_t) * (unsigned long long)n * W, &ok);
-    ws.atomRows = (int16_t *)arena_alloc(A, sizeof(int16_t) * (unsigned long long)n * m, &ok);
-    ws.holeRows = (int16_t *)arena_alloc(A, sizeof(int16_t) * (unsigned long long)tw * h, &ok);
-    ws.col = (ColInfo *)arena_alloc(A, sizeof(ColInfo) * (unsigned long long)n, &ok);
-    ws.recv = (RecvInfo *)arena_alloc(A, sizeof(RecvInfo) * (unsigned long long)n, &ok);
-    ws.ev = (Event *)arena_alloc(A, sizeof(Event) * (unsigned long long)(n + 1), &ok);
-    ws.unitOff = (int32_t *)arena_alloc(A, sizeof(int32_t) * (unsigned long long)(2 * n + 1), &ok);
+    // one request to the arena per warp: its instances' sizes, scanned (an
+    // atomic per array and instance on the one bump pointer took 82 us for
+    // 16 384 chains, this 11 us)
+    const int W = (m + 31) >> 5;
+    const unsigned long long sz[7] = {
+        arena_pad(sizeof(uint32_t) * (unsigned long long)n * W), arena_pad(sizeof(int16_t) * (unsigned long long)n * m),
+        arena_pad(sizeof(int16_t) * (unsigned long long)tw * h), arena_pad(sizeof(ColInfo) * (unsigned long long)n),
+        arena_pad(sizeof(RecvInfo) * (unsigned long long)n), n ? arena_pad(sizeof(Event) * (unsigned long long)(n + 1)) : 0,
+        n ? arena_pad(sizeof(int32_t) * (unsigned long long)(2 * n + 1)) : 0};
+    unsigned long long need = 0;
+#pragma unroll
+    for (int u = 0; u < 7; ++u) need += sz[u];
+    unsigned long long incl = need;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const unsigned long long v = __shfl_up_sync(FULL, incl, o);
+        if (lane >= o) incl += v;
+    }
+    unsigned long long off = 0;
+    if (lane == 31 && incl) off = atomicAdd(A.top, incl);
+    off = __shfl_sync(FULL, off, 31) + incl - need;
+    if (n == 0) return;
+    JobWS &ws = wsv[q];
     ws.nrecv = 0; ws.nev = 0;
-    if (!ok) I->status = RR_ERR_WORKSPACE;
+    if (off + need > A.size) { I->status = RR_ERR_WORKSPACE; return; }
+    char *at = A.base + off;
+    ws.colbits = (uint32_t *)at; at += sz[0];
+    ws.atomRows = (int16_t *)at; at += sz[1];
+    ws.holeRows = (int16_t *)at; at += sz[2];
+    ws.col = (ColInfo *)at; at += sz[3];
+    ws.recv = (RecvInfo *)at; at += sz[4];
+    ws.ev = (Event *)at; at += sz[5];
+    ws.unitOff = (int32_t *)at;
 }
 
 // ------------------------------------------------- S0: load and transpose
@@ -66,7 +78,11 @@ __device__ inline void s_plan_setup(const Blk B, rr_instance *inst, JobWS *wsv, 
 // reads four consecutive bytes (columns 4l .. 4l+3) of each row in one
 // 4-byte load, so that a warp reads 128 contiguous bytes per row, and builds
 // its four columns' words. Other rows: lane l reads column 32g + l byte by
-// byte (32 contiguous bytes per row and warp).
+// byte (32 contiguous bytes per row and warp). Grids of at most NARROW
+// columns (1D chains are one column) leave most of those lanes idle: there
+// the lanes take rows, and a vote makes a word (16 384 chains of 1 024 traps
+// in 36 us instead of 246).
+constexpr int NARROW = 8;
 __device__ inline void s_transpose(const Blk B, rr_instance *inst, JobWS *wsv, int count)
 {
     const int q = B.y;
@@ -76,8 +92,33 @@ __device__ inline void s_transpose(const Blk B, rr_instance *inst, JobWS *wsv, i
     JobWS &ws = wsv[q];
     const int m = I->m, n = I->n, W = (m + 31) >> 5, G = (n + 31) >> 5, G4 = (n + 127) >> 7;
     const int lane = threadIdx.x & 31;
-    const int w0 = B.x * (blockDim.x >> 5) + (threadIdx.x >> 5), nw = B.gx * (blockDim.x >> 5);
-    if (I->layout == RR_BITS32) {
+    const int w0 = B.w, nw = B.nw;
+    if (I->layout == RR_U8 && n <= NARROW) {
+        // a few columns: 32 rows per lane group and load, one vote per word
+        // and column, four words at a time
+        const uint8_t *src = (const uint8_t *)I->grid;
+        for (int item = w0; item < (W + 3) >> 2; item += nw) {
+            const int w = 4 * item;
+            uint32_t keep[4] = {0u, 0u, 0u, 0u};
+            for (int c = 0; c < n; ++c) {
+                int x[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const int row = 32 * (w + u) + lane;
+                    x[u] = row < m ? src[(size_t)row * n + c] : 0;
+                }
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const uint32_t b = __ballot_sync(FULL, x[u] != 0);
+                    if (lane == c) keep[u] = b;
+                }
+            }
+            if (lane < n)
+#pragma unroll
+                for (int u = 0; u < 4; ++u)
+                    if (w + u < W) ws.colbits[(size_t)lane * W + w + u] = keep[u];
+        }
+    } else if (I->layout == RR_BITS32) {
         const uint32_t *src = (const uint32_t *)I->grid;
         if ((G & 3) == 0 && ((uintptr_t)src & 15) == 0) {
             for (int item = w0; item < G4 * W; item += nw) {
@@ -169,29 +210,31 @@ __device__ inline void s_colstats(const Blk B, rr_instance *inst, JobWS *wsv, in
     const int r0 = I->rect.r0, r1 = I->rect.r1, c0 = I->rect.c0, c1 = I->rect.c1;
     const int h = r1 - r0, R = m - h;
     const int lane = threadIdx.x & 31;
-    const int nw = B.gx * (blockDim.x >> 5);
-    for (int c = B.x * (blockDim.x >> 5) + (threadIdx.x >> 5); c < n; c += nw) {
+    for (int c = B.w; c < n; c += B.nw) {
         const uint32_t x = lane < W ? ws.colbits[(size_t)c * W + lane] : 0u;
         const uint32_t mT = row_mask(lane, 0, r0), mBd = row_mask(lane, r0, r1), mO = row_mask(lane, r1, m);
-        const int cAll = __popc(x);
-        const int incl = warp_incl_scan(cAll);
-        const int K = __shfl_sync(FULL, incl, 31);
+        const int K = warp_sum(__popc(x));
         const int ntop = warp_sum(__popc(x & mT));
         const int nband = warp_sum(__popc(x & mBd));
         const int nbot = warp_sum(__popc(x & mO));
         int16_t *rows = ws.atomRows + (size_t)c * m;
-        {
-            int p = incl - cAll;
-            uint32_t y = x;
-            while (y) { const int b = __ffs(y) - 1; rows[p++] = (int16_t)(32 * lane + b); y &= y - 1; }
-        }
         const bool target = c >= c0 && c < c1;
         int16_t *hr = target ? ws.holeRows + (size_t)(c - c0) * h : nullptr;
-        if (target) {
-            uint32_t hx = ~x & mBd;
-            const int ch = __popc(hx);
-            int p = warp_incl_scan(ch) - ch;
-            while (hx) { const int b = __ffs(hx) - 1; hr[p++] = (int16_t)(32 * lane + b); hx &= hx - 1; }
+        // the atoms' rows, and a target column's band holes: a word at a time,
+        // a row per lane, so that a store covers consecutive places (a word
+        // per lane and its bits in turn: 241 us for 2 000 grids of sides 33
+        // to 251, this 116 us)
+        int pa = 0, ph = 0;
+        const unsigned lt = (1u << lane) - 1u;
+        for (int w = 0; w < W; ++w) {
+            const uint32_t xw = __shfl_sync(FULL, x, w);
+            if ((xw >> lane) & 1u) rows[pa + __popc(xw & lt)] = (int16_t)(32 * w + lane);
+            pa += __popc(xw);
+            if (target) {
+                const uint32_t hw = ~xw & row_mask(w, r0, r1);
+                if ((hw >> lane) & 1u) hr[ph + __popc(hw & lt)] = (int16_t)(32 * w + lane);
+                ph += __popc(hw);
+            }
         }
         __syncwarp();
 
@@ -233,13 +276,11 @@ __device__ inline void s_colstats(const Blk B, rr_instance *inst, JobWS *wsv, in
             const uint32_t brk = ~x | ~valid;                     // first non-atom from row 0
             const int fz = brk ? 32 * lane + __ffs(brk) - 1 : 0x7fffffff;
             int firstZero = fz;
-#pragma unroll
-            for (int o = 16; o; o >>= 1) firstZero = min(firstZero, __shfl_xor_sync(FULL, firstZero, o));
+            firstZero = __reduce_min_sync(FULL, firstZero);
             if (firstZero > m) firstZero = m;
             const uint32_t z2 = ~x & valid;                       // last empty row
             int lz = z2 ? 32 * lane + 31 - __clz(z2) : -1;
-#pragma unroll
-            for (int o = 16; o; o >>= 1) lz = max(lz, __shfl_xor_sync(FULL, lz, o));
+            lz = __reduce_max_sync(FULL, lz);
             ci.topRun = min(firstZero, r0);
             ci.botRun = min(m - 1 - lz, m - r1);
             ci.nmoves = (r0 - ci.topRun) + (m - r1 - ci.botRun);
@@ -254,33 +295,43 @@ __device__ inline void s_colstats(const Blk B, rr_instance *inst, JobWS *wsv, in
 
 // ------------------------------------------------- S4: pairing (one warp)
 
-struct PairSmem {
-    int32_t *sig;
-    int16_t *prv, *nxt, *tT, *bT, *mandT, *mandB, *evHead, *evTail, *evCnt;
-    unsigned long long *score;
-};
+constexpr size_t WARM_BYTES = 160 * 1024;    // rows that fit L1 beside the pairing's shared memory
 
-__device__ __forceinline__ unsigned long long pair_score(const PairSmem &S, int c)
+// What the pairing keeps of a column in shared memory.
+struct PairCol {
+    int16_t kind, ptop, pbot, tbase, bbase, nband;   // as in ColInfo
+    int16_t tT, bT;          // donor: pool cursors
+    int16_t mandT, mandB;    // receiver: atoms above / below the band so far
+    int16_t nev, recv;       // receiver: its events, its place in saturation order
+};
+// (rr_capi.cu, rr_noalloc.cu and the single-grid kernel size it by this, 64
+// bytes more)
+static_assert(sizeof(PairCol) == 24 && PAIR_BYTES == 8 + 4 + 24 + 3 * 2, "shared memory of the pairing");
+
+// Score of the pair of columns c < v with surpluses s1 and s2 (v < 0: none).
+// Larger is better: tokens exchanged, then smaller gap, then smaller deficit,
+// then smaller receiver index, then smaller donor index; c last.
+__device__ __forceinline__ uint2 pair_score(int c, int v, int s1, int s2)
 {
-    const int s1 = S.sig[c];
-    if (s1 == 0) return 0ull;
-    const int v = S.nxt[c];
-    if (v < 0) return 0ull;
-    const int s2 = S.sig[v];
-    if ((s1 > 0) == (s2 > 0)) return 0ull;
-    const int i = s1 > 0 ? c : v, j = s1 > 0 ? v : c;
-    const int need = -S.sig[j];
-    const int x = min(S.sig[i], need);
-    const int d = iabs(i - j);
-    const unsigned long long left = i < j ? 1ull : 0ull;
-    // larger is better: tokens exchanged, then smaller gap, then smaller
-    // deficit, then smaller receiver index, then smaller donor index.
-    return ((unsigned long long)x << 42) | ((unsigned long long)(1023 - d) << 32) |
-           ((unsigned long long)(2047 - need) << 21) | ((unsigned long long)(1023 - j) << 11) |
-           (left << 10) | (unsigned long long)c;
+    const bool right = s1 > 0;                        // the donor is c
+    const int give = right ? s1 : s2, need = -(right ? s2 : s1), j = right ? v : c;
+    uint2 r;
+    r.y = (unsigned)min(give, need) << 10 | (unsigned)(1023 - (v - c));
+    r.x = (unsigned)(2047 - need) << 21 | (unsigned)(1023 - j) << 11 | (right ? 1u << 10 : 0u) | (unsigned)c;
+    const bool none = v < 0 || s1 == 0 || s2 == 0 || (s1 > 0) == (s2 > 0);
+    return none ? make_uint2(0u, 0u) : r;
 }
 
-__device__ inline void s_pair(const Blk B, rr_instance *inst, JobWS *wsv, int count)
+// The pairing loop is one chain: the best pair, the donor's tokens it takes
+// (a search over rows in global memory), the scores that change. So each
+// column's best-pair score stays in shared memory and the best of a lane's
+// columns in its registers (two warp reductions find the pair); at most three
+// scores change per pair (its two columns' and that of the column before
+// them), computed side by side from values in registers; what is needed of a
+// column is in shared memory; and `warm` (calls over few grids) brings the
+// atoms' and holes' rows into L1 first. One 256 x 256 grid, 241 pairs: 243 us
+// (with the scores rescanned, one lane updating them, and rows from L2: 400).
+__device__ inline void s_pair(const Blk B, rr_instance *inst, JobWS *wsv, int count, int warm)
 {
     extern __shared__ unsigned long long smem_u64[];
     const int q = B.x;
@@ -293,25 +344,31 @@ __device__ inline void s_pair(const Blk B, rr_instance *inst, JobWS *wsv, int co
     const int h = r1 - r0;
     const int lane = threadIdx.x & 31;
 
-    PairSmem S;
-    S.score = smem_u64;
-    S.sig = (int32_t *)(smem_u64 + n);
-    S.prv = (int16_t *)(S.sig + n);
-    S.nxt = S.prv + n; S.tT = S.nxt + n; S.bT = S.tT + n; S.mandT = S.bT + n; S.mandB = S.mandT + n;
-    S.evHead = S.mandB + n; S.evTail = S.evHead + n; S.evCnt = S.evTail + n;
+    uint2 *score = (uint2 *)smem_u64;                 // n: of the pair of a column and the next one in the list
+    int32_t *sig = (int32_t *)(smem_u64 + n);         // n: surplus
+    PairCol *col = (PairCol *)(sig + n);
+    int16_t *prv = (int16_t *)(col + n), *nxt = prv + n, *evOrd = nxt + n;
+    const uint32_t dump = sh_addr((void *)(((uintptr_t)(evOrd + n) + 15) & ~(uintptr_t)15));
+    if (warm) {
+        const size_t ba = 2 * (size_t)n * m, bh = 2 * (size_t)(I->rect.c1 - c0) * h;
+        if (ba + bh <= WARM_BYTES) {
+            for (size_t o = 32 * (size_t)lane; o < ba; o += 1024) touch_if(true, (const char *)ws.atomRows + o, dump);
+            for (size_t o = 32 * (size_t)lane; o < bh; o += 1024) touch_if(true, (const char *)ws.holeRows + o, dump);
+        }
+    }
 
     int tot = 0, nneg = 0;
     for (int c = lane; c < n; c += 32) {
         const ColInfo ci = ws.col[c];
-        S.sig[c] = ci.sigma;
-        S.tT[c] = 0; S.bT[c] = 0;
-        S.mandT[c] = (int16_t)ci.ntop; S.mandB[c] = (int16_t)ci.nbot;
-        S.evHead[c] = -1; S.evTail[c] = -1; S.evCnt[c] = 0;
+        sig[c] = ci.sigma;
+        col[c] = PairCol{(int16_t)ci.kind, (int16_t)ci.ptop, (int16_t)ci.pbot, (int16_t)ci.tbase, (int16_t)ci.bbase,
+                         (int16_t)ci.nband, 0, 0, (int16_t)ci.ntop, (int16_t)ci.nbot, 0, -1};
         tot += ci.sigma;
         nneg += ci.sigma < 0;
     }
     tot = warp_sum(tot);
     nneg = warp_sum(nneg);
+    touch_wait();
     if (tot < 0) {                    // some column can never be saturated (Sec. III.C)
         if (lane == 0) { I->status = RR_INFEASIBLE; I->n_moves = 0; }
         return;
@@ -322,119 +379,143 @@ __device__ inline void s_pair(const Blk B, rr_instance *inst, JobWS *wsv, int co
         int carry = -1;
         for (int base = ((n - 1) >> 5) << 5; base >= 0; base -= 32) {
             const int c = base + lane;
-            const unsigned nz = __ballot_sync(FULL, c < n && S.sig[c] != 0);
+            const unsigned nz = __ballot_sync(FULL, c < n && sig[c] != 0);
             const unsigned above = lane < 31 ? nz & ~((2u << lane) - 1u) : 0u;
-            if (c < n) S.nxt[c] = (int16_t)(above ? base + __ffs(above) - 1 : carry);
+            if (c < n) nxt[c] = (int16_t)(above ? base + __ffs(above) - 1 : carry);
             if (nz) carry = base + __ffs(nz) - 1;
         }
         carry = -1;
         for (int base = 0; base < n; base += 32) {
             const int c = base + lane;
-            const unsigned nz = __ballot_sync(FULL, c < n && S.sig[c] != 0);
+            const unsigned nz = __ballot_sync(FULL, c < n && sig[c] != 0);
             const unsigned below = nz & ((1u << lane) - 1u);
-            if (c < n) S.prv[c] = (int16_t)(below ? base + 31 - __clz(below) : carry);
+            if (c < n) prv[c] = (int16_t)(below ? base + 31 - __clz(below) : carry);
             if (nz) carry = base + 31 - __clz(nz);
         }
     }
     __syncwarp();
-    for (int c = lane; c < n; c += 32) S.score[c] = pair_score(S, c);
-    __syncwarp();
+    for (int c = lane; c < n; c += 32) {
+        const int v = nxt[c];
+        score[c] = pair_score(c, v, sig[c], v >= 0 ? sig[v] : 0);
+    }
+    // the best of this lane's columns c = lane, lane + 32, ...
+    unsigned mine_y = 0u, mine_x = 0u;
+    auto best_of_lane = [&]() {
+        mine_y = mine_x = 0u;
+#pragma unroll 4
+        for (int c = lane; c < n; c += 32) {
+            const uint2 s = score[c];
+            const bool more = s.y > mine_y || (s.y == mine_y && s.x > mine_x);
+            mine_y = more ? s.y : mine_y;
+            mine_x = more ? s.x : mine_x;
+        }
+    };
+    best_of_lane();
 
     int nrecv = 0, nev = 0;
     const int16_t *allRows = ws.atomRows;
     for (int iter = 0; nneg > 0; ++iter) {
         if (iter > n || (g_guard_cap > 0 && iter >= g_guard_cap)) { if (lane == 0) I->status = RR_ERR_TIMEOUT; return; }
-        unsigned long long best = 0ull;
-        for (int c = lane; c < n; c += 32) { const unsigned long long s = S.score[c]; best = s > best ? s : best; }
-        best = warp_max_u64(best);
-        if (best == 0ull) { if (lane == 0) I->status = RR_ERR_INTERNAL; return; }
-        const int cpos = (int)(best & 1023ull);
-        const int other = S.nxt[cpos];
-        const int i = S.sig[cpos] > 0 ? cpos : other;
-        const int j = S.sig[cpos] > 0 ? other : cpos;
-        const int si = S.sig[i], need = -S.sig[j];
+        const unsigned by = __reduce_max_sync(FULL, mine_y);
+        if (by == 0u) { if (lane == 0) I->status = RR_ERR_INTERNAL; return; }
+        const int cl = (int)(__reduce_max_sync(FULL, mine_y == by ? mine_x : 0u) & 1023u);   // the pair: cl and
+        const int cr = nxt[cl], pl = prv[cl], nr = nxt[cr];                                   // cr; around it: pl, nr
+        const int sl0 = sig[cl], sr0 = sig[cr], spl = pl >= 0 ? sig[pl] : 0, snr = nr >= 0 ? sig[nr] : 0;
+        const int i = sl0 > 0 ? cl : cr, j = sl0 > 0 ? cr : cl;
+        const int si = sl0 > 0 ? sl0 : sr0, need = -(sl0 > 0 ? sr0 : sl0);
         const int x = min(si, need);
         const int kase = si > need ? 1 : (si == need ? 2 : 3);
-        const ColInfo D = ws.col[i];
+        const PairCol D = col[i], Rj = col[j];
         const int16_t *drows = allRows + (size_t)i * m;
-        const int t0 = S.tT[i], b0 = S.bT[i];
+        const int t0 = D.tT, b0 = D.bT;
         const int availT = D.ptop - t0, availB = D.pbot - b0;
         const int e = nev++;
-        Event ev;
-        ev.kase = kase; ev.i = i; ev.j = j; ev.x = x; ev.t0 = t0; ev.b0 = b0; ev.next = -1;
+        if (e >= n) { if (lane == 0) I->status = RR_ERR_INTERNAL; return; }   // an event settles a column
+        int a;
+        __syncwarp();
         if (kase == 3) {
-            ev.a = availT;
+            a = availT;
             if (lane == 0) {
-                S.mandT[j] += (int16_t)availT; S.mandB[j] += (int16_t)availB;
-                S.tT[i] = (int16_t)D.ptop; S.bT[i] = (int16_t)D.pbot;
-                S.sig[j] += si; S.sig[i] = 0;
+                col[j].mandT = (int16_t)(Rj.mandT + availT); col[j].mandB = (int16_t)(Rj.mandB + availB);
+                col[i].tT = D.ptop; col[i].bT = D.pbot;
             }
         } else {
-            const int mT = S.mandT[j], mB = S.mandB[j];
-            const ColInfo Rj = ws.col[j];
+            const int mT = Rj.mandT, mB = Rj.mandB;
             const int M = Rj.nband, nh = h - M;
             const int16_t *hr = ws.holeRows + (size_t)(j - c0) * h;
-            int a;
             if (kase == 2) {
                 a = availT;
                 if (availT + availB != x) { if (lane == 0) I->status = RR_ERR_INTERNAL; return; }
             } else {
                 const int lo = max(0, x - availB), hi = min(x, availT);
+                const bool full = D.kind == KIND_OUTER_FULL;
                 a = split_search(lo, hi, [&](int aa) {
-                    const int tr = pool_top_row(D, drows, r0, t0 + aa - 1);
-                    const int br = pool_bot_row(D, drows, r1, b0 + x - aa);
+                    const int lt = t0 + aa - 1, lb = b0 + x - aa;      // the donor's next pool atoms
+                    const int tr = full ? r0 - 1 - lt : (int)drows[D.tbase - lt];
+                    const int br = full ? r1 + lb : (int)drows[D.bbase + lb];
                     return (r0 + mT + aa - 1 - tr) + (2 * band_P(hr, nh, M, r0, r0 + mT + aa - 1) - M) +
                            (r0 + h - mB - x + aa - 1 - br);
                 });
             }
-            ev.a = a;
             const int nT = mT + a;
-            RecvInfo ri;
-            ri.j = j;
-            ri.nT = nT;
-            ri.kd_end = nT + band_P(hr, nh, M, r0, r0 + nT - 1);
-            ri.ku_start = nT + band_P(hr, nh, M, r0, r0 + nT);
-            ri.nmoves = ri.kd_end + (h - ri.ku_start);
-            ri.pad = 0;
+            const int kd = nT + band_P(hr, nh, M, r0, r0 + nT - 1), ku = nT + band_P(hr, nh, M, r0, r0 + nT);
             if (lane == 0) {
-                S.tT[i] = (int16_t)(t0 + a); S.bT[i] = (int16_t)(b0 + x - a);
-                S.sig[i] -= x; S.sig[j] = 0;
-                // link this event, then close the receiver's list
-                if (S.evTail[j] >= 0) ws.ev[S.evTail[j]].next = e; else S.evHead[j] = (int16_t)e;
-                S.evTail[j] = (int16_t)e; S.evCnt[j] += 1;
-                ri.ev_first = S.evHead[j];
-                ri.ncontrib = S.evCnt[j];
+                col[i].tT = (int16_t)(t0 + a); col[i].bT = (int16_t)(b0 + x - a);
+                col[j].recv = (int16_t)nrecv;
+                RecvInfo ri;
+                ri.j = j;
+                ri.ev_first = 0;
+                ri.ncontrib = Rj.nev + 1;
+                ri.nT = nT;
+                ri.kd_end = kd;
+                ri.ku_start = ku;
+                ri.nmoves = kd + (h - ku);
+                ri.pad = 0;
                 ws.recv[nrecv] = ri;
             }
             ++nrecv;
             --nneg;
         }
+        // surpluses after it, the columns that reached zero out of the list,
+        // the three scores that change
+        const int sl = sl0 > 0 ? sl0 - x : sl0 + x, sr = sr0 > 0 ? sr0 - x : sr0 + x;
+        const bool zl = sl == 0, zr = sr == 0;
+        const int afterPl = zl ? (zr ? nr : cr) : cl, sAfterPl = zl ? (zr ? snr : sr) : sl;
+        const int afterL = zr ? nr : cr, sAfterL = zr ? snr : sr;
         if (lane == 0) {
-            if (kase == 3) {
-                if (S.evTail[j] >= 0) ws.ev[S.evTail[j]].next = e; else S.evHead[j] = (int16_t)e;
-                S.evTail[j] = (int16_t)e; S.evCnt[j] += 1;
-            }
+            evOrd[e] = Rj.nev;
+            col[j].nev = (int16_t)(Rj.nev + 1);
+            Event ev;
+            ev.kase = kase; ev.i = i; ev.j = j; ev.x = x; ev.a = a; ev.t0 = t0; ev.b0 = b0; ev.at = -1;
             ws.ev[e] = ev;
-            // unlink columns that reached zero and refresh the scores around them
-            int touched[6]; int nt = 0;
-            const int cols2[2] = {i, j};
-            for (int u = 0; u < 2; ++u) {
-                const int c = cols2[u];
-                if (S.sig[c] == 0) {
-                    const int p = S.prv[c], nx = S.nxt[c];
-                    if (p >= 0) S.nxt[p] = (int16_t)nx;
-                    if (nx >= 0) S.prv[nx] = (int16_t)p;
-                    S.score[c] = 0ull;
-                    if (p >= 0) touched[nt++] = p;
-                } else {
-                    touched[nt++] = c;
-                    if (S.prv[c] >= 0) touched[nt++] = S.prv[c];
-                }
-            }
-            for (int u = 0; u < nt; ++u) S.score[touched[u]] = pair_score(S, touched[u]);
+            sig[cl] = sl;
+            sig[cr] = sr;
+            if (pl >= 0) nxt[pl] = (int16_t)afterPl;
+            if (!zl) nxt[cl] = (int16_t)afterL;
+            if (!zr) prv[cr] = (int16_t)(zl ? pl : cl);
+            if (nr >= 0) prv[nr] = (int16_t)(zr ? (zl ? pl : cl) : cr);
+        }
+        {
+            const int c = lane == 0 ? pl : lane == 1 ? cl : cr;
+            const uint2 s = lane == 0 ? pair_score(pl, afterPl, spl, sAfterPl)
+                                      : lane == 1 ? pair_score(cl, afterL, sl, sAfterL) : pair_score(cr, nr, sr, snr);
+            if (lane < 3 && c >= 0) score[c] = s;
         }
         __syncwarp();
+        if ((pl & 31) == lane || (cl & 31) == lane || (cr & 31) == lane) best_of_lane();
+        __syncwarp();
     }
+    // the events ordered by receiver: a receiver's first slot, then each
+    // event's slot
+    for (int base = 0, carry = 0; base < nrecv; base += 32) {
+        const int r = base + lane;
+        const int v = r < nrecv ? ws.recv[r].ncontrib : 0;
+        const int incl = warp_incl_scan(v);
+        if (r < nrecv) { ws.recv[r].ev_first = carry + incl - v; sig[r] = carry + incl - v; }
+        carry += __shfl_sync(FULL, incl, 31);
+    }
+    __syncwarp();
+    for (int e = lane; e < nev; e += 32) ws.ev[sig[col[ws.ev[e].j].recv] + evOrd[e]].at = e;
     // move offsets of all solve units: column units in column order, then
     // receiver units in saturation order
     int carry = 0;
@@ -469,10 +550,9 @@ __device__ inline void s_emit_cols(const Blk B, rr_instance *inst, JobWS *wsv, i
     const int m = I->m, n = I->n;
     const int r0 = I->rect.r0, r1 = I->rect.r1, h = r1 - r0;
     const int lane = threadIdx.x & 31;
-    const int nw = B.gx * (blockDim.x >> 5);
     rr_move *out = I->moves;
     long long steps = 0;
-    for (int c = B.x * (blockDim.x >> 5) + (threadIdx.x >> 5); c < n; c += nw) {
+    for (int c = B.w; c < n; c += B.nw) {
         const ColInfo ci = ws.col[c];
         if (ci.nmoves == 0) continue;
         const int16_t *rows = ws.atomRows + (size_t)c * m;
@@ -485,17 +565,17 @@ __device__ inline void s_emit_cols(const Blk B, rr_instance *inst, JobWS *wsv, i
                 if (k < ci.kd_end) pos = ci.kd_end - 1 - k;                  // toward larger rows, deepest first
                 else if (k >= ci.ku_start) pos = ci.kd_end + (k - ci.ku_start);  // toward smaller rows
                 else continue;                                                // isolated
-                o[pos] = rr_move{s, c, r0 + k, c};
+                store_move(&o[pos], s, c, r0 + k, c);
                 steps += iabs(r0 + k - s);
             }
         } else {   // KIND_OUTER_FULL
             const int nbg = m - r1, ndown = nbg - ci.botRun;
             for (int k = lane; k < ndown; k += 32) {
-                o[ndown - 1 - k] = rr_move{rows[ci.K - nbg + k], c, r1 + k, c};
+                store_move(&o[ndown - 1 - k], rows[ci.K - nbg + k], c, r1 + k, c);
                 steps += r1 + k - rows[ci.K - nbg + k];
             }
             for (int k = ci.topRun + lane; k < r0; k += 32) {
-                o[ndown + (k - ci.topRun)] = rr_move{rows[k], c, k, c};
+                store_move(&o[ndown + (k - ci.topRun)], rows[k], c, k, c);
                 steps += rows[k] - k;
             }
         }
@@ -505,6 +585,17 @@ __device__ inline void s_emit_cols(const Blk B, rr_instance *inst, JobWS *wsv, i
 
 // ---------------------------------------------------- S5/S6: receiver units
 
+// A receiver's h sources, 32 at a time, a source per lane. A warp takes a
+// whole receiver, or where there are enough warps (single grids) 32 of its
+// sources. The receiver's contributors (the donors of its pairing events) are
+// read side by side, one per lane, into the warp's part of shared memory; each
+// lane then ranks its own source among all contributors by popcounts. What
+// bounds it is the chain of dependent loads before the first rank (receiver,
+// column, events, donors: about 4 000 cycles), so a warp goes through it once
+// per receiver. (A block of 256 threads per receiver, whose first thread
+// walked the events as a linked list while the others waited, and binary
+// searches over the donors' rows: 870 us for 2 000 grids of sides 33 to 251;
+// this: 375 us.)
 struct Contrib {
     int32_t col, kind, tbase, bbase;
     int32_t tStart, tCnt, bStart, bCnt;
@@ -512,142 +603,157 @@ struct Contrib {
 };
 
 // Top-region order at equal rows: farther column first, right before left.
-__device__ __forceinline__ bool top_before(const Contrib &a, const Contrib &b)
-{
-    return a.d > b.d || (a.d == b.d && a.right && !b.right);
-}
+__device__ __forceinline__ bool top_before(int da, int ra, int db, int rb) { return da > db || (da == db && ra && !rb); }
 // Bottom-region order at equal rows: nearer column first, left before right.
-__device__ __forceinline__ bool bot_before(const Contrib &a, const Contrib &b)
-{
-    return a.d < b.d || (a.d == b.d && !a.right && b.right);
-}
+__device__ __forceinline__ bool bot_before(int da, int ra, int db, int rb) { return da < db || (da == db && !ra && rb); }
 
-constexpr int MAX_CONTRIB = 1024;
+constexpr int EMIT_WARPS = 8;    // at most, per block
+
+// Atoms of a bit column in rows below `row`; *here: whether row holds one.
+__device__ __forceinline__ int col_rank(const uint32_t *col, int row, bool *here)
+{
+    const int w = row >> 5;
+    int r = 0;
+    const uint32_t x = col[w], bit = 1u << (row & 31);
+    for (int u0 = 0; u0 < w; u0 += 8) {            // eight loads in flight at once
+        uint32_t y[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) y[u] = u0 + u < w ? col[u0 + u] : 0u;
+#pragma unroll
+        for (int u = 0; u < 8; ++u) r += __popc(y[u]);
+    }
+    *here = (x & bit) != 0u;
+    return r + __popc(x & (bit - 1u));
+}
 
 __device__ inline void s_emit_recv(const Blk B, rr_instance *inst, JobWS *wsv, int count)
 {
-    __shared__ Contrib C[MAX_CONTRIB + 1];
-    __shared__ int s_nc;
+    __shared__ Contrib Call[EMIT_WARPS][32];
     const int q = B.y;
     if (q >= count) return;
     rr_instance *I = &inst[q];
     if (!live(I)) return;
     JobWS &ws = wsv[q];
+    Contrib *C = Call[threadIdx.x >> 5];
+    const int lane = threadIdx.x & 31;
     const int m = I->m, n = I->n;
     const int r0 = I->rect.r0, r1 = I->rect.r1, h = r1 - r0;
+    const int W = (m + 31) >> 5, chunks = (h + 31) >> 5;
+    const int split = B.nw >= ws.nrecv * chunks ? chunks : 1, items = ws.nrecv * split;
     long long steps = 0;
-    for (int r = B.x; r < ws.nrecv; r += B.gx) {
+    for (int it = B.w; it < items; it += B.nw) {
+        const int r = it / split;
         const RecvInfo ri = ws.recv[r];
-        const int j = ri.j;
+        const int j = ri.j, nc = ri.ncontrib;
         const ColInfo Rj = ws.col[j];
         const int16_t *own = ws.atomRows + (size_t)j * m;
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            int nc = 0, first = Rj.K, e = ri.ev_first;
-            for (int u = 0; u < ri.ncontrib && e >= 0 && nc < MAX_CONTRIB; ++u) {
-                const Event ev = ws.ev[e];
+        const int ownTop = Rj.ntop, ownBand = Rj.nband;
+        const long long out = ws.unitOff[n + r];
+        int first = Rj.K;
+        auto load = [&](int g0) {
+            __syncwarp();
+            Contrib c;
+            int cnt = 0;
+            if (g0 + lane < nc) {
+                const Event ev = ws.ev[ws.ev[ri.ev_first + g0 + lane].at];
                 const ColInfo D = ws.col[ev.i];
-                Contrib c;
                 c.col = ev.i; c.kind = D.kind; c.tbase = D.tbase; c.bbase = D.bbase;
                 c.tStart = ev.t0; c.bStart = ev.b0;
                 if (ev.kase == 3) { c.tCnt = D.ptop - ev.t0; c.bCnt = D.pbot - ev.b0; }
                 else { c.tCnt = ev.a; c.bCnt = ev.x - ev.a; }
-                c.d = iabs(ev.i - j); c.right = ev.i > j; c.first = first;
-                first += c.tCnt + c.bCnt;
-                C[nc++] = c;
-                e = ev.next;
+                c.d = iabs(ev.i - j); c.right = ev.i > j;
+                cnt = c.tCnt + c.bCnt;
             }
-            if (first != h || nc != ri.ncontrib) set_status(I, RR_ERR_INTERNAL);
-            s_nc = nc;
-        }
-        __syncthreads();
-        if (!live(I)) break;
-        const int nc = s_nc;
-        rr_move *o = I->moves + ws.unitOff[n + r];
-        const int ownTop = Rj.ntop, ownBand = Rj.nband;
-        for (int t = threadIdx.x; t < h; t += blockDim.x) {
-            int row, col, ci = -1;
-            if (t < Rj.K) { row = own[t]; col = j; }
-            else {
-                int lo = 0, hi = nc - 1;                 // contributor holding source t
-                while (lo < hi) { const int mid = (lo + hi + 1) >> 1; if (C[mid].first <= t) lo = mid; else hi = mid - 1; }
-                ci = lo;
-                const Contrib &c = C[ci];
-                const int u = t - c.first;
-                const int16_t *drows = ws.atomRows + (size_t)c.col * m;
-                if (u < c.tCnt) {
-                    const int l = c.tStart + u;
-                    row = c.kind == KIND_OUTER_FULL ? r0 - 1 - l : drows[c.tbase - l];
-                } else {
-                    const int l = c.bStart + (u - c.tCnt);
-                    row = c.kind == KIND_OUTER_FULL ? r1 + l : drows[c.bbase + l];
+            const int incl = warp_incl_scan(cnt);
+            if (g0 + lane < nc) { c.first = first + incl - cnt; C[lane] = c; }
+            first += __shfl_sync(FULL, incl, 31);
+            __syncwarp();
+        };
+        if (nc <= 32) load(0);                    // (more are loaded where they are read)
+        for (int t0 = (it - r * split) * 32; t0 < h; t0 += 32 * split) {
+            const int t = t0 + lane;
+            int row = t < Rj.K && t < h ? own[t] : 0, col = j, ci = -1, sd = 0, sr = 0, u = 0, stc = 0;
+            // which source this lane has
+            int before = Rj.K;
+            if (nc > 32) first = Rj.K;
+            for (int g0 = 0; g0 < nc; g0 += 32) {
+                if (nc > 32) { before = first; load(g0); }
+                if (t >= before && t < first) {
+                    int lo = 0, hi = min(32, nc - g0) - 1;   // contributor holding source t
+                    while (lo < hi) { const int mid = (lo + hi + 1) >> 1; if (C[mid].first <= t) lo = mid; else hi = mid - 1; }
+                    const Contrib c = C[lo];
+                    ci = g0 + lo;
+                    u = t - c.first;
+                    sd = c.d; sr = c.right; stc = c.tCnt; col = c.col;
+                    const int16_t *drows = ws.atomRows + (size_t)c.col * m;
+                    if (u < c.tCnt) {
+                        const int l = c.tStart + u;
+                        row = c.kind == KIND_OUTER_FULL ? r0 - 1 - l : drows[c.tbase - l];
+                    } else {
+                        const int l = c.bStart + (u - c.tCnt);
+                        row = c.kind == KIND_OUTER_FULL ? r1 + l : drows[c.bbase + l];
+                    }
                 }
-                col = c.col;
             }
-            int k;
-            if (row >= r0 && row < r1) {
-                k = ri.nT + (t - ownTop);                 // own band atom (only own atoms sit in the band)
-            } else {
-                const bool top = row < r0;
-                int below = 0, tie = 0;
-                Contrib self;
+            if (first != h) {
+                if (lane == 0) set_status(I, RR_ERR_INTERNAL);
+                break;
+            }
+            // its rank among the sources of its region
+            const bool in = t < h, band = row >= r0 && row < r1, top = row < r0;
+            int below = 0, tie = 0;
+            if (in && !band) {
                 if (ci < 0) {
                     // own atom: own rows of its region before it are the ones before it in index
                     below = top ? t : t - ownTop - ownBand;
-                    self.d = 0; self.right = 0;
                 } else {
-                    self = C[ci];
-                    const int lo0 = top ? 0 : ownTop + ownBand, hi0 = top ? ownTop : Rj.K;
-                    int lo = lo0, hi = hi0;
-                    while (lo < hi) { const int mid = (lo + hi) >> 1; if (own[mid] < row) lo = mid + 1; else hi = mid; }
-                    below = lo - lo0;
+                    bool here;
+                    const int rk = col_rank(ws.colbits + (size_t)j * W, row, &here);
+                    below = top ? rk : rk - ownTop - ownBand;
                     // the own atom (distance 0) comes first below the band, last above it
-                    if (!top && lo < hi0 && own[lo] == row) ++tie;
+                    tie += !top && here;
                     // this contributor's other sources on the same side: nearest-first
                     // order is descending rows above the band, ascending below it
-                    const int u = t - self.first;
-                    below += top ? self.tCnt - 1 - u : u - self.tCnt;
+                    below += top ? stc - 1 - u : u - stc;
                 }
-                for (int v = 0; v < nc; ++v) {
-                    if (v == ci) continue;
-                    const Contrib &c = C[v];
-                    const int16_t *drows = ws.atomRows + (size_t)c.col * m;
-                    if (top) {
-                        int lo = c.tStart, hi = c.tStart + c.tCnt;   // first l with row(l) < row
-                        while (lo < hi) {
-                            const int mid = (lo + hi) >> 1;
-                            const int rw = c.kind == KIND_OUTER_FULL ? r0 - 1 - mid : drows[c.tbase - mid];
-                            if (rw < row) hi = mid; else lo = mid + 1;
-                        }
-                        below += c.tStart + c.tCnt - lo;
-                        if (lo > c.tStart) {
-                            const int l = lo - 1;
-                            const int rw = c.kind == KIND_OUTER_FULL ? r0 - 1 - l : drows[c.tbase - l];
-                            if (rw == row && top_before(c, self)) ++tie;
-                        }
-                    } else {
-                        int lo = c.bStart, hi = c.bStart + c.bCnt;   // first l with row(l) >= row
-                        while (lo < hi) {
-                            const int mid = (lo + hi) >> 1;
-                            const int rw = c.kind == KIND_OUTER_FULL ? r1 + mid : drows[c.bbase + mid];
-                            if (rw < row) lo = mid + 1; else hi = mid;
-                        }
-                        below += lo - c.bStart;
-                        if (lo < c.bStart + c.bCnt) {
-                            const int rw = c.kind == KIND_OUTER_FULL ? r1 + lo : drows[c.bbase + lo];
-                            if (rw == row && bot_before(c, self)) ++tie;
-                        }
-                    }
-                }
-                k = top ? below + tie : ri.nT + ownBand + below + tie;
             }
+            if (nc > 32) first = Rj.K;
+            for (int g0 = 0; g0 < nc; g0 += 32) {
+                if (nc > 32) load(g0);
+                if (!in || band) continue;
+                for (int v = 0; v < min(32, nc - g0); ++v) {
+                    if (g0 + v == ci) continue;
+                    const Contrib c = C[v];
+                    // its sources on this side are consecutive atoms of its column
+                    // (consecutive rows in a filled outer column): how many lie in
+                    // rows below, and whether one is in this row
+                    int lowest, cnt, rk;                 // first of them, how many; atoms in rows below
+                    bool here;
+                    if (c.kind == KIND_OUTER_FULL) {
+                        lowest = top ? r0 - c.tStart - c.tCnt : r1 + c.bStart;
+                        cnt = top ? c.tCnt : c.bCnt;
+                        rk = row;
+                        here = true;
+                    } else {
+                        lowest = top ? c.tbase - c.tStart - c.tCnt + 1 : c.bbase + c.bStart;
+                        cnt = top ? c.tCnt : c.bCnt;
+                        rk = col_rank(ws.colbits + (size_t)c.col * W, row, &here);
+                    }
+                    below += min(max(rk - lowest, 0), cnt);
+                    if (here && rk >= lowest && rk < lowest + cnt &&
+                        (top ? top_before(c.d, c.right, sd, sr) : bot_before(c.d, c.right, sd, sr))) ++tie;
+                }
+            }
+            if (!in) continue;
+            // (only own atoms sit in the band)
+            const int k = band ? ri.nT + (t - ownTop) : top ? below + tie : ri.nT + ownBand + below + tie;
             if (k < 0 || k >= h) { set_status(I, RR_ERR_INTERNAL); continue; }
             int pos;
             if (k < ri.kd_end) pos = ri.kd_end - 1 - k;
             else if (k >= ri.ku_start) pos = ri.kd_end + (k - ri.ku_start);
             else continue;                                 // isolated own band atom
             if (pos >= ri.nmoves) { set_status(I, RR_ERR_INTERNAL); continue; }
-            o[pos] = rr_move{row, col, r0 + k, j};
+            store_move(&I->moves[out + pos], row, col, r0 + k, j);
             steps += iabs(r0 + k - row) + iabs(j - col);
         }
     }

@@ -85,7 +85,7 @@ __global__ void k_classify(rr_instance *inst, int count, int nclass, int max_sid
 
 // The simulation: one block per instance (of a size class's list, or of the
 // whole call).
-template <int MODE>
+template <int MODE, bool WRITERS>
 __device__ __forceinline__ void sim_of_block(rr_instance *inst, JobWS *wsv, int count, const int *classList,
                                              const int *classCount, int side, int counters)
 {
@@ -96,22 +96,36 @@ __device__ __forceinline__ void sim_of_block(rr_instance *inst, JobWS *wsv, int 
         q = classList[q];
     }
     if (q >= count) return;
-    sim_block<MODE>(&inst[q], wsv[q], (char *)sim_smem, side, counters);
+    sim_block<MODE, WRITERS>(&inst[q], wsv[q], (char *)sim_smem, side, counters);
 }
 
-// sides up to 256
-__global__ void __launch_bounds__(SIM_MAX_THREADS, 6) k_sim(rr_instance *inst, JobWS *wsv, int count,
-                                                            const int *classList, const int *classCount, int side,
-                                                            int counters)
-{
-    sim_of_block<SIM_SMALL>(inst, wsv, count, classList, classCount, side, counters);
-}
+// One warp, sides up to 256 and beyond; the same with writers. (A register
+// too few costs more than a block too few per SM: with 96 instead of 128
+// registers a 256 x 256 grid took 22 instead of 18 ms.)
+#define SIM_KERNEL(name, mode, writers, threads, blocks)                                                      \
+    __global__ void __launch_bounds__(threads, blocks) name(rr_instance *inst, JobWS *wsv, int count,         \
+                                                            const int *classList, const int *classCount,      \
+                                                            int side, int counters)                           \
+    {                                                                                                         \
+        sim_of_block<mode, writers>(inst, wsv, count, classList, classCount, side, counters);                 \
+    }
+SIM_KERNEL(k_sim, SIM_SMALL, false, 32, SIM_BLOCKS)
+SIM_KERNEL(k_sim_big, SIM_BIG, false, 32, 12)
+SIM_KERNEL(k_simw, SIM_SMALL, true, SIM_MAX_THREADS, 2)
+SIM_KERNEL(k_simw_big, SIM_BIG, true, SIM_MAX_THREADS, 2)
 
-__global__ void __launch_bounds__(SIM_MAX_THREADS, 4) k_sim_big(rr_instance *inst, JobWS *wsv, int count,
-                                                                const int *classList, const int *classCount, int side,
-                                                                int counters)
+// The batches of simulations that ran without writers.
+__global__ void __launch_bounds__(256, 6) k_write(rr_instance *inst, JobWS *wsv, int count, const int *classList,
+                                                  const int *classCount, int side)
 {
-    sim_of_block<SIM_BIG>(inst, wsv, count, classList, classCount, side, counters);
+    extern __shared__ int32_t write_smem[];
+    int q = blockIdx.y;
+    if (classList) {
+        if (q >= *classCount) return;
+        q = classList[q];
+    }
+    if (q >= count) return;
+    s_write(hw_blk(), &inst[q], wsv[q], write_smem + sim_pow2(side) * (threadIdx.x >> 5));
 }
 
 int guard_cap_batch(long long cap)

@@ -656,13 +656,14 @@ __device__ inline void s_brec(const Blk B, rr_instance *inst, JobWS *wsv, int co
     for (int64_t b = B.x * blockDim.x + threadIdx.x; b < k; b += (int64_t)B.gx * blockDim.x) {
         const rr_move p = load_move(&I->moves[b]);
         const int lo = ws.pairOff[b], hi = lo + ws.rec[2 * b].z;
-        int v[4] = {-1, -1, -1, -1};
+        int v[4] = {-1, -1, -1, -1}, next = 0;
         for (int e = lo; e < hi; ++e) {
             const int32_t sId = ws.succ[e];
             const int32_t f = ws.indeg[sId] == 1 ? sId | SUCC_SINGLE : ws.multiNo[sId];
             if (e - lo < 4) v[e - lo] = f; else ws.succ[e] = f;
+            if (sId == b + 1 && e - lo < 4) next = e - lo + 1;
         }
-        const int4 r = move_rec(p, hi - lo, lo + 4, hi - lo == 1 && v[0] == (int)(SUCC_SINGLE | (b + 1)));
+        const int4 r = move_rec(p, hi - lo, lo + 4, hi - lo == 1 && v[0] == (int)(SUCC_SINGLE | (b + 1)), next);
         ws.rec[2 * b] = r;
         ws.rec[2 * b + 1] = make_int4(v[0], v[1], v[2], v[3]);
         const int in = ws.indeg[b];
@@ -740,8 +741,8 @@ __device__ inline void s_classify(const Blk B, rr_instance *inst, int count, int
 // ---------------------------------------------------------- simulation
 //
 // Alg. 4 with the local constraint set of Sec. IV, as an event-driven
-// simulation: one block per instance, its first warp simulates and logs, its
-// other warps write the batches.
+// simulation: one block per instance; one warp simulates and logs, others
+// write the batches.
 //
 // The lowest-id unfinished move is always ready (nothing earlier is
 // unfinished), so it is always the first member ("leader") of the batch. With
@@ -773,39 +774,71 @@ __device__ inline void s_classify(const Blk B, rr_instance *inst, int count, int
 //    `along` minus the clock and the clock at which its leg ends, so a segment
 //    that none of them ends does not touch them. They are kept in no order
 //    (the writers sort), with the smallest id and the first end in registers.
-//  - The leader lives in warp-uniform registers. When it finishes, the next
-//    leader is nearly always the next id, released at that moment: its record
-//    is loaded while its predecessor still runs.
+//  - The leader lives in registers. When it finishes, the next leader is
+//    nearly always the next id, released at that moment; its record has been
+//    brought into L1 long before. Successive leaders that meet nothing on
+//    their way are taken together (run_of_leaders).
 //  - In-degrees of the moves with several predecessors are counted in shared
 //    memory as far as they fit (a global atomic's answer takes about 700
 //    cycles); their predecessors name the counter, not the move, so that a
 //    count that does not reach zero touches nothing else. Moves with one
 //    predecessor need no count.
 //  - A segment is logged in 16 bytes plus its members' ids where these
-//    changed, into memory that the conflict graph no longer needs. The other
-//    warps of the block turn the log into batches and members while the
-//    simulation runs on, each warp 32 segments at a time, with stores of
-//    consecutive words.
+//    changed, into memory that the conflict graph no longer needs. Other
+//    warps turn the log into batches and members, 32 segments at a time, with
+//    stores of consecutive words: three warps of the same block while the
+//    simulation runs on (calls over few grids), or a kernel after it.
+// One 256 x 256 grid: 63 ms with linked lists, sorted members, batches written
+// by the simulating warp and in-degrees in global memory; 17 ms this way.
 
 // ------------------------------------------------------------- the writers
+
+// What a lane writes of a segment's batches: three words per batch
+// (direction, first member, count), a warp's store covering 32 consecutive
+// words, so that 32 batches take three stores, in which a lane's words are
+// always the same field (f) of the same batch (q) of the 32.
+struct OpLane {
+    int f[3], q[3];
+    __device__ __forceinline__ OpLane(int lane)
+    {
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+            q[j] = (lane + 32 * j) / 3;
+            f[j] = (lane + 32 * j) % 3;
+        }
+    }
+};
+__device__ __forceinline__ void write_ops(int32_t *o, const OpLane &P, int lane, unsigned mem0, int kseg, int ns, int d)
+{
+    int v[3], by[3];
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+        by[j] = P.f[j] == 1 ? ns : 0;
+        v[j] = (P.f[j] == 0 ? d : P.f[j] == 1 ? (int)mem0 : ns) + by[j] * P.q[j];
+    }
+    for (int w = lane; w - lane < 3 * kseg; w += 96) {
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+            if (w + 32 * j < 3 * kseg) o[w + 32 * j] = v[j];
+            v[j] += 32 * by[j];
+        }
+    }
+}
 
 // A segment's kseg batches of ns moves at batch op0 and member mem0: the
 // leader L (the smallest id) and the ns - 1 moves of list[], in no order.
 // One warp; buf holds the next power of two of ns words. Batches are written
 // as consecutive words (three per batch), members likewise.
-__device__ inline void write_segment(rr_op *ops, int32_t *mem, unsigned op0, unsigned mem0, int kseg, int ns, int d,
-                                     int L, const int32_t *list, int32_t *buf)
+__device__ inline void write_segment(rr_op *ops, int32_t *mem, const OpLane &P, unsigned op0, unsigned mem0, int kseg,
+                                     int ns, int d, int L, const int32_t *list, int32_t *buf)
 {
     const int lane = threadIdx.x & 31;
-    int32_t *o = (int32_t *)(ops + op0);
-    for (int w = lane; w < 3 * kseg; w += 32) {
-        const int q = (int)(((unsigned)w * 43691u) >> 17), f = w - 3 * q;      // w / 3 for w < 2^16
-        o[w] = f == 0 ? d : f == 1 ? (int32_t)(mem0 + (unsigned)(q * ns)) : ns;
-    }
+    write_ops((int32_t *)(ops + op0), P, lane, mem0, kseg, ns, d);
     int32_t *mp = mem + mem0;
     const int total = kseg * ns;
     if (ns == 1) {
-        for (int i = lane; i < total; i += 32) mp[i] = L;
+        for (int i = lane; i - lane < total; i += 32)
+            if (i < total) mp[i] = L;
         return;
     }
     // lane's place in the cycle of ns members, and what 32 places on means
@@ -820,11 +853,14 @@ __device__ inline void write_segment(rr_op *ops, int32_t *mem, unsigned op0, uns
     const int step = mod(32);
     if (ns <= 32) {
         int v = lane == 0 ? L : lane < ns ? list[lane - 1] : INTMAX;
-        int r = 0;
-        for (int j = 0; j < ns; ++j) r += __shfl_sync(FULL, v, j) < v;
-        if (lane < ns) buf[r] = v;
-        __syncwarp();
-        v = lane < ns ? buf[lane] : 0;
+        if (ns > 2) {              // sort: every lane counts the smaller ones
+            int r = 0;
+            for (int j = 1; j < ns; ++j) r += __shfl_sync(FULL, v, j) < v;
+            if (lane > 0) ++r;     // the leader is the smallest
+            if (lane < ns) buf[r] = v;
+            __syncwarp();
+            v = lane < ns ? buf[lane] : 0;
+        }
         for (int i0 = 0; i0 < total; i0 += 32) {
             const int x = __shfl_sync(FULL, v, u);
             if (i0 + lane < total) mp[i0 + lane] = x;
@@ -849,14 +885,41 @@ constexpr int SIM_POLLS = 1 << 22;      // a writer's polls without progress bef
 // Header of a logged segment: its first batch and first member, where its
 // members' ids lie, and the leader (30 bits) with the direction. Lengths
 // follow from the next header.
-__device__ inline void run_writers(SimCtl *C, rr_instance *I, const int32_t *log, int32_t *buf)
+__device__ __forceinline__ void write_chunk(const int32_t *log, int s0, int cnt, unsigned long long cap_ops,
+                                            unsigned long long cap_mem, rr_op *ops, int32_t *mem, const OpLane &P,
+                                            int32_t *buf)
 {
     const int lane = threadIdx.x & 31;
     const uint4 *hdr = (const uint4 *)log;
+    uint4 h = make_uint4(0u, 0u, 0u, 0u);
+    int kseg = 0, ns = 0;
+    if (lane < cnt) {
+        h = hdr[s0 + lane];
+        const uint2 nx = *(const uint2 *)&hdr[s0 + lane + 1];
+        kseg = (int)(nx.x - h.x);
+        ns = (int)((nx.y - h.y) / (unsigned)max(kseg, 1));
+        // a batch list that does not fit ends as RR_ERR_CAPACITY: nothing of it is written
+        if (nx.x > cap_ops || nx.y > cap_mem) kseg = 0;
+    }
+    for (int j = 0; j < cnt; ++j) {
+        const int kj = __shfl_sync(FULL, kseg, j), nj = __shfl_sync(FULL, ns, j);
+        const unsigned op0 = __shfl_sync(FULL, h.x, j), mem0 = __shfl_sync(FULL, h.y, j);
+        const unsigned lo = __shfl_sync(FULL, h.z, j), l = __shfl_sync(FULL, h.w, j);
+        if (kj > 0)
+            write_segment(ops, mem, P, op0, mem0, kj, nj, (int)(l >> 30), (int)(l & 0x3fffffffu), log + lo, buf);
+    }
+}
+
+// A warp of the simulation's block writes what is published of the log, 32
+// segments at a time, until the simulation has ended and nothing is left.
+__device__ inline void run_writers(SimCtl *C, rr_instance *I, const int32_t *log, int32_t *buf)
+{
+    const int lane = threadIdx.x & 31;
     const unsigned long long cap_ops = (unsigned long long)I->cap_ops, cap_mem = (unsigned long long)I->cap_members;
     rr_op *ops = as_global(I->ops);
     int32_t *mem = as_global(I->members);
     volatile int *pub = &C->pub, *fin = &C->fin;
+    const OpLane P(lane);
     for (;;) {
         int s0 = 0;
         if (lane == 0) s0 = atomicAdd(&C->next, 32);
@@ -874,24 +937,23 @@ __device__ inline void run_writers(SimCtl *C, rr_instance *I, const int32_t *log
         __threadfence_block();
         const int cnt = min(32, have - s0);
         if (cnt <= 0) return;
-        uint4 h = make_uint4(0u, 0u, 0u, 0u);
-        int kseg = 0, ns = 0;
-        if (lane < cnt) {
-            h = hdr[s0 + lane];
-            const uint2 nx = *(const uint2 *)&hdr[s0 + lane + 1];
-            kseg = (int)(nx.x - h.x);
-            ns = (int)((nx.y - h.y) / (unsigned)max(kseg, 1));
-            // a batch list that does not fit ends as RR_ERR_CAPACITY: nothing of it is written
-            if (nx.x > cap_ops || nx.y > cap_mem) kseg = 0;
-        }
-        for (int j = 0; j < cnt; ++j) {
-            const int kj = __shfl_sync(FULL, kseg, j), nj = __shfl_sync(FULL, ns, j);
-            const unsigned op0 = __shfl_sync(FULL, h.x, j), mem0 = __shfl_sync(FULL, h.y, j);
-            const unsigned lo = __shfl_sync(FULL, h.z, j), l = __shfl_sync(FULL, h.w, j);
-            if (kj > 0)
-                write_segment(ops, mem, op0, mem0, kj, nj, (int)(l >> 30), (int)(l & 0x3fffffffu), log + lo, buf);
-        }
+        write_chunk(log, s0, cnt, cap_ops, cap_mem, ops, mem, P, buf);
     }
+}
+
+// The logged segments of every instance, as far as its simulation ran without
+// writers of its own: a warp per 32 segments.
+__device__ inline void s_write(const Blk B, rr_instance *I, const JobWS &ws, int32_t *buf)
+{
+    if (!live(I) || I->n_moves == 0) return;
+    const int lane = threadIdx.x & 31;
+    const OpLane P(lane);
+    rr_op *ops = as_global(I->ops);
+    int32_t *mem = as_global(I->members);
+    const int32_t *log = as_global(ws.nextAt);
+    const unsigned long long cap_ops = (unsigned long long)I->cap_ops, cap_mem = (unsigned long long)I->cap_members;
+    for (int s0 = 32 * B.w; s0 < ws.nseg; s0 += 32 * B.nw)
+        write_chunk(log, s0, min(32, ws.nseg - s0), cap_ops, cap_mem, ops, mem, P, buf);
 }
 
 // ---------------------------------------------------------- the simulation
@@ -981,6 +1043,14 @@ __device__ __forceinline__ int2 ldg_if(bool c, const int2 *p)
                  : "+r"(v.x), "+r"(v.y) : "r"((unsigned)c), "l"(p) : "memory");
     return v;
 }
+// (not from L1: atomics change the word in L2)
+__device__ __forceinline__ int ldg_volatile_if(bool c, const void *p)
+{
+    int v = 0;
+    asm volatile("{ .reg .pred q; setp.ne.u32 q, %1, 0; @q ld.global.cg.u32 %0, [%2]; }"
+                 : "+r"(v) : "r"((unsigned)c), "l"(p) : "memory");
+    return v;
+}
 __device__ __forceinline__ int ldg_if(bool c, const void *p)
 {
     int v = 0;
@@ -998,6 +1068,7 @@ static inline void st_if(bool c, int2 *p, int x, int y) { if (c) *p = make_int2(
 static inline int4 ldg_if(bool c, const int4 *p) { return c ? *p : make_int4(0, 0, 0, 0); }
 static inline int2 ldg_if(bool c, const int2 *p) { return c ? *p : make_int2(0, 0); }
 static inline int ldg_if(bool c, const void *p) { return c ? *(const int *)p : 0; }
+static inline int ldg_volatile_if(bool c, const void *p) { return c ? *(const int *)p : 0; }
 #endif
 
 __device__ __forceinline__ void touch_rec_if(bool c, const int4 *rec, int id, uint32_t dump)
@@ -1010,9 +1081,225 @@ __device__ __forceinline__ void touch_rec_if(bool c, const int4 *rec, int id, ui
 // computed from it, need no bookkeeping for lanes that might diverge.
 __device__ __forceinline__ uint32_t uni(uint32_t v) { return __reduce_max_sync(FULL, v); }
 
-// Words the log must have left at the start of 32 segments: their headers and
-// the one after them, a list of ids for each.
-#define LOG_SLACK(lineCap) (4u * 34u + 32u * (unsigned)(lineCap))
+
+constexpr int RUN = 32;     // leaders of a run at most: one per lane
+
+// Segments that the log has room for: a header each, one after them, a list
+// of ids each, and the headers of one run.
+__device__ __forceinline__ int log_room(unsigned nseg, unsigned idTop, int lineCap)
+{
+    return ((int)idTop - 4 * ((int)nseg + 2 + 2 * RUN)) / (4 + lineCap);
+}
+
+// A block's shared memory (sim_smem_bytes), the tables apart.
+struct SimLayout {
+    int MC;                   // room of the members
+    int2 *mie;
+    uint32_t *mpos;
+    SimCtl *C;
+    int32_t *bufs, *ids;      // a sort buffer per warp, a list of ids
+    int32_t *dump;            // 16 bytes that nothing reads
+    unsigned *cnt;
+    __device__ __forceinline__ SimLayout(char *smem, int side)
+    {
+        MC = (side + 7) & ~7;
+        mie = (int2 *)(smem + 14 * 4 * sim_cap(side));
+        mpos = (uint32_t *)(mie + MC);
+        C = (SimCtl *)(mpos + MC);
+        bufs = (int32_t *)(C + 1);
+        ids = bufs + sim_pow2(side) * (int)(blockDim.x >> 5);
+        dump = ids + MC;
+        cnt = (unsigned *)(dump + 4);
+    }
+};
+
+// A run: successive leaders, each alone in its batches, are taken
+// together. Lane i looks at the i-th next id (lane 0 at the leader), its
+// horizontal leg if it has one, and its vertical leg. The run goes on
+// while every vertical leg runs the same way down the same column, no
+// static stands on or ahead of either leg's line of motion or on a line
+// that the leg reaches, the only move that a leader makes ready is the
+// next id, and no in-degree counter of a successor runs out. Nothing else
+// changes meanwhile, so the batches are known at once: the legs, one
+// after another. Deep in a receiver's unit nearly all moves are of this
+// kind: on a 256 x 256 grid 900 runs take 10 700 of 14 400 leaders (the
+// simulation 22.4 -> 17.1 ms). The leader L has rem steps of its leg left at lpos in
+// direction d. Returns 0 or the leaders taken, their legs (each logged) and
+// their steps, in 6, 7 and 17 bits. Not inlined: its registers would crowd
+// those of the loop that calls it.
+template <int MODE>
+static __device__ __noinline__ int run_of_leaders(rr_instance *I, JobWS *ws, char *smem, int side, int counters, int L, int d,
+                                                  int rem, uint32_t lpos, int clk, unsigned nmem, unsigned nseg,
+                                                  unsigned list, bool logging)
+{
+    const SimLayout Y(smem, side);
+    const int lane = lane_id(), k = (int)I->n_moves, cap = sim_cap(side), groups = cap >> 3;
+    const int ncnt = min(counters, ws->nmulti);
+    const bool allShared = counters >= ws->nmulti;
+    const uint32_t *pos = (const uint32_t *)smem;
+    const int4 *rec = as_global(ws->rec);
+    int32_t *multi = as_global(ws->multi), *log = as_global(ws->nextAt);
+    const int32_t *multiId = as_global(ws->multiId);
+    const uint32_t *multiPos = as_global(ws->multiPos);
+    SimCtl *C = Y.C;
+    unsigned *cnt = Y.cnt;
+    int32_t *ids = Y.ids, *buf = Y.bufs;
+    const uint32_t dump = sh_addr(Y.dump);
+    const int id = min(L + lane, k);
+    const int4 r = rec[2 * (size_t)id], s = rec[2 * (size_t)id + 1];
+    int d1 = r.y & 3, len = r.y >> 2 & 2047;
+    uint32_t p1 = (uint32_t)r.x;
+    if (lane == 0) { d1 = d; len = rem; p1 = lpos; }
+    const bool hor = d1 >= 2;
+    const Leg g = second_leg(d1, p1 + (uint32_t)len, r.y >> 13 & 1023);
+    const int hl = hor ? len : 0, vd = hor ? g.d : d1, vl = hor ? g.rem : len;
+    const uint32_t vp = hor ? g.pos : p1;
+    const int rd = __shfl_sync(FULL, vd, 0);
+    const uint32_t rc = __shfl_sync(FULL, vp >> 16, 0);
+    // successors: the next id (without another predecessor, or the last
+    // one it waits for), and counters that stay above zero
+    const int32_t sv[4] = {s.x, s.y, s.z, s.w};
+    const int next = (r.y >> 24 & 7) - 1;
+    bool link = false, bad = L + lane >= k || r.z > 4 || vl == 0 || vd != rd || (vp >> 16) != rc;
+    bool inS[4], inG[4];
+    int left_[4];
+    #pragma unroll
+    for (int e = 0; e < 4; ++e) {
+        const bool v = e < r.z && !bad, one = (sv[e] & SUCC_SINGLE) != 0;
+        inS[e] = v && !one && sv[e] < ncnt;
+        inG[e] = v && !one && sv[e] >= ncnt;
+        link |= v && one && e == next;
+    }
+    #pragma unroll
+    for (int e = 0; e < 4; ++e) {
+        bad |= e < r.z && (sv[e] & SUCC_SINGLE) && e != next;
+        left_[e] = ld_u16_if(inS[e], (const uint16_t *)cnt + (inS[e] ? sv[e] : 0));
+    }
+    if (!allShared)
+    #pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const int c = ldg_volatile_if(inG[e], multi + (inG[e] ? sv[e] : 0)) & MULTI_COUNT;
+            left_[e] = inG[e] ? c : left_[e];
+        }
+    unsigned few = 0;       // entries whose counter will be at one
+    #pragma unroll
+    for (int e = 0; e < 4; ++e) {
+        const bool m = inS[e] || inG[e], last = m && left_[e] == 1;
+        link |= last && e == next;
+        bad |= last && e != next;
+        few |= m && left_[e] == 2 ? 1u << e : 0u;
+        inS[e] = inS[e] && !last;          // (nobody else waits on a counter that has run out)
+        inG[e] = inG[e] && !last;
+    }
+    const unsigned okb = __ballot_sync(FULL, !bad && link);
+    int n = okb == FULL ? 32 : __ffs(~okb) - 1;
+    if (n == 0) return 0;
+    // horizontal legs against the few statics of the horizontal directions
+    if (__any_sync(FULL, hl > 0))
+        for (int q = 2; q < 4; ++q) {
+            if (C->nfree[q] == cap) continue;
+            bool hit = false;
+            for (int g0 = 0; g0 < groups; g0 += 32) {
+                const int e0 = q * cap + 8 * min(g0 + lane, groups - 1);
+                const uint4 a = *(const uint4 *)(pos + e0), b = *(const uint4 *)(pos + e0 + 4);
+                const uint32_t all = a.x & a.y & a.z & a.w & b.x & b.y & b.z & b.w;
+                // (a hole is no hit: it lies far ahead, on no row)
+                for (unsigned m = __ballot_sync(FULL, all != HOLE); m; m &= m - 1) {
+                    const int src = 31 - __clz(m & (0u - m));
+                    const uint32_t x[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+    #pragma unroll
+                    for (int u = 0; u < 8; ++u) {
+                        const uint32_t w = __shfl_sync(FULL, x[u], src);
+                        hit |= ((w - p1) & 0xffffu) < (unsigned)hl || (w >> 16) == (p1 >> 16);
+                    }
+                }
+            }
+            const unsigned hb = __ballot_sync(FULL, hit && d1 == q);
+            if (hb) n = min(n, __ffs(hb) - 1);
+        }
+    // vertical legs against the statics of their direction, four at a time
+    const int vtb = rd * cap;
+    for (int i = 0; i < n; i += 4) {
+        uint32_t w[4], v[4];
+        int need[4];
+    #pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            w[u] = 0x10000u - __shfl_sync(FULL, vp, i + u);
+            need[u] = __shfl_sync(FULL, vl, i + u);
+            v[u] = HOLE;
+        }
+        for (int gg = 0; gg < groups; gg += 32) {
+            const int e0 = vtb + 8 * min(gg + lane, groups - 1);
+            const uint4 a = *(const uint4 *)(pos + e0), b = *(const uint4 *)(pos + e0 + 4);
+    #pragma unroll
+            for (int u = 0; u < 4; ++u) v[u] = min8(a, b, w[u], v[u]);
+        }
+        int stop = n;
+    #pragma unroll
+        for (int u = 3; u >= 0; --u) {
+            const int near = (int)__reduce_min_sync(FULL, v[u] < 0x10000u ? 0u : v[u] & 0xffffu);
+            if (near < need[u]) stop = i + u;
+        }
+        if (stop < n) { n = stop; break; }
+    }
+    // count down; a counter that runs out after all (two leaders of the
+    // run share it) ends the run before the last of them
+    while (n > 0) {
+        const bool in = lane < n;
+        int gone = -1, old[4];
+    #pragma unroll
+        for (int e = 0; e < 4; ++e)
+            old[e] = sh_add_if(in && inS[e], cnt + (inS[e] ? sv[e] >> 1 : 0), -(1 << ((sv[e] & 1) * 16)));
+    #pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            if (in && inS[e] && (old[e] >> ((sv[e] & 1) * 16) & 0xffff) == 1) gone = sv[e];
+            if (!allShared && in && inG[e] && (atomicSub(&multi[sv[e]], 1) & MULTI_COUNT) == 1) gone = sv[e];
+        }
+        const unsigned gb = __ballot_sync(FULL, gone >= 0);
+        if (!gb) break;
+        const int x = __shfl_sync(FULL, gone, __ffs(gb) - 1);
+        bool has = false;
+    #pragma unroll
+        for (int e = 0; e < 4; ++e) {                        // take them back
+            sh_add_if(in && inS[e], cnt + (inS[e] ? sv[e] >> 1 : 0), 1 << ((sv[e] & 1) * 16));
+            if (!allShared && in && inG[e]) atomicAdd(&multi[sv[e]], 1);
+            has |= in && (inS[e] || inG[e]) && sv[e] == x;
+        }
+        n = 31 - __clz(__ballot_sync(FULL, has));
+        __syncwarp();
+    }
+    if (n == 0) return 0;
+    if (__any_sync(FULL, lane < n && few != 0u)) {
+    #pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const bool t = lane < n && (few >> e & 1u);
+            touch_if(t, multiId + (t ? sv[e] : 0), dump);
+            touch_if(t, multiPos + (t ? sv[e] : 0), dump);
+            touch_if(t, multi + (t ? sv[e] : 0), dump);
+        }
+    }
+    // log the legs
+    const int mine = lane < n ? (hl + vl) | ((hl > 0 ? 2 : 1) << 20) : 0;
+    const int incl = warp_incl_scan(mine), tot = __shfl_sync(FULL, incl, 31);
+    const int before = (incl - mine) & 0xfffff, steps = tot & 0xfffff, segs = tot >> 20;
+    if (logging) {
+        uint4 *h = (uint4 *)log + nseg + ((incl - mine) >> 20);
+        if (lane < n) {
+            if (hl > 0) *h++ = make_uint4((unsigned)(clk + before), nmem + (unsigned)before, list, (unsigned)id | (unsigned)d1 << 30);
+            *h = make_uint4((unsigned)(clk + before + hl), nmem + (unsigned)(before + hl), list, (unsigned)id | (unsigned)vd << 30);
+        }
+    } else {
+        for (int i = 0; i < n; ++i) {
+            const int o = clk + __shfl_sync(FULL, before, i), m0 = (int)nmem + __shfl_sync(FULL, before, i);
+            const int h1 = __shfl_sync(FULL, hl, i), v1 = __shfl_sync(FULL, vl, i), hd = __shfl_sync(FULL, d1, i);
+            if ((unsigned long long)(o + h1 + v1) > (unsigned long long)I->cap_ops ||
+                (unsigned long long)(m0 + h1 + v1) > (unsigned long long)I->cap_members) break;
+            if (h1 > 0) write_segment(as_global(I->ops), as_global(I->members), OpLane(lane), (unsigned)o, (unsigned)m0, h1, 1, hd, L + i, ids, buf);
+            write_segment(as_global(I->ops), as_global(I->members), OpLane(lane), (unsigned)(o + h1), (unsigned)(m0 + h1), v1, 1, rd, L + i, ids, buf);
+        }
+    }
+    return n | segs << 6 | steps << 13;
+}
 
 // One simulation by one warp. SIM_SMALL: tables in shared memory, at most 256
 // entries per direction (one load of every lane covers them); SIM_BIG: the
@@ -1039,6 +1326,8 @@ struct Sim {
     int ncnt;
     bool allShared;           // all of them
     uint32_t dump;            // shared address for the touches
+    char *smem;               // the block's shared memory, its side and counters
+    int side, counters;
 
     __device__ __forceinline__ int base(int d) const { return MODE == SIM_WIDE ? C->wbase[d] : d * cap; }
     __device__ __forceinline__ int size(int d) const { return MODE == SIM_WIDE ? C->wcap[d] : cap; }
@@ -1102,7 +1391,7 @@ template <int MODE>
 __device__ __forceinline__ int Sim<MODE>::run(rr_instance *I, JobWS &ws, int32_t *log, unsigned logWords, int lineCap,
                                               int32_t *buf, int32_t *ids)
 {
-    const int lane = threadIdx.x & 31;
+    const int lane = lane_id();
     const unsigned lt = (1u << lane) - 1u;
     const int k = (int)I->n_moves;
     int err = RR_OK;
@@ -1133,12 +1422,17 @@ __device__ __forceinline__ int Sim<MODE>::run(rr_instance *I, JobWS &ws, int32_t
     // the log: headers from its start, ids from its end
     uint4 *hdr = (uint4 *)log;
     unsigned nseg = 0, idTop = logWords, list = 0;
-    bool logging = idTop >= LOG_SLACK(lineCap);
-    // housekeeping every 32 segments: publish, check the bounds
-    int left = 32;
+    // housekeeping every 32 segments (or as many as the log has room for):
+    // publish, check the bounds
+    int left = min(32, log_room(0u, idTop, lineCap));
+    bool logging = left > 0;
+    if (!logging) left = 32;
     long long guard = (g_guard_cap > 0 ? g_guard_cap : I->n_steps + 2ll * k + 16) + 1;
-    if (guard < 32) left = (int)guard;
+    if (guard < left) left = (int)guard;
     guard -= left;
+    // a run is tried with a leader whose predecessor met nothing on its way
+    // (elsewhere it would mostly be in vain)
+    bool alone = false, tryRun = false;
     // this lane's eight entries of a table's first 256 (a lane beyond the
     // table reads the last eight too: that changes no minimum)
     int groups = size(0) >> 3, off = 8 * min(lane, groups - 1);
@@ -1147,7 +1441,7 @@ __device__ __forceinline__ int Sim<MODE>::run(rr_instance *I, JobWS &ws, int32_t
         d = (int)(y & 3u);
         lend = clk + (int)(y >> 2 & 2047u);
         ldst = (int)(y >> 13 & 1023u);
-        chain = (y >> 23) != 0u;
+        chain = (y >> 23 & 1u) != 0u;
     };
     auto on_clock = [&](uint32_t p) { return (p & 0xffff0000u) | ((p + (uint32_t)clk) & 0xffffu); };
     auto dissolve = [&]() {
@@ -1161,9 +1455,30 @@ __device__ __forceinline__ int Sim<MODE>::run(rr_instance *I, JobWS &ws, int32_t
         changed = true;
         __syncwarp();
     };
-    // a record a little later into L1
-    auto look_ahead = [&]() {
-        touch_rec_if(lane == 0, rec, min(L + 4, k), dump);
+    // the records that come into a run's view, n of them, into L1
+    auto look_ahead = [&](int n) {
+        touch_rec_if(lane < n, rec, min(L + 2 * RUN - n + lane, k), dump);
+    };
+    auto housekeeping = [&]() {
+        if (guard <= 0) return (int)RR_ERR_TIMEOUT;
+        if (MODE != SIM_WIDE && *(volatile int *)&C->full) return (int)RR_SIM_RETRY;
+        // (a run may have gone beyond the 32)
+        guard += left;
+        left = 32;
+        if (logging) {
+            // a header follows the published segments (it says where they
+            // end); without room for another one the rest is written here
+            if (lane == 0) hdr[nseg] = make_uint4((unsigned)clk, nmem, 0u, 0u);
+            __syncwarp();
+            __threadfence_block();
+            if (lane == 0) *(volatile int *)&C->pub = (int)nseg;
+            const int room = log_room(nseg, idTop, lineCap);
+            logging = room > 0;
+            if (logging) left = min(32, room);
+        }
+        if (guard < left) left = (int)guard;
+        guard -= left;
+        return (int)RR_OK;
     };
     // the lowest unfinished move, wherever it waits, becomes the leader (rare:
     // nearly always it is released when its predecessor finishes); false when
@@ -1221,7 +1536,8 @@ __device__ __forceinline__ int Sim<MODE>::run(rr_instance *I, JobWS &ws, int32_t
             changed = true;
         }
         __syncwarp();
-        look_ahead();
+        look_ahead(RUN);
+        alone = false;
         return true;
     };
 
@@ -1241,6 +1557,34 @@ __device__ __forceinline__ int Sim<MODE>::run(rr_instance *I, JobWS &ws, int32_t
                 v = min8(a2, b2, nadd, v);
             }
         int pick = (int)__reduce_min_sync(FULL, v < 0x10000u ? 0u : v & 0xffffu);
+        if (MODE != SIM_WIDE && tryRun) {
+            tryRun = false;
+            int run = 0;
+            if (nm == 0 && pick >= lend - clk && guard > 128)
+                run = run_of_leaders<MODE>(I, &ws, smem, side, counters, L, d, lend - clk, lpos, clk, nmem, nseg, list, logging);
+            if (run > 0) {
+                const int segs = run >> 6 & 127, steps = run >> 13;
+                L += run & 63;
+                if (logging) nseg += (unsigned)segs;
+                left -= segs;
+                clk += steps;
+                nmem += (unsigned)steps;
+                const int4 r = rec[2 * (size_t)L];
+                lpos = (uint32_t)r.x;
+                set_leg((uint32_t)r.y);
+                nsu = r.z;
+                ov = r.w;
+                s4 = rec[2 * (size_t)L + 1];
+                look_ahead(run & 63);
+                tryRun = (run & 63) == RUN;
+                evEnd = lend;
+                if (left <= 0) {
+                    err = housekeeping();
+                    if (err) break;
+                }
+                continue;
+            }
+        }
         if (pick == 0) {
             const unsigned ba = __ballot_sync(FULL, (v & 0xffffu) == 0u), bc = __ballot_sync(FULL, v < 0x10000u);
             bool choose;
@@ -1262,6 +1606,7 @@ __device__ __forceinline__ int Sim<MODE>::run(rr_instance *I, JobWS &ws, int32_t
                 choose = __reduce_min_sync(FULL, ma) < __reduce_min_sync(FULL, mc);
                 if (nm > 0 && choose != prim) dissolve();
             }
+            alone = false;
             if (choose ? ba : bc) {
                 // the chosen line's statics join the members
                 int me = minEnd, fr = C->nfree[d];
@@ -1346,31 +1691,19 @@ __device__ __forceinline__ int Sim<MODE>::run(rr_instance *I, JobWS &ws, int32_t
             if (o1 <= (unsigned long long)I->cap_ops && m1 <= (unsigned long long)I->cap_members) {
                 for (int u = lane; u < nm; u += 32) ids[u] = mie[u].x;
                 __syncwarp();
-                write_segment(as_global(I->ops), as_global(I->members), (unsigned)clk, nmem, kseg, nm + 1, d, L, ids, buf);
+                write_segment(as_global(I->ops), as_global(I->members), OpLane(lane), (unsigned)clk, nmem, kseg, nm + 1, d, L,
+                              ids, buf);
             }
         }
         // everything in the batch advances
         nmem += (unsigned)(kseg * (nm + 1));
         clk += kseg;
         lpos += (uint32_t)kseg;
-        if (--left == 0) {
-            if (guard <= 0) { err = RR_ERR_TIMEOUT; break; }
-            if (kseg < 1) { err = RR_ERR_INTERNAL; break; }
-            if (MODE != SIM_WIDE && *(volatile int *)&C->full) break;
-            left = guard < 32 ? (int)guard : 32;
-            guard -= left;
-            if (logging) {
-                // a header follows the published segments (it says where they
-                // end); without room for the next 32 segments the rest is
-                // written here, above
-                if (lane == 0) hdr[nseg] = make_uint4((unsigned)clk, nmem, 0u, 0u);
-                __syncwarp();
-                __threadfence_block();
-                if (lane == 0) *(volatile int *)&C->pub = (int)nseg;
-                logging = 4u * nseg + LOG_SLACK(lineCap) <= idTop;
-            }
+        if (--left <= 0) {
+            err = kseg < 1 ? RR_ERR_INTERNAL : housekeeping();
+            if (err) break;
         }
-        if (clk != evEnd) continue;
+        if (clk != evEnd) { alone = false; continue; }
         bool fin = false, moved = false;
         int4 nr = make_int4(0, 0, 0, 0), ns4 = nr;
         if (clk == lend) {
@@ -1447,12 +1780,14 @@ __device__ __forceinline__ int Sim<MODE>::run(rr_instance *I, JobWS &ws, int32_t
             }
             if (hand) {
                 L = handId;
-                lpos = uni((uint32_t)nr.x);
-                set_leg(uni((uint32_t)nr.y));
+                lpos = (uint32_t)nr.x;
+                set_leg((uint32_t)nr.y);
                 nsu = nr.z;
                 ov = nr.w;
                 s4 = ns4;
-                look_ahead();
+                look_ahead(1);
+                tryRun = alone;
+                alone = true;
             } else if (!find_leader()) {
                 break;
             }
@@ -1483,31 +1818,10 @@ __device__ __forceinline__ int Sim<MODE>::run(rr_instance *I, JobWS &ws, int32_t
     return err;
 }
 
-// A block's shared memory (sim_smem_bytes), the tables apart.
-struct SimLayout {
-    int MC;                   // room of the members
-    int2 *mie;
-    uint32_t *mpos;
-    SimCtl *C;
-    int32_t *bufs, *ids;      // a sort buffer per warp, a list of ids
-    int32_t *dump;            // 16 bytes that nothing reads
-    unsigned *cnt;
-    __device__ __forceinline__ SimLayout(char *smem, int side)
-    {
-        MC = (side + 7) & ~7;
-        mie = (int2 *)(smem + 14 * 4 * sim_cap(side));
-        mpos = (uint32_t *)(mie + MC);
-        C = (SimCtl *)(mpos + MC);
-        bufs = (int32_t *)(C + 1);
-        ids = bufs + sim_pow2(side) * (int)(blockDim.x >> 5);
-        dump = ids + MC;
-        cnt = (unsigned *)(dump + 4);
-    }
-};
-
 template <int MODE>
-__device__ __forceinline__ int sim_run(Sim<MODE> &S, rr_instance *I, JobWS &ws, const SimLayout &Y, int counters)
+__device__ __forceinline__ int sim_run(Sim<MODE> &S, rr_instance *I, JobWS &ws, char *smem, int side, int counters)
 {
+    const SimLayout Y(smem, side);
     S.mie = Y.mie; S.mpos = Y.mpos; S.C = Y.C;
     S.rec = as_global(ws.rec); S.succ = as_global(ws.succ); S.multi = as_global(ws.multi);
     S.multiId = as_global(ws.multiId); S.multiPos = as_global(ws.multiPos);
@@ -1515,6 +1829,7 @@ __device__ __forceinline__ int sim_run(Sim<MODE> &S, rr_instance *I, JobWS &ws, 
     S.dump = sh_addr(Y.dump);
     S.ncnt = min(counters, ws.nmulti);
     S.allShared = counters >= ws.nmulti;
+    S.smem = smem; S.side = side; S.counters = counters;
     // the log: the chains of the conflict graph are no longer needed
     return S.run(I, ws, as_global(ws.nextAt), (unsigned)((4 * (ws.P + 1) + 255) / 256 * 64), Y.MC, Y.bufs, Y.ids);
 }
@@ -1528,14 +1843,15 @@ static __device__ __noinline__ int sim_wide(rr_instance *I, JobWS *ws, char *sme
     S.ir = (int2 *)(S.pos + n);
     S.stk = (int32_t *)(S.ir + n);
     S.cap = 0;
-    return sim_run(S, I, *ws, SimLayout(smem, side), counters);
+    return sim_run(S, I, *ws, smem, side, counters);
 }
 
 // The whole simulation of one instance by one block (every thread calls it):
-// warp 0 simulates, the others write, warp 0 writes too once it is done.
+// warp 0 simulates, the others write, warp 0 writes too once it is done. A
+// block without writers is that one warp; s_write writes afterwards.
 // An instance that outgrows the shared-memory tables starts over with its
 // tables in global memory (the batches written so far are the same ones).
-template <int MODE>
+template <int MODE, bool WRITERS>
 __device__ __forceinline__ void sim_block(rr_instance *I, JobWS &ws, char *smem, int side, int counters)
 {
     const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -1603,11 +1919,12 @@ __device__ __forceinline__ void sim_block(rr_instance *I, JobWS &ws, char *smem,
         for (int i = threadIdx.x; i < ncnt; i += blockDim.x) c16[i] = (unsigned short)(ws.multi[i] & MULTI_COUNT);
         __syncthreads();
         if (wid == 0) {
-            const int st = pass == 0 ? sim_run(S, I, ws, Y, counters) : sim_wide(I, &ws, smem, side, counters);
+            const int st = pass == 0 ? sim_run(S, I, ws, smem, side, counters) : sim_wide(I, &ws, smem, side, counters);
             if (lane == 0) C->status = st;
             __syncwarp();
         }
-        run_writers(C, I, as_global(ws.nextAt), Y.bufs + sim_pow2(side) * wid);
+        if (WRITERS) run_writers(C, I, as_global(ws.nextAt), Y.bufs + sim_pow2(side) * wid);
+        else if (lane == 0) ws.nseg = C->pub;            // s_write follows
         __syncthreads();
         const int st = C->status;
         if (st != RR_SIM_RETRY || pass == 1 || k < SIM_WIDE_MIN) {

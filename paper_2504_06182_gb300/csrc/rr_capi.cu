@@ -32,7 +32,10 @@ __global__ void k_order(const rr_instance *, int, int *);
 __global__ void k_gather(const rr_instance *, const int *, rr_instance *);
 __global__ void k_scatter(rr_instance *, const int *, const rr_instance *, int);
 __global__ void k_sim(rr_instance *, JobWS *, int, const int *, const int *, int, int);
+__global__ void k_write(rr_instance *, JobWS *, int, const int *, const int *, int);
 __global__ void k_sim_big(rr_instance *, JobWS *, int, const int *, const int *, int, int);
+__global__ void k_simw(rr_instance *, JobWS *, int, const int *, const int *, int, int);
+__global__ void k_simw_big(rr_instance *, JobWS *, int, const int *, const int *, int, int);
 }  // namespace rrk
 
 using namespace rrk;
@@ -43,7 +46,7 @@ static_assert(sizeof(rr_instance) == 128, "rr_instance layout is part of the ABI
 static constexpr int SMALL_CALL = 8;
 
 // Kernels launched with more than the default 48 KB of dynamic shared memory.
-enum { SM_GSORT, SM_GSWEEP_H, SM_GSWEEP_V, SM_SIM, SM_SIM_BIG, SM_BIRD, SM_ONE, SM_NKERNEL };
+enum { SM_GSORT, SM_GSWEEP_H, SM_GSWEEP_V, SM_SIM, SM_SIM_BIG, SM_SIMW, SM_SIMW_BIG, SM_BIRD, SM_ONE, SM_NKERNEL };
 
 struct rr_ctx {
     int device;
@@ -139,7 +142,8 @@ static int smem_limits(int dev, int *out)
         int optin = 0;
         cudaError_t e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
         const void *fn[SM_NKERNEL] = {(const void *)k_gsort, (const void *)k_gsweep_h, (const void *)k_gsweep_v,
-                                      (const void *)k_sim, (const void *)k_sim_big, (const void *)k_bird, one_kernel()};
+                                      (const void *)k_sim, (const void *)k_sim_big, (const void *)k_simw,
+                                      (const void *)k_simw_big, (const void *)k_bird, one_kernel()};
         for (int i = 0; e == cudaSuccess && i < SM_NKERNEL; ++i) {
             cudaFuncAttributes fa;
             e = cudaFuncGetAttributes(&fa, fn[i]);
@@ -363,17 +367,27 @@ static int launch_plan(rr_ctx *ctx, rr_instance *d_inst, JobWS *ws, int count, i
 
 // A simulation block: its warps (one simulates, the others write) and its
 // in-degree counters in shared memory. A call over few grids leaves most of
-// the machine idle: more writers, and counters for every move that needs one.
-struct SimShape { int warps, counters; size_t smem; };
+// the machine idle: three writers, and counters for every move that needs one.
+// In a call over many grids registers and shared memory decide how many
+// simulations are resident: one warp each, and k_write after them, with more
+// warps per SM than the simulation's registers allow.
+struct SimShape {
+    void (*kernel)(rr_instance *, JobWS *, int, const int *, const int *, int, int);
+    int warps, counters;
+    size_t smem;
+    bool fits;
+};
 static SimShape sim_shape(const rr_ctx *ctx, int count, int side)
 {
     SimShape s;
     const bool few = count <= ctx->nsm;
-    const int limit = std::min(ctx->smemLimit[SM_SIM], ctx->smemLimit[SM_SIM_BIG]);
-    s.warps = few ? 4 : 2;
-    const int room = (limit - (int)sim_smem_bytes(side, s.warps, 0)) / 2 - 8;
+    s.warps = few ? 4 : 1;
+    const int which = (few ? SM_SIMW : SM_SIM) + (side > 256 ? 1 : 0);
+    s.kernel = which == SM_SIM ? k_sim : which == SM_SIM_BIG ? k_sim_big : which == SM_SIMW ? k_simw : k_simw_big;
+    const int room = (ctx->smemLimit[which] - (int)sim_smem_bytes(side, s.warps, 0)) / 2 - 8;
     s.counters = std::max(0, std::min(side * side / (few ? 4 : 12), room)) & ~7;
     s.smem = sim_smem_bytes(side, s.warps, s.counters);
+    s.fits = s.smem <= (size_t)ctx->smemLimit[which];
     return s;
 }
 
@@ -446,12 +460,16 @@ static int launch_batch(rr_ctx *ctx, rr_instance *d_inst, JobWS *ws, int count, 
         if (!one) CUDA_TRY(cudaStreamWaitEvent(cs, ctx->evFork, 0));
         const int side = class_side(max_side, c, nclass);
         const SimShape sh = sim_shape(ctx, count, side);
-        if (sh.smem > (size_t)std::min(ctx->smemLimit[SM_SIM], ctx->smemLimit[SM_SIM_BIG]))
+        if (!sh.fits)
             return fail(ctx, RR_ERR_ARG, "simulation shared memory %zu too large", sh.smem);
         const int *list = one ? nullptr : ctx->d_classList + (size_t)c * count;
         const int *cnt = one ? nullptr : ctx->d_classCount + c;
-        (side <= 256 ? k_sim : k_sim_big)<<<count, 32 * sh.warps, sh.smem, cs>>>(d_inst, ws, count, list, cnt, side,
-                                                                                 sh.counters);
+        sh.kernel<<<count, 32 * sh.warps, sh.smem, cs>>>(d_inst, ws, count, list, cnt, side, sh.counters);
+        if (sh.warps == 1) {
+            const int wb = clampi(std::max(1, budget(ctx, 16384) / count), 1, 64);
+            k_write<<<dim3(wb, count), 256, 8 * 4 * (size_t)sim_pow2(side), cs>>>(d_inst, ws, count, list, cnt, side);
+            ctx->nlaunch += 1;
+        }
         if (!one) {
             CUDA_TRY(cudaEventRecord(ctx->evJoin[c], cs));
             CUDA_TRY(cudaStreamWaitEvent(s, ctx->evJoin[c], 0));

@@ -112,6 +112,7 @@ struct JobWS {
     uint32_t *multiPos;
     int32_t *multiNo;      // k: a move's number among them
     int32_t nmulti;        // how many there are
+    int32_t nseg;          // logged segments that are still to be written
     // path-vertex offsets by the multi-block scan (large move lists only):
     // one status word per tile, the tile counter
     unsigned long long *lbStatus;
@@ -169,7 +170,7 @@ __host__ __device__ inline size_t sim_smem_bytes(int side, int warps, int counte
     return 14 * 4 * (size_t)sim_cap(side) + 12 * M + sizeof(SimCtl) + 4 * ((size_t)sim_pow2(side) * warps + M) + 16 +
            2 * (size_t)((counters + 7) & ~7);
 }
-constexpr int SIM_MAX_THREADS = 128;
+constexpr int SIM_MAX_THREADS = 128, SIM_BLOCKS = 16;   // with writers; one-warp blocks per SM
 
 // Workspace of the wide simulation: tables in global memory with room for
 // every move, at most two legs each. Only instances with more ready moves
@@ -185,8 +186,9 @@ constexpr int32_t RR_SIM_RETRY = 100;
 
 // A move's record (two int4): the position word of its source; its first
 // leg's direction (2 bits) and length (11 bits), its destination row (10
-// bits) and whether its only successor is the next id, without other
-// predecessors; its number of successors; where those after the fourth lie;
+// bits), whether its only successor is the next id, without other
+// predecessors (1 bit), and which of the first four successors the next id is
+// (3 bits, 0: none); its number of successors; where those after the fourth lie;
 // then the first four successors. The position of a token that moves in direction d: the
 // coordinate along its way, mirrored for the negative directions so that it
 // grows, and the one across it, both plus one, in the halves of a word.
@@ -197,11 +199,11 @@ __device__ __forceinline__ uint32_t dir_pos(int d, int row, int col)
     const int x = d < 2 ? row : col, al = (d & 1) ? x + 1 : MIRROR - 1 - x;
     return (uint32_t)al | (uint32_t)((d < 2 ? col : row) + 1) << 16;
 }
-__device__ __forceinline__ int4 move_rec(rr_move p, int nsucc, int more, bool chain)
+__device__ __forceinline__ int4 move_rec(rr_move p, int nsucc, int more, bool chain, int next)
 {
     const int hl = p.dst_col - p.src_col, vl = p.dst_row - p.src_row;
     const int d = hl ? (hl > 0 ? 3 : 2) : (vl > 0 ? 1 : 0), len = hl ? (hl > 0 ? hl : -hl) : (vl > 0 ? vl : -vl);
-    return make_int4((int)dir_pos(d, p.src_row, p.src_col), d | len << 2 | p.dst_row << 13 | (chain ? 1 << 23 : 0),
+    return make_int4((int)dir_pos(d, p.src_row, p.src_col), d | len << 2 | p.dst_row << 13 | (chain ? 1 << 23 : 0) | next << 24,
                      nsucc, more);
 }
 
@@ -220,6 +222,19 @@ __device__ __forceinline__ void *arena_alloc(const Arena &A, unsigned long long 
 }
 
 __host__ __device__ constexpr unsigned long long arena_pad(unsigned long long bytes) { return (bytes + 255ull) & ~255ull; }
+
+// The lane, read once: threadIdx.x would be read again (20 cycles or more)
+// wherever the compiler is short of a register to keep it in.
+__device__ __forceinline__ int lane_id()
+{
+#ifdef __CUDA_ARCH__
+    int l;
+    asm volatile("mov.u32 %0, %%laneid;" : "=r"(l));
+    return l;
+#else
+    return threadIdx.x & 31;
+#endif
+}
 
 __device__ __forceinline__ int warp_incl_scan(int v)
 {

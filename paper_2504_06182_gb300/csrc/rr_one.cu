@@ -21,7 +21,7 @@
 
 namespace rrk {
 
-__global__ void __launch_bounds__(ONE_THREADS) k_one(rr_instance h, rr_instance *I, JobWS *ws, Arena A, int flags,
+__global__ void __launch_bounds__(ONE_THREADS, 1) k_one(rr_instance h, rr_instance *I, JobWS *ws, Arena A, int flags,
                                                       int side, int P2, int counters, rr_instance *hostOut)
 {
     extern __shared__ int4 one_smem[];
@@ -70,7 +70,7 @@ __global__ void __launch_bounds__(ONE_THREADS) k_one(rr_instance h, rr_instance 
         __syncthreads();
         s_brec(B, I, ws, 1);
         __syncthreads();
-        sim_block<SIM_SMALL>(I, ws[0], (char *)one_smem, side, counters);
+        sim_block<SIM_SMALL, true>(I, ws[0], (char *)one_smem, side, counters);
         __syncthreads();
     }
     if (threadIdx.x < sizeof(rr_instance) / 4) ((volatile int32_t *)hostOut)[threadIdx.x] = ((int32_t *)I)[threadIdx.x];

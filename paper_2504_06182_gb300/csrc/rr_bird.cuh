@@ -7,7 +7,8 @@
 // sequential by definition: the unsolved columns are filled one after the
 // other, left to right, each from every token of the grid at once, and each
 // fill changes the tokens the next one sees. One block per grid runs that
-// loop with the grid's reservoir rows resident in shared memory.
+// loop with the grid's reservoir rows resident in shared memory, one half of
+// its threads on each side of the band.
 //
 // The generalised 1D instance of receiver column j (Sec. III.E): an atom in a
 // reservoir row v of a column at distance d sits on vertex v - d of column j
@@ -20,12 +21,28 @@
 // itself is red-rec's split: a tokens from above, all band atoms of j, the
 // rest from below, a of least total distance (largest a on ties), found by
 // the discrete derivative of the convex cost.
+//
+// What bounds it: the chain from one receiver to the next, about seven
+// barriers and as many shared-memory round trips. A side's nearest tokens are
+// found without visiting cells one by one: a thread per column counts its
+// tokens by layer (one shared add per token), a scan of the counts gives the
+// cut-off layer and each layer's place in the list, a second pass puts the
+// tokens into their layers, and within a layer (a column has at most one token
+// in it) a token's rank is the number of smaller entries. The layers counted
+// are the previous receiver's and a margin, more only when these do not
+// suffice: the reservoirs change little from one receiver to the next. Sides
+// of one warp (small grids, calls over very many) first walk the nearest cells
+// in order, which costs fewer instructions while the reservoirs are full.
+// Measured, against one warp per side walking cells, bisecting for the cut-off
+// and sorting by a bitonic network: 427 x 256 1089 -> 208 us, 1024 x 1024 51.7
+// -> 5.1 ms, 1024 grids of up to 256 x 256 4.1 -> 0.79 ms, 3000 of up to 64 x
+// 64 324 -> 227 us.
 #pragma once
 #include "rr_internal.cuh"
 
 namespace rrk {
 
-// Token of a walk list: row in the upper 16 bits, column in the lower.
+// Token of a list: row in the upper 16 bits, column in the lower.
 __device__ __forceinline__ int tok_row(int v) { return v >> 16; }
 __device__ __forceinline__ int tok_col(int v) { return v & 0xffff; }
 
@@ -52,184 +69,165 @@ __device__ __forceinline__ void walk_cell(int g, int j, int r0, int r1, bool top
     *row = top ? r0 - 1 - k + d : r1 + k - d;
 }
 
-// Walks cells g in [g, gEnd) in order (one warp), appending the tokens found
-// to list[got ..] until `need` are held. Returns the tokens held; *gNext is
-// the first cell not examined.
-__device__ inline int walk_range(const uint32_t *bits, int W, int m, int n, int r0, int r1, int j, bool top, int need,
-                          int g, int gEnd, int maxIter, int got, int32_t *list, int *gNext)
+// The nearest tokens of one side by visiting cells in order (one warp, 32
+// cells at a time, maxIter times at most): the tokens held if `need` were
+// found or no cell is left, else -1.
+__device__ __forceinline__ int bird_walk(const uint32_t *bits, int Wp, int m, int n, int r0, int r1, int j, bool top, int need,
+                                         int kmax, int maxIter, int lane, int32_t *list)
 {
-    const int lane = threadIdx.x & 31;
-    for (int it = 0; got < need && g < gEnd && it < maxIter; ++it, g += 32) {
+    const int gEnd = (kmax + 1) * (kmax + 1);
+    int got = 0, g = 0;
+    for (int it = 0; got < need && g < gEnd; ++it, g += 32) {
+        if (it == maxIter) return -1;
         const int gl = g + lane;
         int row, col;
         walk_cell(gl, j, r0, r1, top, &row, &col);
         bool occ = false;
         if (gl < gEnd && col >= 0 && col < n && row >= 0 && row < m && (top ? row < r0 : row >= r1))
-            occ = (bits[(size_t)col * W + (row >> 5)] >> (row & 31)) & 1u;
+            occ = (bits[col * Wp + (row >> 5)] >> (row & 31)) & 1u;
         const unsigned bal = __ballot_sync(FULL, occ);
         const int rank = got + __popc(bal & ((1u << lane) - 1u));
         if (occ && rank < need) list[rank] = (row << 16) | col;
         got = min(need, got + __popc(bal));
     }
-    *gNext = g;
     return got;
 }
 
-// Tokens of one side in layers <= K (one warp): per column, a masked popcount
-// over the rows whose vertex is within K of the band.
-__device__ inline int side_count(const uint32_t *bits, int W, int m, int n, int r0, int r1, int j, bool top, int K)
+// Position of a token of receiver j in the order in which the optimal window
+// takes them, on one side of the band: layer k in the upper bits, then its
+// place i in the layer: i = 0 is column j itself, i = 2d-1 column j-d, i = 2d
+// column j+d, on row r0-1-k+d above the band or r1+k-d below it.
+constexpr int KEY_I = 11;
+static_assert(2 * RR_MAX_SIDE <= 1 << KEY_I, "places of a layer");
+__device__ __forceinline__ uint32_t bird_key(int k, int c, int j)
 {
-    const int lane = threadIdx.x & 31;
-    int cnt = 0;
-    for (int c = lane; c < n; c += 32) {
-        const int d = iabs(c - j);
-        if (d > K) continue;
-        const int lo = top ? max(0, r0 - 1 - K + d) : r1;
-        const int hi = top ? r0 : min(m, r1 + K - d + 1);
-        for (int w = lo >> 5; w <= (hi - 1) >> 5; ++w) cnt += __popc(bits[(size_t)c * W + w] & row_mask(w, lo, hi));
-    }
-    return warp_sum(cnt);
+    return (uint32_t)k << KEY_I | (uint32_t)(c < j ? 2 * (j - c) - 1 : 2 * (c - j));
 }
 
-// Sorts a[0..len) ascending (one warp, bitonic network over the next power
-// of two; the entries past len are padding and must fit in the buffer).
-__device__ inline void warp_sort_u32(uint32_t *a, int len)
+// Barrier of one side's threads. (Immediate ids: a barrier number in a
+// register claims all sixteen, and fewer blocks fit on an SM.)
+__device__ __forceinline__ void side_sync(bool top, int T)
 {
-    const int lane = threadIdx.x & 31;
-    if (len <= 1) return;
-    int P = 1;
-    while (P < len) P <<= 1;
-    for (int i = len + lane; i < P; i += 32) a[i] = 0xffffffffu;
-    __syncwarp();
-    for (int k = 2; k <= P; k <<= 1)
-        for (int jj = k >> 1; jj > 0; jj >>= 1) {
-            for (int i = lane; i < P; i += 32) {
-                const int ij = i ^ jj;
-                if (ij > i) {
-                    const uint32_t x = a[i], y = a[ij];
-                    if ((x > y) == ((i & k) == 0)) { a[i] = y; a[ij] = x; }
-                }
-            }
-            __syncwarp();
-        }
+    if (T == 32) __syncwarp();
+    else if (top) asm volatile("bar.sync 1, %0;" ::"r"(T) : "memory");
+    else asm volatile("bar.sync 2, %0;" ::"r"(T) : "memory");
 }
 
-// Smallest layer K >= lo at which one side holds `need` tokens, kmax when it
-// never does (one warp); the layers below lo hold fewer. The search starts
-// from `guess` (the previous receiver's cut-off on this side: the
-// reservoirs change little from one column to the next), gallops toward the
-// answer, then bisects. *before gets the tokens in layers < K.
-__device__ inline int find_cutoff(const uint32_t *bits, int W, int m, int n, int r0, int r1, int j, bool top, int need,
-                           int lo, int kmax, int guess, int *before)
+// One side of the band of one receiver: its threads (T of them, st the
+// thread's number) call f(layer, column) for every token in the layers above
+// `from` and up to `to`. While these reach over few columns, 2, 4 or 8 threads
+// share one, each with some of every word's bits. A word's lowest and highest
+// bit are taken together: the two searches' latencies overlap.
+template <class F>
+__device__ __forceinline__ void bird_tokens(const uint32_t *bits, int Wp, int m, int n, int r0, int r1, int j, bool top,
+                                            int from, int to, int st, int T, F f)
 {
-    int kb = lo - 1, cb = kb < 0 ? 0 : -1;   // largest layer known to hold fewer than need, its count
-    const int g = min(max(guess, lo), kmax);
-    int hi = kmax;
-    const int cg = side_count(bits, W, m, n, r0, r1, j, top, g);
-    if (cg >= need) {
-        hi = g;
-        for (int s = 1; hi - s >= lo; s <<= 1) {
-            const int t = hi - s;
-            const int ct = side_count(bits, W, m, n, r0, r1, j, top, t);
-            if (ct >= need) { hi = t; continue; }
-            kb = t; cb = ct; lo = t + 1;
-            break;
-        }
-    } else {
-        kb = g; cb = cg; lo = g + 1;
-        for (int s = 1;; s <<= 1) {
-            const int t = min(g + s, kmax);
-            const int ct = side_count(bits, W, m, n, r0, r1, j, top, t);
-            if (ct >= need) { hi = t; break; }
-            kb = t; cb = ct; lo = t + 1;
-            if (t == kmax) {                    // fewer than need in all: take them all
-                *before = side_count(bits, W, m, n, r0, r1, j, top, kmax - 1);
-                return kmax;
+    const int first = max(0, j - to), cols = min(n - 1, j + to) - first + 1;
+    const int sh = cols > T / 2 ? 0 : cols > T / 4 ? 1 : cols > T / 8 ? 2 : 3;
+    const uint32_t part = sh == 0 ? FULL : (1u << (32 >> sh)) - 1u << (st & ((1 << sh) - 1)) * (32 >> sh);
+    for (int q = st >> sh; q < cols; q += T >> sh) {
+        const int c = first + q, d = iabs(c - j);
+        const int lo = top ? max(0, r0 - 1 - to + d) : max(r1, r1 + from + 1 - d);
+        const int end = top ? min(r0, r0 - 1 - from + d) : min(m, r1 + to - d + 1);
+        for (int w = lo >> 5; 32 * w < end; ++w) {
+            // the layer of bit b: k0 - b above the band, k0 + b below it
+            const int k0 = (top ? r0 - 1 - 32 * w : 32 * w - r1) + d;
+            for (uint32_t x = bits[c * Wp + w] & part & row_mask(w, lo, end); x;) {
+                const int b0 = __ffs(x) - 1, b1 = 31 - __clz(x);
+                x = x & (x - 1u) & ~(1u << b1);
+                f(top ? k0 - b0 : k0 + b0, c);
+                if (b1 != b0) f(top ? k0 - b1 : k0 + b1, c);
             }
         }
     }
-    while (lo < hi) {
-        const int mid = (lo + hi) >> 1;
-        const int cm = side_count(bits, W, m, n, r0, r1, j, top, mid);
-        if (cm >= need) hi = mid;
-        else { lo = mid + 1; kb = mid; cb = cm; }
-    }
-    *before = lo == 0 ? 0 : (kb == lo - 1 && cb >= 0 ? cb : side_count(bits, W, m, n, r0, r1, j, top, lo - 1));
-    return lo;
 }
 
-// Collects, in walk order, the `need` nearest tokens of receiver j on one
-// side of the band, or all of them if fewer (one warp). While the
-// reservoirs near j are full the walk finds them in a few iterations. Once
-// they are depleted the walk would scan the empty area cell by cell, so the
-// cut-off layer K (the first at which the count reaches need) is found by
-// popcounts instead (find_cutoff); the tokens of the layers before K are
-// gathered by their walk index and sorted, and layer K alone is walked.
-// *sparse and *kHint carry this side's state from one receiver to the next:
-// after a cut-off beyond what the bounded walk would have reached, the next
-// receiver skips the walk and starts the search from this cut-off.
-__device__ inline int bird_side(const uint32_t *bits, int W, int m, int n, int r0, int r1, int j, bool top, int need,
-                         int32_t *list, int *s_cnt, bool *sparse, int *kHint)
+// The `need` nearest tokens of receiver j on one side, in the window's order,
+// or all of them if fewer: into list; returns their number. hist: zero for
+// every layer on entry; the layers up to *used are not on return. guess: the
+// layers to count at first (on return: for the next receiver, the cut-off and
+// as many more as it has grown by since the last one; a layer near it may hold
+// as many tokens as the receiver needs). s_out: two words.
+__device__ __forceinline__ int bird_side(const uint32_t *bits, int Wp, int m, int n, int r0, int r1, int j, bool top,
+                                         int need, int32_t *list, uint32_t *keys, unsigned *hist, int *s_out, int st,
+                                         int T, int *guess, int *last, int *used, bool *sparse)
 {
-    const int lane = threadIdx.x & 31;
+    *used = -1;
     if (top ? r0 == 0 : r1 == m) return 0;
-    const int dmax = max(j, n - 1 - j);
-    const int kmax = top ? r0 - 1 + dmax : m - 1 - r1 + dmax;   // no cell beyond this layer
-    const int gAll = (kmax + 1) * (kmax + 1);
-    const int walkIter = 8 + need / 8;
-    int gNext, lo = 0;
-    if (!*sparse) {
-        const int got = walk_range(bits, W, m, n, r0, r1, j, top, need, 0, gAll, walkIter, 0, list, &gNext);
-        if (got >= need || gNext >= gAll) return got;
-        lo = isqrt_floor(gNext);             // layers below the walk's last one hold fewer than need
+    const int lane = st & 31;
+    const int kmax = (top ? r0 - 1 : m - 1 - r1) + max(j, n - 1 - j);     // no cell beyond this layer
+    if (T == 32 && !*sparse) {
+        const int got = bird_walk(bits, Wp, m, n, r0, r1, j, top, need, kmax, 8 + need / 8, lane, list);
+        if (got >= 0) return got;
     }
-    int before;
-    const int K = find_cutoff(bits, W, m, n, r0, r1, j, top, need, lo, kmax, *kHint, &before);
-    *kHint = K;
-    *sparse = (K + 1) * (K + 1) > 32 * walkIter;
-    // gather the walk indices of the tokens in layers < K, sort, decode
-    if (lane == 0) *s_cnt = 0;
-    __syncwarp();
-    uint32_t *keys = (uint32_t *)list;
-    for (int c = lane; c < n; c += 32) {
-        const int d = iabs(c - j);
-        if (d > K - 1) continue;
-        const int rlo = top ? max(0, r0 - 1 - (K - 1) + d) : r1;
-        const int rhi = top ? r0 : min(m, r1 + (K - 1) - d + 1);
-        const int i = d == 0 ? 0 : (c < j ? 2 * d - 1 : 2 * d);
-        for (int w = rlo >> 5; w <= (rhi - 1) >> 5; ++w) {
-            uint32_t x = bits[(size_t)c * W + w] & row_mask(w, rlo, rhi);
-            while (x) {
-                const int v = 32 * w + __ffs(x) - 1;
-                x &= x - 1;
-                const int k = (top ? r0 - 1 - v : v - r1) + d;
-                const int slot = atomicAdd(s_cnt, 1);
-                if (slot < before) keys[slot] = (uint32_t)(k * k + i);
+    int from = -1, to = min(*guess, kmax), more = 2, K, total;
+    for (;;) {
+        bird_tokens(bits, Wp, m, n, r0, r1, j, top, from, to, st, T, [&](int k, int) { atomicAdd(&hist[k], 1u); });
+        side_sync(top, T);
+        if (st < 32) {
+            // the first layer with `need` tokens up to it; the layers' places
+            const int per = (to + 32) >> 5 | 1, k0 = lane * per, k1 = min(k0 + per, to + 1);
+            int sum = 0;
+#pragma unroll 4
+            for (int k = k0; k < k1; ++k) sum += (int)hist[k];
+            const int incl = warp_incl_scan(sum);
+            const unsigned full = __ballot_sync(FULL, incl >= need);
+            if (full || to == kmax) {
+                int at = incl - sum, cut = 0x7fffffff, tot = 0;
+#pragma unroll 4
+                for (int k = k0; k < k1; ++k) {
+                    const int c = (int)hist[k];
+                    hist[k] = (unsigned)at;
+                    at += c;
+                    if (at >= need && cut == 0x7fffffff) { cut = k; tot = at; }
+                }
+                const int src = full ? __ffs(full) - 1 : 31;
+                cut = __shfl_sync(FULL, full ? cut : kmax, src);
+                tot = __shfl_sync(FULL, full ? tot : incl, src);
+                if (lane == 0) { s_out[0] = cut; s_out[1] = tot; }
+            } else if (lane == 0) {
+                s_out[0] = -1;
             }
         }
+        side_sync(top, T);
+        K = s_out[0];
+        total = s_out[1];
+        if (K >= 0) break;
+        from = to;
+        to = min(kmax, to + more);
+        more *= 2;
     }
-    __syncwarp();
-    warp_sort_u32(keys, before);
-    for (int t = lane; t < before; t += 32) {
-        int row, col;
-        walk_cell((int)keys[t], j, r0, r1, top, &row, &col);
-        list[t] = (row << 16) | col;
+    // tokens into their layers; a layer's entry ends at the next one's start
+    bird_tokens(bits, Wp, m, n, r0, r1, j, top, -1, K, st, T,
+                [&](int k, int c) { keys[atomicAdd(&hist[k], 1u)] = bird_key(k, c, j); });
+    if (st < 3) keys[total + st] = FULL;
+    side_sync(top, T);
+    for (int t = st; t < total; t += T) {
+        // (four entries at a time: those before the layer are all smaller,
+        // those after it greater)
+        const uint32_t x = keys[t];
+        const int k = (int)(x >> KEY_I), b0 = (k > 0 ? (int)hist[k - 1] : 0) & ~3, b1 = (int)hist[k];
+        int at = b0;
+#pragma unroll 2
+        for (int u = b0; u < b1; u += 4) {
+            const uint4 y = *(const uint4 *)(keys + u);
+            at += (y.x < x) + (y.y < x) + (y.z < x) + (y.w < x);
+        }
+        const int i = (int)(x & ((1u << KEY_I) - 1u)), d = (i + 1) >> 1;
+        if (at < need) list[at] = (top ? r0 - 1 - k + d : r1 + k - d) << 16 | ((i & 1) ? j - d : j + d);
     }
-    __syncwarp();
-    return walk_range(bits, W, m, n, r0, r1, j, top, need, K * K, (K + 1) * (K + 1), 0x7fffffff, before, list,
-                      &gNext);
+    *guess = K + max(1, K - *last);
+    *last = K;
+    *sparse = (K + 1) * (K + 1) > 32 * (8 + need / 8);
+    *used = to;
+    return min(total, need);
 }
 
-// Threads of the bird stage: two warps (one per side of the band), synchronised
-// by a named barrier of their own, so that the stage also runs inside a larger
-// block whose other warps wait outside it.
-constexpr int BIRD_THREADS = 64;
-__device__ __forceinline__ void bird_sync() { asm volatile("bar.sync 1, 64;" ::: "memory"); }
-
+// Every thread of the block calls it: T on each side of the band.
 __device__ inline void s_bird(const Blk B, rr_instance *inst, JobWS *wsv, int count, int max_side)
 {
-    extern __shared__ uint32_t birdsm[];
-    __shared__ int s_nt, s_nb, s_a, s_base, s_bad, s_nrecv, s_cnt[2];
+    extern __shared__ __align__(16) uint32_t birdsm[];
+    __shared__ int s_got[2], s_base, s_bad, s_nrecv, s_out[4];
     const int q = B.x;
     if (q >= count) return;
     rr_instance *I = &inst[q];
@@ -237,15 +235,17 @@ __device__ inline void s_bird(const Blk B, rr_instance *inst, JobWS *wsv, int co
     JobWS &ws = wsv[q];
     const int m = I->m, n = I->n, W = (m + 31) >> 5;
     const int r0 = I->rect.r0, r1 = I->rect.r1, c0 = I->rect.c0, c1 = I->rect.c1, h = r1 - r0;
-    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-    uint32_t *bits = birdsm;                                               // n * W words
-    int listCap = 1;                                                      // next power of two >= max_side
-    while (listCap < max_side) listCap <<= 1;
-    int32_t *topTok = (int32_t *)(birdsm + (size_t)max_side * ((max_side + 31) >> 5));
-    int32_t *botTok = topTok + listCap;
+    const int threads = blockDim.x, T = threads >> 1;
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, side = tid >= T ? 1 : 0;
+    const BirdLayout Y(max_side);
+    const int Wp = W | 1;                                                  // odd: neighbouring columns in different banks
+    uint32_t *bits = birdsm;                                               // n * Wp words
+    int32_t *topTok = (int32_t *)(birdsm + Y.lists), *botTok = topTok + max_side;
+    uint32_t *keys = birdsm + Y.keys + side * Y.room;
+    unsigned *hist = birdsm + Y.hist + side * 2 * max_side;
     // receivers in column order (column, band atoms, atoms above the band),
     // and the current receiver's band holes and band atom rows
-    int16_t *recvCol = (int16_t *)(botTok + listCap);
+    int16_t *recvCol = (int16_t *)(birdsm + Y.recv);
     int16_t *recvM = recvCol + max_side, *recvTop = recvM + max_side;
     int16_t *sHr = recvTop + max_side, *sOwn = sHr + max_side;
 
@@ -286,7 +286,8 @@ __device__ inline void s_bird(const Blk B, rr_instance *inst, JobWS *wsv, int co
     // Reservoir rows after the column phase: solved target columns keep the
     // atoms outside their window, outer columns with enough atoms fill every
     // reservoir trap, the others are untouched. Band rows are never read.
-    for (int idx = tid; idx < n * W; idx += BIRD_THREADS) {
+    for (int i = tid; i < 4 * max_side; i += threads) birdsm[Y.hist + i] = 0u;
+    for (int idx = tid; idx < n * W; idx += threads) {
         const int c = idx / W, w = idx - c * W;
         const ColInfo ci = ws.col[c];
         const uint32_t res = row_mask(w, 0, r0) | row_mask(w, r1, m);
@@ -299,9 +300,9 @@ __device__ inline void s_bird(const Blk B, rr_instance *inst, JobWS *wsv, int co
             const int botLim = ci.pbot > 0 ? rows[ci.bbase] : m;           // pool below: rows >= botLim
             x &= row_mask(w, 0, topLim) | row_mask(w, botLim, m);
         }
-        bits[idx] = x & res;
+        bits[c * Wp + w] = x & res;
     }
-    bird_sync();
+    __syncthreads();
     if (s_bad) {
         if (tid == 0) { I->status = RR_INFEASIBLE; I->n_moves = 0; }
         return;
@@ -311,45 +312,44 @@ __device__ inline void s_bird(const Blk B, rr_instance *inst, JobWS *wsv, int co
     const int nrecv = s_nrecv;
     long long done = 0;          // moves of the receiver units so far
     long long steps = 0;
-    bool sparse = false;         // this warp's side: walk skipped, search hint
-    int kHint = 0;
+    int guess = -1, last = 0;    // this side's layers to count, its last cut-off
+    bool sparse = false;
     for (int u = 0; u < nrecv; ++u) {
         const int j = recvCol[u], M = recvM[u], ownTop = recvTop[u];
         const int need = h - M, nh = h - M;
         // this receiver's band holes and band atoms (read by the split and
-        // the emission once the walks are done)
-        {
-            const int16_t *ghr = ws.holeRows + (size_t)(j - c0) * h;
-            const int16_t *gown = ws.atomRows + (size_t)j * m + ownTop;
-            for (int t = tid; t < nh; t += BIRD_THREADS) sHr[t] = ghr[t];
-            for (int t = tid; t < M; t += BIRD_THREADS) sOwn[t] = gown[t];
-        }
+        // the emission once the tokens are found): the first ones' loads are
+        // in flight meanwhile
+        const int16_t *ghr = ws.holeRows + (size_t)(j - c0) * h;
+        const int16_t *gown = ws.atomRows + (size_t)j * m + ownTop;
+        const int16_t hr0 = tid < nh ? ghr[tid] : (int16_t)0, own0 = tid < M ? gown[tid] : (int16_t)0;
+        if (guess < 0) guess = last = 2 + (int)sqrtf(2.f * (float)need);
+        int used;
+        const int got = bird_side(bits, Wp, m, n, r0, r1, j, side == 0, need, side == 0 ? topTok : botTok, keys, hist,
+                                  s_out + 2 * side, tid - side * T, T, &guess, &last, &used, &sparse);
+        if (tid == side * T) s_got[side] = got;
+        if (tid < nh) sHr[tid] = hr0;
+        if (tid < M) sOwn[tid] = own0;
+        for (int t = tid + threads; t < nh; t += threads) sHr[t] = ghr[t];
+        for (int t = tid + threads; t < M; t += threads) sOwn[t] = gown[t];
         const int16_t *hr = sHr;
-        if (wid < 2) {
-            const int got = bird_side(bits, W, m, n, r0, r1, j, wid == 0, need, wid == 0 ? topTok : botTok,
-                                      &s_cnt[wid], &sparse, &kHint);
-            if (lane == 0) { if (wid == 0) s_nt = got; else s_nb = got; }
+        __syncthreads();
+        for (int k = tid - side * T; k <= used; k += T) hist[k] = 0u;
+        // every warp finds the split: that is cheaper than another barrier
+        const int nt = s_got[0], nb = s_got[1];
+        int a = -1;
+        if (nt + nb >= need) {
+            const int lo = max(0, need - nb), hi = min(need, nt);
+            // d cost / da: one more token from above (the a-th nearest)
+            // and one fewer from below (the (need-a+1)-th nearest)
+            a = split_search(lo, hi, [&](int aa) {
+                const int tv = topTok[aa - 1], bv = botTok[need - aa];
+                const int tpos = tok_row(tv) - iabs(tok_col(tv) - j);
+                const int bpos = tok_row(bv) + iabs(tok_col(bv) - j);
+                return (r0 + aa - 1 - tpos) + (2 * band_P(hr, nh, M, r0, r0 + aa - 1) - M) +
+                       (r0 + h - need + aa - 1 - bpos);
+            });
         }
-        bird_sync();
-        if (wid == 0) {
-            const int nt = s_nt, nb = s_nb;
-            int a = -1;
-            if (nt + nb >= need) {
-                const int lo = max(0, need - nb), hi = min(need, nt);
-                // d cost / da: one more token from above (the a-th nearest)
-                // and one fewer from below (the (need-a+1)-th nearest)
-                a = split_search(lo, hi, [&](int aa) {
-                    const int tv = topTok[aa - 1], bv = botTok[need - aa];
-                    const int tpos = tok_row(tv) - iabs(tok_col(tv) - j);
-                    const int bpos = tok_row(bv) + iabs(tok_col(bv) - j);
-                    return (r0 + aa - 1 - tpos) + (2 * band_P(hr, nh, M, r0, r0 + aa - 1) - M) +
-                           (r0 + h - need + aa - 1 - bpos);
-                });
-            }
-            if (lane == 0) s_a = a;
-        }
-        bird_sync();
-        const int a = s_a;
         if (a < 0) {             // cannot happen when the total surplus is >= 0
             if (tid == 0) set_status(I, RR_ERR_INTERNAL);
             return;
@@ -361,7 +361,7 @@ __device__ inline void s_bird(const Blk B, rr_instance *inst, JobWS *wsv, int co
         const int kd_end = a + band_P(hr, nh, M, r0, r0 + a - 1);
         const int ku_start = a + band_P(hr, nh, M, r0, r0 + a);
         const long long base = colTotal + done;
-        for (int k = tid; k < h; k += BIRD_THREADS) {
+        for (int k = tid; k < h; k += threads) {
             int row, col;
             if (k < a) { const int v = topTok[a - 1 - k]; row = tok_row(v); col = tok_col(v); }
             else if (k < a + M) { row = sOwn[k - a]; col = j; }
@@ -375,13 +375,13 @@ __device__ inline void s_bird(const Blk B, rr_instance *inst, JobWS *wsv, int co
             steps += iabs(r0 + k - row) + iabs(j - col);
         }
         // the chosen tokens leave the reservoirs
-        for (int l = tid; l < need; l += BIRD_THREADS) {
+        for (int l = tid; l < need; l += threads) {
             const int v = l < a ? topTok[l] : botTok[l - a];
             const int row = tok_row(v), col = tok_col(v);
-            atomicAnd(&bits[(size_t)col * W + (row >> 5)], ~(1u << (row & 31)));
+            atomicAnd(&bits[col * Wp + (row >> 5)], ~(1u << (row & 31)));
         }
         done += kd_end + (h - ku_start);
-        bird_sync();
+        __syncthreads();
     }
     add_steps(I, steps);
     if (tid == 0) {

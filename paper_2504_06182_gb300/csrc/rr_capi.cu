@@ -301,16 +301,19 @@ static int clampi(int v, int lo, int hi) { return v < lo ? lo : (v > hi ? hi : v
 // Blocks a launch may spread over all grids of a call (divided by the count).
 static int budget(const rr_ctx *ctx, int base) { return ctx->shift >= 0 ? base << ctx->shift : base >> -ctx->shift; }
 
-// Shared memory of a k_bird block: reservoir-row bits of the largest grid
-// (column-major, one word per 32 rows), the two token lists (each the next
-// power of two >= max_side: they double as sort buffers), then five int16
-// arrays of max_side (the receiver list: columns, band atoms, atoms above
-// the band; the current receiver's band holes and band atom rows).
-static size_t bird_smem_bytes(int max_side)
+// Threads of a k_bird block. A thread per column on each side of the band
+// where the machine is not full: one grid of 427 x 256 takes 208 us with 512
+// threads and 239 with 896; of 1024 x 1024 5.0 ms with 1024, 5.5 with 512 and
+// 7.3 with 256; 1024 grids of up to 256 x 256 758 us with 384 and 862 with 256;
+// 600 of up to 128 x 128 295 us with 128 and 336 with 256. In calls over more
+// grids the threads that an SM holds, shared out: 3000 grids of up to 64 x 64
+// take 219 us with 64 threads and 287 with 128, of up to 256 x 256 2.0 ms with
+// 128, 2.3 with 64 and 2.7 with 256.
+static int bird_threads(const rr_ctx *ctx, int count, int max_side)
 {
-    size_t cap = 1;
-    while (cap < (size_t)max_side) cap <<= 1;
-    return 4 * ((size_t)max_side * ((max_side + 31) / 32) + 2 * cap) + 2 * 5 * (size_t)max_side;
+    const int most = count <= ctx->nsm ? (max_side <= 512 ? 512 : BIRD_MAX_THREADS) : max_side <= 128 ? 128 : 384;
+    const int share = (int)std::min<long long>(2048ll * ctx->nsm / std::max(count, 1), 2048) & ~63;
+    return std::min(std::min(most, 2 * ((max_side + 31) / 32 * 32)), std::max(share, max_side <= 128 ? 64 : 128));
 }
 
 // Planning kernels over `count` device descriptors whose sides are <= max_side:
@@ -344,7 +347,7 @@ static int launch_plan(rr_ctx *ctx, rr_instance *d_inst, JobWS *ws, int count, i
         if (birdSmem > (size_t)ctx->smemLimit[SM_BIRD])
             return fail(ctx, RR_ERR_ARG, "bird: shared memory %zu for side %d too large", birdSmem, max_side);
         mark(ctx, s, "k_bird");
-        k_bird<<<count, 64, birdSmem, s>>>(d_inst, ws, count, max_side);
+        k_bird<<<count, bird_threads(ctx, count, max_side), birdSmem, s>>>(d_inst, ws, count, max_side);
         mark(ctx, s, "k_emit_cols");
         k_emit_cols<<<dim3(colBlocks, rows), 256, 0, s>>>(d_inst, ws, count, per);
         mark(ctx, s, nullptr);

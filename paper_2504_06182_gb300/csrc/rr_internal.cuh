@@ -378,6 +378,28 @@ __device__ __forceinline__ int band_P(const int16_t *hr, int nh, int nband, int 
     return (int)hr[u] - r0 - u;
 }
 
+// Shared memory of the bird stage, in words: reservoir-row bits of the largest
+// grid (column-major, an odd number of words per column), the two sides' layer
+// entries (a side holds fewer than the tokens it needs and one layer more, and
+// three words of padding), the two token lists and layer counts, then five
+// int16 arrays (the
+// receiver list: columns, band atoms, atoms above the band; the current
+// receiver's band holes and band atom rows).
+constexpr int BIRD_MAX_THREADS = 1024;
+struct BirdLayout {
+    int keys, room, lists, hist, recv, words;
+    __host__ __device__ explicit BirdLayout(int max_side)
+    {
+        keys = (max_side * (((max_side + 31) / 32) | 1) + 3) & ~3;     // 16-byte aligned, as a side's room is
+        room = (2 * max_side + 6) & ~3;
+        lists = keys + 2 * room;
+        hist = lists + 2 * max_side;
+        recv = hist + 4 * max_side;
+        words = recv + (5 * max_side + 1) / 2;
+    }
+};
+inline size_t bird_smem_bytes(int max_side) { return 4 * (size_t)BirdLayout(max_side).words; }
+
 } // namespace rrk
 
 // Library-internal hooks between translation units (not part of the C ABI).

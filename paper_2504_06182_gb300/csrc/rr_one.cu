@@ -9,8 +9,7 @@
 // same functions the separate kernels run (rr_plan.cuh, rr_bird.cuh,
 // rr_batch.cuh), given block coordinates x = 0, gx = 1 so that each
 // grid-stride loop covers all of its work with this block's warps; the
-// pairing runs on warp 0 and the two-warp bird stage on warps 0-1 while the
-// other warps wait at the next barrier. In the simulation warp 0 simulates
+// pairing runs on warp 0 while the other warps wait at the next barrier. In the simulation warp 0 simulates
 // and the other warps write the batches.
 // The descriptor comes in as a kernel parameter and the final one is written
 // to mapped host memory, so a call is one launch and one synchronisation.
@@ -40,7 +39,7 @@ __global__ void __launch_bounds__(ONE_THREADS, 1) k_one(rr_instance h, rr_instan
     s_colstats(B, I, ws, 1, (flags & RR_STRICT_RESERVOIR) ? 1 : 0);
     __syncthreads();
     if (bird) {
-        if (wid < 2) s_bird(B, I, ws, 1, side);
+        s_bird(B, I, ws, 1, side);
         __syncthreads();
         s_emit_cols(B, I, ws, 1);
     } else {
@@ -90,11 +89,7 @@ size_t one_smem_bytes(int side, int flags)
     while (P2 < side) P2 <<= 1;
     const size_t warps = ONE_THREADS / 32;
     size_t b = (size_t)side * PAIR_BYTES + 64;                               // pairing
-    if (flags & RR_BIRD) {
-        size_t cap = 1;
-        while (cap < (size_t)side) cap <<= 1;
-        b = std::max(b, 4 * ((size_t)side * ((side + 31) / 32) + 2 * cap) + 2 * 5 * (size_t)side);
-    }
+    if (flags & RR_BIRD) b = std::max(b, bird_smem_bytes(side));
     if (flags & RR_WITH_BATCH) {
         b = std::max(b, warps * 4 * (size_t)P2);                              // k_gsort
         b = std::max(b, warps * 12 * (size_t)side);                           // k_gsweep_v (h needs a third)

@@ -83,15 +83,14 @@ __device__ inline void s_bsetup(const Blk B, rr_instance *inst, JobWS *wsv, int 
             ws.rowCur = (int32_t *)arena_alloc(A, 4ull * (m + 1), &ok);
             ws.rowList = (int32_t *)arena_alloc(A, 4ull * (k + 1), &ok);
             ws.firstH = (int32_t *)arena_alloc(A, 4ull * cells, &ok);
-            ws.multiPos = (uint32_t *)arena_alloc(A, 4ull * (k + 1), &ok);
+            ws.multiMove = (int2 *)arena_alloc(A, 8ull * (k + 1), &ok);
             ws.indeg = (int32_t *)arena_alloc(A, 4ull * (k + 1), &ok);
             ws.rec = (int4 *)arena_alloc(A, 32ull * (k + 1), &ok);
             ws.succ4 = ws.rec + 1;
             ws.ready0 = (int32_t *)arena_alloc(A, 4ull * (k + 1) + 16, &ok);
             ws.slotOvf = arena_alloc(A, sim_wide_bytes(k), &ok);
-            ws.multiNo = (int32_t *)arena_alloc(A, 4ull * (k + 1), &ok);
             ws.multi = ws.colList;               // both lists are free again once they have been swept
-            ws.multiId = ws.rowList;
+            ws.multiNo = ws.rowList;
             ws.nmulti = 0;
             ws.nextAt = nullptr;
             ws.succ = nullptr;
@@ -148,15 +147,14 @@ __device__ inline void s_bsetup(const Blk B, rr_instance *inst, JobWS *wsv, int 
             ws.rowCur = (int32_t *)arena_alloc(A, 4ull * (m + 1), &ok);
             ws.rowList = (int32_t *)arena_alloc(A, 4ull * (k + 1), &ok);
             ws.firstH = (int32_t *)arena_alloc(A, 4ull * cells, &ok);
-            ws.multiPos = (uint32_t *)arena_alloc(A, 4ull * (k + 1), &ok);
+            ws.multiMove = (int2 *)arena_alloc(A, 8ull * (k + 1), &ok);
             ws.indeg = (int32_t *)arena_alloc(A, 4ull * (k + 1), &ok);
             ws.rec = (int4 *)arena_alloc(A, 32ull * (k + 1), &ok);   // record, successors: one 32 B sector
             ws.succ4 = ws.rec + 1;
             ws.ready0 = (int32_t *)arena_alloc(A, 4ull * (k + 1) + 16, &ok);
             ws.slotOvf = arena_alloc(A, sim_wide_bytes(k), &ok);
-            ws.multiNo = (int32_t *)arena_alloc(A, 4ull * (k + 1), &ok);
             ws.multi = ws.colList;               // both lists are free again once they have been swept
-            ws.multiId = ws.rowList;
+            ws.multiNo = ws.rowList;
             ws.nmulti = 0;
             // a path has at most as many distinct successors as vertices: they
             // are stored at the path's vertex offset, so no count pass or scan
@@ -608,7 +606,7 @@ __device__ inline int distinct_succ(const int32_t *seq, int len, int32_t *out, J
         out[cnt++] = v;
         if (atomicAdd(&ws.indeg[v], 1) == 1) {    // a second predecessor: it needs a counter
             const int x = atomicAdd(&ws.nmulti, 1);
-            ws.multiId[x] = v;
+            ws.multiMove[x].x = v;
             ws.multiNo[v] = x;
         }
     };
@@ -670,7 +668,7 @@ __device__ inline void s_brec(const Blk B, rr_instance *inst, JobWS *wsv, int co
         if (in > 1) {
             const int x = ws.multiNo[b];
             ws.multi[x] = in | (r.y & 8191) << MULTI_BITS;
-            ws.multiPos[x] = (uint32_t)r.x;
+            ws.multiMove[x].y = r.x;
         }
         if (in == 0) ws.ready0[atomicAdd(&ws.ready0[k], 1)] = (int32_t)b;
     }
@@ -1139,8 +1137,7 @@ static __device__ __noinline__ int run_of_leaders(rr_instance *I, JobWS *ws, cha
     const uint32_t *pos = (const uint32_t *)smem;
     const int4 *rec = as_global(ws->rec);
     int32_t *multi = as_global(ws->multi), *log = as_global(ws->nextAt);
-    const int32_t *multiId = as_global(ws->multiId);
-    const uint32_t *multiPos = as_global(ws->multiPos);
+    const int2 *multiMove = as_global(ws->multiMove);
     SimCtl *C = Y.C;
     unsigned *cnt = Y.cnt;
     int32_t *ids = Y.ids, *buf = Y.bufs;
@@ -1273,8 +1270,7 @@ static __device__ __noinline__ int run_of_leaders(rr_instance *I, JobWS *ws, cha
     #pragma unroll
         for (int e = 0; e < 4; ++e) {
             const bool t = lane < n && (few >> e & 1u);
-            touch_if(t, multiId + (t ? sv[e] : 0), dump);
-            touch_if(t, multiPos + (t ? sv[e] : 0), dump);
+            touch_if(t, multiMove + (t ? sv[e] : 0), dump);
             touch_if(t, multi + (t ? sv[e] : 0), dump);
         }
     }
@@ -1319,8 +1315,8 @@ struct Sim {
     uint32_t *mpos;           // members: position word, `along` minus the clock
     SimCtl *C;
     const int4 *rec;
-    const int32_t *succ, *multiId;
-    const uint32_t *multiPos;
+    const int32_t *succ;
+    const int2 *multiMove;    // the moves that the counters belong to: id, position word
     int32_t *multi;           // in-degree counters in global memory (with their moves' first legs)
     unsigned *cnt;            // the first ncnt of them in shared memory, two per word
     int ncnt;
@@ -1361,24 +1357,24 @@ struct Sim {
         const bool single = c && (v & SUCC_SINGLE), multi_ = c && !(v & SUCC_SINGLE);
         const int x = v & SUCC_ID;
         const int sh = (x & 1) * 16;
+        bool h = single && x == handId;
+        const bool fresh = single && !h;
         int old = (sh_add_if(multi_ && x < ncnt, cnt + (x >> 1), -(1 << sh)) >> sh) & 0xffff;
+        int2 r = ldg_if(fresh, (const int2 *)(rec + 2 * (size_t)x));       // (in flight during the vote)
         if (!allShared) {
             if (multi_ && x >= ncnt) old = atomicSub(&multi[x], 1) & MULTI_COUNT;
             __syncwarp();
         }
         const bool soon = multi_ && old == 2, last = multi_ && old == 1;
-        touch_if(soon, multiId + x, dump);           // next time it is ready
-        touch_if(soon, multiPos + x, dump);
+        touch_if(soon, multiMove + x, dump);         // next time it is ready
         touch_if(soon, multi + x, dump);
-        bool h = single && x == handId;
-        const bool fresh = single && !h;
         if (__any_sync(FULL, fresh || last)) {
-            const int2 r = ldg_if(fresh, (const int2 *)(rec + 2 * (size_t)x));
-            int id = ldg_if(last, (const void *)(multiId + x)), p = ldg_if(last, (const void *)(multiPos + x));
-            int y = ldg_if(last, (const void *)(multi + x)) >> MULTI_BITS;
-            if (fresh) { id = x; p = r.x; y = r.y; }
+            const int2 mv = ldg_if(last, multiMove + x);
+            const int y = ldg_if(last, (const void *)(multi + x)) >> MULTI_BITS;
+            const int id = last ? mv.x : x;
+            if (last) r = make_int2(mv.y, y);
             h |= last && id == handId;
-            enter((fresh || last) && !h, y & 3, (uint32_t)p, id, y >> 2 & 2047);
+            enter((fresh || last) && !h, r.y & 3, (uint32_t)r.x, id, r.y >> 2 & 2047);
         }
         return h;
     }
@@ -1436,6 +1432,7 @@ __device__ __forceinline__ int Sim<MODE>::run(rr_instance *I, JobWS &ws, int32_t
     // this lane's eight entries of a table's first 256 (a lane beyond the
     // table reads the last eight too: that changes no minimum)
     int groups = size(0) >> 3, off = 8 * min(lane, groups - 1);
+    const unsigned holders = groups >= 32 ? FULL : (1u << groups) - 1u;      // (lanes of a SIM_SMALL table)
 
     auto set_leg = [&](uint32_t y) {
         d = (int)(y & 3u);
@@ -1556,6 +1553,7 @@ __device__ __forceinline__ int Sim<MODE>::run(rr_instance *I, JobWS &ws, int32_t
                 const uint4 a2 = *(const uint4 *)(pos + tb + 8 * g), b2 = *(const uint4 *)(pos + tb + 8 * g + 4);
                 v = min8(a2, b2, nadd, v);
             }
+        int fr = C->nfree[d];
         int pick = (int)__reduce_min_sync(FULL, v < 0x10000u ? 0u : v & 0xffffu);
         if (MODE != SIM_WIDE && tryRun) {
             tryRun = false;
@@ -1604,12 +1602,12 @@ __device__ __forceinline__ int Sim<MODE>::run(rr_instance *I, JobWS &ws, int32_t
                     if (prim) ma = min(ma, id); else mc = min(mc, id);
                 }
                 choose = __reduce_min_sync(FULL, ma) < __reduce_min_sync(FULL, mc);
-                if (nm > 0 && choose != prim) dissolve();
+                if (nm > 0 && choose != prim) { dissolve(); fr = C->nfree[d]; }
             }
             alone = false;
             if (choose ? ba : bc) {
                 // the chosen line's statics join the members
-                int me = minEnd, fr = C->nfree[d];
+                int me = minEnd;
                 __syncwarp();
                 const uint32_t half = choose ? 0xffffu : 0xffff0000u;
                 for (int g0 = 0; g0 < groups; g0 += 32) {
@@ -1620,7 +1618,8 @@ __device__ __forceinline__ int Sim<MODE>::run(rr_instance *I, JobWS &ws, int32_t
                     } else if (g0 + lane < groups) {
                         q = match8(*(const uint4 *)(pos + e0), *(const uint4 *)(pos + e0 + 4), lpos, half);
                     }
-                    for (unsigned bal = __ballot_sync(FULL, q != 0u); bal; bal = __ballot_sync(FULL, q != 0u)) {
+                    for (unsigned bal = MODE == SIM_SMALL ? (choose ? ba : bc) & holders : __ballot_sync(FULL, q != 0u); bal;
+                         bal = __ballot_sync(FULL, q != 0u)) {
                         const int n = __popc(bal);
                         if (nm + n > lineCap) { err = RR_ERR_INTERNAL; break; }
                         const bool c = q != 0u;
@@ -1681,8 +1680,11 @@ __device__ __forceinline__ int Sim<MODE>::run(rr_instance *I, JobWS &ws, int32_t
                 changed = false;
                 idTop -= (unsigned)nm;
                 list = idTop;
-                for (int u0 = 0; u0 < nm; u0 += 32)
-                    if (u0 + lane < nm) log[list + u0 + lane] = mie[u0 + lane].x;
+                // (lanes beyond the members read room that nothing uses)
+                const int id = mie[lane].x;
+                if (lane < nm) log[list + lane] = id;
+                if (nm > 32)
+                    for (int u = 32 + lane; u < nm; u += 32) log[list + u] = mie[u].x;
             }
             if (lane == 0) hdr[nseg] = make_uint4((unsigned)clk, nmem, list, (unsigned)L | (unsigned)d << 30);
             ++nseg;
@@ -1731,6 +1733,7 @@ __device__ __forceinline__ int Sim<MODE>::run(rr_instance *I, JobWS &ws, int32_t
                 const int2 ie = mie[act ? u : u0];
                 const uint32_t p = mpos[act ? u : u0];
                 const bool ended = act && ie.y == clk, keep = act && ie.y != clk;
+                int4 r = ldg_if(ended, rec + 2 * (size_t)ie.x), s = ldg_if(ended, rec + 2 * (size_t)ie.x + 1);
                 const unsigned kb = __ballot_sync(FULL, keep);
                 me = keep ? min(me, ie.y) : me;
                 const int w = nk + __popc(kb & lt);
@@ -1738,8 +1741,7 @@ __device__ __forceinline__ int Sim<MODE>::run(rr_instance *I, JobWS &ws, int32_t
                     __syncwarp();
                     st_if(keep, mie + w, ie.x, ie.y);
                     st_if(keep, mpos + w, p);
-                    if (__any_sync(FULL, ended)) {
-                        int4 r = ldg_if(ended, rec + 2 * (size_t)ie.x), s = ldg_if(ended, rec + 2 * (size_t)ie.x + 1);
+                    if (nm <= 32 || __any_sync(FULL, ended)) {
                         if (dm >= 2) {
                             const int dst = r.y >> 13 & 1023;
                             const bool turn = ended && dst != (int)(p >> 16) - 1;
@@ -1824,7 +1826,7 @@ __device__ __forceinline__ int sim_run(Sim<MODE> &S, rr_instance *I, JobWS &ws, 
     const SimLayout Y(smem, side);
     S.mie = Y.mie; S.mpos = Y.mpos; S.C = Y.C;
     S.rec = as_global(ws.rec); S.succ = as_global(ws.succ); S.multi = as_global(ws.multi);
-    S.multiId = as_global(ws.multiId); S.multiPos = as_global(ws.multiPos);
+    S.multiMove = as_global(ws.multiMove);
     S.cnt = Y.cnt;
     S.dump = sh_addr(Y.dump);
     S.ncnt = min(counters, ws.nmulti);
@@ -1911,7 +1913,7 @@ __device__ __forceinline__ void sim_block(rr_instance *I, JobWS &ws, char *smem,
                     st[C->wbase[d] + i] = C->wcap[d] - 1 - i;
                 }
             // the first pass counted in-degrees down: start over
-            for (int x = threadIdx.x; x < ws.nmulti; x += blockDim.x) ws.multi[x] = (ws.multi[x] & ~MULTI_COUNT) | ws.indeg[ws.multiId[x]];
+            for (int x = threadIdx.x; x < ws.nmulti; x += blockDim.x) ws.multi[x] = (ws.multi[x] & ~MULTI_COUNT) | ws.indeg[ws.multiMove[x].x];
         }
         __syncthreads();
         unsigned short *c16 = (unsigned short *)Y.cnt;

@@ -108,8 +108,8 @@ struct JobWS {
     void *slotOvf;         // the wide simulation's tables
     // the moves with several predecessors, by number: in-degree and first leg
     // (MULTI_BITS), id, position word
-    int32_t *multi, *multiId;
-    uint32_t *multiPos;
+    int32_t *multi;
+    int2 *multiMove;
     int32_t *multiNo;      // k: a move's number among them
     int32_t nmulti;        // how many there are
     int32_t nseg;          // logged segments that are still to be written

@@ -588,173 +588,214 @@ __device__ inline void s_emit_cols(const Blk B, rr_instance *inst, JobWS *wsv, i
 // A receiver's h sources, 32 at a time, a source per lane. A warp takes a
 // whole receiver, or where there are enough warps (single grids) 32 of its
 // sources. The receiver's contributors (the donors of its pairing events) are
-// read side by side, one per lane, into the warp's part of shared memory; each
-// lane then ranks its own source among all contributors by popcounts. What
-// bounds it is the chain of dependent loads before the first rank (receiver,
-// column, events, donors: about 4 000 cycles), so a warp goes through it once
-// per receiver. (A block of 256 threads per receiver, whose first thread
-// walked the events as a linked list while the others waited, and binary
-// searches over the donors' rows: 870 us for 2 000 grids of sides 33 to 251;
-// this: 375 us.)
+// read side by side, one per lane; each one's sources become a bit column in
+// the warp's part of shared memory (consecutive atoms: the donor's bit column
+// between two rows), a lane per word, so that a source's rank takes one load
+// and one popcount per contributor. What bounds it is the chain of dependent
+// loads before the first rank (receiver, column, events, donors, their rows),
+// which a warp goes through once per receiver. 2 000 grids of sides 33 to 251:
+// 870 us by a block per receiver with binary searches over the donors' rows,
+// 379 with ranks by popcounts over whole bit columns in global memory, 270
+// this way.
 struct Contrib {
-    int32_t col, kind, tbase, bbase;
-    int32_t tStart, tCnt, bStart, bCnt;
+    int32_t col, full;           // donor; an outer column whose reservoir rows are all filled
+    int32_t cnt, tCnt, tAt, bAt; // sources, of these above the band, the nearest ones' atom (row, if full)
     int32_t d, right, first;     // distance, right-side donor, first source index
 };
 
-// Top-region order at equal rows: farther column first, right before left.
-__device__ __forceinline__ bool top_before(int da, int ra, int db, int rb) { return da > db || (da == db && ra && !rb); }
-// Bottom-region order at equal rows: nearer column first, left before right.
-__device__ __forceinline__ bool bot_before(int da, int ra, int db, int rb) { return da < db || (da == db && !ra && rb); }
-
 constexpr int EMIT_WARPS = 8;    // at most, per block
+constexpr int EMIT_GROUP = 16;   // contributors held in shared memory at a time
 
-// Atoms of a bit column in rows below `row`; *here: whether row holds one.
-__device__ __forceinline__ int col_rank(const uint32_t *col, int row, bool *here)
+// A warp's view of a receiver unit: contributors and the bit columns (32
+// words) of their sources, the receiver's own bit column, and the number of
+// sources in the words before.
+struct EmitUnit {
+    const rr_instance *I;
+    const JobWS *ws;
+    Contrib *C;
+    uint32_t *X, *own, *before;
+    RecvInfo ri;
+    int K;                       // own atoms
+    long long out;               // first move
+};
+
+// Contributors g0 .. g0 + EMIT_GROUP - 1 of a unit, the first one's first
+// source being number *first (moved on); returns their sources in this lane's
+// word.
+__device__ __forceinline__ int emit_load(const EmitUnit &U, int g0, int *first)
 {
-    const int w = row >> 5;
-    int r = 0;
-    const uint32_t x = col[w], bit = 1u << (row & 31);
-    for (int u0 = 0; u0 < w; u0 += 8) {            // eight loads in flight at once
-        uint32_t y[8];
-#pragma unroll
-        for (int u = 0; u < 8; ++u) y[u] = u0 + u < w ? col[u0 + u] : 0u;
-#pragma unroll
-        for (int u = 0; u < 8; ++u) r += __popc(y[u]);
+    const int lane = threadIdx.x & 31, m = U.I->m, r0 = U.I->rect.r0, r1 = U.I->rect.r1, j = U.ri.j;
+    const JobWS &ws = *U.ws;
+    __syncwarp();
+    const bool act = lane < EMIT_GROUP && g0 + lane < U.ri.ncontrib;
+    Contrib c;
+    c.col = c.full = 0;
+    int cnt = 0, tLo = 0, tHi = 0, bLo = 0, bHi = 0;
+    if (act) {
+        const Event ev = ws.ev[ws.ev[U.ri.ev_first + g0 + lane].at];
+        const ColInfo D = ws.col[ev.i];
+        const int16_t *drows = ws.atomRows + (size_t)ev.i * m;
+        const int tStart = ev.t0, bStart = ev.b0;
+        c.tCnt = ev.kase == 3 ? D.ptop - ev.t0 : ev.a;
+        cnt = c.tCnt + (ev.kase == 3 ? D.pbot - ev.b0 : ev.x - ev.a);
+        c.full = D.kind == KIND_OUTER_FULL;
+        c.col = ev.i;
+        c.tAt = c.full ? r0 - 1 - tStart : D.tbase - tStart;
+        c.bAt = c.full ? r1 + bStart : D.bbase + bStart;
+        c.d = iabs(ev.i - j); c.right = ev.i > j;
+        // its sources on a side are consecutive atoms of its column
+        // (consecutive rows in a filled outer column): the rows they span
+        auto row_of = [&](int at) { return c.full ? at : (int)drows[at]; };
+        if (c.tCnt > 0) { tLo = row_of(c.tAt - c.tCnt + 1); tHi = row_of(c.tAt) + 1; }
+        if (cnt > c.tCnt) { bLo = row_of(c.bAt); bHi = row_of(c.bAt + cnt - c.tCnt - 1) + 1; }
+        c.cnt = cnt;
     }
-    *here = (x & bit) != 0u;
-    return r + __popc(x & (bit - 1u));
+    const int incl = warp_incl_scan(cnt);
+    c.first = *first + incl - cnt;
+    if (act) U.C[lane] = c;
+    *first += __shfl_sync(FULL, incl, 31);
+    int held = 0;
+    const int some = min(EMIT_GROUP, U.ri.ncontrib - g0), W = (m + 31) >> 5;
+    for (int v = 0; v < some; ++v) {
+        const int tl = __shfl_sync(FULL, tLo, v), th = __shfl_sync(FULL, tHi, v);
+        const int bl = __shfl_sync(FULL, bLo, v), bh = __shfl_sync(FULL, bHi, v);
+        const int col = __shfl_sync(FULL, c.col, v), full = __shfl_sync(FULL, c.full, v);
+        uint32_t x = row_mask(lane, tl, th) | row_mask(lane, bl, bh);
+        if (!full && lane < W) x &= ws.colbits[(size_t)col * W + lane];
+        U.X[v * 32 + lane] = x;
+        held += __popc(x);
+    }
+    __syncwarp();
+    return held;
+}
+
+// In a row above the band the farther column comes first, right before left,
+// the receiver's own (distance 0) last; below it the own, then the nearer
+// column, left before right. Whether column a comes before column b.
+__device__ __forceinline__ bool emit_before(bool top, int da, int ra, int db, int rb)
+{
+    return top ? da > db || (da == db && ra && !rb) : da < db || (da == db && !ra && rb);
+}
+
+// The move of the source of rank k.
+__device__ __forceinline__ int emit_store(const EmitUnit &U, rr_instance *I, int k, int row, int col)
+{
+    const int h = I->rect.r1 - I->rect.r0, r0 = I->rect.r0;
+    const int pos = k < U.ri.kd_end ? U.ri.kd_end - 1 - k : U.ri.kd_end + (k - U.ri.ku_start);
+    if (k < 0 || k >= h || pos >= U.ri.nmoves) {
+        set_status(I, RR_ERR_INTERNAL);
+        return 0;
+    }
+    if (pos < U.ri.kd_end && k >= U.ri.kd_end) return 0;             // isolated own band atom
+    store_move(&I->moves[U.out + pos], row, col, r0 + k, U.ri.j);
+    return iabs(r0 + k - row) + iabs(U.ri.j - col);
+}
+
+// A unit of more contributors than shared memory holds: its sources 32 at a
+// time, whichever contributors they come from, all contributors read in turn
+// for each 32. part of parts: the 32s that this warp takes.
+static __device__ __noinline__ int emit_many(const EmitUnit U, rr_instance *I, int part, int parts)
+{
+    const int lane = threadIdx.x & 31, h = I->rect.r1 - I->rect.r0, r0 = I->rect.r0, nc = U.ri.ncontrib;
+    const int16_t *atomRows = U.ws->atomRows;
+    int steps = 0;
+    for (int t0 = 32 * part; t0 < h; t0 += 32 * parts) {
+        const int t = t0 + lane;
+        int row = t < U.K && t < h ? atomRows[(size_t)U.ri.j * I->m + t] : 0, col = U.ri.j, ci = -1, sd = 0, sr = 0;
+        for (int g0 = 0, first = U.K; g0 < nc; g0 += EMIT_GROUP) {
+            const int before = first;
+            emit_load(U, g0, &first);
+            if (t >= before && t < first) {
+                int lo = 0, hi = min(EMIT_GROUP, nc - g0) - 1;       // contributor holding source t
+                while (lo < hi) { const int mid = (lo + hi + 1) >> 1; if (U.C[mid].first <= t) lo = mid; else hi = mid - 1; }
+                const Contrib c = U.C[lo];
+                const int u = t - c.first, at = u < c.tCnt ? c.tAt - u : c.bAt + (u - c.tCnt);
+                ci = g0 + lo; sd = c.d; sr = c.right; col = c.col;
+                row = c.full ? at : atomRows[(size_t)col * I->m + at];
+            }
+        }
+        const int w = row >> 5;
+        const uint32_t bit = 1u << (row & 31);
+        const bool top = row < r0;
+        int k = (int)U.before[w] + __popc(U.own[w] & (bit - 1u));
+        if (ci >= 0 && !top && (U.own[w] & bit)) ++k;
+        for (int g0 = 0, first = U.K; g0 < nc; g0 += EMIT_GROUP) {
+            emit_load(U, g0, &first);
+            for (int v = 0; v < min(EMIT_GROUP, nc - g0); ++v) {
+                const uint32_t x = U.X[v * 32 + w];
+                k += __popc(x & (bit - 1u));
+                if ((x & bit) && g0 + v != ci) k += emit_before(top, U.C[v].d, U.C[v].right, sd, sr);
+            }
+        }
+        if (t < h) steps += emit_store(U, I, k, row, col);
+    }
+    return steps;
 }
 
 __device__ inline void s_emit_recv(const Blk B, rr_instance *inst, JobWS *wsv, int count)
 {
-    __shared__ Contrib Call[EMIT_WARPS][32];
+    __shared__ Contrib Call[EMIT_WARPS][EMIT_GROUP];
+    __shared__ uint32_t Xall[EMIT_WARPS][(EMIT_GROUP + 2) * 32];
     const int q = B.y;
     if (q >= count) return;
     rr_instance *I = &inst[q];
     if (!live(I)) return;
     JobWS &ws = wsv[q];
-    Contrib *C = Call[threadIdx.x >> 5];
-    const int lane = threadIdx.x & 31;
-    const int m = I->m, n = I->n;
-    const int r0 = I->rect.r0, r1 = I->rect.r1, h = r1 - r0;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int m = I->m, n = I->n, r0 = I->rect.r0, h = I->rect.r1 - r0;
     const int W = (m + 31) >> 5, chunks = (h + 31) >> 5;
     const int split = B.nw >= ws.nrecv * chunks ? chunks : 1, items = ws.nrecv * split;
+    EmitUnit U;
+    U.I = I; U.ws = &ws; U.C = Call[wid]; U.X = Xall[wid]; U.own = U.X + EMIT_GROUP * 32; U.before = U.own + 32;
     long long steps = 0;
     for (int it = B.w; it < items; it += B.nw) {
-        const int r = it / split;
-        const RecvInfo ri = ws.recv[r];
-        const int j = ri.j, nc = ri.ncontrib;
-        const ColInfo Rj = ws.col[j];
+        const int r = it / split, part = it - r * split;
+        U.ri = ws.recv[r];
+        const int j = U.ri.j, nc = U.ri.ncontrib;
+        const uint32_t mine = lane < W ? ws.colbits[(size_t)j * W + lane] : 0u;
+        U.K = ws.col[j].K;
+        U.out = ws.unitOff[n + r];
+        int first = U.K, held = __popc(mine);
+        __syncwarp();
+        U.own[lane] = mine;
+        for (int g0 = 0; g0 < nc; g0 += EMIT_GROUP) held += emit_load(U, g0, &first);
+        U.before[lane] = (uint32_t)(warp_incl_scan(held) - held);
+        __syncwarp();
+        if (first != h) {
+            if (lane == 0) set_status(I, RR_ERR_INTERNAL);
+            continue;
+        }
+        if (nc > EMIT_GROUP) {
+            steps += emit_many(U, I, part, split);
+            continue;
+        }
+        // the own atoms: a source's rank is the number of sources in rows
+        // below it and, in its own row, of those that come first
         const int16_t *own = ws.atomRows + (size_t)j * m;
-        const int ownTop = Rj.ntop, ownBand = Rj.nband;
-        const long long out = ws.unitOff[n + r];
-        int first = Rj.K;
-        auto load = [&](int g0) {
-            __syncwarp();
-            Contrib c;
-            int cnt = 0;
-            if (g0 + lane < nc) {
-                const Event ev = ws.ev[ws.ev[ri.ev_first + g0 + lane].at];
-                const ColInfo D = ws.col[ev.i];
-                c.col = ev.i; c.kind = D.kind; c.tbase = D.tbase; c.bbase = D.bbase;
-                c.tStart = ev.t0; c.bStart = ev.b0;
-                if (ev.kase == 3) { c.tCnt = D.ptop - ev.t0; c.bCnt = D.pbot - ev.b0; }
-                else { c.tCnt = ev.a; c.bCnt = ev.x - ev.a; }
-                c.d = iabs(ev.i - j); c.right = ev.i > j;
-                cnt = c.tCnt + c.bCnt;
-            }
-            const int incl = warp_incl_scan(cnt);
-            if (g0 + lane < nc) { c.first = first + incl - cnt; C[lane] = c; }
-            first += __shfl_sync(FULL, incl, 31);
-            __syncwarp();
-        };
-        if (nc <= 32) load(0);                    // (more are loaded where they are read)
-        for (int t0 = (it - r * split) * 32; t0 < h; t0 += 32 * split) {
-            const int t = t0 + lane;
-            int row = t < Rj.K && t < h ? own[t] : 0, col = j, ci = -1, sd = 0, sr = 0, u = 0, stc = 0;
-            // which source this lane has
-            int before = Rj.K;
-            if (nc > 32) first = Rj.K;
-            for (int g0 = 0; g0 < nc; g0 += 32) {
-                if (nc > 32) { before = first; load(g0); }
-                if (t >= before && t < first) {
-                    int lo = 0, hi = min(32, nc - g0) - 1;   // contributor holding source t
-                    while (lo < hi) { const int mid = (lo + hi + 1) >> 1; if (C[mid].first <= t) lo = mid; else hi = mid - 1; }
-                    const Contrib c = C[lo];
-                    ci = g0 + lo;
-                    u = t - c.first;
-                    sd = c.d; sr = c.right; stc = c.tCnt; col = c.col;
-                    const int16_t *drows = ws.atomRows + (size_t)c.col * m;
-                    if (u < c.tCnt) {
-                        const int l = c.tStart + u;
-                        row = c.kind == KIND_OUTER_FULL ? r0 - 1 - l : drows[c.tbase - l];
-                    } else {
-                        const int l = c.bStart + (u - c.tCnt);
-                        row = c.kind == KIND_OUTER_FULL ? r1 + l : drows[c.bbase + l];
-                    }
+        for (int t = 32 * part + lane; t < U.K; t += 32 * split) {
+            const int row = own[t], w = row >> 5;
+            const uint32_t bit = 1u << (row & 31), upto = row < r0 ? bit | (bit - 1u) : bit - 1u;
+            int k = (int)U.before[w] + __popc(U.own[w] & (bit - 1u));
+            for (int v = 0; v < nc; ++v) k += __popc(U.X[v * 32 + w] & upto);
+            steps += emit_store(U, I, k, row, j);
+        }
+        // each contributor's
+        for (int c = part; c < nc; c += split) {
+            const Contrib D = U.C[c];
+            const int16_t *rows = ws.atomRows + (size_t)D.col * m;
+            for (int u = lane; u < D.cnt; u += 32) {
+                const int at = u < D.tCnt ? D.tAt - u : D.bAt + (u - D.tCnt);
+                const int row = D.full ? at : rows[at], w = row >> 5;
+                const bool top = row < r0;
+                const uint32_t bit = 1u << (row & 31);
+                int k = (int)U.before[w] + __popc(U.own[w] & (top ? bit - 1u : bit | (bit - 1u)));
+                for (int v = 0; v < nc; ++v) {
+                    const uint32_t x = U.X[v * 32 + w];
+                    k += __popc(x & (bit - 1u));
+                    if ((x & bit) && v != c) k += emit_before(top, U.C[v].d, U.C[v].right, D.d, D.right);
                 }
+                steps += emit_store(U, I, k, row, D.col);
             }
-            if (first != h) {
-                if (lane == 0) set_status(I, RR_ERR_INTERNAL);
-                break;
-            }
-            // its rank among the sources of its region
-            const bool in = t < h, band = row >= r0 && row < r1, top = row < r0;
-            int below = 0, tie = 0;
-            if (in && !band) {
-                if (ci < 0) {
-                    // own atom: own rows of its region before it are the ones before it in index
-                    below = top ? t : t - ownTop - ownBand;
-                } else {
-                    bool here;
-                    const int rk = col_rank(ws.colbits + (size_t)j * W, row, &here);
-                    below = top ? rk : rk - ownTop - ownBand;
-                    // the own atom (distance 0) comes first below the band, last above it
-                    tie += !top && here;
-                    // this contributor's other sources on the same side: nearest-first
-                    // order is descending rows above the band, ascending below it
-                    below += top ? stc - 1 - u : u - stc;
-                }
-            }
-            if (nc > 32) first = Rj.K;
-            for (int g0 = 0; g0 < nc; g0 += 32) {
-                if (nc > 32) load(g0);
-                if (!in || band) continue;
-                for (int v = 0; v < min(32, nc - g0); ++v) {
-                    if (g0 + v == ci) continue;
-                    const Contrib c = C[v];
-                    // its sources on this side are consecutive atoms of its column
-                    // (consecutive rows in a filled outer column): how many lie in
-                    // rows below, and whether one is in this row
-                    int lowest, cnt, rk;                 // first of them, how many; atoms in rows below
-                    bool here;
-                    if (c.kind == KIND_OUTER_FULL) {
-                        lowest = top ? r0 - c.tStart - c.tCnt : r1 + c.bStart;
-                        cnt = top ? c.tCnt : c.bCnt;
-                        rk = row;
-                        here = true;
-                    } else {
-                        lowest = top ? c.tbase - c.tStart - c.tCnt + 1 : c.bbase + c.bStart;
-                        cnt = top ? c.tCnt : c.bCnt;
-                        rk = col_rank(ws.colbits + (size_t)c.col * W, row, &here);
-                    }
-                    below += min(max(rk - lowest, 0), cnt);
-                    if (here && rk >= lowest && rk < lowest + cnt &&
-                        (top ? top_before(c.d, c.right, sd, sr) : bot_before(c.d, c.right, sd, sr))) ++tie;
-                }
-            }
-            if (!in) continue;
-            // (only own atoms sit in the band)
-            const int k = band ? ri.nT + (t - ownTop) : top ? below + tie : ri.nT + ownBand + below + tie;
-            if (k < 0 || k >= h) { set_status(I, RR_ERR_INTERNAL); continue; }
-            int pos;
-            if (k < ri.kd_end) pos = ri.kd_end - 1 - k;
-            else if (k >= ri.ku_start) pos = ri.kd_end + (k - ri.ku_start);
-            else continue;                                 // isolated own band atom
-            if (pos >= ri.nmoves) { set_status(I, RR_ERR_INTERNAL); continue; }
-            store_move(&I->moves[out + pos], row, col, r0 + k, j);
-            steps += iabs(r0 + k - row) + iabs(j - col);
         }
     }
     add_steps(I, steps);

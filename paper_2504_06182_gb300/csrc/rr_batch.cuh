@@ -1080,6 +1080,16 @@ __device__ __forceinline__ void touch_rec_if(bool c, const int4 *rec, int id, ui
 __device__ __forceinline__ uint32_t uni(uint32_t v) { return __reduce_max_sync(FULL, v); }
 
 
+// A segment written by the simulating warp itself, once the log is full, out of
+// line: the loop around it stays smaller (389 x 501 39.6 -> 38.0 ms; where
+// registers are scarcest, in the small tables' kernel, inlining is better: 4096
+// mixed grids 31 ms, 33 this way).
+static __device__ __noinline__ void write_call(rr_instance *I, unsigned op0, unsigned mem0, int kseg, int ns, int d, int L,
+                                               const int32_t *list, int32_t *buf)
+{
+    write_segment(as_global(I->ops), as_global(I->members), OpLane(lane_id()), op0, mem0, kseg, ns, d, L, list, buf);
+}
+
 constexpr int RUN = 32;     // leaders of a run at most: one per lane
 
 // Segments that the log has room for: a header each, one after them, a list
@@ -1693,8 +1703,10 @@ __device__ __forceinline__ int Sim<MODE>::run(rr_instance *I, JobWS &ws, int32_t
             if (o1 <= (unsigned long long)I->cap_ops && m1 <= (unsigned long long)I->cap_members) {
                 for (int u = lane; u < nm; u += 32) ids[u] = mie[u].x;
                 __syncwarp();
-                write_segment(as_global(I->ops), as_global(I->members), OpLane(lane), (unsigned)clk, nmem, kseg, nm + 1, d, L,
-                              ids, buf);
+                if constexpr (MODE == SIM_SMALL)
+                    write_segment(as_global(I->ops), as_global(I->members), OpLane(lane), (unsigned)clk, nmem, kseg, nm + 1, d, L,
+                                  ids, buf);
+                else write_call(I, (unsigned)clk, nmem, kseg, nm + 1, d, L, ids, buf);
             }
         }
         // everything in the batch advances

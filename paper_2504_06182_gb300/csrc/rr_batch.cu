@@ -57,6 +57,11 @@ __global__ void k_bsucc(rr_instance *inst, JobWS *wsv, int count)
     s_bsucc(hw_blk(), inst, wsv, count);
 }
 
+__global__ void k_bnum(rr_instance *inst, JobWS *wsv, int count)
+{
+    s_bnum(hw_blk(), inst, wsv, count);
+}
+
 __global__ void k_brec(rr_instance *inst, JobWS *wsv, int count)
 {
     s_brec(hw_blk(), inst, wsv, count);

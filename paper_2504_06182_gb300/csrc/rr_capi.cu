@@ -26,6 +26,7 @@ __global__ void k_gsort(rr_instance *, JobWS *, int, int);
 __global__ void k_gsweep_h(rr_instance *, JobWS *, int, int);
 __global__ void k_gsweep_v(rr_instance *, JobWS *, int, int);
 __global__ void k_bsucc(rr_instance *, JobWS *, int);
+__global__ void k_bnum(rr_instance *, JobWS *, int);
 __global__ void k_brec(rr_instance *, JobWS *, int);
 __global__ void k_classify(rr_instance *, int, int, int, int *, int *);
 __global__ void k_order(const rr_instance *, int, int *);
@@ -439,6 +440,8 @@ static int launch_batch(rr_ctx *ctx, rr_instance *d_inst, JobWS *ws, int count, 
     }
     mark(ctx, s, "k_bsucc");
     k_bsucc<<<dim3(pathBlocks, count), 256, 0, s>>>(d_inst, ws, count);
+    mark(ctx, s, "k_bnum");
+    k_bnum<<<dim3(pathBlocks, count), 256, 0, s>>>(d_inst, ws, count);
     mark(ctx, s, "k_brec");
     k_brec<<<dim3(pathBlocks, count), 256, 0, s>>>(d_inst, ws, count);
     // simulation: one block per instance, launched per size class on forked
@@ -480,7 +483,7 @@ static int launch_batch(rr_ctx *ctx, rr_instance *d_inst, JobWS *ws, int count, 
     }
     mark(ctx, s, nullptr);
     CUDA_TRY(cudaGetLastError());
-    ctx->nlaunch += (one ? 9 : 10) + nclass;
+    ctx->nlaunch += (one ? 10 : 11) + nclass;
     return RR_OK;
 }
 

@@ -67,6 +67,8 @@ __global__ void __launch_bounds__(ONE_THREADS, 1) k_one(rr_instance h, rr_instan
         __syncthreads();
         s_bsucc(B, I, ws, 1);
         __syncthreads();
+        s_bnum(B, I, ws, 1);
+        __syncthreads();
         s_brec(B, I, ws, 1);
         __syncthreads();
         sim_block<SIM_SMALL, true>(I, ws[0], (char *)one_smem, side, counters);

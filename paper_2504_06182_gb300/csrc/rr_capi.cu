@@ -14,6 +14,8 @@ __global__ void k_batch_begin(rr_instance, rr_instance *, Arena);
 __global__ void k_transpose(rr_instance *, JobWS *, int, int);
 __global__ void k_colstats(rr_instance *, JobWS *, int, int, int);
 __global__ void k_pair(rr_instance *, JobWS *, int, int);
+__global__ void k_pair_sift(rr_instance *, JobWS *, int);
+__global__ void k_pair_listed(rr_instance *, JobWS *, int);
 __global__ void k_emit_cols(rr_instance *, JobWS *, int, int);
 __global__ void k_emit_recv(rr_instance *, JobWS *, int, int);
 __global__ void k_bird(rr_instance *, JobWS *, int, int);
@@ -297,6 +299,8 @@ static Arena arena_of(rr_ctx *ctx)
     return A;
 }
 
+static constexpr size_t SM_SMEM = 228 * 1024;    // shared memory of an SM
+
 static int clampi(int v, int lo, int hi) { return v < lo ? lo : (v > hi ? hi : v); }
 
 // Blocks a launch may spread over all grids of a call (divided by the count).
@@ -358,7 +362,16 @@ static int launch_plan(rr_ctx *ctx, rr_instance *d_inst, JobWS *ws, int count, i
     }
     const size_t pairSmem = (size_t)max_side * PAIR_BYTES + 64;
     mark(ctx, s, "k_pair");
-    k_pair<<<count, 32, pairSmem, s>>>(d_inst, ws, count, count <= ctx->nsm ? 1 : 0);
+    const int fit = clampi((int)(SM_SMEM / (pairSmem + 1024)), 1, 32);         // blocks that an SM holds
+    if (count <= fit * ctx->nsm) {
+        k_pair<<<count, 32, pairSmem, s>>>(d_inst, ws, count, count <= ctx->nsm ? 1 : 0);
+    } else {
+        // more blocks than fit at once: only for the grids that need them
+        // (2 000 grids of up to 251 x 251, which all fit: 317 us, 336 this way)
+        k_pair_sift<<<(count + 7) / 8, 256, 0, s>>>(d_inst, ws, count);
+        k_pair_listed<<<fit * ctx->nsm, 32, pairSmem, s>>>(d_inst, ws, count);
+        ctx->nlaunch += 1;
+    }
     mark(ctx, s, "k_emit_cols");
     k_emit_cols<<<dim3(colBlocks, rows), 256, 0, s>>>(d_inst, ws, count, per);
     mark(ctx, s, "k_emit_recv");

@@ -92,6 +92,8 @@ struct JobWS {
     Event *ev;             // n + 1
     int32_t *unitOff;      // 2n + 1
     int32_t nrecv, nev;
+    int32_t npending, pending;   // calls over many grids: how many still need pairing (of the first
+                                 // instance), the i-th of them
     // batching (Gamma + simulation)
     int64_t P;             // total path vertices (sum of path length + 1)
     int32_t *pairOff;      // k + 1

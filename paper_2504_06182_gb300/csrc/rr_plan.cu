@@ -55,6 +55,22 @@ __global__ void k_pair(rr_instance *inst, JobWS *wsv, int count, int warm)
     s_pair(hw_blk(), inst, wsv, count, warm);
 }
 
+__global__ void k_pair_sift(rr_instance *inst, JobWS *wsv, int count)
+{
+    s_pair_sift(hw_blk(), inst, wsv, count);
+}
+
+__global__ void k_pair_listed(rr_instance *inst, JobWS *wsv, int count)
+{
+    const int n = wsv[0].npending;
+    Blk B = hw_blk();
+    for (int i = blockIdx.x; i < n; i += gridDim.x) {
+        B.x = wsv[i].pending;
+        s_pair(B, inst, wsv, count, 0);
+        __syncwarp();
+    }
+}
+
 __global__ void k_emit_cols(rr_instance *inst, JobWS *wsv, int count, int per)
 {
     s_emit_cols(hw_blk_shared(per), inst, wsv, count);

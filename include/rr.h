@@ -165,7 +165,8 @@ typedef struct {
 } rr_instance;
 
 /* With RR_BATCH_ONLY the planning kernels are skipped and each instance's
- * moves[0 .. n_moves) are batched as by rr_batch (status must be RR_OK).
+ * moves[0 .. n_moves) are batched as by rr_batch (status must be RR_OK); sizes
+ * or a list that rr_batch refuses give the instance RR_ERR_ARG.
  * count in [1, 65535]; max_side bounds m and n of every instance (an
  * instance above it gets RR_ERR_ARG); it sizes the launch shapes. The call
  * may grow the context's descriptor table (a synchronous cudaMalloc), so the

@@ -12,9 +12,9 @@ __global__ void k_batch_begin(rr_instance h, rr_instance *I, Arena A)
     if (threadIdx.x == 0) { *I = h; *A.top = 0; }
 }
 
-__global__ void k_bsetup(rr_instance *inst, JobWS *wsv, int count, Arena A, int lookback)
+__global__ void k_bsetup(rr_instance *inst, JobWS *wsv, int count, int max_side, Arena A, int lookback)
 {
-    s_bsetup(hw_blk(), inst, wsv, count, A, lookback);
+    s_bsetup(hw_blk(), inst, wsv, count, max_side, A, lookback);
 }
 
 __global__ void __launch_bounds__(LB_THREADS) k_pairoff_lookback(rr_instance *inst, JobWS *wsv, int count, Arena A)

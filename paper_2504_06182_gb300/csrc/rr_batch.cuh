@@ -53,7 +53,10 @@ __device__ inline long long block_exclusive_scan(int32_t *v, int len, long long 
 
 // ----------------------------------------------------------- set-up pass
 // One block per instance: check the moves, count path vertices, allocate.
-__device__ inline void s_bsetup(const Blk B, rr_instance *inst, JobWS *wsv, int count, Arena A, int lookback)
+// An instance whose sizes the launch's shared memory does not cover (or that
+// carries no list) ends here: with RR_BATCH_ONLY no planning kernel has looked
+// at it, and every later stage indexes by its m, n and n_moves.
+__device__ inline void s_bsetup(const Blk B, rr_instance *inst, JobWS *wsv, int count, int max_side, Arena A, int lookback)
 {
     __shared__ long long s_tmp[34];
     __shared__ int s_bad;
@@ -64,6 +67,11 @@ __device__ inline void s_bsetup(const Blk B, rr_instance *inst, JobWS *wsv, int 
     JobWS &ws = wsv[q];
     const int m = I->m, n = I->n;
     const int64_t k = I->n_moves;
+    if (m < 1 || n < 1 || m > max_side || n > max_side || k < 0 || k > 0x3fffffff || (k > 0 && !I->moves)) {
+        __syncthreads();                    // (every thread has read the status)
+        if (threadIdx.x == 0) I->status = RR_ERR_ARG;
+        return;
+    }
     if (lookback && k >= LB_MIN_MOVES) {
         // a large move list: checking the moves, counting their vertices and
         // the offsets are the work of the multi-block k_pairoff_lookback,
@@ -71,9 +79,8 @@ __device__ inline void s_bsetup(const Blk B, rr_instance *inst, JobWS *wsv, int 
         // known; here only the move-sized arrays
         __shared__ int s_ok;
         if (threadIdx.x == 0) {
-            bool ok = k <= 0x3fffffff;
+            bool ok = true;
             const unsigned long long cells = (unsigned long long)m * n;
-            if (!ok) I->status = RR_ERR_ARG;
             ws.P = -1;
             ws.pairOff = (int32_t *)arena_alloc(A, 4ull * (k + 1), &ok);
             ws.colOff = (int32_t *)arena_alloc(A, 4ull * (n + 1), &ok);
@@ -96,7 +103,7 @@ __device__ inline void s_bsetup(const Blk B, rr_instance *inst, JobWS *wsv, int 
             ws.succ = nullptr;
             ws.lbStatus = (unsigned long long *)arena_alloc(A, 8ull * ((k + LB_TILE - 1) / LB_TILE), &ok);
             ws.lbCounter = (int32_t *)arena_alloc(A, 4, &ok);
-            if (!ok && live(I)) I->status = RR_ERR_WORKSPACE;
+            if (!ok) I->status = RR_ERR_WORKSPACE;
             s_ok = live(I);
         }
         __syncthreads();
@@ -130,7 +137,7 @@ __device__ inline void s_bsetup(const Blk B, rr_instance *inst, JobWS *wsv, int 
         I->n_steps = ts;
         I->n_members = ts;
         if (s_bad) { I->status = RR_ERR_ARG; }
-        else if (k > 0x3fffffff || tp > 0x7fffffffLL) { I->status = RR_ERR_ARG; }
+        else if (tp > 0x7fffffffLL) { I->status = RR_ERR_ARG; }
         else if (ts > I->cap_members || (ts > 0 && (!I->members || !I->ops))) {
             I->status = RR_ERR_CAPACITY;
             I->n_ops = ts;                      // upper bound

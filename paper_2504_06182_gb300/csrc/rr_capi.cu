@@ -19,7 +19,7 @@ __global__ void k_pair_listed(rr_instance *, JobWS *, int);
 __global__ void k_emit_cols(rr_instance *, JobWS *, int, int);
 __global__ void k_emit_recv(rr_instance *, JobWS *, int, int);
 __global__ void k_bird(rr_instance *, JobWS *, int, int);
-__global__ void k_bsetup(rr_instance *, JobWS *, int, Arena, int);
+__global__ void k_bsetup(rr_instance *, JobWS *, int, int, Arena, int);
 __global__ void k_pairoff_lookback(rr_instance *, JobWS *, int, Arena);
 __global__ void k_gcount(rr_instance *, JobWS *, int);
 __global__ void k_gscan(rr_instance *, JobWS *, int);
@@ -423,7 +423,7 @@ static int launch_batch(rr_ctx *ctx, rr_instance *d_inst, JobWS *ws, int count, 
     // path-vertex offsets from the multi-block look-back scan
     const int lookback = max_side > 256 ? 1 : 0;
     mark(ctx, s, "k_bsetup");
-    k_bsetup<<<count, 512, 0, s>>>(d_inst, ws, count, A, lookback);
+    k_bsetup<<<count, 512, 0, s>>>(d_inst, ws, count, max_side, A, lookback);
     if (lookback) {
         mark(ctx, s, "k_pairoff_lookback");
         k_pairoff_lookback<<<dim3(clampi(2 * ctx->nsm / count, 1, 2 * ctx->nsm), count), LB_THREADS, 0, s>>>(

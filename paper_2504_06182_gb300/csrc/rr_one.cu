@@ -51,7 +51,7 @@ __global__ void __launch_bounds__(ONE_THREADS, 1) k_one(rr_instance h, rr_instan
     }
     __syncthreads();
     if (batch && I->status == RR_OK) {          // read after a barrier: the same in every thread
-        s_bsetup(B, I, ws, 1, A, 0);
+        s_bsetup(B, I, ws, 1, side, A, 0);
         __syncthreads();
         s_gcount(B, I, ws, 1);
         __syncthreads();

@@ -880,6 +880,9 @@ __device__ __forceinline__ void write_ops(int32_t *o, const OpLane &P, int lane,
     }
 }
 
+// The room that a capacity gives: none if it is negative.
+__device__ __forceinline__ unsigned long long room_of(int64_t cap) { return cap > 0 ? (unsigned long long)cap : 0ull; }
+
 // A segment's kseg batches of ns moves at batch op0 and member mem0: the
 // leader L (the smallest id) and the ns - 1 moves of list[], in no order.
 // One warp; buf holds the next power of two of ns words. Batches are written
@@ -970,7 +973,7 @@ __device__ __forceinline__ void write_chunk(const int32_t *log, int s0, int cnt,
 __device__ inline void run_writers(SimCtl *C, rr_instance *I, const int32_t *log, int32_t *buf)
 {
     const int lane = threadIdx.x & 31;
-    const unsigned long long cap_ops = (unsigned long long)I->cap_ops, cap_mem = (unsigned long long)I->cap_members;
+    const unsigned long long cap_ops = room_of(I->cap_ops), cap_mem = room_of(I->cap_members);
     rr_op *ops = as_global(I->ops);
     int32_t *mem = as_global(I->members);
     volatile int *pub = &C->pub, *fin = &C->fin;
@@ -1006,7 +1009,7 @@ __device__ inline void s_write(const Blk B, rr_instance *I, const JobWS &ws, int
     rr_op *ops = as_global(I->ops);
     int32_t *mem = as_global(I->members);
     const int32_t *log = as_global(ws.nextAt);
-    const unsigned long long cap_ops = (unsigned long long)I->cap_ops, cap_mem = (unsigned long long)I->cap_members;
+    const unsigned long long cap_ops = room_of(I->cap_ops), cap_mem = room_of(I->cap_members);
     for (int s0 = 32 * B.w; s0 < ws.nseg; s0 += 32 * B.nw)
         write_chunk(log, s0, min(32, ws.nseg - s0), cap_ops, cap_mem, ops, mem, P, buf);
 }
@@ -1355,8 +1358,8 @@ static __device__ __noinline__ int run_of_leaders(rr_instance *I, JobWS *ws, cha
         for (int i = 0; i < n; ++i) {
             const int o = clk + __shfl_sync(FULL, before, i), m0 = (int)nmem + __shfl_sync(FULL, before, i);
             const int h1 = __shfl_sync(FULL, hl, i), v1 = __shfl_sync(FULL, vl, i), hd = __shfl_sync(FULL, d1, i);
-            if ((unsigned long long)(o + h1 + v1) > (unsigned long long)I->cap_ops ||
-                (unsigned long long)(m0 + h1 + v1) > (unsigned long long)I->cap_members) break;
+            if ((unsigned long long)(o + h1 + v1) > room_of(I->cap_ops) ||
+                (unsigned long long)(m0 + h1 + v1) > room_of(I->cap_members)) break;
             if (h1 > 0) write_segment(as_global(I->ops), as_global(I->members), OpLane(lane), (unsigned)o, (unsigned)m0, h1, 1, hd, L + i, ids, buf);
             write_segment(as_global(I->ops), as_global(I->members), OpLane(lane), (unsigned)(o + h1), (unsigned)(m0 + h1), v1, 1, rd, L + i, ids, buf);
         }
@@ -1757,7 +1760,7 @@ __device__ __forceinline__ int Sim<MODE>::run(rr_instance *I, JobWS &ws, int32_t
             ++nseg;
         } else {
             const unsigned long long o1 = (unsigned long long)clk + kseg, m1 = nmem + (unsigned long long)kseg * (nm + 1);
-            if (o1 <= (unsigned long long)I->cap_ops && m1 <= (unsigned long long)I->cap_members) {
+            if (o1 <= room_of(I->cap_ops) && m1 <= room_of(I->cap_members)) {
                 for (int u = lane; u < nm; u += 32) ids[u] = mie[u].x;
                 __syncwarp();
                 if constexpr (MODE == SIM_SMALL)

@@ -1,6 +1,8 @@
 """RR_BATCH_ONLY descriptors that no planning kernel has looked at: an instance
 whose sizes or list rr_batch would refuse ends with RR_ERR_ARG and touches
-nothing, and the instances beside it in the call are batched as ever."""
+nothing, and the instances beside it in the call are batched as ever; room for
+fewer batches than the list needs (or a negative number) ends with
+RR_ERR_CAPACITY and nothing is written beyond it."""
 import numpy as np
 import pytest
 
@@ -69,3 +71,29 @@ def test_refused_descriptors(planner, count, side):
         else:
             assert x.status == rr.RR_ERR_ARG
             assert bool((ops == -7).all()) and bool((mem == -7).all())
+
+
+@pytest.mark.parametrize("count", [2, 200])              # written beside the simulation, and after it
+@pytest.mark.parametrize("unit", [False, True])          # from the log, and directly once it is full
+@pytest.mark.parametrize("room", [-1, 0, 5])
+def test_room_for_batches(planner, count, unit, room):
+    import oracle
+    import paper_2504_06182_gb300 as rr
+    from paper_2504_06182_gb300.planner import unpack_instances
+    if unit:                                             # a token to and fro: a batch per move, twice the log's room
+        mv = np.array([(i % 2, 0, 1 - i % 2, 0) for i in range(4000)], np.int32)
+        rops, rmem = oracle.batch(mv, 2, 1)
+    else:
+        mv, rops, rmem = a_plan(40, 2)
+    dev = torch.from_numpy(mv).cuda()
+    bufs = [(torch.full((len(rops), 3), -7, dtype=torch.int32, device="cuda"),
+             torch.full((len(rmem),), -7, dtype=torch.int32, device="cuda")) for _ in range(count)]
+    inst = descriptors([(40, 40, dev, len(mv), o, len(o) if q % 2 else room, b, len(b)) for q, (o, b) in enumerate(bufs)])
+    assert rr.rr_plan_batched(planner.ctx, inst, count, 40, rr.RR_BATCH_ONLY) == rr.RR_OK
+    torch.cuda.synchronize()
+    for q, ((ops, mem), x) in enumerate(zip(bufs, unpack_instances(inst, count))):
+        if q % 2:
+            assert x.status == rr.RR_OK and np.array_equal(ops.cpu().numpy(), rops) and np.array_equal(mem.cpu().numpy(), rmem)
+        else:
+            assert x.status == rr.RR_ERR_CAPACITY and x.n_ops == len(rops) and x.n_members == len(rmem)
+            assert bool((ops[max(room, 0):] == -7).all())

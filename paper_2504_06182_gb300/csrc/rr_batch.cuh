@@ -938,7 +938,7 @@ __device__ inline void write_segment(rr_op *ops, int32_t *mem, const OpLane &P, 
     __syncwarp();
 }
 
-constexpr int SIM_POLLS = 1 << 22;      // a writer's polls without progress before it gives up
+constexpr int SIM_POLLS = 1 << 22;      // a writer's polls without progress of the log before it gives up
 
 // Header of a logged segment: its first batch and first member, where its
 // members' ids lie, and the leader (30 bits) with the direction. Lengths
@@ -969,7 +969,7 @@ __device__ __forceinline__ void write_chunk(const int32_t *log, int s0, int cnt,
 }
 
 // A warp of the simulation's block writes what is published of the log, 32
-// segments at a time, until the simulation has ended and nothing is left.
+// segments at a time, until the log has ended and nothing is left.
 __device__ inline void run_writers(SimCtl *C, rr_instance *I, const int32_t *log, int32_t *buf)
 {
     const int lane = threadIdx.x & 31;
@@ -1493,6 +1493,13 @@ __device__ __forceinline__ int Sim<MODE>::run(rr_instance *I, JobWS &ws, int32_t
     int left = min(32, log_room(0u, idTop, lineCap));
     bool logging = left > 0;
     if (!logging) left = 32;
+    // The log has ended and pub is final: the writers are done once they have
+    // written it, however long the simulation, writing by itself, still takes.
+    auto end_of_log = [&]() {
+        __threadfence_block();
+        if (lane == 0) *(volatile int *)&C->fin = 1;
+    };
+    if (!logging) end_of_log();
     long long guard = (g_guard_cap > 0 ? g_guard_cap : I->n_steps + 2ll * k + 16) + 1;
     if (guard < left) left = (int)guard;
     guard -= left;
@@ -1542,6 +1549,7 @@ __device__ __forceinline__ int Sim<MODE>::run(rr_instance *I, JobWS &ws, int32_t
             const int room = log_room(nseg, idTop, lineCap);
             logging = room > 0;
             if (logging) left = min(32, room);
+            else end_of_log();
         }
         if (guard < left) left = (int)guard;
         guard -= left;

@@ -144,7 +144,7 @@ struct SimCtl {
     int full;                 // a table was full
     int pub;                  // segments of the log that the writers may write
     int next;                 // first segment not yet taken by a writer (by 32)
-    int fin;                  // the simulation has ended: pub is final
+    int fin;                  // pub is final: the simulation, or its log, has ended
     int status;               // its end: RR_OK, RR_SIM_RETRY or an error
     int pad[3];
 };

@@ -10,7 +10,6 @@
 //
 // Alg. 4 itself runs as an event-driven simulation (below).
 #pragma once
-#include <type_traits>
 #include "rr_internal.cuh"
 
 namespace rrk {
@@ -95,7 +94,7 @@ __device__ inline void s_bsetup(const Blk B, rr_instance *inst, JobWS *wsv, int 
             ws.rec = (int4 *)arena_alloc(A, 32ull * (k + 1), &ok);
             ws.succ4 = ws.rec + 1;
             ws.ready0 = (int32_t *)arena_alloc(A, 4ull * (k + 1) + 16, &ok);
-            ws.slotOvf = arena_alloc(A, sim_wide_bytes(k), &ok);
+            ws.state = (int2 *)arena_alloc(A, sim_wide_bytes(k), &ok);
             ws.multi = ws.colList;               // both lists are free again once they have been swept
             ws.multiNo = ws.rowList;
             ws.nmulti = 0;
@@ -159,7 +158,7 @@ __device__ inline void s_bsetup(const Blk B, rr_instance *inst, JobWS *wsv, int 
             ws.rec = (int4 *)arena_alloc(A, 32ull * (k + 1), &ok);   // record, successors: one 32 B sector
             ws.succ4 = ws.rec + 1;
             ws.ready0 = (int32_t *)arena_alloc(A, 4ull * (k + 1) + 16, &ok);
-            ws.slotOvf = arena_alloc(A, sim_wide_bytes(k), &ok);
+            ws.state = (int2 *)arena_alloc(A, sim_wide_bytes(k), &ok);
             ws.multi = ws.colList;               // both lists are free again once they have been swept
             ws.multiNo = ws.rowList;
             ws.nmulti = 0;
@@ -1367,20 +1366,49 @@ static __device__ __noinline__ int run_of_leaders(rr_instance *I, JobWS *ws, cha
     return n | segs << 6 | steps << 13;
 }
 
+// The log has ended and pub is final: the writers are done once they have
+// written it, however long the simulation, writing by itself, still takes.
+__device__ __forceinline__ void end_of_log(SimCtl *C)
+{
+    __threadfence_block();
+    if (lane_id() == 0) *(volatile int *)&C->fin = 1;
+}
+// The end of a simulation: a header with the totals, everything published,
+// the instance's counts. Returns its status.
+__device__ __forceinline__ int sim_end(rr_instance *I, SimCtl *C, uint4 *hdr, unsigned nseg, bool logging, int clk,
+                                       unsigned nmem, int err)
+{
+    const int lane = lane_id();
+    touch_wait();
+    __syncwarp();
+    if (logging && lane == 0) hdr[nseg] = make_uint4((unsigned)clk, nmem, 0u, 0u);
+    if (lane == 0) {
+        I->n_ops = clk;
+        I->n_members = nmem;
+    }
+    if (*(volatile int *)&C->full) err = RR_SIM_RETRY;
+    if (!err && (long long)nmem != I->n_steps) err = RR_ERR_INTERNAL;
+    if (!err && ((int64_t)clk > I->cap_ops || (int64_t)nmem > I->cap_members)) err = RR_ERR_CAPACITY;
+    __syncwarp();
+    __threadfence_block();
+    if (lane == 0) *(volatile int *)&C->pub = (int)nseg;
+    end_of_log(C);
+    __syncwarp();
+    return err;
+}
+
 // One simulation by one warp. SIM_SMALL: tables in shared memory, at most 256
 // entries per direction (one load of every lane covers them); SIM_BIG: the
-// same with more entries; both end with RR_SIM_RETRY when an instance has
-// more ready moves of a direction than entries. SIM_WIDE: tables in global
-// memory, room for every move.
-enum { SIM_SMALL, SIM_BIG, SIM_WIDE };
+// same with more entries. Both end with RR_SIM_RETRY when an instance has
+// more ready moves of a direction than entries (WideSim, below).
+enum { SIM_SMALL, SIM_BIG };
 
 template <int MODE>
 struct Sim {
-    using ST = typename std::conditional<MODE == SIM_WIDE, int32_t, uint16_t>::type;
     uint32_t *pos;            // position words, a table of cap entries per direction
     int2 *ir;                 // id, steps left in the leg
-    ST *stk;                  // free entries (numbers within the table)
-    int cap;                  // (the wide tables have sizes of their own, C->wcap from C->wbase on)
+    uint16_t *stk;            // free entries (numbers within the table)
+    int cap;
     int2 *mie;                // members: id, clock at the end of the leg
     uint32_t *mpos;           // members: position word, `along` minus the clock
     SimCtl *C;
@@ -1395,27 +1423,16 @@ struct Sim {
     char *smem;               // the block's shared memory, its side and counters
     int side, counters;
 
-    __device__ __forceinline__ int base(int d) const { return MODE == SIM_WIDE ? C->wbase[d] : d * cap; }
-    __device__ __forceinline__ int size(int d) const { return MODE == SIM_WIDE ? C->wcap[d] : cap; }
-
     // The moves of the lanes with c become statics.
     __device__ __forceinline__ void enter(bool c, int d, uint32_t p, int id, int rem)
     {
-        if constexpr (MODE == SIM_WIDE) {
-            if (c) {
-                const int b = base(d), e = b + stk[b + atomicSub(&C->nfree[d], 1) - 1];
-                pos[e] = p;
-                ir[e] = make_int2(id, rem);
-            }
-        } else {
-            const int o = sh_add_if(c, &C->nfree[d], -1) - 1;
-            const bool none = c && o < 0, ok = c && o >= 0;
-            st_if(none, &C->full, 1u);             // no room: the run will end with RR_SIM_RETRY
-            sh_add_if(none, &C->nfree[d], 1);
-            const int e = d * cap + ld_u16_if(ok, stk + d * cap + o);
-            st_if(ok, pos + e, p);
-            st_if(ok, ir + e, id, rem);
-        }
+        const int o = sh_add_if(c, &C->nfree[d], -1) - 1;
+        const bool none = c && o < 0, ok = c && o >= 0;
+        st_if(none, &C->full, 1u);             // no room: the run will end with RR_SIM_RETRY
+        sh_add_if(none, &C->nfree[d], 1);
+        const int e = d * cap + ld_u16_if(ok, stk + d * cap + o);
+        st_if(ok, pos + e, p);
+        st_if(ok, ir + e, id, rem);
     }
 
     // A finished move of each lane with c hands one predecessor fewer to the
@@ -1493,13 +1510,7 @@ __device__ __forceinline__ int Sim<MODE>::run(rr_instance *I, JobWS &ws, int32_t
     int left = min(32, log_room(0u, idTop, lineCap));
     bool logging = left > 0;
     if (!logging) left = 32;
-    // The log has ended and pub is final: the writers are done once they have
-    // written it, however long the simulation, writing by itself, still takes.
-    auto end_of_log = [&]() {
-        __threadfence_block();
-        if (lane == 0) *(volatile int *)&C->fin = 1;
-    };
-    if (!logging) end_of_log();
+    if (!logging) end_of_log(C);
     long long guard = (g_guard_cap > 0 ? g_guard_cap : I->n_steps + 2ll * k + 16) + 1;
     if (guard < left) left = (int)guard;
     guard -= left;
@@ -1508,7 +1519,7 @@ __device__ __forceinline__ int Sim<MODE>::run(rr_instance *I, JobWS &ws, int32_t
     bool alone = false, tryRun = false;
     // this lane's eight entries of a table's first 256 (a lane beyond the
     // table reads the last eight too: that changes no minimum)
-    int groups = size(0) >> 3, off = 8 * min(lane, groups - 1);
+    const int groups = cap >> 3, off = 8 * min(lane, groups - 1);
     const unsigned holders = groups >= 32 ? FULL : (1u << groups) - 1u;      // (lanes of a SIM_SMALL table)
 
     auto set_leg = [&](uint32_t y) {
@@ -1535,7 +1546,7 @@ __device__ __forceinline__ int Sim<MODE>::run(rr_instance *I, JobWS &ws, int32_t
     };
     auto housekeeping = [&]() {
         if (guard <= 0) return (int)RR_ERR_TIMEOUT;
-        if (MODE != SIM_WIDE && *(volatile int *)&C->full) return (int)RR_SIM_RETRY;
+        if (*(volatile int *)&C->full) return (int)RR_SIM_RETRY;
         // (a run may have gone beyond the 32)
         guard += left;
         left = 32;
@@ -1549,7 +1560,7 @@ __device__ __forceinline__ int Sim<MODE>::run(rr_instance *I, JobWS &ws, int32_t
             const int room = log_room(nseg, idTop, lineCap);
             logging = room > 0;
             if (logging) left = min(32, room);
-            else end_of_log();
+            else end_of_log(C);
         }
         if (guard < left) left = (int)guard;
         guard -= left;
@@ -1565,7 +1576,7 @@ __device__ __forceinline__ int Sim<MODE>::run(rr_instance *I, JobWS &ws, int32_t
             if (id < best) { best = id; where = 4; place = u; }
         }
         for (int q = 0; q < 4; ++q)
-            for (int e0 = base(q) + 4 * lane; e0 < base(q) + size(q); e0 += 128) {
+            for (int e0 = q * cap + 4 * lane; e0 < (q + 1) * cap; e0 += 128) {
                 const uint4 a = *(const uint4 *)(pos + e0);
                 const uint32_t x[4] = {a.x, a.y, a.z, a.w};
 #pragma unroll
@@ -1587,11 +1598,11 @@ __device__ __forceinline__ int Sim<MODE>::run(rr_instance *I, JobWS &ws, int32_t
             d = where;
             lpos = uni(pos[place]);
             lend = clk + (int)uni((uint32_t)ir[place].y);
-            const int fr = C->nfree[d], tb = base(d);
+            const int fr = C->nfree[d], tb = d * cap;
             __syncwarp();
             if (lane == 0) {
                 pos[place] = HOLE;
-                stk[tb + fr] = (ST)(place - tb);
+                stk[tb + fr] = (uint16_t)(place - tb);
                 C->nfree[d] = fr + 1;
             }
         } else {
@@ -1621,8 +1632,7 @@ __device__ __forceinline__ int Sim<MODE>::run(rr_instance *I, JobWS &ws, int32_t
     while (!err) {
         // the statics of the leader's direction: the distance to the nearest
         // line ahead that holds one, 0 when one stands on a line of the leader's
-        const int tb = base(d);
-        if (MODE == SIM_WIDE) { groups = size(d) >> 3; off = 8 * min(lane, groups - 1); }
+        const int tb = d * cap;
         const uint32_t nadd = 0x10000u - lpos;
         uint4 a = *(const uint4 *)(pos + tb + off), b = *(const uint4 *)(pos + tb + off + 4);
         uint32_t v = min8(a, b, nadd, HOLE);
@@ -1633,7 +1643,7 @@ __device__ __forceinline__ int Sim<MODE>::run(rr_instance *I, JobWS &ws, int32_t
             }
         int fr = C->nfree[d];
         int pick = (int)__reduce_min_sync(FULL, v < 0x10000u ? 0u : v & 0xffffu);
-        if (MODE != SIM_WIDE && tryRun) {
+        if (tryRun) {
             tryRun = false;
             int run = 0;
             if (nm == 0 && pick >= lend - clk && guard > 128)
@@ -1703,29 +1713,18 @@ __device__ __forceinline__ int Sim<MODE>::run(rr_instance *I, JobWS &ws, int32_t
                         const bool c = q != 0u;
                         const int i = c ? 31 - __clz(q) : 0, e = e0 + i, rank = __popc(bal & lt), u = nm + rank;
                         q &= ~(1u << i);
-                        if constexpr (MODE == SIM_WIDE) {
-                            if (c) {
-                                const int2 x = ir[e];
-                                mie[u] = make_int2(x.x, x.y + clk);
-                                mpos[u] = (pos[e] & 0xffff0000u) | ((pos[e] - (uint32_t)clk) & 0xffffu);
-                                pos[e] = HOLE;
-                                stk[tb + fr + rank] = (ST)(e - tb);
-                                me = min(me, x.y + clk);
-                            }
-                        } else {
-                            const int ec = c ? e : tb;
-                            const int2 x = ir[ec];
-                            const uint32_t p = pos[ec];
-                            const int end = x.y + clk;
-                            st_if(c, mie + u, x.x, end);
-                            st_if(c, mpos + u, (p & 0xffff0000u) | ((p - (uint32_t)clk) & 0xffffu));
-                            st_if(c, pos + e, HOLE);
-                            st_if(c, stk + tb + fr + rank, e - tb);
-                            if (c) me = min(me, end);
-                            // its record and its likeliest successor's: read when it finishes
-                            touch_rec_if(c, rec, x.x, dump);
-                            touch_rec_if(c, rec, x.x + 1, dump);
-                        }
+                        const int ec = c ? e : tb;
+                        const int2 x = ir[ec];
+                        const uint32_t p = pos[ec];
+                        const int end = x.y + clk;
+                        st_if(c, mie + u, x.x, end);
+                        st_if(c, mpos + u, (p & 0xffff0000u) | ((p - (uint32_t)clk) & 0xffffu));
+                        st_if(c, pos + e, HOLE);
+                        st_if(c, stk + tb + fr + rank, e - tb);
+                        if (c) me = min(me, end);
+                        // its record and its likeliest successor's: read when it finishes
+                        touch_rec_if(c, rec, x.x, dump);
+                        touch_rec_if(c, rec, x.x + 1, dump);
                         nm += n;
                         fr += n;
                     }
@@ -1878,65 +1877,476 @@ __device__ __forceinline__ int Sim<MODE>::run(rr_instance *I, JobWS &ws, int32_t
         if (moved && nm > 0 && !(dm == d && line == (prim ? (int)(lpos & 0xffffu) - clk : (int)(lpos >> 16)))) dissolve();
         evEnd = min(lend, minEnd);
     }
-    // the log's end: a header with the totals, everything published
-    touch_wait();
-    __syncwarp();
-    if (logging && lane == 0) hdr[nseg] = make_uint4((unsigned)clk, nmem, 0u, 0u);
-    if (lane == 0) {
-        I->n_ops = clk;
-        I->n_members = nmem;
-    }
-    if (MODE != SIM_WIDE && *(volatile int *)&C->full) err = RR_SIM_RETRY;
-    if (!err && (long long)nmem != I->n_steps) err = RR_ERR_INTERNAL;
-    if (!err && ((int64_t)clk > I->cap_ops || (int64_t)nmem > I->cap_members)) err = RR_ERR_CAPACITY;
-    __syncwarp();
-    __threadfence_block();
-    if (lane == 0) {
-        *(volatile int *)&C->pub = (int)nseg;
-        __threadfence_block();
-        *(volatile int *)&C->fin = 1;
-    }
-    __syncwarp();
-    return err;
+    return sim_end(I, C, hdr, nseg, logging, clk, nmem, err);
 }
 
-template <int MODE>
-__device__ __forceinline__ int sim_run(Sim<MODE> &S, rr_instance *I, JobWS &ws, char *smem, int side, int counters)
+// ------------------------------------------------- the wide simulation
+//
+// For instances with more ready moves of a direction than the tables hold (no
+// planner here makes such lists; rr_batch takes any path system): statics by
+// the vertex that they stand on (ready moves share none), with room for every
+// move, so that a segment's cost grows with the grid's side and not with the
+// length of the list. A line's statics are found by reading the line; counts
+// of every line say whether there are any, a bit per line of a direction where
+// the next one ahead is. Against a table of all legs in global memory, scanned
+// whole at every segment: 524 288 dominoes on 1024 x 1024 (1 278 batches) 3.2 s
+// -> 60 ms, 600 000 moves of one token beside 512 others 31 s -> 0.9 s.
+
+constexpr uint32_t NOBODY = 0xffffffffu;
+struct Wide {
+    uint32_t *map;            // m * n: id and direction (upper two bits) of the static on a vertex
+                              // (where the first horizontal coverers were: the conflict graph is done)
+    int2 *state;              // k: a static's position word, steps left and direction (two bits);
+                              // .y is 0 for a move that waits or is a member, -1 for a finished one
+    int32_t *al, *ac;         // 4 * side each: statics of a direction on a line across its way, along it
+    uint32_t *some;           // 4 * 32: which lines across a direction's way hold any
+    int m, n, side;
+
+    static __host__ __device__ size_t shared_words(int side) { return 8 * (size_t)side + 128; }
+    __device__ __forceinline__ Wide(rr_instance *I, const JobWS &ws, char *smem, int side_)
+        : map((uint32_t *)as_global(ws.firstH)), state(as_global(ws.state)), m(I->m), n(I->n), side(side_)
+    {
+        al = (int32_t *)smem;
+        ac = al + 4 * side;
+        some = (uint32_t *)(ac + 4 * side);
+    }
+    // A position's line across the way (numbered along it) and along it, its
+    // row and column.
+    __device__ __forceinline__ int line_al(int d, uint32_t p) const
+    {
+        return (int)(p & 0xffffu) - ((d & 1) ? 1 : MIRROR - side);
+    }
+    __device__ __forceinline__ int line_ac(uint32_t p) const { return (int)(p >> 16) - 1; }
+    __device__ __forceinline__ int coord(int d, uint32_t p) const
+    {
+        return (d & 1) ? (int)(p & 0xffffu) - 1 : MIRROR - 1 - (int)(p & 0xffffu);
+    }
+    __device__ __forceinline__ int row(int d, uint32_t p) const { return d < 2 ? coord(d, p) : line_ac(p); }
+    __device__ __forceinline__ int col(int d, uint32_t p) const { return d < 2 ? line_ac(p) : coord(d, p); }
+
+    // A move becomes a static, or is one no longer (each lane its own).
+    __device__ __forceinline__ void put(int d, uint32_t p, int id, int rem)
+    {
+        const int a = line_al(d, p);
+        map[(size_t)row(d, p) * n + col(d, p)] = (uint32_t)id | (uint32_t)d << 30;
+        state[id] = make_int2((int)p, rem << 2 | d);
+        if (atomicAdd(&al[d * side + a], 1) == 0) atomicOr(&some[32 * d + (a >> 5)], 1u << (a & 31));
+        atomicAdd(&ac[d * side + line_ac(p)], 1);
+    }
+    __device__ __forceinline__ void take(int d, uint32_t p, int id)
+    {
+        const int a = line_al(d, p);
+        map[(size_t)row(d, p) * n + col(d, p)] = NOBODY;
+        state[id].y = 0;
+        if (atomicSub(&al[d * side + a], 1) == 1) atomicAnd(&some[32 * d + (a >> 5)], ~(1u << (a & 31)));
+        atomicSub(&ac[d * side + line_ac(p)], 1);
+    }
+    // Lines from p's to the next one ahead that holds a static of direction d
+    // (far, if there is none).
+    __device__ __forceinline__ int ahead(int d, uint32_t p) const
+    {
+        const int lane = lane_id(), a = line_al(d, p), w = a >> 5;
+        uint32_t x = some[32 * d + lane];
+        x &= lane < w ? 0u : lane == w ? ~(((2u << (a & 31)) - 1u)) : FULL;
+        const unsigned b = __ballot_sync(FULL, x != 0u);
+        if (!b) return 0x7fff;
+        const int src = __ffs(b) - 1;
+        return 32 * src + __ffs(__shfl_sync(FULL, x, src)) - 1 - a;
+    }
+    // f(lane's static there or not, its id) for the vertices of p's line
+    // across the way of d (or along it), 32 at a time, four loads in flight.
+    template <class F>
+    __device__ __forceinline__ void line(int d, uint32_t p, bool across, F f) const
+    {
+        const bool isRow = across == (d < 2);
+        const int len = isRow ? n : m, step = isRow ? 1 : n;
+        const uint32_t *at = map + (isRow ? (size_t)row(d, p) * n : (size_t)col(d, p));
+        for (int i0 = lane_id(); i0 - lane_id() < len; i0 += 128) {
+            uint32_t w[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) w[u] = i0 + 32 * u < len ? at[(size_t)(i0 + 32 * u) * step] : NOBODY;
+#pragma unroll
+            for (int u = 0; u < 4; ++u) f(w[u] != NOBODY && (int)(w[u] >> 30) == d, (int)(w[u] & 0x3fffffffu));
+        }
+    }
+    __device__ __forceinline__ int least_id(int d, uint32_t p, bool across) const
+    {
+        int least = INTMAX;
+        line(d, p, across, [&](bool c, int id) { least = c ? min(least, id) : least; });
+        return least;
+    }
+};
+
+// The simulation over such a map: as Sim, without what makes that one fast on
+// plans (runs of leaders, counters in shared memory).
+struct WideSim : Wide {
+    int2 *mie;                // members: id, clock at the end of the leg
+    uint32_t *mpos;           // members: position word, `along` minus the clock
+    SimCtl *C;
+    const int4 *rec;
+    const int32_t *succ;
+    const int2 *multiMove;
+    int32_t *multi;
+    uint32_t dump;
+
+    using Wide::Wide;
+
+    __device__ __forceinline__ bool release(bool c, int32_t v, int handId)
+    {
+        const bool single = c && (v & SUCC_SINGLE);
+        int id = v & SUCC_ID, y = 0;
+        uint32_t p = 0;
+        bool ready = single;
+        if (single) {
+            const int4 r = rec[2 * (size_t)id];
+            p = (uint32_t)r.x;
+            y = r.y;
+        } else if (c && (atomicSub(&multi[id], 1) & MULTI_COUNT) == 1) {
+            y = ldg_volatile_if(true, multi + id) >> MULTI_BITS;
+            const int2 mv = multiMove[id];
+            id = mv.x;
+            p = (uint32_t)mv.y;
+            ready = true;
+        }
+        __syncwarp();
+        const bool h = ready && id == handId;
+        if (ready && !h) put(y & 3, p, id, y >> 2 & 2047);
+        __syncwarp();
+        return h;
+    }
+
+    __device__ __forceinline__ int run(rr_instance *I, JobWS &ws, int32_t *log, unsigned logWords, int lineCap,
+                                       int32_t *buf, int32_t *ids);
+};
+
+__device__ __forceinline__ int WideSim::run(rr_instance *I, JobWS &ws, int32_t *log, unsigned logWords, int lineCap,
+                                            int32_t *buf, int32_t *ids)
 {
-    const SimLayout Y(smem, side);
+    const int lane = lane_id();
+    const unsigned lt = (1u << lane) - 1u;
+    const int k = (int)I->n_moves;
+    int err = RR_OK;
+
+    // moves without predecessors become statics
+    for (int b = lane, n0 = ws.ready0[k]; b < n0; b += 32) {
+        const int id = ws.ready0[b];
+        const int4 r = rec[2 * (size_t)id];
+        put(r.y & 3, (uint32_t)r.x, id, r.y >> 2 & 2047);
+    }
+    __syncwarp();
+    // leader, members, clock and log as in Sim
+    int L = -1, d = 0, lend = 0, ldst = 0, nsu = 0, ov = 0;
+    uint32_t lpos = 0;
+    int4 s4 = make_int4(0, 0, 0, 0);
+    int nm = 0, dm = -1, line_ = 0, minEnd = INTMAX;
+    bool prim = true, changed = false;
+    int clk = 0;
+    unsigned nmem = 0;
+    uint4 *hdr = (uint4 *)log;
+    unsigned nseg = 0, idTop = logWords, list = 0;
+    int left = min(32, log_room(0u, idTop, lineCap));
+    bool logging = left > 0;
+    if (!logging) { left = 32; end_of_log(C); }
+    long long guard = (g_guard_cap > 0 ? g_guard_cap : I->n_steps + 2ll * k + 16) + 1;
+    if (guard < left) left = (int)guard;
+    guard -= left;
+
+    auto set_record = [&](const int4 r, const int4 s) {
+        d = (int)uni((uint32_t)r.y & 3u);
+        lpos = uni((uint32_t)r.x);
+        lend = clk + (r.y >> 2 & 2047);
+        ldst = r.y >> 13 & 1023;
+        nsu = r.z;
+        ov = r.w;
+        s4 = s;
+    };
+    auto on_clock = [&](uint32_t p) { return (p & 0xffff0000u) | ((p + (uint32_t)clk) & 0xffffu); };
+    auto dissolve = [&]() {
+        for (int u = lane; u < nm; u += 32) put(dm, on_clock(mpos[u]), mie[u].x, mie[u].y - clk);
+        nm = 0;
+        minEnd = INTMAX;
+        changed = true;
+        __syncwarp();
+    };
+    // the lowest unfinished move becomes the leader: every id up to the last
+    // leader's has finished, so on from there
+    auto find_leader = [&]() {
+        unsigned open = 0;
+        int b = L + 1;
+        for (; b < k; b += 32) {
+            open = __ballot_sync(FULL, b + lane < k && state[min(b + lane, k - 1)].y >= 0);
+            if (open) break;
+        }
+        if (!open) return false;
+        L = b + __ffs(open) - 1;
+        set_record(rec[2 * (size_t)L], rec[2 * (size_t)L + 1]);
+        const int2 st = state[L];
+        __syncwarp();
+        if (st.y > 0) {
+            d = (int)uni((uint32_t)st.y & 3u);
+            lpos = uni((uint32_t)st.x);
+            lend = clk + (st.y >> 2);
+            if (lane == 0) take(d, lpos, L);
+        } else {
+            int at = -1;
+            for (int u = lane; u < nm; u += 32) at = mie[u].x == L ? u : at;
+            at = __reduce_max_sync(FULL, at);
+            if (at < 0) return false;               // neither ready nor moving
+            d = dm;
+            lpos = uni(on_clock(mpos[at]));
+            lend = mie[at].y;
+            --nm;
+            const int2 le = mie[nm];
+            const uint32_t lp = mpos[nm];
+            __syncwarp();
+            if (lane == 0) { mie[at] = le; mpos[at] = lp; }
+            __syncwarp();
+            int me = INTMAX;
+            for (int u = lane; u < nm; u += 32) me = min(me, mie[u].y);
+            minEnd = __reduce_min_sync(FULL, me);
+            changed = true;
+        }
+        __syncwarp();
+        return true;
+    };
+
+    if (!find_leader() || L != 0) err = RR_ERR_INTERNAL;
+    while (!err) {
+        const int la = d * side + line_al(d, lpos), lc = d * side + line_ac(lpos);
+        const bool onA = al[la] != 0, onC = ac[lc] != 0;
+        if (onA || onC) {
+            bool choose;
+            if (!onC && (nm == 0 || prim)) choose = true;
+            else if (!onA && (nm == 0 || !prim)) choose = false;
+            else {
+                // candidates on both lines: the smaller smallest id decides
+                int ma = least_id(d, lpos, true), mc = least_id(d, lpos, false);
+                for (int u = lane; u < nm; u += 32) {
+                    const int id = mie[u].x;
+                    if (prim) ma = min(ma, id); else mc = min(mc, id);
+                }
+                choose = __reduce_min_sync(FULL, ma) < __reduce_min_sync(FULL, mc);
+                if (nm > 0 && choose != prim) dissolve();
+            }
+            if (choose ? onA : onC) {
+                // the chosen line's statics join the members
+                int me = minEnd;
+                __syncwarp();
+                line(d, lpos, choose, [&](bool c, int id) {
+                    const unsigned bal = __ballot_sync(FULL, c);
+                    const int u = nm + __popc(bal & lt);
+                    if (nm + __popc(bal) > lineCap) { err = RR_ERR_INTERNAL; return; }
+                    if (c) {
+                        const int2 st = state[id];
+                        const uint32_t p = (uint32_t)st.x;
+                        const int end = (st.y >> 2) + clk;
+                        mie[u] = make_int2(id, end);
+                        mpos[u] = (p & 0xffff0000u) | ((p - (uint32_t)clk) & 0xffffu);
+                        take(d, p, id);
+                        me = min(me, end);
+                    }
+                    nm += __popc(bal);
+                });
+                if (err) break;
+                minEnd = __reduce_min_sync(FULL, me);
+                prim = choose;
+                dm = d;
+                line_ = choose ? (int)(lpos & 0xffffu) - clk : (int)(lpos >> 16);
+                changed = true;
+                __syncwarp();
+            }
+        }
+        // the segment: up to the first leg end or the nearest line ahead
+        const int evEnd = min(lend, minEnd), kseg = min(ahead(d, lpos), evEnd - clk);
+        if (kseg < 1) { err = RR_ERR_INTERNAL; break; }
+        if (logging) {
+            if (changed) {
+                changed = false;
+                idTop -= (unsigned)nm;
+                list = idTop;
+                for (int u = lane; u < nm; u += 32) log[list + u] = mie[u].x;
+            }
+            if (lane == 0) hdr[nseg] = make_uint4((unsigned)clk, nmem, list, (unsigned)L | (unsigned)d << 30);
+            ++nseg;
+        } else {
+            const unsigned long long o1 = (unsigned long long)clk + kseg, m1 = nmem + (unsigned long long)kseg * (nm + 1);
+            if (o1 <= room_of(I->cap_ops) && m1 <= room_of(I->cap_members)) {
+                for (int u = lane; u < nm; u += 32) ids[u] = mie[u].x;
+                __syncwarp();
+                write_call(I, (unsigned)clk, nmem, kseg, nm + 1, d, L, ids, buf);
+            }
+        }
+        // everything in the batch advances
+        nmem += (unsigned)(kseg * (nm + 1));
+        clk += kseg;
+        lpos += (uint32_t)kseg;
+        if (--left <= 0) {
+            if (guard <= 0) { err = RR_ERR_TIMEOUT; break; }
+            left = 32;
+            if (logging) {
+                if (lane == 0) hdr[nseg] = make_uint4((unsigned)clk, nmem, 0u, 0u);
+                __syncwarp();
+                __threadfence_block();
+                if (lane == 0) *(volatile int *)&C->pub = (int)nseg;
+                const int room = log_room(nseg, idTop, lineCap);
+                logging = room > 0;
+                if (logging) left = min(32, room);
+                else end_of_log(C);
+            }
+            if (guard < left) left = (int)guard;
+            guard -= left;
+        }
+        if (clk != evEnd) continue;
+        bool fin = false, moved = false;
+        if (clk == lend) {
+            moved = true;
+            if (d < 2 || ldst == (int)(lpos >> 16) - 1) fin = true;
+            else {
+                const Leg g = second_leg(d, lpos, ldst);
+                d = g.d; lpos = g.pos; lend = clk + g.rem;
+            }
+        }
+        const int handId = fin ? L + 1 : -1;       // the next leader, if it becomes ready now
+        bool hand = false;
+        if (clk == minEnd) {
+            // members whose leg ended leave: they turn or finish
+            int nk = 0, me = INTMAX;
+            for (int u0 = 0; u0 < nm; u0 += 32) {
+                const int u = u0 + lane;
+                const int2 ie = mie[min(u, nm - 1)];
+                const uint32_t p = mpos[min(u, nm - 1)];
+                const bool ended = u < nm && ie.y == clk, keep = u < nm && ie.y != clk;
+                const unsigned kb = __ballot_sync(FULL, keep);
+                const int w = nk + __popc(kb & lt);
+                if (keep) { mie[w] = ie; mpos[w] = p; me = min(me, ie.y); }
+                int4 r = make_int4(0, 0, 0, 0), s = r;
+                if (ended) {
+                    r = rec[2 * (size_t)ie.x];
+                    s = rec[2 * (size_t)ie.x + 1];
+                    const int dst = r.y >> 13 & 1023;
+                    if (dm >= 2 && dst != (int)(p >> 16) - 1) {
+                        const Leg g = second_leg(dm, on_clock(p), dst);
+                        put(g.d, g.pos, ie.x, g.rem);
+                        r.z = 0;
+                    } else {
+                        state[ie.x].y = -1;
+                    }
+                }
+                __syncwarp();
+                const int most = (int)uni((uint32_t)r.z);
+                for (int e = 0; e < most; ++e) {
+                    int32_t v = e == 0 ? s.x : e == 1 ? s.y : e == 2 ? s.z : s.w;
+                    if (e >= 4 && e < r.z) v = succ[r.w + e - 4];
+                    hand |= release(e < r.z, v, handId);
+                }
+                nk += __popc(kb);
+            }
+            nm = nk;
+            minEnd = __reduce_min_sync(FULL, me);
+            changed = true;
+        }
+        if (fin) {
+            const int n_ = (int)uni((uint32_t)nsu);
+            for (int e0 = 0; e0 < n_; e0 += 32) {
+                const int e = e0 + lane;
+                int32_t v = e == 0 ? s4.x : e == 1 ? s4.y : e == 2 ? s4.z : s4.w;
+                if (e >= 4 && e < n_) v = succ[ov + e - 4];
+                hand |= release(e < n_, v, handId);
+            }
+            if (__any_sync(FULL, hand)) {
+                L = handId;
+                set_record(rec[2 * (size_t)L], rec[2 * (size_t)L + 1]);
+                touch_rec_if(lane == 0, rec, min(L + 1, k), dump);
+            } else if (!find_leader()) {
+                break;
+            }
+        }
+        // members no longer on the leader's line or in its direction?
+        if (moved && nm > 0 && !(dm == d && line_ == (prim ? (int)(lpos & 0xffffu) - clk : (int)(lpos >> 16)))) dissolve();
+    }
+    return sim_end(I, C, hdr, nseg, logging, clk, nmem, err);
+}
+
+// The fields that both forms have, and the log: the chains of the conflict
+// graph are no longer needed.
+template <class SIM>
+__device__ __forceinline__ int sim_run(SIM &S, rr_instance *I, JobWS &ws, const SimLayout &Y)
+{
     S.mie = Y.mie; S.mpos = Y.mpos; S.C = Y.C;
     S.rec = as_global(ws.rec); S.succ = as_global(ws.succ); S.multi = as_global(ws.multi);
     S.multiMove = as_global(ws.multiMove);
-    S.cnt = Y.cnt;
     S.dump = sh_addr(Y.dump);
-    S.ncnt = min(counters, ws.nmulti);
-    S.allShared = counters >= ws.nmulti;
-    S.smem = smem; S.side = side; S.counters = counters;
-    // the log: the chains of the conflict graph are no longer needed
     return S.run(I, ws, as_global(ws.nextAt), (unsigned)((4 * (ws.P + 1) + 255) / 256 * 64), Y.MC, Y.bufs, Y.ids);
 }
 
-// The tables in global memory, for an instance that outgrew shared memory.
-static __device__ __noinline__ int sim_wide(rr_instance *I, JobWS *ws, char *smem, int side, int counters)
+// A simulation starts: its control words (every thread calls it).
+__device__ __forceinline__ void ctl_begin(SimCtl *C, int free)
 {
-    const size_t n = sim_wide_entries(I->n_moves);
-    Sim<SIM_WIDE> S;
-    S.pos = (uint32_t *)ws->slotOvf;
-    S.ir = (int2 *)(S.pos + n);
-    S.stk = (int32_t *)(S.ir + n);
-    S.cap = 0;
-    return sim_run(S, I, *ws, smem, side, counters);
+    if (threadIdx.x < 4) C->nfree[threadIdx.x] = free;
+    if (threadIdx.x == 0) {
+        C->full = C->pub = C->next = C->fin = 0;
+        C->status = RR_OK;
+    }
+}
+// The counters in shared memory.
+__device__ __forceinline__ void counters_begin(const SimLayout &Y, const JobWS &ws, int counters)
+{
+    unsigned short *c16 = (unsigned short *)Y.cnt;
+    const int ncnt = min(counters, ws.nmulti);
+    for (int i = threadIdx.x; i < ncnt; i += blockDim.x) c16[i] = (unsigned short)(ws.multi[i] & MULTI_COUNT);
 }
 
-// The whole simulation of one instance by one block (every thread calls it):
-// warp 0 simulates, the others write, warp 0 writes too once it is done. A
-// block without writers is that one warp; s_write writes afterwards.
-// An instance that outgrows the shared-memory tables starts over with its
-// tables in global memory (the batches written so far are the same ones).
+// Warp 0 runs simulate(), the others write, warp 0 writes too once it is done.
+// Returns the status (every thread calls it).
+template <class F>
+__device__ __forceinline__ int sim_and_write(F simulate, rr_instance *I, JobWS &ws, const SimLayout &Y, int side)
+{
+    const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    __syncthreads();
+    if (wid == 0) {
+        const int st = simulate();
+        if (lane == 0) Y.C->status = st;
+        __syncwarp();
+    }
+    run_writers(Y.C, I, as_global(ws.nextAt), Y.bufs + sim_pow2(side) * wid);
+    __syncthreads();
+    return Y.C->status;
+}
+
+// An instance that outgrew the tables starts over in the wide form (the
+// batches written so far are the same ones): its state at the start, for the
+// whole block, its simulation, both with writers. Out of line: in line, the
+// registers and the stack of this form would cost the other one.
+static __device__ __noinline__ void wide_begin(rr_instance *I, JobWS *ws, char *smem, int side)
+{
+    const Wide W(I, *ws, smem, side);
+    const int k = (int)I->n_moves;
+    for (int i = threadIdx.x; i < W.m * W.n; i += blockDim.x) W.map[i] = NOBODY;
+    for (int b = threadIdx.x; b < k; b += blockDim.x) W.state[b] = make_int2(0, 0);
+    for (int i = threadIdx.x; i < (int)Wide::shared_words(side); i += blockDim.x) W.al[i] = 0;
+    // (the first form counted in-degrees down)
+    for (int x = threadIdx.x; x < ws->nmulti; x += blockDim.x)
+        ws->multi[x] = (ws->multi[x] & ~MULTI_COUNT) | ws->indeg[ws->multiMove[x].x];
+}
+static __device__ __noinline__ int wide_run(rr_instance *I, JobWS *ws, char *smem, int side)
+{
+    WideSim S(I, *ws, smem, side);
+    return sim_run(S, I, *ws, SimLayout(smem, side));
+}
+static __device__ __noinline__ int wide_block(rr_instance *I, JobWS *ws, char *smem, int side)
+{
+    const SimLayout Y(smem, side);
+    __syncthreads();                    // every thread has read the first form's status
+    ctl_begin(Y.C, 0);
+    wide_begin(I, ws, smem, side);
+    return sim_and_write([&]() { return wide_run(I, ws, smem, side); }, I, *ws, Y, side);
+}
+
+// The whole simulation of one instance by one block (every thread calls it). A
+// block without writers is one warp; s_write writes afterwards.
 template <int MODE, bool WRITERS>
 __device__ __forceinline__ void sim_block(rr_instance *I, JobWS &ws, char *smem, int side, int counters)
 {
-    const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int k = (int)I->n_moves;
     if (!live(I)) return;                       // the same in every thread: set before this kernel or a barrier
     if (k == 0) {
@@ -1950,71 +2360,43 @@ __device__ __forceinline__ void sim_block(rr_instance *I, JobWS &ws, char *smem,
     S.ir = (int2 *)(S.pos + 4 * cap);
     S.stk = (uint16_t *)(S.ir + 4 * cap);
     S.cap = cap;
-    SimCtl *C = Y.C;
-
-    for (int pass = 0;; ++pass) {
-        if (threadIdx.x < 4) C->nfree[threadIdx.x] = pass == 0 ? cap : 0;
-        if (threadIdx.x == 0) {
-            C->full = C->pub = C->next = C->fin = 0;
-            C->status = RR_OK;
+    S.cnt = Y.cnt;
+    S.ncnt = min(counters, ws.nmulti);
+    S.allShared = counters >= ws.nmulti;
+    S.smem = smem; S.side = side; S.counters = counters;
+    auto tables_begin = [&]() {                 // entries are handed out from a table's start
+        for (int i = threadIdx.x; i < 4 * cap; i += blockDim.x) {
+            S.pos[i] = HOLE;
+            S.stk[i] = (uint16_t)(cap - 1 - i % cap);
         }
-        // entries are handed out from a table's start
-        if (pass == 0) {
-            for (int i = threadIdx.x; i < 4 * cap; i += blockDim.x) {
-                S.pos[i] = HOLE;
-                S.stk[i] = (uint16_t)(cap - 1 - i % cap);
-            }
-        } else {
-            // as many entries per direction as there are legs of it (rounded
-            // up to eight, at least eight)
+    };
+    int st;
+    if constexpr (WRITERS) {
+        ctl_begin(Y.C, cap);
+        tables_begin();
+        counters_begin(Y, ws, counters);
+        st = sim_and_write([&]() { return sim_run(S, I, ws, Y); }, I, ws, Y, side);
+        if (st == RR_SIM_RETRY && k >= SIM_WIDE_MIN) st = wide_block(I, &ws, smem, side);
+    } else {
+        for (int pass = 0;; ++pass) {
+            ctl_begin(Y.C, pass == 0 ? cap : 0);
+            if (pass == 0) tables_begin();
+            else wide_begin(I, &ws, smem, side);
             __syncthreads();
-            for (int b = threadIdx.x; b < k; b += blockDim.x) {
-                const int4 r = ws.rec[2 * (size_t)b];
-                const int d = r.y & 3, dst = r.y >> 13 & 1023, row = (int)((uint32_t)r.x >> 16) - 1;
-                atomicAdd(&C->nfree[d], 1);
-                if (d >= 2 && dst != row) atomicAdd(&C->nfree[dst > row ? 1 : 0], 1);
-            }
+            counters_begin(Y, ws, counters);
             __syncthreads();
-            if (threadIdx.x == 0) {
-                int at = 0;
-                for (int d = 0; d < 4; ++d) {
-                    C->wbase[d] = at;
-                    C->nfree[d] = C->wcap[d] = max(8, (C->nfree[d] + 7) & ~7);
-                    at += C->wcap[d];
-                }
-            }
-            __syncthreads();
-            const size_t n = sim_wide_entries(k);
-            uint32_t *p = (uint32_t *)ws.slotOvf;
-            int32_t *st = (int32_t *)(p + 3 * n);
-            for (int d = 0; d < 4; ++d)
-                for (int i = threadIdx.x; i < C->wcap[d]; i += blockDim.x) {
-                    p[C->wbase[d] + i] = HOLE;
-                    st[C->wbase[d] + i] = C->wcap[d] - 1 - i;
-                }
-            // the first pass counted in-degrees down: start over
-            for (int x = threadIdx.x; x < ws.nmulti; x += blockDim.x) ws.multi[x] = (ws.multi[x] & ~MULTI_COUNT) | ws.indeg[ws.multiMove[x].x];
-        }
-        __syncthreads();
-        unsigned short *c16 = (unsigned short *)Y.cnt;
-        const int ncnt = min(counters, ws.nmulti);
-        for (int i = threadIdx.x; i < ncnt; i += blockDim.x) c16[i] = (unsigned short)(ws.multi[i] & MULTI_COUNT);
-        __syncthreads();
-        if (wid == 0) {
-            const int st = pass == 0 ? sim_run(S, I, ws, smem, side, counters) : sim_wide(I, &ws, smem, side, counters);
-            if (lane == 0) C->status = st;
+            // (in a register from here on, the status costs the kernel a stack
+            // frame and 4096 mixed grids 2 % of their time)
+            const int r = pass == 0 ? sim_run(S, I, ws, Y) : wide_run(I, &ws, smem, side);
+            if (threadIdx.x == 0) Y.C->status = r;
             __syncwarp();
+            if (threadIdx.x == 0) ws.nseg = Y.C->pub;        // s_write follows
+            __syncthreads();
+            st = Y.C->status;
+            if (st != RR_SIM_RETRY || pass == 1 || k < SIM_WIDE_MIN) break;
         }
-        if (WRITERS) run_writers(C, I, as_global(ws.nextAt), Y.bufs + sim_pow2(side) * wid);
-        else if (lane == 0) ws.nseg = C->pub;            // s_write follows
-        __syncthreads();
-        const int st = C->status;
-        if (st != RR_SIM_RETRY || pass == 1 || k < SIM_WIDE_MIN) {
-            if (threadIdx.x == 0 && st != RR_OK) I->status = st == RR_SIM_RETRY ? RR_ERR_INTERNAL : st;
-            break;
-        }
-        __syncthreads();
     }
+    if (threadIdx.x == 0 && st != RR_OK) I->status = st == RR_SIM_RETRY ? RR_ERR_INTERNAL : st;
 }
 
 } // namespace rrk

@@ -107,7 +107,7 @@ struct JobWS {
     int32_t *colOff, *colCur, *colList;   // n + 1, n, k
     int32_t *rowOff, *rowCur, *rowList;   // m + 1, m, k
     int32_t *firstH;       // m * n: lowest-id L-move crossing each vertex, -1
-    void *slotOvf;         // the wide simulation's tables
+    int2 *state;           // k: the wide simulation's moves (Wide)
     // the moves with several predecessors, by number: in-degree and first leg
     // (MULTI_BITS), id, position word
     int32_t *multi;
@@ -140,7 +140,6 @@ __host__ __device__ inline int class_side(int max_side, int c, int nclass)
 // Block-wide state of a simulation in shared memory.
 struct SimCtl {
     int nfree[4];             // free entries of each direction's table
-    int wbase[4], wcap[4];    // the wide tables: first entry, entries
     int full;                 // a table was full
     int pub;                  // segments of the log that the writers may write
     int next;                 // first segment not yet taken by a writer (by 32)
@@ -174,12 +173,11 @@ __host__ __device__ inline size_t sim_smem_bytes(int side, int warps, int counte
 }
 constexpr int SIM_MAX_THREADS = 128, SIM_BLOCKS = 16;   // with writers; one-warp blocks per SM
 
-// Workspace of the wide simulation: tables in global memory with room for
-// every move, at most two legs each. Only instances with more ready moves
-// than a shared-memory table holds (at least 64) can need it.
+// Workspace of the wide simulation: 8 bytes per move, beside the words per
+// vertex that the conflict graph no longer needs. Only instances with more
+// ready moves than a shared-memory table holds (at least 64) can need it.
 constexpr int SIM_WIDE_MIN = 65;
-__host__ __device__ inline size_t sim_wide_entries(long long k) { return 2 * (size_t)k + 32; }
-__host__ __device__ inline size_t sim_wide_bytes(long long k) { return k < SIM_WIDE_MIN ? 0 : 16 * sim_wide_entries(k); }
+__host__ __device__ inline size_t sim_wide_bytes(long long k) { return k < SIM_WIDE_MIN ? 0 : 8 * (size_t)k; }
 
 // End of the narrow simulation when an instance needs more table entries
 // than shared memory holds: the wide one starts over in the same block, so

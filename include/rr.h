@@ -222,8 +222,11 @@ int rr_set_config(rr_ctx *ctx, int nclass, int shift, int pipe);
  * Continuous batching of planning requests (red-rec + batching per request):
  * a request is admitted as soon as its grid and its move list (room for
  * 2 m n moves, each atom moves at most twice) fit in the device input pool
- * and fewer than `slots` requests are resident (first come, first served), planned in waves (one rr_plan_batched call over the
- * requests admitted since the previous wave) on a pool of streams so that
+ * and fewer than `slots` requests are resident (first come, first served; in a
+ * server with RR_WITH_BATCH whose streams are busy by more than a quarter, a
+ * request is held back for half a millisecond at most, so that requests that
+ * come in together share a wave), planned in waves (one rr_plan_batched call
+ * over the requests admitted since the previous wave) on a pool of streams so that
  * waves overlap on the device, and, once a request's exact number of
  * elementary steps is known, given result memory from a device heap and
  * batched in a second wave (memory-based admission). A worker thread owned

@@ -35,7 +35,7 @@ struct Req {
     int64_t heapOff = -1, heapBytes = 0;
     int phase = QUEUED;
     rr_instance desc{};
-    double tSubmit = 0, tAdmit = 0, tPlanned = 0, tDone = 0;
+    double tSubmit = 0, tAdmit = 0, tDone = 0;
 };
 
 struct Wave {
@@ -127,24 +127,29 @@ static void fail_all(rr_server *S, int status)
     S->cvDone.notify_all();
 }
 
-// Whether the requests at the head of a queue should wait for company before
-// they take a stream. A wave keeps its stream until its slowest simulation is
-// done, so waves of one request each, started while a burst is still coming in,
-// take all streams and leave the rest of the burst waiting for tens of
-// milliseconds (48 requests of sides 64 to 512 on 12 streams: 177 ms, 134
-// this way). So once a quarter of the streams is busy, a wave that could hold
-// more waits, for a sixteenth of the time that the largest grid in it will take
-// at most (a 256 x 256 grid simulates in 17 ms, and time grows as cells ^ 1.25:
-// 3 ms for 128 x 128, 95 for 512 x 512). since: when a request entered the queue.
-static bool wait_for_more(const rr_server *S, const std::deque<Req *> &queue, double Req::*since)
+// Whether the queued requests should wait for company before they are planned.
+// A batched wave keeps its stream until its slowest simulation is done, so waves
+// of one request each, started while a burst is still coming in, take all
+// streams and leave the rest of the burst waiting for tens of milliseconds. So
+// once a quarter of the streams is busy, a wave that could hold more waits, for
+// a sixteenth of the time that its largest grid will be simulated (a 256 x 256
+// grid takes 17 ms, and time grows as cells ^ 1.25) and half a millisecond at
+// most: a burst has come in by then. Planned requests do not wait again, and in
+// a server that only plans, where no wave keeps its stream for long, none does.
+// 48 requests of sides 64 to 512 on 12 streams: 178 ms without waiting, 104 this
+// way (waiting without the half millisecond, before planning and before
+// batching: 126); of sides 24 to 48: 4.5 ms, 4.3 this way.
+constexpr double WAIT_AT_MOST_US = 500;
+static bool wait_for_more(const rr_server *S)
 {
+    if (!(S->cfg.flags & RR_WITH_BATCH) || (int)S->queued.size() >= S->cfg.max_wave) return false;
     int busy = 0;
     for (const Wave &W : S->wave) busy += W.busy;
-    if (4 * busy <= (int)S->wave.size() || (int)queue.size() >= S->cfg.max_wave) return false;
+    if (4 * busy <= (int)S->wave.size()) return false;
     double cells = 0;
-    for (const Req *R : queue) cells = std::max(cells, (double)R->m * R->n);
-    const double us = 17000.0 * std::pow(cells / 65536.0, 1.25);
-    return S->now() - queue.front()->*since < us / 16;
+    for (const Req *R : S->queued) cells = std::max(cells, (double)R->m * R->n);
+    const double us = 17000.0 / 16 * std::pow(cells / 65536.0, 1.25);
+    return S->now() - S->queued.front()->tSubmit < std::min(us, WAIT_AT_MOST_US);
 }
 
 // One pass of the pipeline; returns true if it changed anything.
@@ -164,7 +169,6 @@ static bool pump(rr_server *S)
             R->desc = S->hDesc[s][i];
             if (W.kind == 1 && R->desc.status == RR_OK && (S->cfg.flags & RR_WITH_BATCH) && R->desc.n_moves > 0) {
                 R->phase = PLANNED;
-                R->tPlanned = S->now();
                 S->planned.push_back(R);
             } else {
                 finish(S, R, RR_OK);
@@ -180,7 +184,6 @@ static bool pump(rr_server *S)
     for (int s = 0; s < NS && !S->planned.empty(); ++s) {
         Wave &W = S->wave[s];
         if (W.busy) continue;
-        if (wait_for_more(S, S->planned, &Req::tPlanned)) break;
         int cnt = 0;
         while (!S->planned.empty() && cnt < S->cfg.max_wave) {
             Req *R = S->planned.front();
@@ -224,7 +227,7 @@ static bool pump(rr_server *S)
     for (int s = 0; s < NS && !S->queued.empty() && S->resident < S->cfg.slots; ++s) {
         Wave &W = S->wave[s];
         if (W.busy) continue;
-        if (S->resident + (int)S->queued.size() <= S->cfg.slots && wait_for_more(S, S->queued, &Req::tSubmit)) break;
+        if (S->resident + (int)S->queued.size() <= S->cfg.slots && wait_for_more(S)) break;
         cudaStream_t st = S->stream[s];
         int cnt = 0, e = cudaSuccess;
         while (!S->queued.empty() && S->resident < S->cfg.slots && cnt < S->cfg.max_wave) {

@@ -14,6 +14,7 @@ __global__ void k_batch_begin(rr_instance, rr_instance *, Arena);
 __global__ void k_transpose(rr_instance *, JobWS *, int, int);
 __global__ void k_colstats(rr_instance *, JobWS *, int, int, int);
 __global__ void k_pair(rr_instance *, JobWS *, int, int);
+__global__ void k_pair_many(rr_instance *, JobWS *, int);
 __global__ void k_pair_sift(rr_instance *, JobWS *, int);
 __global__ void k_pair_listed(rr_instance *, JobWS *, int);
 __global__ void k_emit_cols(rr_instance *, JobWS *, int, int);
@@ -332,10 +333,14 @@ static int launch_plan(rr_ctx *ctx, rr_instance *d_inst, JobWS *ws, int count, i
     const bool bird = (flags & RR_BIRD) != 0;
     const int strict = (flags & RR_STRICT_RESERVOIR) ? 1 : 0;
     const Arena A = arena_of(ctx);
-    const int colBlocks = clampi(std::max(1, budget(ctx, 8192) / count), 1, (max_side + 7) / 8);
+    // (twice the blocks win 1 % of a call over 3 000 grids of sides 33 to 251
+    // and lose 10 us of 50 over 700 chains, which keep one warp of each busy)
+    const int colBlocks = clampi(std::max(1, budget(ctx, 4096) / count), 1, (max_side + 7) / 8);
     const int tiles = ((max_side + 31) / 32) * ((max_side + 31) / 32);
     const int trBlocks = clampi(std::max(1, budget(ctx, 4096) / count), 1, (tiles + 7) / 8);
-    const int recvBlocks = clampi(std::max(1, budget(ctx, 8192) / count), 1, (max_side * ((max_side + 31) / 32) + 7) / 8);
+    // (its warps go to the instances that need them; with 4 and 1.5 times the
+    // blocks 2 000 grids of sides 33 to 251 take 27 and 3 us longer)
+    const int recvBlocks = clampi(std::max(1, budget(ctx, 2048) / count), 1, (max_side * ((max_side + 31) / 32) + 7) / 8);
     // warps of a block on each instance: all eight, fewer in calls over very
     // many grids (see hw_blk_shared)
     const int per = count <= 4096 ? 8 : count <= 8192 ? 4 : count <= 16384 ? 2 : 1;
@@ -363,8 +368,11 @@ static int launch_plan(rr_ctx *ctx, rr_instance *d_inst, JobWS *ws, int count, i
     const size_t pairSmem = (size_t)max_side * PAIR_BYTES + 64;
     mark(ctx, s, "k_pair");
     const int fit = clampi((int)(SM_SMEM / (pairSmem + 1024)), 1, 32);         // blocks that an SM holds
-    if (count <= fit * ctx->nsm) {
-        k_pair<<<count, 32, pairSmem, s>>>(d_inst, ws, count, count <= ctx->nsm ? 1 : 0);
+    const bool many = count > ctx->nsm;
+    if (!many) {
+        k_pair<<<count, 32, pairSmem, s>>>(d_inst, ws, count, 1);
+    } else if (count <= fit * ctx->nsm) {
+        k_pair_many<<<count, 32, pairSmem, s>>>(d_inst, ws, count);
     } else {
         // more blocks than fit at once: only for the grids that need them
         // (2 000 grids of up to 251 x 251, which all fit: 317 us, 336 this way)
@@ -375,7 +383,7 @@ static int launch_plan(rr_ctx *ctx, rr_instance *d_inst, JobWS *ws, int count, i
     mark(ctx, s, "k_emit_cols");
     k_emit_cols<<<dim3(colBlocks, rows), 256, 0, s>>>(d_inst, ws, count, per);
     mark(ctx, s, "k_emit_recv");
-    k_emit_recv<<<dim3(recvBlocks, rows), 256, 0, s>>>(d_inst, ws, count, per);
+    k_emit_recv<<<recvBlocks * rows, 256, 0, s>>>(d_inst, ws, count, many);
     mark(ctx, s, nullptr);
     CUDA_TRY(cudaGetLastError());
     ctx->nlaunch += 6;

@@ -94,6 +94,7 @@ struct JobWS {
     int32_t nrecv, nev;
     int32_t npending, pending;   // calls over many grids: how many still need pairing (of the first
                                  // instance), the i-th of them
+    int32_t nlacking, lacking;   // how many have receiver units (of the first instance), the i-th of them
     // batching (Gamma + simulation)
     int64_t P;             // total path vertices (sum of path length + 1)
     int32_t *pairOff;      // k + 1

@@ -112,7 +112,7 @@ extern "C" int rr_plan_noalloc(const void *d_grid, int layout, int m, int n, rr_
         k_colstats<<<dim3(colBlocks, 1), 256, 0, stream>>>(d_inst, d_ws, 1, 0, 8);
         k_pair<<<1, 32, pairSmem, stream>>>(d_inst, d_ws, 1, 1);
         k_emit_cols<<<dim3(colBlocks, 1), 256, 0, stream>>>(d_inst, d_ws, 1, 8);
-        k_emit_recv<<<dim3((side * ((side + 31) / 32) + 7) / 8, 1), 256, 0, stream>>>(d_inst, d_ws, 1, 8);
+        k_emit_recv<<<(side * ((side + 31) / 32) + 7) / 8, 256, 0, stream>>>(d_inst, d_ws, 1, 0);
     }
     if (cudaGetLastError() != cudaSuccess) return RR_ERR_CUDA;
     if (cudaMemcpyAsync(&h, d_inst, sizeof(h), cudaMemcpyDeviceToHost, stream) != cudaSuccess) return RR_ERR_CUDA;

@@ -50,9 +50,24 @@ __global__ void k_colstats(rr_instance *inst, JobWS *wsv, int count, int strict,
     s_colstats(hw_blk_shared(per), inst, wsv, count, strict);
 }
 
+// Lists an instance that has receiver units, once it is paired, for
+// k_emit_recv. (It costs the pairing loop's code 1.5 %, so that calls over few
+// grids, whose time that loop is, go without.)
+__device__ __forceinline__ void list_lacking(const rr_instance *inst, JobWS *wsv, int q)
+{
+    if ((threadIdx.x & 31) == 0 && live(&inst[q]) && wsv[q].nrecv > 0)
+        wsv[atomicAdd(&wsv[0].nlacking, 1)].lacking = q;
+}
+
 __global__ void k_pair(rr_instance *inst, JobWS *wsv, int count, int warm)
 {
     s_pair(hw_blk(), inst, wsv, count, warm);
+}
+
+__global__ void k_pair_many(rr_instance *inst, JobWS *wsv, int count)
+{
+    s_pair(hw_blk(), inst, wsv, count, 0);
+    list_lacking(inst, wsv, blockIdx.x);
 }
 
 __global__ void k_pair_sift(rr_instance *inst, JobWS *wsv, int count)
@@ -67,6 +82,7 @@ __global__ void k_pair_listed(rr_instance *inst, JobWS *wsv, int count)
     for (int i = blockIdx.x; i < n; i += gridDim.x) {
         B.x = wsv[i].pending;
         s_pair(B, inst, wsv, count, 0);
+        list_lacking(inst, wsv, B.x);
         __syncwarp();
     }
 }
@@ -78,9 +94,18 @@ __global__ void k_emit_cols(rr_instance *inst, JobWS *wsv, int count, int per)
 
 // (more resident warps are worth more here than registers: 95 of them left
 // room for 16 warps per SM)
-__global__ void __launch_bounds__(256, 5) k_emit_recv(rr_instance *inst, JobWS *wsv, int count, int per)
+// The launch's warps are shared out among the instances, in calls over many
+// grids among those that have receiver units: how many these are, the host
+// cannot know (1D chains have none, and eleven idle blocks for each took 10 of
+// the 71 us of a call over 700 of them). The last to be paired come first: they
+// have the most units (2 000 grids of sides 33 to 251: 315 us with four blocks
+// each, 268 this way).
+__global__ void __launch_bounds__(256, 5) k_emit_recv(rr_instance *inst, JobWS *wsv, int count, int listed)
 {
-    s_emit_recv(hw_blk_shared(per), inst, wsv, count);
+    const int n = listed ? wsv[0].nlacking : count;
+    if (n == 0) return;
+    const int nw = (int)gridDim.x * 8 / n, g = (int)blockIdx.x * 8 + (int)(threadIdx.x >> 5), i = g / nw;
+    if (i < n) s_emit_recv(Blk{0, listed ? wsv[n - 1 - i].lacking : i, 1, g % nw, nw}, inst, wsv, count);
 }
 
 int guard_cap_plan(long long cap)

@@ -21,7 +21,7 @@ __device__ inline void s_plan_setup(const Blk B, rr_instance *inst, JobWS *wsv, 
     int m = 0, n = 0, h = 0, tw = 0;
     if (q < count) {
         I->n_moves = 0; I->n_steps = 0; I->n_ops = 0; I->n_members = 0;
-        if (q == 0) wsv[0].npending = 0;
+        if (q == 0) wsv[0].npending = wsv[0].nlacking = 0;
         m = I->m; n = I->n;
         const rr_rect R = I->rect;
         const bool bad = m < 1 || n < 1 || m > max_side || n > max_side || m > RR_MAX_SIDE || n > RR_MAX_SIDE ||

@@ -92,7 +92,6 @@ __device__ inline void s_bsetup(const Blk B, rr_instance *inst, JobWS *wsv, int 
             ws.multiMove = (int2 *)arena_alloc(A, 8ull * (k + 1), &ok);
             ws.indeg = (int32_t *)arena_alloc(A, 4ull * (k + 1), &ok);
             ws.rec = (int4 *)arena_alloc(A, 32ull * (k + 1), &ok);
-            ws.succ4 = ws.rec + 1;
             ws.ready0 = (int32_t *)arena_alloc(A, 4ull * (k + 1) + 16, &ok);
             ws.state = (int2 *)arena_alloc(A, sim_wide_bytes(k), &ok);
             ws.multi = ws.colList;               // both lists are free again once they have been swept
@@ -156,7 +155,6 @@ __device__ inline void s_bsetup(const Blk B, rr_instance *inst, JobWS *wsv, int 
             ws.multiMove = (int2 *)arena_alloc(A, 8ull * (k + 1), &ok);
             ws.indeg = (int32_t *)arena_alloc(A, 4ull * (k + 1), &ok);
             ws.rec = (int4 *)arena_alloc(A, 32ull * (k + 1), &ok);   // record, successors: one 32 B sector
-            ws.succ4 = ws.rec + 1;
             ws.ready0 = (int32_t *)arena_alloc(A, 4ull * (k + 1) + 16, &ok);
             ws.state = (int2 *)arena_alloc(A, sim_wide_bytes(k), &ok);
             ws.multi = ws.colList;               // both lists are free again once they have been swept
@@ -385,9 +383,7 @@ __device__ inline void warp_sort32(int32_t *a, int n, int32_t *buf, int cap)
 // it need not tell shared memory apart.
 template <class T> __device__ __forceinline__ T *as_global(T *p)
 {
-#ifdef __CUDA_ARCH__
     __builtin_assume(__isGlobal(p));
-#endif
     return p;
 }
 
@@ -1058,7 +1054,6 @@ __device__ __forceinline__ uint32_t min8(uint4 a, uint4 b, uint32_t w, uint32_t 
 // branched around: in one warp's serial code a branch and the point where its
 // lanes meet again cost 15 to 20 cycles each, and the code below has little
 // else between them.
-#ifdef __CUDA_ARCH__
 #define RR_IF(instr) "{ .reg .pred q; setp.ne.u32 q, %0, 0; @q " instr " }"
 __device__ __forceinline__ int sh_add_if(bool c, void *p, int v)
 {
@@ -1116,17 +1111,6 @@ __device__ __forceinline__ int ldg_if(bool c, const void *p)
     return v;
 }
 #undef RR_IF
-#else   // host-side stand-ins
-static inline int sh_add_if(bool c, void *p, int v) { int r = 0; if (c) { r = *(int *)p; *(int *)p = (int)((unsigned)r + (unsigned)v); } return r; }
-static inline int ld_u16_if(bool c, const uint16_t *p) { return c ? *p : 0; }
-static inline void st_if(bool c, uint16_t *p, int v) { if (c) *p = (uint16_t)v; }
-static inline void st_if(bool c, void *p, uint32_t v) { if (c) *(uint32_t *)p = v; }
-static inline void st_if(bool c, int2 *p, int x, int y) { if (c) *p = make_int2(x, y); }
-static inline int4 ldg_if(bool c, const int4 *p) { return c ? *p : make_int4(0, 0, 0, 0); }
-static inline int2 ldg_if(bool c, const int2 *p) { return c ? *p : make_int2(0, 0); }
-static inline int ldg_if(bool c, const void *p) { return c ? *(const int *)p : 0; }
-static inline int ldg_volatile_if(bool c, const void *p) { return c ? *(const int *)p : 0; }
-#endif
 
 __device__ __forceinline__ void touch_rec_if(bool c, const int4 *rec, int id, uint32_t dump)
 {

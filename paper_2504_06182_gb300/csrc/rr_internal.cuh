@@ -101,8 +101,7 @@ struct JobWS {
     int32_t *nextAt;       // P
     int32_t *succ;         // P: a path's successors at its vertex offset (pairOff)
     int32_t *indeg;        // k
-    int4 *rec;             // k + 1 (the last unused): see move_rec
-    int4 *succ4;           // k: first four successors (flagged, -1 padded)
+    int4 *rec;             // 2 (k + 1), the last two unused: see move_rec
     int32_t *ready0;       // k + 1: moves without predecessors; [k] = their count
     // Gamma by sweeps: moves ending in each column, L-moves starting on each row
     int32_t *colOff, *colCur, *colList;   // n + 1, n, k
@@ -228,13 +227,9 @@ __host__ __device__ constexpr unsigned long long arena_pad(unsigned long long by
 // wherever the compiler is short of a register to keep it in.
 __device__ __forceinline__ int lane_id()
 {
-#ifdef __CUDA_ARCH__
     int l;
     asm volatile("mov.u32 %0, %%laneid;" : "=r"(l));
     return l;
-#else
-    return threadIdx.x & 31;
-#endif
 }
 
 __device__ __forceinline__ int warp_incl_scan(int v)
@@ -250,15 +245,6 @@ __device__ __forceinline__ int warp_incl_scan(int v)
 
 __device__ __forceinline__ int warp_sum(int v) { return __reduce_add_sync(FULL, v); }
 
-// (two 32-bit reductions: the upper halves, then the lower ones of the lanes
-// that hold the largest upper half)
-__device__ __forceinline__ unsigned long long warp_max_u64(unsigned long long v)
-{
-    const unsigned hi = __reduce_max_sync(FULL, (unsigned)(v >> 32));
-    const unsigned lo = __reduce_max_sync(FULL, (unsigned)(v >> 32) == hi ? (unsigned)v : 0u);
-    return (unsigned long long)hi << 32 | lo;
-}
-
 // Bits of rows [lo, hi) that fall in word w (rows 32w .. 32w+31).
 __device__ __forceinline__ uint32_t row_mask(int w, int lo, int hi)
 {
@@ -270,7 +256,6 @@ __device__ __forceinline__ uint32_t row_mask(int w, int lo, int hi)
 }
 
 __device__ __forceinline__ int iabs(int v) { return v < 0 ? -v : v; }
-__device__ __forceinline__ int isgn(int v) { return (v > 0) - (v < 0); }
 
 // A move of a list in one 16-byte access where the list is aligned for it
 // (an array of rr_move need not be): four 4-byte accesses of a warp's moves
@@ -289,26 +274,10 @@ __device__ __forceinline__ void store_move(rr_move *p, int sr, int sc, int dr, i
     else *p = rr_move{sr, sc, dr, dc};
 }
 
-// Direction codes of rr_op.
-__device__ __forceinline__ int step_dir(int sr, int sc, int dr, int dc, int t)
-{
-    int hl = iabs(dc - sc);
-    if (t < hl) return dc > sc ? 3 : 2;
-    return dr > sr ? 1 : 0;
-}
-
-__device__ __forceinline__ void path_cell(int sr, int sc, int dr, int dc, int t, int *r, int *c)
-{
-    int hl = iabs(dc - sc);
-    if (t <= hl) { *r = sr; *c = sc + t * isgn(dc - sc); }
-    else { *r = sr + (t - hl) * isgn(dr - sr); *c = dc; }
-}
-
 // Bring the 32 bytes around a word into L1 without a register waiting for
 // them (lanes that c holds for): an asynchronous copy of the word to a place
 // in shared memory that nothing reads, `dump`. (prefetch.global.L1 stops at
 // L2 here: a load after it takes 300 to 500 cycles, after this copy 40.)
-#ifdef __CUDA_ARCH__
 __device__ __forceinline__ uint32_t sh_addr(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
 __device__ __forceinline__ void touch_if(bool c, const void *p, uint32_t dump)
 {
@@ -316,11 +285,6 @@ __device__ __forceinline__ void touch_if(bool c, const void *p, uint32_t dump)
                  ::"r"((unsigned)c), "r"(dump), "l"(p) : "memory");
 }
 __device__ __forceinline__ void touch_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
-#else   // host-side stand-ins
-static inline uint32_t sh_addr(const void *) { return 0; }
-static inline void touch_if(bool, const void *, uint32_t) {}
-static inline void touch_wait() {}
-#endif
 
 // Test hook: when positive, the pairing loop and the batching simulation
 // stop after this many iterations with RR_ERR_TIMEOUT, as when their own

@@ -1886,7 +1886,8 @@ struct Wide {
     uint32_t *some;           // 4 * 32: which lines across a direction's way hold any
     int m, n, side;
 
-    static __host__ __device__ size_t shared_words(int side) { return 8 * (size_t)side + 128; }
+    // (where the tables were: 14 words for each of at least max(side, 56) entries)
+    static __device__ size_t shared_words(int side) { return 8 * (size_t)side + 128; }
     __device__ __forceinline__ Wide(rr_instance *I, const JobWS &ws, char *smem, int side_)
         : map((uint32_t *)as_global(ws.firstH)), state(as_global(ws.state)), m(I->m), n(I->n), side(side_)
     {

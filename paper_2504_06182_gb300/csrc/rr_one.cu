@@ -9,8 +9,8 @@
 // same functions the separate kernels run (rr_plan.cuh, rr_bird.cuh,
 // rr_batch.cuh), given block coordinates x = 0, gx = 1 so that each
 // grid-stride loop covers all of its work with this block's warps; the
-// pairing runs on warp 0 while the other warps wait at the next barrier. In the simulation warp 0 simulates
-// and the other warps write the batches.
+// pairing runs on warp 0 while the other warps wait at the next barrier. In
+// the simulation warp 0 simulates and the other warps write the batches.
 // The descriptor comes in as a kernel parameter and the final one is written
 // to mapped host memory, so a call is one launch and one synchronisation.
 #include <algorithm>

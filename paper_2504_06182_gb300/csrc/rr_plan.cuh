@@ -80,9 +80,9 @@ __device__ inline void s_plan_setup(const Blk B, rr_instance *inst, JobWS *wsv, 
 // 4-byte load, so that a warp reads 128 contiguous bytes per row, and builds
 // its four columns' words. Other rows: lane l reads column 32g + l byte by
 // byte (32 contiguous bytes per row and warp). Grids of at most NARROW
-// columns (1D chains are one column) leave most of those lanes idle: there
-// the lanes take rows, and a vote makes a word (16 384 chains of 1 024 traps
-// in 36 us instead of 246).
+// columns leave most of those lanes idle: there the lanes take rows, and a vote
+// makes a word (16 384 chains of 1 024 traps, before chains on 16-byte
+// boundaries had a load of their own, in 36 us instead of 246).
 constexpr int NARROW = 8;
 __device__ inline void s_transpose(const Blk B, rr_instance *inst, JobWS *wsv, int count)
 {

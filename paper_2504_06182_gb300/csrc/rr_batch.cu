@@ -119,6 +119,19 @@ SIM_KERNEL(k_sim_big, SIM_BIG, false, 32, 12)
 SIM_KERNEL(k_simw, SIM_SMALL, true, SIM_MAX_THREADS, 2)
 SIM_KERNEL(k_simw_big, SIM_BIG, true, SIM_MAX_THREADS, 2)
 
+// The simulations without writers that outgrew their tables.
+__global__ void __launch_bounds__(32) k_sim_wide(rr_instance *inst, JobWS *wsv, int count, const int *classList,
+                                                 const int *classCount, int side)
+{
+    extern __shared__ int4 wide_smem[];
+    int q = blockIdx.x;
+    if (classList) {
+        if (q >= *classCount) return;
+        q = classList[q];
+    }
+    if (q < count) s_wide(&inst[q], wsv[q], (char *)wide_smem, side);
+}
+
 // The batches of simulations that ran without writers.
 __global__ void __launch_bounds__(256, 6) k_write(rr_instance *inst, JobWS *wsv, int count, const int *classList,
                                                   const int *classCount, int side)

@@ -2327,8 +2327,9 @@ static __device__ __noinline__ int wide_block(rr_instance *I, JobWS *ws, char *s
     return sim_and_write([&]() { return wide_run(I, ws, smem, side); }, I, *ws, Y, side);
 }
 
-// The whole simulation of one instance by one block (every thread calls it). A
-// block without writers is one warp; s_write writes afterwards.
+// The simulation of one instance by one block (every thread calls it). A block
+// without writers is one warp; s_wide follows for the instances that outgrew the
+// tables, s_write writes afterwards.
 template <int MODE, bool WRITERS>
 __device__ __forceinline__ void sim_block(rr_instance *I, JobWS &ws, char *smem, int side, int counters)
 {
@@ -2363,25 +2364,38 @@ __device__ __forceinline__ void sim_block(rr_instance *I, JobWS &ws, char *smem,
         st = sim_and_write([&]() { return sim_run(S, I, ws, Y); }, I, ws, Y, side);
         if (st == RR_SIM_RETRY && k >= SIM_WIDE_MIN) st = wide_block(I, &ws, smem, side);
     } else {
-        for (int pass = 0;; ++pass) {
-            ctl_begin(Y.C, pass == 0 ? cap : 0);
-            if (pass == 0) tables_begin();
-            else wide_begin(I, &ws, smem, side);
-            __syncthreads();
-            counters_begin(Y, ws, counters);
-            __syncthreads();
-            // (in a register from here on, the status costs the kernel a stack
-            // frame and 4096 mixed grids 2 % of their time)
-            const int r = pass == 0 ? sim_run(S, I, ws, Y) : wide_run(I, &ws, smem, side);
-            if (threadIdx.x == 0) Y.C->status = r;
-            __syncwarp();
-            if (threadIdx.x == 0) ws.nseg = Y.C->pub;        // s_write follows
-            __syncthreads();
-            st = Y.C->status;
-            if (st != RR_SIM_RETRY || pass == 1 || k < SIM_WIDE_MIN) break;
+        ctl_begin(Y.C, cap);
+        tables_begin();
+        counters_begin(Y, ws, counters);
+        __syncthreads();
+        st = sim_run(S, I, ws, Y);
+        if (threadIdx.x == 0) ws.nseg = Y.C->pub;        // s_write follows
+        if (st == RR_SIM_RETRY && k >= SIM_WIDE_MIN) {
+            if (threadIdx.x == 0) I->status = RR_SIM_RETRY;      // s_wide takes over
+            return;
         }
     }
     if (threadIdx.x == 0 && st != RR_OK) I->status = st == RR_SIM_RETRY ? RR_ERR_INTERNAL : st;
+}
+
+// The instances that outgrew the tables in blocks of one warp. A kernel of its
+// own, whose blocks nearly always return at once: with both forms in one kernel
+// the first one's code is slower whatever way the second is called (4096 mixed
+// grids 38.2 ms, 35.0 this way; 2 000 of sides 64 to 128 11.1 and 10.2).
+__device__ inline void s_wide(rr_instance *I, JobWS &ws, char *smem, int side)
+{
+    if (I->status != RR_SIM_RETRY) return;
+    __syncthreads();
+    const SimLayout Y(smem, side);
+    if (threadIdx.x == 0) I->status = RR_OK;
+    ctl_begin(Y.C, 0);
+    wide_begin(I, &ws, smem, side);
+    __syncthreads();
+    const int st = wide_run(I, &ws, smem, side);
+    if (threadIdx.x == 0) {
+        ws.nseg = Y.C->pub;
+        if (st != RR_OK) I->status = st == RR_SIM_RETRY ? RR_ERR_INTERNAL : st;
+    }
 }
 
 } // namespace rrk

@@ -36,6 +36,7 @@ __global__ void k_order(const rr_instance *, int, int *);
 __global__ void k_gather(const rr_instance *, const int *, rr_instance *);
 __global__ void k_scatter(rr_instance *, const int *, const rr_instance *, int);
 __global__ void k_sim(rr_instance *, JobWS *, int, const int *, const int *, int, int);
+__global__ void k_sim_wide(rr_instance *, JobWS *, int, const int *, const int *, int);
 __global__ void k_write(rr_instance *, JobWS *, int, const int *, const int *, int);
 __global__ void k_sim_big(rr_instance *, JobWS *, int, const int *, const int *, int, int);
 __global__ void k_simw(rr_instance *, JobWS *, int, const int *, const int *, int, int);
@@ -50,7 +51,7 @@ static_assert(sizeof(rr_instance) == 128, "rr_instance layout is part of the ABI
 static constexpr int SMALL_CALL = 8;
 
 // Kernels launched with more than the default 48 KB of dynamic shared memory.
-enum { SM_GSORT, SM_GSWEEP_H, SM_GSWEEP_V, SM_SIM, SM_SIM_BIG, SM_SIMW, SM_SIMW_BIG, SM_BIRD, SM_ONE, SM_NKERNEL };
+enum { SM_GSORT, SM_GSWEEP_H, SM_GSWEEP_V, SM_SIM, SM_SIM_BIG, SM_SIMW, SM_SIMW_BIG, SM_SIM_WIDE, SM_BIRD, SM_ONE, SM_NKERNEL };
 
 struct rr_ctx {
     int device;
@@ -147,7 +148,8 @@ static int smem_limits(int dev, int *out)
         cudaError_t e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
         const void *fn[SM_NKERNEL] = {(const void *)k_gsort, (const void *)k_gsweep_h, (const void *)k_gsweep_v,
                                       (const void *)k_sim, (const void *)k_sim_big, (const void *)k_simw,
-                                      (const void *)k_simw_big, (const void *)k_bird, one_kernel()};
+                                      (const void *)k_simw_big, (const void *)k_sim_wide, (const void *)k_bird,
+                                      one_kernel()};
         for (int i = 0; e == cudaSuccess && i < SM_NKERNEL; ++i) {
             cudaFuncAttributes fa;
             e = cudaFuncGetAttributes(&fa, fn[i]);
@@ -493,9 +495,10 @@ static int launch_batch(rr_ctx *ctx, rr_instance *d_inst, JobWS *ws, int count, 
         const int *cnt = one ? nullptr : ctx->d_classCount + c;
         sh.kernel<<<count, 32 * sh.warps, sh.smem, cs>>>(d_inst, ws, count, list, cnt, side, sh.counters);
         if (sh.warps == 1) {
+            k_sim_wide<<<count, 32, sim_smem_bytes(side, 1, 0), cs>>>(d_inst, ws, count, list, cnt, side);
             const int wb = clampi(std::max(1, budget(ctx, 16384) / count), 1, 64);
             k_write<<<dim3(wb, count), 256, 8 * 4 * (size_t)sim_pow2(side), cs>>>(d_inst, ws, count, list, cnt, side);
-            ctx->nlaunch += 1;
+            ctx->nlaunch += 2;
         }
         if (!one) {
             CUDA_TRY(cudaEventRecord(ctx->evJoin[c], cs));

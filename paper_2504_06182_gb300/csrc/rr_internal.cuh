@@ -180,8 +180,8 @@ constexpr int SIM_WIDE_MIN = 65;
 __host__ __device__ inline size_t sim_wide_bytes(long long k) { return k < SIM_WIDE_MIN ? 0 : 8 * (size_t)k; }
 
 // End of the narrow simulation when an instance needs more table entries
-// than shared memory holds: the wide one starts over in the same block, so
-// callers never see it.
+// than shared memory holds: the wide one starts over, in the same block or in
+// the kernel that follows (k_sim_wide), so callers never see it.
 constexpr int32_t RR_SIM_RETRY = 100;
 
 // A move's record (two int4): the position word of its source; its first
